@@ -271,6 +271,23 @@ ptq_status_t ptq_calibrate(int K, int N, int T, const void *xcal_fp16, int Bc,
                            float *smooth_out, float *act_step_out, void *stream);
 
 /*
+ * The four calibrations (ptq_calibrate, ptq_calibrate_per_tensor, ptq_calibrate_asym, ptq_calibrate_w4a4) in a device
+ * workspace of the caller, which a program that calibrates layer after layer keeps: nothing is allocated.  Same
+ * arguments, results and errors.
+ *   scheme        PTQ_CALIB_PTS .. PTQ_CALIB_W4A4; w_q is [N,K] int8, or [N, (K+1)/2] packed bytes for W4A4
+ *   act_zero_out  host, [T] int32, asymmetric only (else NULL)
+ *   workspace     device, 256-byte aligned, at least ptq_calibrate_workspace_bytes(K, N, T) bytes (0: out of range)
+ */
+#define PTQ_CALIB_PTS        0
+#define PTQ_CALIB_PER_TENSOR 1
+#define PTQ_CALIB_ASYM       2
+#define PTQ_CALIB_W4A4       3
+size_t ptq_calibrate_workspace_bytes(int K, int N, int T);
+ptq_status_t ptq_calibrate_in(int scheme, int K, int N, int T, const void *xcal_fp16, int Bc, const void *w_q,
+                              const float *w_step, float *smooth_out, float *act_step_out, int32_t *act_zero_out,
+                              void *workspace, size_t workspace_bytes, void *stream);
+
+/*
  * Comparator: per-TENSOR static quantization (the coarsest granularity of the latency table of Sec. 6
  * and of Fig. 5: one step for the whole activation tensor).  Same s[k] as ptq_calibrate, and
  *   step = max( max_{b,t,k} |xcal[b,t,k] / s[k]|, 1e-5 ) / 127
@@ -337,6 +354,12 @@ ptq_status_t ptq_quantize_packed4(const ptq_linear_t *h, const void *x_fp16, int
 ptq_status_t ptq_search_act_step(int K, int T, const void *xcal_fp16, int Bc, const float *smooth,
                                  const float *base_step, int n_grid, int j_lo, float *act_step_out,
                                  int32_t *best_out, double *loss_out, void *stream);
+/* The same in a device workspace of the caller (256-byte aligned); nothing is allocated on the device. */
+size_t ptq_search_workspace_bytes(int K, int T, int n_grid, int j_lo);
+ptq_status_t ptq_search_act_step_in(int K, int T, const void *xcal_fp16, int Bc, const float *smooth,
+                                    const float *base_step, int n_grid, int j_lo, float *act_step_out,
+                                    int32_t *best_out, double *loss_out, void *workspace, size_t workspace_bytes,
+                                    void *stream);
 
 /*
  * Q0 for asymmetric layers: s[k] as in ptq_calibrate; per token position the range [lo, hi] of x/s over

@@ -54,8 +54,6 @@ def load_library() -> ctypes.CDLL:
     L.ptq_linear_create.argtypes = [ctypes.POINTER(vp), ci, ci, ci, vp, vp, vp, vp, vp, cu]
     L.ptq_linear_create_asym.restype = ci
     L.ptq_linear_create_asym.argtypes = [ctypes.POINTER(vp), ci, ci, ci, vp, vp, vp, vp, vp, vp, cu]
-    L.ptq_calibrate_asym.restype = ci
-    L.ptq_calibrate_asym.argtypes = [ci, ci, ci, vp, ci, vp, vp, vp, vp, vp, vp]
     L.ptq_linear_destroy.restype = None
     L.ptq_linear_destroy.argtypes = [vp]
     L.ptq_linear_workspace_bytes.restype = sz
@@ -86,18 +84,20 @@ def load_library() -> ctypes.CDLL:
     L.ptq_linear_forward_debug.argtypes = [vp, vp, ci, vp, vp, vp, vp, sz, cu, vp]
     L.ptq_calibrate.restype = ci
     L.ptq_calibrate.argtypes = [ci, ci, ci, vp, ci, vp, vp, vp, vp, vp]
+    L.ptq_calibrate_workspace_bytes.restype = sz
+    L.ptq_calibrate_workspace_bytes.argtypes = [ci, ci, ci]
+    L.ptq_calibrate_in.restype = ci
+    L.ptq_calibrate_in.argtypes = [ci, ci, ci, ci, vp, ci, vp, vp, vp, vp, vp, vp, sz, vp]
+    L.ptq_search_workspace_bytes.restype = sz
+    L.ptq_search_workspace_bytes.argtypes = [ci, ci, ci, ci]
+    L.ptq_search_act_step_in.restype = ci
+    L.ptq_search_act_step_in.argtypes = [ci, ci, vp, ci, vp, vp, ci, ci, vp, vp, vp, vp, sz, vp]
     L.ptq_linear_create_w4a4.restype = ci
     L.ptq_linear_create_w4a4.argtypes = [ctypes.POINTER(vp), ci, ci, ci, vp, vp, vp, vp, vp, cu]
     L.ptq_linear_selftest_wait_timeout.restype = ci
     L.ptq_linear_selftest_wait_timeout.argtypes = [vp, ctypes.c_uint, vp, vp]
-    L.ptq_calibrate_per_tensor.restype = ci
-    L.ptq_calibrate_per_tensor.argtypes = [ci, ci, ci, vp, ci, vp, vp, vp, vp, vp]
-    L.ptq_calibrate_w4a4.restype = ci
-    L.ptq_calibrate_w4a4.argtypes = [ci, ci, ci, vp, ci, vp, vp, vp, vp, vp]
     L.ptq_quantize_packed4.restype = ci
     L.ptq_quantize_packed4.argtypes = [vp, vp, ci, vp, vp, sz, vp]
-    L.ptq_search_act_step.restype = ci
-    L.ptq_search_act_step.argtypes = [ci, ci, vp, ci, vp, vp, ci, ci, vp, vp, vp, vp]
     L.ptq_linear_describe.restype = ci
     L.ptq_linear_describe.argtypes = [vp, ctypes.c_char_p, ci]
     L.ptq_linear_device_status.restype = ci
@@ -363,78 +363,65 @@ class PtqLinear:
         return y, q, acc
 
 
-def calibrate(xcal, w_q, w_step, stream=None, per_tensor: bool = False):
-    """``ptq_calibrate``: device fp16 [Bc,T,K] -> (s fp32 [K], dx fp32 [T]) as numpy arrays.
-    ``per_tensor=True`` calls ``ptq_calibrate_per_tensor`` (one step, repeated T times)."""
+def _xcal(xcal, K=None):
     import torch
-    L = load_library()
-    if xcal.dtype != torch.float16 or not xcal.is_cuda or not xcal.is_contiguous() or xcal.dim() != 3:
+    if xcal.dtype != torch.float16 or not xcal.is_cuda or not xcal.is_contiguous() or xcal.dim() != 3 or (
+            K is not None and xcal.shape[2] != K):
         raise ValueError("xcal must be a contiguous CUDA float16 tensor [Bc,T,K]")
-    Bc, T, K = (int(v) for v in xcal.shape)
-    w_q = _host(w_q, np.int8)
-    N = int(w_q.shape[0])
-    if w_q.shape != (N, K):
+    return tuple(int(v) for v in xcal.shape)
+
+
+CALIB_PTS, CALIB_PER_TENSOR, CALIB_ASYM, CALIB_W4A4 = 0, 1, 2, 3
+
+
+def _calibrate(scheme, xcal, w, w_step, stream, packed_K=None):
+    """``ptq_calibrate_in`` in a workspace from torch's caching allocator (a device allocation per call costs more than
+    the calibration)."""
+    L = load_library()
+    Bc, T, K = _xcal(xcal, packed_K)
+    w = _host(w, np.uint8 if scheme == CALIB_W4A4 else np.int8)
+    N = int(w.shape[0])
+    if scheme == CALIB_W4A4:
+        if w.shape != (N, (K + 1) // 2):
+            raise ValueError("packed w_q must be [N, (K+1)//2] bytes")
+    elif w.shape != (N, K):
         raise ValueError("w_q must be [N,K]")
     w_step = _host(w_step, np.float32, (N,))
     s = np.empty(K, np.float32)
     dx = np.empty(T, np.float32)
-    fn = L.ptq_calibrate_per_tensor if per_tensor else L.ptq_calibrate
-    _check(fn(K, N, T, xcal.data_ptr(), Bc, _hp(w_q), _hp(w_step), _hp(s), _hp(dx), _stream_ptr(stream)))
-    return s, dx
+    z = np.empty(T, np.int32) if scheme == CALIB_ASYM else None
+    ws = _scratch(L.ptq_calibrate_workspace_bytes(K, N, T), xcal.device, stream)
+    _check(L.ptq_calibrate_in(scheme, K, N, T, xcal.data_ptr(), Bc, _hp(w), _hp(w_step), _hp(s), _hp(dx), _hp(z),
+                              ws.data_ptr(), ws.numel(), _stream_ptr(stream)))
+    return (s, dx) if z is None else (s, dx, z)
+
+
+def calibrate(xcal, w_q, w_step, stream=None, per_tensor: bool = False):
+    """``ptq_calibrate``: device fp16 [Bc,T,K] -> (s fp32 [K], dx fp32 [T]) as numpy arrays.
+    ``per_tensor=True``: ``ptq_calibrate_per_tensor`` (one step, repeated T times)."""
+    return _calibrate(CALIB_PER_TENSOR if per_tensor else CALIB_PTS, xcal, w_q, w_step, stream)
 
 
 def calibrate_asym(xcal, w_q, w_step, stream=None):
     """``ptq_calibrate_asym``: device fp16 [Bc,T,K] -> (s fp32 [K], dx fp32 [T], z int32 [T])."""
-    import torch
-    L = load_library()
-    if xcal.dtype != torch.float16 or not xcal.is_cuda or not xcal.is_contiguous() or xcal.dim() != 3:
-        raise ValueError("xcal must be a contiguous CUDA float16 tensor [Bc,T,K]")
-    Bc, T, K = (int(v) for v in xcal.shape)
-    w_q = _host(w_q, np.int8)
-    N = int(w_q.shape[0])
-    if w_q.shape != (N, K):
-        raise ValueError("w_q must be [N,K]")
-    w_step = _host(w_step, np.float32, (N,))
-    s = np.empty(K, np.float32)
-    dx = np.empty(T, np.float32)
-    z = np.empty(T, np.int32)
-    _check(L.ptq_calibrate_asym(K, N, T, xcal.data_ptr(), Bc, _hp(w_q), _hp(w_step), _hp(s), _hp(dx), _hp(z),
-                                _stream_ptr(stream)))
-    return s, dx, z
+    return _calibrate(CALIB_ASYM, xcal, w_q, w_step, stream)
 
 
 def search_act_step(xcal, smooth, base_step, n_grid: int = 100, j_lo: int = 20, want_loss: bool = False, stream=None):
     """``ptq_search_act_step``: device fp16 [Bc,T,K] -> (dx fp32 [T], best j int32 [T], loss fp64 [T,C] or None)."""
-    import torch
     L = load_library()
-    if xcal.dtype != torch.float16 or not xcal.is_cuda or not xcal.is_contiguous() or xcal.dim() != 3:
-        raise ValueError("xcal must be a contiguous CUDA float16 tensor [Bc,T,K]")
-    Bc, T, K = (int(v) for v in xcal.shape)
+    Bc, T, K = _xcal(xcal)
     smooth = _host(smooth, np.float32, (K,))
     base_step = _host(base_step, np.float32, (T,))
     dx = np.empty(T, np.float32)
     best = np.empty(T, np.int32)
     loss = np.empty((T, max(n_grid - j_lo + 1, 1)), np.float64) if want_loss else None
-    _check(L.ptq_search_act_step(K, T, xcal.data_ptr(), Bc, smooth.ctypes.data, base_step.ctypes.data, n_grid, j_lo,
-                                 dx.ctypes.data, best.ctypes.data,
-                                 loss.ctypes.data if loss is not None else None, _stream_ptr(stream)))
+    ws = _scratch(L.ptq_search_workspace_bytes(K, T, n_grid, j_lo), xcal.device, stream)
+    _check(L.ptq_search_act_step_in(K, T, xcal.data_ptr(), Bc, _hp(smooth), _hp(base_step), n_grid, j_lo, _hp(dx),
+                                    _hp(best), _hp(loss), ws.data_ptr(), ws.numel(), _stream_ptr(stream)))
     return dx, best, loss
 
 
 def calibrate_w4a4(xcal, w_q_packed, K: int, w_step, stream=None):
     """``ptq_calibrate_w4a4``: device fp16 [Bc,T,K], packed 4-bit weights -> (s fp32 [K], dx fp32 [T] = max|x/s|/7)."""
-    import torch
-    L = load_library()
-    if xcal.dtype != torch.float16 or not xcal.is_cuda or not xcal.is_contiguous() or xcal.dim() != 3 or xcal.shape[2] != K:
-        raise ValueError("xcal must be a contiguous CUDA float16 tensor [Bc,T,K]")
-    Bc, T = int(xcal.shape[0]), int(xcal.shape[1])
-    w_q_packed = _host(w_q_packed, np.uint8)
-    N = int(w_q_packed.shape[0])
-    if w_q_packed.shape != (N, (K + 1) // 2):
-        raise ValueError("packed w_q must be [N, (K+1)//2] bytes")
-    w_step = _host(w_step, np.float32, (N,))
-    s = np.empty(K, np.float32)
-    dx = np.empty(T, np.float32)
-    _check(L.ptq_calibrate_w4a4(K, N, T, xcal.data_ptr(), Bc, w_q_packed.ctypes.data, w_step.ctypes.data,
-                                s.ctypes.data, dx.ctypes.data, _stream_ptr(stream)))
-    return s, dx
+    return _calibrate(CALIB_W4A4, xcal, w_q_packed, w_step, stream, packed_K=int(K))

@@ -673,6 +673,22 @@ ptq_status_t static_scratch_address(int device, void **out)
     return PTQ_OK;
 }
 
+template <int kVec>
+void launch_calib_rowrange(bool asym, const __half *x, int Bc, int K, int T, int sms, const float *s, unsigned *hi,
+                           unsigned *nlo, cudaStream_t stream)
+{
+    // two blocks per SM where there are few positions, but at least eight images per block
+    int splits = (2 * sms + T - 1) / T;
+    const int most = (Bc + 7) / 8;
+    if (splits > most) splits = most;
+    const int per = (Bc + splits - 1) / splits;
+    const dim3 grid(static_cast<unsigned>(T), static_cast<unsigned>((Bc + per - 1) / per));
+    if (asym)
+        ptq::ptq_calib_rowrange_kernel<kVec, true><<<grid, 128, 0, stream>>>(x, Bc, per, K, T, s, hi, nlo);
+    else
+        ptq::ptq_calib_rowrange_kernel<kVec, false><<<grid, 128, 0, stream>>>(x, Bc, per, K, T, s, hi, nlo);
+}
+
 ptq_status_t validate_forward(const ptq_linear *h, const void *x, int B, const void *y)
 {
     if (!h || !x || !y) return fail(PTQ_ERR_NULL, "handle, x and y must not be NULL");
@@ -1007,9 +1023,30 @@ ptq_status_t ptq_linear_forward_static(const ptq_linear_t *h, const void *x_fp16
     return launch_gemm(h, scratch, M, y_fp16, nullptr, s);
 }
 
-ptq_status_t ptq_search_act_step(int K, int T, const void *xcal_fp16, int Bc, const float *smooth,
-                                 const float *base_step, int n_grid, int j_lo, float *act_step_out,
-                                 int32_t *best_out, double *loss_out, void *stream)
+// Device workspace of the step search: [K] s, [T] base, then [T] dx, [T] best, then the losses [T, C].
+struct SearchLayout {
+    size_t in, out, loss, total;
+};
+static SearchLayout search_layout(int K, int T, int C)
+{
+    auto up = [](size_t v) { return (v + 255) / 256 * 256; };
+    SearchLayout l;
+    l.in = 0;
+    l.out = up(sizeof(float) * (static_cast<size_t>(K) + static_cast<size_t>(T)));
+    l.loss = l.out + up(2 * sizeof(float) * static_cast<size_t>(T));
+    l.total = l.loss + up(sizeof(double) * static_cast<size_t>(T) * C);
+    return l;
+}
+
+size_t ptq_search_workspace_bytes(int K, int T, int n_grid, int j_lo)
+{
+    if (K < 1 || K > PTQ_MAX_K || T < 1 || T > PTQ_MAX_T || n_grid < 1 || n_grid > PTQ_MAX_SEARCH_GRID || j_lo < 1 || j_lo > n_grid)
+        return 0;
+    return search_layout(K, T, n_grid - j_lo + 1).total;
+}
+
+static ptq_status_t search_check(int K, int T, const void *xcal_fp16, int Bc, const float *smooth, const float *base_step,
+                                 int n_grid, int j_lo, const float *act_step_out)
 {
     if (!xcal_fp16 || !smooth || !base_step || !act_step_out)
         return fail(PTQ_ERR_NULL, "search: pointers must not be NULL");
@@ -1026,43 +1063,68 @@ ptq_status_t ptq_search_act_step(int K, int T, const void *xcal_fp16, int Bc, co
     for (int t = 0; t < T; ++t)
         if (!(base_step[t] >= 1e-30f) || !std::isfinite(base_step[t]))
             return fail(PTQ_ERR_VALUE, "search: base_step[%d] = %g is not in [1e-30, inf)", t, base_step[t]);
-    cudaStream_t s = static_cast<cudaStream_t>(stream);
+    return PTQ_OK;
+}
+
+ptq_status_t ptq_search_act_step_in(int K, int T, const void *xcal_fp16, int Bc, const float *smooth,
+                                    const float *base_step, int n_grid, int j_lo, float *act_step_out,
+                                    int32_t *best_out, double *loss_out, void *workspace, size_t workspace_bytes,
+                                    void *stream)
+{
+    const ptq_status_t st = search_check(K, T, xcal_fp16, Bc, smooth, base_step, n_grid, j_lo, act_step_out);
+    if (st != PTQ_OK) return st;
     const int C = n_grid - j_lo + 1;
-    float *d_f = nullptr;      // [K] s, [T] base, [T] dx
-    int *d_best = nullptr;     // [T]
-    double *d_loss = nullptr;  // [T, C]
-    auto body = [&]() -> ptq_status_t {
-        PTQ_CUDA(cudaMalloc(reinterpret_cast<void **>(&d_f), sizeof(float) * (K + 2 * static_cast<size_t>(T))));
-        PTQ_CUDA(cudaMalloc(reinterpret_cast<void **>(&d_best), sizeof(int) * static_cast<size_t>(T)));
-        PTQ_CUDA(cudaMalloc(reinterpret_cast<void **>(&d_loss), sizeof(double) * static_cast<size_t>(T) * C));
-        PTQ_CUDA(cudaMemcpyAsync(d_f, smooth, sizeof(float) * K, cudaMemcpyHostToDevice, s));
-        PTQ_CUDA(cudaMemcpyAsync(d_f + K, base_step, sizeof(float) * T, cudaMemcpyHostToDevice, s));
-        ptq::SearchParams p;
-        p.x = static_cast<const __half *>(xcal_fp16);
-        p.s = d_f;
-        p.base = d_f + K;
-        p.loss = d_loss;
-        p.Bc = Bc;
-        p.T = T;
-        p.K = K;
-        p.n_grid = n_grid;
-        p.j_lo = j_lo;
-        const dim3 grid(static_cast<unsigned>(T), static_cast<unsigned>((C + ptq::kSearchCandPerBlock - 1) / ptq::kSearchCandPerBlock));
-        ptq::ptq_search_loss_kernel<<<grid, ptq::kSearchThreads, 0, s>>>(p);
-        ptq::ptq_search_pick_kernel<<<(T + 127) / 128, 128, 0, s>>>(d_loss, d_f + K, T, n_grid, j_lo, d_best, d_f + K + T);
-        g_launches.fetch_add(2, std::memory_order_relaxed);
-        PTQ_CUDA(cudaGetLastError());
-        PTQ_CUDA(cudaMemcpyAsync(act_step_out, d_f + K + T, sizeof(float) * T, cudaMemcpyDeviceToHost, s));
-        if (best_out) PTQ_CUDA(cudaMemcpyAsync(best_out, d_best, sizeof(int) * T, cudaMemcpyDeviceToHost, s));
-        if (loss_out)
-            PTQ_CUDA(cudaMemcpyAsync(loss_out, d_loss, sizeof(double) * static_cast<size_t>(T) * C, cudaMemcpyDeviceToHost, s));
-        PTQ_CUDA(cudaStreamSynchronize(s));
-        return PTQ_OK;
-    };
-    const ptq_status_t st = body();
-    cudaFree(d_f);
-    cudaFree(d_best);
-    cudaFree(d_loss);
+    const SearchLayout l = search_layout(K, T, C);
+    if (!workspace) return fail(PTQ_ERR_NULL, "search: workspace must not be NULL");
+    if (workspace_bytes < l.total)
+        return fail(PTQ_ERR_SHAPE, "search: workspace has %zu bytes, %zu needed", workspace_bytes, l.total);
+    if (reinterpret_cast<uintptr_t>(workspace) % 256) return fail(PTQ_ERR_ALIGN, "search: workspace must be 256-byte aligned");
+    cudaStream_t s = static_cast<cudaStream_t>(stream);
+    unsigned char *base = static_cast<unsigned char *>(workspace);
+    float *d_s = reinterpret_cast<float *>(base + l.in), *d_base = d_s + K;
+    float *d_dx = reinterpret_cast<float *>(base + l.out);
+    int *d_best = reinterpret_cast<int *>(d_dx + T);
+    double *d_loss = reinterpret_cast<double *>(base + l.loss);
+    std::vector<float> in(static_cast<size_t>(K) + T), out(2 * static_cast<size_t>(T));   // one copy each way
+    std::memcpy(in.data(), smooth, sizeof(float) * K);
+    std::memcpy(in.data() + K, base_step, sizeof(float) * T);
+    PTQ_CUDA(cudaMemcpyAsync(d_s, in.data(), sizeof(float) * in.size(), cudaMemcpyHostToDevice, s));
+    ptq::SearchParams p;
+    p.x = static_cast<const __half *>(xcal_fp16);
+    p.s = d_s;
+    p.base = d_base;
+    p.loss = d_loss;
+    p.Bc = Bc;
+    p.T = T;
+    p.K = K;
+    p.n_grid = n_grid;
+    p.j_lo = j_lo;
+    const dim3 grid(static_cast<unsigned>(T), static_cast<unsigned>((C + ptq::kSearchCandPerBlock - 1) / ptq::kSearchCandPerBlock));
+    ptq::ptq_search_loss_kernel<<<grid, ptq::kSearchThreads, 0, s>>>(p);
+    ptq::ptq_search_pick_kernel<<<(T + 127) / 128, 128, 0, s>>>(d_loss, d_base, T, n_grid, j_lo, d_best, d_dx);
+    g_launches.fetch_add(2, std::memory_order_relaxed);
+    PTQ_CUDA(cudaGetLastError());
+    PTQ_CUDA(cudaMemcpyAsync(out.data(), d_dx, sizeof(float) * out.size(), cudaMemcpyDeviceToHost, s));
+    if (loss_out)
+        PTQ_CUDA(cudaMemcpyAsync(loss_out, d_loss, sizeof(double) * static_cast<size_t>(T) * C, cudaMemcpyDeviceToHost, s));
+    PTQ_CUDA(cudaStreamSynchronize(s));
+    std::memcpy(act_step_out, out.data(), sizeof(float) * T);
+    if (best_out) std::memcpy(best_out, out.data() + T, sizeof(int32_t) * T);
+    return PTQ_OK;
+}
+
+ptq_status_t ptq_search_act_step(int K, int T, const void *xcal_fp16, int Bc, const float *smooth,
+                                 const float *base_step, int n_grid, int j_lo, float *act_step_out,
+                                 int32_t *best_out, double *loss_out, void *stream)
+{
+    ptq_status_t st = search_check(K, T, xcal_fp16, Bc, smooth, base_step, n_grid, j_lo, act_step_out);
+    if (st != PTQ_OK) return st;
+    const size_t bytes = ptq_search_workspace_bytes(K, T, n_grid, j_lo);
+    void *ws = nullptr;
+    PTQ_CUDA(cudaMalloc(&ws, bytes));
+    st = ptq_search_act_step_in(K, T, xcal_fp16, Bc, smooth, base_step, n_grid, j_lo, act_step_out, best_out, loss_out, ws,
+                                bytes, stream);
+    cudaFree(ws);
     return st;
 }
 
@@ -1251,91 +1313,148 @@ ptq_status_t ptq_probe(int kind, void *buf, size_t bytes, int iters, double *res
     return PTQ_OK;
 }
 
-static ptq_status_t calibrate_impl(int K, int N, int T, const void *xcal_fp16, int Bc, const int8_t *w_q,
-                                   const float *w_step, float *smooth_out, float *act_step_out,
-                                   int32_t *act_zero_out, void *stream, float qmax = 127.0f,
-                                   bool per_tensor = false)
+// Device workspace of a calibration: accumulators (zeroed per call), results, weight steps, weights.
+struct CalibLayout {
+    size_t bits, out, dw, w, total;     // byte offsets and size
+};
+static CalibLayout calib_layout(int K, int N, int T)
 {
-    if (!xcal_fp16 || !w_q || !w_step || !smooth_out || !act_step_out)
+    auto up = [](size_t v) { return (v + 255) / 256 * 256; };
+    CalibLayout l;
+    l.bits = 0;                                                                  // [K] maxX, [T] mu (or hi), [T] -lo, [K] maxW
+    l.out = up(sizeof(unsigned) * (2 * static_cast<size_t>(K) + 2 * static_cast<size_t>(T)));   // [K] s, [T] dx, [T] z
+    l.dw = l.out + up(sizeof(float) * (static_cast<size_t>(K) + 2 * static_cast<size_t>(T)));
+    l.w = l.dw + up(sizeof(float) * static_cast<size_t>(N));
+    l.total = l.w + up(static_cast<size_t>(N) * K);
+    return l;
+}
+
+size_t ptq_calibrate_workspace_bytes(int K, int N, int T)
+{
+    if (K < 1 || K > PTQ_MAX_K || N < 1 || N > PTQ_MAX_N || T < 1 || T > PTQ_MAX_T) return 0;
+    return calib_layout(K, N, T).total;
+}
+
+ptq_status_t ptq_calibrate_in(int scheme, int K, int N, int T, const void *xcal_fp16, int Bc, const void *w_q,
+                              const float *w_step, float *smooth_out, float *act_step_out, int32_t *act_zero_out,
+                              void *workspace, size_t workspace_bytes, void *stream)
+{
+    const bool asym = scheme == PTQ_CALIB_ASYM, packed = scheme == PTQ_CALIB_W4A4;
+    if (scheme < PTQ_CALIB_PTS || scheme > PTQ_CALIB_W4A4) return fail(PTQ_ERR_VALUE, "calibrate: unknown scheme %d", scheme);
+    if (!xcal_fp16 || !w_q || !w_step || !smooth_out || !act_step_out || (asym && !act_zero_out) || !workspace)
         return fail(PTQ_ERR_NULL, "calibrate: pointers must not be NULL");
     if (K < 1 || K > PTQ_MAX_K || N < 1 || N > PTQ_MAX_N || T < 1 || T > PTQ_MAX_T || Bc < 1)
         return fail(PTQ_ERR_SHAPE, "calibrate: dimensions out of range (K=%d N=%d T=%d Bc=%d)", K, N, T, Bc);
     if (reinterpret_cast<uintptr_t>(xcal_fp16) % 2) return fail(PTQ_ERR_ALIGN, "xcal must be 2-byte aligned");
+    const CalibLayout l = calib_layout(K, N, T);
+    if (workspace_bytes < l.total)
+        return fail(PTQ_ERR_SHAPE, "calibrate: workspace has %zu bytes, %zu needed", workspace_bytes, l.total);
+    if (reinterpret_cast<uintptr_t>(workspace) % 256) return fail(PTQ_ERR_ALIGN, "calibrate: workspace must be 256-byte aligned");
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     int dev = -1, sms = 0;
     PTQ_CUDA(cudaGetDevice(&dev));
     PTQ_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     const long long M = static_cast<long long>(Bc) * T;
+    const __half *x = static_cast<const __half *>(xcal_fp16);
+    unsigned char *base = static_cast<unsigned char *>(workspace);
+    unsigned *d_xbits = reinterpret_cast<unsigned *>(base + l.bits), *d_hi = d_xbits + K, *d_nlo = d_hi + T, *d_wbits = d_nlo + T;
+    float *d_s = reinterpret_cast<float *>(base + l.out), *d_dx = d_s + K;
+    int *d_z = reinterpret_cast<int *>(d_dx + T);
+    float *d_dw = reinterpret_cast<float *>(base + l.dw);
+    uint8_t *d_w = base + l.w;
+    const int row_bytes = packed ? (K + 1) / 2 : K;
 
-    unsigned *d_bits = nullptr;   // [K] maxX bits, then [T] mu (or hi) bits, then [T] -lo bits, then [K] maxW bits
-    float *d_out = nullptr;       // [K] s, then [T] dx, then [T] z (int)
-    float *d_dw = nullptr;
-    int8_t *d_w = nullptr;
-    ptq_status_t st = PTQ_OK;
-    auto body = [&]() -> ptq_status_t {
-        PTQ_CUDA(cudaMalloc(reinterpret_cast<void **>(&d_bits), sizeof(unsigned) * (2 * K + 2 * T)));
-        PTQ_CUDA(cudaMalloc(reinterpret_cast<void **>(&d_out), sizeof(float) * (K + 2 * T)));
-        PTQ_CUDA(cudaMalloc(reinterpret_cast<void **>(&d_dw), sizeof(float) * N));
-        PTQ_CUDA(cudaMalloc(reinterpret_cast<void **>(&d_w), static_cast<size_t>(N) * K));
-        PTQ_CUDA(cudaMemsetAsync(d_bits, 0, sizeof(unsigned) * (2 * K + 2 * T), s));
-        PTQ_CUDA(cudaMemcpyAsync(d_dw, w_step, sizeof(float) * N, cudaMemcpyHostToDevice, s));
-        PTQ_CUDA(cudaMemcpyAsync(d_w, w_q, static_cast<size_t>(N) * K, cudaMemcpyHostToDevice, s));
-        const __half *x = static_cast<const __half *>(xcal_fp16);
-        long long want = (M + 7) / 8;
-        if (want > sms * 8ll) want = sms * 8ll;
-        const int grid = static_cast<int>(want < 1 ? 1 : want);
-        ptq::ptq_calib_colmax_kernel<<<grid, 256, 0, s>>>(x, M, K, d_bits);
-        unsigned *d_wbits = d_bits + K + 2 * T;
-        const dim3 wgrid(static_cast<unsigned>((K + 127) / 128),
-                         static_cast<unsigned>((N + ptq::kCalibRowsPerBlock - 1) / ptq::kCalibRowsPerBlock));
-        ptq::ptq_calib_wmax_kernel<<<wgrid, 128, 0, s>>>(d_w, d_dw, N, K, d_wbits);
-        ptq::ptq_calib_smooth_kernel<<<(K + 127) / 128, 128, 0, s>>>(d_bits, d_wbits, K, d_out);
-        if (act_zero_out) {
-            ptq::ptq_calib_rowrange_kernel<<<grid, 256, 0, s>>>(x, M, K, T, d_out, d_bits + K, d_bits + K + T);
-            ptq::ptq_calib_step_asym_kernel<<<(T + 127) / 128, 128, 0, s>>>(d_bits + K, d_bits + K + T, T, d_out + K,
-                                                                           reinterpret_cast<int *>(d_out + K + T));
-        } else {
-            ptq::ptq_calib_rowmax_kernel<<<grid, 256, 0, s>>>(x, M, K, T, d_out, d_bits + K);
-            if (per_tensor)
-                ptq::ptq_calib_step_tensor_kernel<<<1, 256, 0, s>>>(d_bits + K, T, d_out + K, qmax);
-            else
-                ptq::ptq_calib_step_kernel<<<(T + 127) / 128, 128, 0, s>>>(d_bits + K, T, d_out + K, qmax);
-        }
-        g_launches.fetch_add(5, std::memory_order_relaxed);
-        PTQ_CUDA(cudaGetLastError());
-        PTQ_CUDA(cudaMemcpyAsync(smooth_out, d_out, sizeof(float) * K, cudaMemcpyDeviceToHost, s));
-        PTQ_CUDA(cudaMemcpyAsync(act_step_out, d_out + K, sizeof(float) * T, cudaMemcpyDeviceToHost, s));
-        if (act_zero_out)
-            PTQ_CUDA(cudaMemcpyAsync(act_zero_out, d_out + K + T, sizeof(int32_t) * T, cudaMemcpyDeviceToHost, s));
-        PTQ_CUDA(cudaStreamSynchronize(s));
-        return PTQ_OK;
-    };
-    st = body();
-    cudaFree(d_bits);
-    cudaFree(d_out);
-    cudaFree(d_dw);
-    cudaFree(d_w);
+    // The activations' column maxima first: they run while the weights are on their way from the host.
+    PTQ_CUDA(cudaMemsetAsync(d_xbits, 0, sizeof(unsigned) * (2 * static_cast<size_t>(K) + 2 * static_cast<size_t>(T)), s));
+    const bool vec = K % 8 == 0 && reinterpret_cast<uintptr_t>(x) % 16 == 0;
+    const int cpr = vec ? K / 8 : K;
+    const long long rp = 256 / (cpr < 256 ? cpr : 256);
+    long long rpb = (M + 2 * sms - 1) / (2 * sms);
+    if (rpb < 4 * rp) rpb = 4 * rp;
+    const int cgrid = static_cast<int>((M + rpb - 1) / rpb);
+    if (vec)
+        ptq::ptq_calib_colmax_kernel<8><<<cgrid, 256, 0, s>>>(x, M, K, static_cast<int>(rpb), d_xbits);
+    else
+        ptq::ptq_calib_colmax_kernel<1><<<cgrid, 256, 0, s>>>(x, M, K, static_cast<int>(rpb), d_xbits);
+    PTQ_CUDA(cudaMemcpyAsync(d_dw, w_step, sizeof(float) * N, cudaMemcpyHostToDevice, s));
+    PTQ_CUDA(cudaMemcpyAsync(d_w, w_q, static_cast<size_t>(N) * row_bytes, cudaMemcpyHostToDevice, s));
+    const bool w4 = row_bytes % 4 == 0;
+    const int groups = w4 ? row_bytes / 4 : row_bytes;
+    const dim3 wgrid(static_cast<unsigned>((groups + 127) / 128),
+                     static_cast<unsigned>((N + ptq::kCalibRowsPerBlock - 1) / ptq::kCalibRowsPerBlock));
+    if (packed && w4)
+        ptq::ptq_calib_wmax_kernel<4, true><<<wgrid, 128, 0, s>>>(d_w, d_dw, N, K, d_wbits);
+    else if (packed)
+        ptq::ptq_calib_wmax_kernel<1, true><<<wgrid, 128, 0, s>>>(d_w, d_dw, N, K, d_wbits);
+    else if (w4)
+        ptq::ptq_calib_wmax_kernel<4, false><<<wgrid, 128, 0, s>>>(d_w, d_dw, N, K, d_wbits);
+    else
+        ptq::ptq_calib_wmax_kernel<1, false><<<wgrid, 128, 0, s>>>(d_w, d_dw, N, K, d_wbits);
+    ptq::ptq_calib_smooth_kernel<<<(K + 127) / 128, 128, 0, s>>>(d_xbits, d_wbits, K, d_s);
+    if (vec)
+        launch_calib_rowrange<8>(asym, x, Bc, K, T, sms, d_s, d_hi, d_nlo, s);
+    else
+        launch_calib_rowrange<1>(asym, x, Bc, K, T, sms, d_s, d_hi, d_nlo, s);
+    if (asym)
+        ptq::ptq_calib_step_asym_kernel<<<(T + 127) / 128, 128, 0, s>>>(d_hi, d_nlo, T, d_dx, d_z);
+    else if (scheme == PTQ_CALIB_PER_TENSOR)
+        ptq::ptq_calib_step_tensor_kernel<<<1, 256, 0, s>>>(d_hi, T, d_dx, 127.0f);
+    else
+        ptq::ptq_calib_step_kernel<<<(T + 127) / 128, 128, 0, s>>>(d_hi, T, d_dx, packed ? 7.0f : 127.0f);
+    g_launches.fetch_add(5, std::memory_order_relaxed);
+    PTQ_CUDA(cudaGetLastError());
+    // one copy back: s, dx and (asymmetric) z are adjacent
+    const size_t words = static_cast<size_t>(K) + static_cast<size_t>(T) * (asym ? 2 : 1);
+    std::vector<float> got(words);
+    PTQ_CUDA(cudaMemcpyAsync(got.data(), d_s, sizeof(float) * words, cudaMemcpyDeviceToHost, s));
+    PTQ_CUDA(cudaStreamSynchronize(s));
+    std::memcpy(smooth_out, got.data(), sizeof(float) * K);
+    std::memcpy(act_step_out, got.data() + K, sizeof(float) * T);
+    if (asym) std::memcpy(act_zero_out, got.data() + K + T, sizeof(int32_t) * T);
+    return PTQ_OK;
+}
+
+// The entry points without a caller workspace: one temporary device allocation around ptq_calibrate_in.
+static ptq_status_t calibrate_alloc(int scheme, int K, int N, int T, const void *xcal_fp16, int Bc, const void *w_q,
+                                    const float *w_step, float *smooth_out, float *act_step_out, int32_t *act_zero_out,
+                                    void *stream)
+{
+    if (!xcal_fp16 || !w_q || !w_step || !smooth_out || !act_step_out || (scheme == PTQ_CALIB_ASYM && !act_zero_out))
+        return fail(PTQ_ERR_NULL, "calibrate: pointers must not be NULL");
+    const size_t bytes = ptq_calibrate_workspace_bytes(K, N, T);
+    if (bytes == 0 || Bc < 1)
+        return fail(PTQ_ERR_SHAPE, "calibrate: dimensions out of range (K=%d N=%d T=%d Bc=%d)", K, N, T, Bc);
+    void *ws = nullptr;
+    PTQ_CUDA(cudaMalloc(&ws, bytes));
+    const ptq_status_t st = ptq_calibrate_in(scheme, K, N, T, xcal_fp16, Bc, w_q, w_step, smooth_out, act_step_out,
+                                             act_zero_out, ws, bytes, stream);
+    cudaFree(ws);
     return st;
 }
 
 ptq_status_t ptq_calibrate(int K, int N, int T, const void *xcal_fp16, int Bc, const int8_t *w_q,
                            const float *w_step, float *smooth_out, float *act_step_out, void *stream)
 {
-    return calibrate_impl(K, N, T, xcal_fp16, Bc, w_q, w_step, smooth_out, act_step_out, nullptr, stream);
+    return calibrate_alloc(PTQ_CALIB_PTS, K, N, T, xcal_fp16, Bc, w_q, w_step, smooth_out, act_step_out, nullptr, stream);
 }
 
 ptq_status_t ptq_calibrate_per_tensor(int K, int N, int T, const void *xcal_fp16, int Bc, const int8_t *w_q,
                                       const float *w_step, float *smooth_out, float *act_step_out, void *stream)
 {
-    return calibrate_impl(K, N, T, xcal_fp16, Bc, w_q, w_step, smooth_out, act_step_out, nullptr, stream, 127.0f, true);
+    return calibrate_alloc(PTQ_CALIB_PER_TENSOR, K, N, T, xcal_fp16, Bc, w_q, w_step, smooth_out, act_step_out, nullptr, stream);
 }
 
 ptq_status_t ptq_calibrate_asym(int K, int N, int T, const void *xcal_fp16, int Bc, const int8_t *w_q,
                                 const float *w_step, float *smooth_out, float *act_step_out,
                                 int32_t *act_zero_out, void *stream)
 {
-    if (!act_zero_out) return fail(PTQ_ERR_NULL, "calibrate: pointers must not be NULL");
-    return calibrate_impl(K, N, T, xcal_fp16, Bc, w_q, w_step, smooth_out, act_step_out, act_zero_out, stream);
+    return calibrate_alloc(PTQ_CALIB_ASYM, K, N, T, xcal_fp16, Bc, w_q, w_step, smooth_out, act_step_out, act_zero_out, stream);
+}
+
+ptq_status_t ptq_calibrate_w4a4(int K, int N, int T, const void *xcal_fp16, int Bc, const uint8_t *w_q_packed,
+                                const float *w_step, float *smooth_out, float *act_step_out, void *stream)
+{
+    return calibrate_alloc(PTQ_CALIB_W4A4, K, N, T, xcal_fp16, Bc, w_q_packed, w_step, smooth_out, act_step_out, nullptr, stream);
 }
 
 // Sign-extending unpack of rows of 4-bit values, two per byte, low nibble = even column.
@@ -1362,17 +1481,6 @@ ptq_status_t ptq_linear_create_w4a4(ptq_linear_t **out, int K, int N, int T, con
     std::vector<int8_t> w;
     unpack_int4_host(w_q_packed, N, K, w);
     return create_impl(out, K, N, T, w.data(), w_step, smooth, act_step, nullptr, bias, flags, 4);
-}
-
-ptq_status_t ptq_calibrate_w4a4(int K, int N, int T, const void *xcal_fp16, int Bc, const uint8_t *w_q_packed,
-                                const float *w_step, float *smooth_out, float *act_step_out, void *stream)
-{
-    if (!w_q_packed) return fail(PTQ_ERR_NULL, "calibrate: pointers must not be NULL");
-    if (K < 1 || K > PTQ_MAX_K || N < 1 || N > PTQ_MAX_N)
-        return fail(PTQ_ERR_SHAPE, "calibrate: dimensions out of range (K=%d N=%d)", K, N);
-    std::vector<int8_t> w;
-    unpack_int4_host(w_q_packed, N, K, w);
-    return calibrate_impl(K, N, T, xcal_fp16, Bc, w.data(), w_step, smooth_out, act_step_out, nullptr, stream, 7.0f);
 }
 
 ptq_status_t ptq_quantize_packed4(const ptq_linear_t *h, const void *x_fp16, int B, void *q_packed, void *workspace,

@@ -24,53 +24,115 @@ __device__ __forceinline__ float warp_max(float v)
     return v;
 }
 
-// maxX: each warp walks rows with a stride; lanes cover channels k = lane, lane+32, ...
-// Per-lane running maxima live in registers (8 channels per lane per pass over K), then one
-// atomicMax per (warp, channel).
-__global__ void __launch_bounds__(256) ptq_calib_colmax_kernel(const __half *x, long long M, int K,
+// kVec consecutive channels of one row, held as packed binary16 pairs (kVec = 8: one 16-byte load, needs K % 8 == 0 and
+// a 16-byte aligned x; kVec = 1: any K and alignment).
+template <int kVec>
+struct __align__(16) CalibChunk {
+    __half2 h[kVec == 8 ? 4 : 1];
+};
+template <int kVec>
+__device__ __forceinline__ CalibChunk<kVec> calib_load(const __half *p)
+{
+    CalibChunk<kVec> c;
+    if (kVec == 8) {
+        const uint4 v = __ldg(reinterpret_cast<const uint4 *>(p));
+        *reinterpret_cast<uint4 *>(&c) = v;
+    } else {
+        c.h[0] = __half2half2(__ldg(p));
+    }
+    return c;
+}
+template <int kVec>
+__device__ __forceinline__ float calib_channel(const CalibChunk<kVec> &c, int i)
+{
+    return (i & 1) ? __high2float(c.h[kVec == 8 ? i >> 1 : 0]) : __low2float(c.h[kVec == 8 ? i >> 1 : 0]);
+}
+
+// maxX[k].  A block takes `rows_per_block` consecutive rows; a thread keeps one group of kVec channels in binary16
+// registers (max.f16x2 drops NaN, and a maximum of binary16 values is exact in binary16) over every rp-th of those
+// rows, the block merges its rp row lanes in shared memory and issues one global atomicMax per channel.
+// Bound: memory latency at calibration sizes (8 images: 0.6 - 4.8 MB, a few loads deep per thread).
+template <int kVec>
+__global__ void __launch_bounds__(256) ptq_calib_colmax_kernel(const __half *x, long long M, int K, int rows_per_block,
                                                                unsigned *max_x_bits)
 {
-    const int lane = threadIdx.x & 31;
-    const int warps_per_block = blockDim.x >> 5;
-    const long long warp = static_cast<long long>(blockIdx.x) * warps_per_block + (threadIdx.x >> 5);
-    const long long nwarps = static_cast<long long>(gridDim.x) * warps_per_block;
-    for (int k0 = 0; k0 < K; k0 += 32 * 8) {
-        float mx[8];
+    __shared__ unsigned best[256 * kVec];
+    const int cpr = K / kVec;
+    const int tpr = min(cpr, 256);                       // threads along a row
+    const int rp = 256 / tpr;                            // rows side by side
+    const int r = static_cast<int>(threadIdx.x) / tpr;
+    const int c = static_cast<int>(threadIdx.x) - r * tpr;
+    const long long m0 = static_cast<long long>(blockIdx.x) * rows_per_block;
+    const int rows = static_cast<int>(M - m0 < rows_per_block ? M - m0 : rows_per_block);
+    for (int c0 = 0; c0 < cpr; c0 += tpr) {
+        const bool on = r < rp && c0 + c < cpr;
+        CalibChunk<kVec> mx;
 #pragma unroll
-        for (int j = 0; j < 8; ++j) mx[j] = 0.0f;
-        for (long long m = warp; m < M; m += nwarps) {
-            const __half *row = x + m * K;
+        for (int i = 0; i < (kVec == 8 ? 4 : 1); ++i) mx.h[i] = __float2half2_rn(0.0f);
+        if (on) {
+            const __half *p = x + (m0 + r) * K + static_cast<long long>(c0 + c) * kVec;
+#pragma unroll 4
+            for (int m = r; m < rows; m += rp, p += static_cast<long long>(rp) * K) {
+                const CalibChunk<kVec> v = calib_load<kVec>(p);
 #pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                const int k = k0 + j * 32 + lane;
-                if (k < K) mx[j] = fmaxf(mx[j], fabsf(__half2float(row[k])));   // fmaxf drops NaN
+                for (int i = 0; i < (kVec == 8 ? 4 : 1); ++i) mx.h[i] = __hmax2(mx.h[i], __habs2(v.h[i]));
             }
         }
+        if (rp > 1) {
+            __syncthreads();
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            const int k = k0 + j * 32 + lane;
-            if (k < K && mx[j] > 0.0f) atomicMax(max_x_bits + k, __float_as_uint(mx[j]));
+            for (int i = 0; i < kVec; ++i) best[threadIdx.x * kVec + i] = 0u;
+            __syncthreads();
+            if (on) {
+#pragma unroll
+                for (int i = 0; i < kVec; ++i) atomicMax(&best[c * kVec + i], __float_as_uint(calib_channel<kVec>(mx, i)));
+            }
+            __syncthreads();
+            for (int k = threadIdx.x; k < tpr * kVec && c0 * kVec + k < K; k += 256)
+                if (best[k] != 0u) atomicMax(max_x_bits + c0 * kVec + k, best[k]);
+        } else if (on) {
+#pragma unroll
+            for (int i = 0; i < kVec; ++i) {
+                const unsigned bits = __float_as_uint(calib_channel<kVec>(mx, i));
+                if (bits != 0u) atomicMax(max_x_bits + (c0 + c) * kVec + i, bits);
+            }
         }
     }
 }
 
-// maxW[k] = max_n |Wq[n,k]| * dw[n]: grid (channel blocks, row blocks); a thread scans kCalibRowsPerBlock
-// weight rows of its channel (coalesced across the block's channels) and merges with one atomicMax.
+// maxW[k] = max_n |Wq[n,k]| * dw[n]: grid (byte-group blocks, row blocks); a thread scans kCalibRowsPerBlock weight rows
+// of kBytes adjacent bytes (coalesced across the block) and merges with one atomicMax per channel.  kPacked: two
+// signed 4-bit weights per byte, low nibble = even channel, rows of (K+1)/2 bytes.
 constexpr int kCalibRowsPerBlock = 32;
 
-__global__ void __launch_bounds__(128) ptq_calib_wmax_kernel(const int8_t *wq, const float *dw, int N, int K,
+template <int kBytes, bool kPacked>
+__global__ void __launch_bounds__(128) ptq_calib_wmax_kernel(const uint8_t *wq, const float *dw, int N, int K,
                                                              unsigned *max_w_bits)
 {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= K) return;
+    constexpr int kChan = kPacked ? 2 * kBytes : kBytes;
+    const int row_bytes = kPacked ? (K + 1) / 2 : K;
+    const int j = (blockIdx.x * blockDim.x + threadIdx.x) * kBytes;
+    if (j >= row_bytes) return;
     const int n0 = blockIdx.y * kCalibRowsPerBlock;
     const int n1 = min(N, n0 + kCalibRowsPerBlock);
-    float mw = 0.0f;
-    for (int n = n0; n < n1; ++n) {
-        const float a = __fmul_rn(fabsf(static_cast<float>(wq[static_cast<long long>(n) * K + k])), __ldg(dw + n));
-        mw = fmaxf(mw, a);
+    float mw[kChan];
+#pragma unroll
+    for (int i = 0; i < kChan; ++i) mw[i] = 0.0f;
+    const uint8_t *p = wq + static_cast<long long>(n0) * row_bytes + j;
+#pragma unroll 8
+    for (int n = n0; n < n1; ++n, p += row_bytes) {
+        const uint32_t w = kBytes == 4 ? __ldg(reinterpret_cast<const uint32_t *>(p)) : static_cast<uint32_t>(__ldg(p));
+        const float d = __ldg(dw + n);
+#pragma unroll
+        for (int i = 0; i < kChan; ++i) {
+            const int q = kPacked ? static_cast<int>(w << (28 - 4 * i)) >> 28 : static_cast<int>(w << (24 - 8 * i)) >> 24;
+            mw[i] = fmaxf(mw[i], __fmul_rn(fabsf(static_cast<float>(q)), d));
+        }
     }
-    if (mw > 0.0f) atomicMax(max_w_bits + k, __float_as_uint(mw));
+    const int k0 = kPacked ? 2 * j : j;
+#pragma unroll
+    for (int i = 0; i < kChan; ++i)
+        if (k0 + i < K && mw[i] > 0.0f) atomicMax(max_w_bits + k0 + i, __float_as_uint(mw[i]));
 }
 
 // s[k] from maxX[k] and maxW[k]; one thread per channel.
@@ -84,21 +146,53 @@ __global__ void __launch_bounds__(128) ptq_calib_smooth_kernel(const unsigned *m
     s[k] = __fsqrt_rn(__fdiv_rn(mx, mw));
 }
 
-// mu[t] = max_{b,k} |x[b,t,k] / s[k]|: one warp per row, shuffle reduction, one atomicMax per row.
-__global__ void __launch_bounds__(256) ptq_calib_rowmax_kernel(const __half *x, long long M, int K, int T,
-                                                               const float *s, unsigned *mu_bits)
+// Largest and smallest x/s of a token position over the images of a block's share, both widened to zero; grid
+// (T, image splits).  A correctly rounded division by a positive s is monotone, so the maximum over the images is taken
+// on the binary16 inputs and only the one survivor per (position, channel) is divided: the same bits as dividing every
+// element, with 1/Bc of the divisions.
+//   kAsym = false: mu[t] = max |x/s| in hi_bits;   kAsym = true: hi[t] in hi_bits, -lo[t] in nlo_bits
+template <int kVec, bool kAsym>
+__global__ void __launch_bounds__(128) ptq_calib_rowrange_kernel(const __half *x, int Bc, int imgs_per_block, int K, int T,
+                                                                 const float *s, unsigned *hi_bits, unsigned *nlo_bits)
 {
-    const int lane = threadIdx.x & 31;
-    const int warps_per_block = blockDim.x >> 5;
-    const long long warp = static_cast<long long>(blockIdx.x) * warps_per_block + (threadIdx.x >> 5);
-    const long long nwarps = static_cast<long long>(gridDim.x) * warps_per_block;
-    for (long long m = warp; m < M; m += nwarps) {
-        const __half *row = x + m * K;
-        float mu = 0.0f;
-        for (int k = lane; k < K; k += 32)
-            mu = fmaxf(mu, fabsf(__fdiv_rn(__half2float(row[k]), __ldg(s + k))));
-        mu = warp_max(mu);
-        if (lane == 0 && mu > 0.0f) atomicMax(mu_bits + static_cast<int>(m % T), __float_as_uint(mu));
+    const int t = blockIdx.x;
+    const int b0 = blockIdx.y * imgs_per_block;
+    const int nb = min(imgs_per_block, Bc - b0);
+    const int cpr = K / kVec;
+    const int tpr = min(cpr, 128);
+    const int ip = 128 / tpr;                            // images side by side
+    const int img = static_cast<int>(threadIdx.x) / tpr;
+    const int c = static_cast<int>(threadIdx.x) - img * tpr;
+    const long long img_step = static_cast<long long>(T) * K;
+    float hi = 0.0f, nlo = 0.0f;
+    if (img < ip) {
+        for (int c0 = c; c0 < cpr; c0 += tpr) {
+            CalibChunk<kVec> mx, mn;
+#pragma unroll
+            for (int i = 0; i < (kVec == 8 ? 4 : 1); ++i) mx.h[i] = mn.h[i] = __float2half2_rn(0.0f);
+            const __half *p = x + (static_cast<long long>(b0 + img) * T + t) * K + static_cast<long long>(c0) * kVec;
+#pragma unroll 8
+            for (int b = img; b < nb; b += ip, p += ip * img_step) {
+                const CalibChunk<kVec> v = calib_load<kVec>(p);
+#pragma unroll
+                for (int i = 0; i < (kVec == 8 ? 4 : 1); ++i) {
+                    mx.h[i] = __hmax2(mx.h[i], kAsym ? v.h[i] : __habs2(v.h[i]));     // NaN is dropped
+                    if (kAsym) mn.h[i] = __hmin2(mn.h[i], v.h[i]);
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < kVec; ++i) {
+                const float sv = __ldg(s + c0 * kVec + i);
+                hi = fmaxf(hi, __fdiv_rn(calib_channel<kVec>(mx, i), sv));
+                if (kAsym) nlo = fmaxf(nlo, -__fdiv_rn(calib_channel<kVec>(mn, i), sv));
+            }
+        }
+    }
+    hi = warp_max(hi);
+    if (kAsym) nlo = warp_max(nlo);
+    if ((threadIdx.x & 31) == 0) {
+        if (hi > 0.0f) atomicMax(hi_bits + t, __float_as_uint(hi));
+        if (kAsym && nlo > 0.0f) atomicMax(nlo_bits + t, __float_as_uint(nlo));
     }
 }
 
@@ -130,32 +224,6 @@ __global__ void __launch_bounds__(256) ptq_calib_step_tensor_kernel(const unsign
 // --- asymmetric variant: per-token-position range [lo, hi] of x/s, always containing zero ----------
 //   hi[t] = max(0, max x/s),  nlo[t] = max(0, max -(x/s))   (both non-negative: atomicMax on the bits)
 //   dx[t] = max(hi + nlo, 1e-5) / 255,   z[t] = clip(rne(nlo / dx[t]), 0, 255)
-__global__ void __launch_bounds__(256) ptq_calib_rowrange_kernel(const __half *x, long long M, int K, int T,
-                                                                 const float *s, unsigned *hi_bits,
-                                                                 unsigned *nlo_bits)
-{
-    const int lane = threadIdx.x & 31;
-    const int warps_per_block = blockDim.x >> 5;
-    const long long warp = static_cast<long long>(blockIdx.x) * warps_per_block + (threadIdx.x >> 5);
-    const long long nwarps = static_cast<long long>(gridDim.x) * warps_per_block;
-    for (long long m = warp; m < M; m += nwarps) {
-        const __half *row = x + m * K;
-        float hi = 0.0f, nlo = 0.0f;
-        for (int k = lane; k < K; k += 32) {
-            const float u = __fdiv_rn(__half2float(row[k]), __ldg(s + k));
-            hi = fmaxf(hi, u);          // fmaxf drops NaN
-            nlo = fmaxf(nlo, -u);
-        }
-        hi = warp_max(hi);
-        nlo = warp_max(nlo);
-        if (lane == 0) {
-            const int t = static_cast<int>(m % T);
-            if (hi > 0.0f) atomicMax(hi_bits + t, __float_as_uint(hi));
-            if (nlo > 0.0f) atomicMax(nlo_bits + t, __float_as_uint(nlo));
-        }
-    }
-}
-
 __global__ void __launch_bounds__(128) ptq_calib_step_asym_kernel(const unsigned *hi_bits, const unsigned *nlo_bits,
                                                                   int T, float *dx, int *z)
 {
