@@ -13,6 +13,7 @@
 #include <cstring>
 #include <mutex>
 #include <new>
+#include <type_traits>
 #include <utility>
 #include <vector>
 
@@ -97,7 +98,6 @@ ptq_status_t make_map_2d(CUtensorMap *map, CUtensorMapDataType dt, int elem_byte
 #endif
 
 inline int round_up(int v, int m) { return (v + m - 1) / m * m; }
-inline int gcd_int(int a, int b) { while (b) { int t = a % b; a = b; b = t; } return a; }
 
 bool ranges_overlap(const void *a, size_t na, const void *b, size_t nb)
 {
@@ -286,64 +286,38 @@ ptq_status_t launch_quantize(const ptq_linear *h, const void *x, long long M, vo
     p.T = h->T;
     p.q_pitch = q_pitch;
     const long long B = M / h->T;
-    // Vector kernel: thread count = S * (chunks per image), S images apart between a thread's chunks.
-    // S is the multiple of `mult` (which makes the thread count a multiple of 256) that brings the grid
-    // closest to one resident wave without exceeding it; shapes for which even the smallest S
-    // overshoots the wave by far go to the scalar kernel.
-    bool vec = (h->K % 8 == 0) && (reinterpret_cast<uintptr_t>(x) % 16 == 0) &&
-               (reinterpret_cast<uintptr_t>(q) % 8 == 0) && (q_pitch % 8 == 0);
-    long long cpi = 0, S = 0;
-    if (vec) {
-        cpi = static_cast<long long>(h->T) * (h->K / 8);
-        const long long wave = static_cast<long long>(h->num_sms) * ptq::kQuantCtasPerSm * 256;
-        const long long mult = 256 / gcd_int(static_cast<int>(cpi % 256 == 0 ? 256 : cpi % 256), 256);
-        S = wave / cpi / mult * mult;
-        if (S < mult) S = mult;
-        const long long bcap = (B + mult - 1) / mult * mult;      // more than B images apart is idle threads only
-        if (S > bcap) S = bcap;
-        if (S * cpi > 4 * wave) vec = false;
-    }
+    // Thread count = S * (chunks per image), S images apart between a thread's chunks: the smallest S that needs no more
+    // rounds than one resident wave of threads does (at least one image at a time, however large).
+    const bool vec = (h->K % 8 == 0) && (reinterpret_cast<uintptr_t>(x) % 16 == 0) &&
+                     (reinterpret_cast<uintptr_t>(q) % 8 == 0) && (q_pitch % 8 == 0);
+    const int cpr = (h->K + 7) / 8;
+    const long long cpi = static_cast<long long>(h->T) * cpr;
+    const long long wave = static_cast<long long>(h->num_sms) * ptq::kQuantCtasPerSm * 256;
+    long long S = wave / cpi;
+    if (S < 1) S = 1;
+    const long long rounds = (B + S - 1) / S;
+    S = (B + rounds - 1) / rounds;
     p.B = static_cast<int>(B);
     p.imgs_per_iter = static_cast<int>(S);
-    p.fd_cpi = ptq::make_fastdiv(static_cast<unsigned>(vec ? cpi : 1));
-    p.fd_cpr = ptq::make_fastdiv(static_cast<unsigned>(vec ? h->K / 8 : 1));
-    if (vec) {
-        const int grid = static_cast<int>(S * cpi / 256);
-        if (h->act_bits == 4) {
-            if (h->fast_div)
-                PTQ_CUDA(launch_pdl(ptq::ptq_quantize_vec8_kernel<true, ptq::kCodeS4>, grid, 256, 0, stream, p));
-            else
-                PTQ_CUDA(launch_pdl(ptq::ptq_quantize_vec8_kernel<false, ptq::kCodeS4>, grid, 256, 0, stream, p));
-        } else if (h->asym) {
-            if (h->fast_div)
-                PTQ_CUDA(launch_pdl(ptq::ptq_quantize_vec8_kernel<true, ptq::kCodeU8>, grid, 256, 0, stream, p));
-            else
-                PTQ_CUDA(launch_pdl(ptq::ptq_quantize_vec8_kernel<false, ptq::kCodeU8>, grid, 256, 0, stream, p));
-        } else if (h->fast_div)
-            PTQ_CUDA(launch_pdl(ptq::ptq_quantize_vec8_kernel<true>, grid, 256, 0, stream, p));
-        else
-            PTQ_CUDA(launch_pdl(ptq::ptq_quantize_vec8_kernel<false>, grid, 256, 0, stream, p));
-    } else {
-        long long want = (M * h->K + 255) / 256;
-        const long long cap = static_cast<long long>(h->num_sms) * 8;
-        if (want > cap) want = cap;
-        if (want < 1) want = 1;
-        const int g = static_cast<int>(want);
-        if (h->act_bits == 4) {
-            if (h->fast_div)
-                PTQ_CUDA(launch_pdl(ptq::ptq_quantize_scalar_kernel<true, ptq::kCodeS4>, g, 256, 0, stream, p));
-            else
-                PTQ_CUDA(launch_pdl(ptq::ptq_quantize_scalar_kernel<false, ptq::kCodeS4>, g, 256, 0, stream, p));
-        } else if (h->asym) {
-            if (h->fast_div)
-                PTQ_CUDA(launch_pdl(ptq::ptq_quantize_scalar_kernel<true, ptq::kCodeU8>, g, 256, 0, stream, p));
-            else
-                PTQ_CUDA(launch_pdl(ptq::ptq_quantize_scalar_kernel<false, ptq::kCodeU8>, g, 256, 0, stream, p));
-        } else if (h->fast_div)
-            PTQ_CUDA(launch_pdl(ptq::ptq_quantize_scalar_kernel<true>, g, 256, 0, stream, p));
-        else
-            PTQ_CUDA(launch_pdl(ptq::ptq_quantize_scalar_kernel<false>, g, 256, 0, stream, p));
-    }
+    p.fd_cpi = ptq::make_fastdiv(static_cast<unsigned>(cpi));
+    p.fd_cpr = ptq::make_fastdiv(static_cast<unsigned>(cpr));
+    const uintptr_t x_align = reinterpret_cast<uintptr_t>(x) | static_cast<uintptr_t>(2 * h->K);
+    p.ld_bytes = x_align % 8 == 0 ? 8 : x_align % 4 == 0 ? 4 : 2;
+    p.st_bytes = (reinterpret_cast<uintptr_t>(q) % 8 == 0 && q_pitch % 8 == 0) ? 8 : 1;
+    const int grid = static_cast<int>((S * cpi + 255) / 256);
+    auto go = [&](auto mode, auto fast) -> cudaError_t {
+        constexpr int kMode = decltype(mode)::value;
+        constexpr bool kFast = decltype(fast)::value;
+        return vec ? launch_pdl(ptq::ptq_quantize_vec8_kernel<kFast, kMode, false>, grid, 256, 0, stream, p)
+                   : launch_pdl(ptq::ptq_quantize_vec8_kernel<kFast, kMode, true>, grid, 256, 0, stream, p);
+    };
+    auto pick = [&](auto mode) { return h->fast_div ? go(mode, std::true_type()) : go(mode, std::false_type()); };
+    if (h->act_bits == 4)
+        PTQ_CUDA(pick(std::integral_constant<int, ptq::kCodeS4>()));
+    else if (h->asym)
+        PTQ_CUDA(pick(std::integral_constant<int, ptq::kCodeU8>()));
+    else
+        PTQ_CUDA(pick(std::integral_constant<int, ptq::kCodeS8>()));
     g_launches.fetch_add(1, std::memory_order_relaxed);
     PTQ_CUDA(cudaGetLastError());
     return PTQ_OK;
@@ -484,6 +458,8 @@ ptq_status_t launch_gemm(const ptq_linear *h, const void *codes, long long M, vo
     p.use_tma_store = tma_store ? 1 : 0;
     p.y_vec2 = (h->N % 2 == 0 && reinterpret_cast<uintptr_t>(y) % 4 == 0) ? 1 : 0;
     p.y_vec8 = 0;   // this kernel always has a staging buffer; 16-byte alignment means TMA stores
+    const uintptr_t y_align = reinterpret_cast<uintptr_t>(y) | static_cast<uintptr_t>(2 * h->N);
+    p.y_copy_bytes = y_align % 8 == 0 ? 8 : y_align % 4 == 0 ? 4 : 2;
     p.zp = h->d_zp;
     p.wsum = h->d_wsum;
     p.fd_T = ptq::make_fastdiv(static_cast<unsigned>(p.T));
@@ -631,6 +607,7 @@ ptq_status_t launch_fused(const ptq_linear *h, const void *x, long long M, void 
     p.use_tma_store = tma_store ? 1 : 0;
     p.y_vec2 = (h->N % 2 == 0 && reinterpret_cast<uintptr_t>(y) % 4 == 0) ? 1 : 0;
     p.y_vec8 = (aligned && !tma_store) ? 1 : 0;
+    p.y_copy_bytes = 2;   // not used by this kernel
     p.zp = nullptr;
     p.wsum = nullptr;
     fp.x = static_cast<const __half *>(x);

@@ -86,6 +86,7 @@ struct GemmParams {
     int use_tma_store; // y is written by TMA (needs N % 8 == 0 and a 16-byte aligned y)
     int y_vec2;        // plain-store path may use 4-byte stores (N even, y 4-byte aligned)
     int y_vec8;        // plain-store path may use 16-byte stores (N % 8 == 0, y 16-byte aligned)
+    int y_copy_bytes;  // streaming kernel without TMA stores: bytes per lane of a row copy (8, 4 or 2: alignment of y's rows)
     // Asymmetric layers (zero offset per token position): the codes are unsigned, the tensor core
     // accumulates sum_k c * Wq, and the epilogue subtracts z[t] * sum_k Wq[n,k] to obtain the offset-free
     // accumulator sum_k (c - z[t]) * Wq[n,k] exactly (all int32).  nullptr for symmetric layers.
@@ -340,6 +341,51 @@ __device__ __forceinline__ void convert_stage64_sw128(const uint32_t (&v0)[32], 
     for (int jj = 0; jj < 8; ++jj) st_shared_v4(row_addr + ((static_cast<uint32_t>(jj) ^ sw) << 4), o[jj]);
 }
 
+// A staged 32-row x 64-column box to y without TMA (N not a multiple of 8, or y not 16-byte aligned): the warp copies it
+// row by row, so that the stores of a row are contiguous and touch each sector once.  Storing from the accumulator
+// layout instead (a thread per row) scatters every store over 32 rows: 129 -> 257 channels, 285 rows, took 32 us.
+__device__ __noinline__ void copy_box_rows(__half *y, long long M, int N, int copy_bytes, uint32_t box, long long m_row0,
+                                           int n_first, int lane)
+{
+    auto at = [&](int r, int c) {
+        return box + static_cast<uint32_t>(r) * 128u + (((static_cast<uint32_t>(c) >> 3) ^ static_cast<uint32_t>(r & 7)) << 4) +
+               (static_cast<uint32_t>(c) & 7u) * 2u;
+    };
+    if (M <= m_row0) return;
+    const int rows = M - m_row0 < 32 ? static_cast<int>(M - m_row0) : 32;
+    __half *yb = y + m_row0 * N + n_first;
+    if (copy_bytes == 8) {                               // N % 4 == 0: 16 lanes per row
+        const int c = (lane & 15) * 4;
+        if (n_first + c >= N) return;
+#pragma unroll 8
+        for (int r = lane >> 4; r < rows; r += 2) {
+            uint32_t a, b;
+            asm volatile("ld.shared.v2.b32 {%0, %1}, [%2];" : "=r"(a), "=r"(b) : "r"(at(r, c)));
+            *reinterpret_cast<uint2 *>(yb + static_cast<long long>(r) * N + c) = make_uint2(a, b);
+        }
+    } else if (copy_bytes == 4) {
+        const int c = lane * 2;
+        if (n_first + c >= N) return;
+#pragma unroll 8
+        for (int r = 0; r < rows; ++r) {
+            uint32_t a;
+            asm volatile("ld.shared.b32 %0, [%1];" : "=r"(a) : "r"(at(r, c)));
+            *reinterpret_cast<uint32_t *>(yb + static_cast<long long>(r) * N + c) = a;
+        }
+    } else {
+        const bool ok0 = n_first + lane < N, ok1 = n_first + lane + 32 < N;
+#pragma unroll 4
+        for (int r = 0; r < rows; ++r) {
+            unsigned short a, b;
+            asm volatile("ld.shared.b16 %0, [%1];" : "=h"(a) : "r"(at(r, lane)));
+            asm volatile("ld.shared.b16 %0, [%1];" : "=h"(b) : "r"(at(r, lane + 32)));
+            __half *row = yb + static_cast<long long>(r) * N;
+            if (ok0) row[lane] = __ushort_as_half(a);
+            if (ok1) row[lane + 32] = __ushort_as_half(b);
+        }
+    }
+}
+
 template <bool kDebugAcc>
 __device__ __forceinline__ uint32_t epilogue_tile_stream(const GemmParams &p, const CUtensorMap *tmY, uint32_t tmem_row,
                                                          long long m_row0, int n0, float dxr, uint32_t staging,
@@ -389,12 +435,18 @@ __device__ __forceinline__ uint32_t epilogue_tile_stream(const GemmParams &p, co
         convert_stage64_sw128(v0, v1, dxr, reinterpret_cast<const float4 *>(dw_s + c0),
                               bias_s != nullptr ? reinterpret_cast<const float4 *>(bias_s + c0) : nullptr,
                               box + static_cast<uint32_t>(lane) * 128u, lane);
-        fence_proxy_async_smem();
-        __syncwarp();
-        if (lane == 0) {
-            if (n_first < p.N && m_row0 < p.M)
-                tma_store_2d(tmY, n_first, static_cast<int>(m_row0), box);   // clipped at N and M
-            bulk_commit_group();
+        if (p.use_tma_store) {
+            fence_proxy_async_smem();
+            __syncwarp();
+            if (lane == 0) {
+                if (n_first < p.N && m_row0 < p.M)
+                    tma_store_2d(tmY, n_first, static_cast<int>(m_row0), box);   // clipped at N and M
+                bulk_commit_group();
+            }
+        } else {
+            __syncwarp();
+            copy_box_rows(p.y, p.M, p.N, p.y_copy_bytes, box, m_row0, n_first, lane);
+            __syncwarp();
         }
         ++nboxes;
     }
@@ -694,14 +746,12 @@ ptq_gemm_dequant_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
             if (lane == 0) mbar_arrive(scale_bar);
         };
         uint32_t buf = 0, bphase = 0, nboxes = 0, it = 0;
-        if (p.use_tma_store) {
-            fetch_scales(blockIdx.x);
-            publish_scales(0u);
-        }
+        fetch_scales(blockIdx.x);
+        publish_scales(0u);
         RowStep rs_next = load_row_step(p, static_cast<int>(fd_div(blockIdx.x, p.fd_n_tiles)), quarter, lane);
         for (int tile = blockIdx.x; tile < total_tiles; tile += gridDim.x, ++it) {
             const int tile_next = tile + static_cast<int>(gridDim.x);
-            if (p.use_tma_store) fetch_scales(tile_next);                            // in flight during this tile
+            fetch_scales(tile_next);                            // in flight during this tile
             const int m_tile = static_cast<int>(fd_div(static_cast<unsigned>(tile), p.fd_n_tiles));
             const int n_tile = tile - m_tile * p.n_tiles;
             const long long m_row0 = static_cast<long long>(m_tile) * kBM + quarter * 32;
@@ -709,23 +759,17 @@ ptq_gemm_dequant_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
             const int zr = rs_next.z;
             if (tile_next < total_tiles)
                 rs_next = load_row_step(p, static_cast<int>(fd_div(static_cast<unsigned>(tile_next), p.fd_n_tiles)), quarter, lane);
-            bool got = true;
             // every epilogue warp has written its share of this tile's scale copies (arrival `it` of the barrier)
-            if (p.use_tma_store) got = mbar_wait(scale_bar, it & 1u, abort_flag, p.status);
+            bool got = mbar_wait(scale_bar, it & 1u, abort_flag, p.status);
             got = got && mbar_wait(tfull_bar(buf), bphase, abort_flag, p.status);
             got = __all_sync(0xffffffffu, got);
             if (!got) break;
             tc_fence_after_sync();
             const uint32_t tmem_row = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) + buf * kMaxBN;
-            if (p.use_tma_store) {
-                const float *dw_s = scale_s + (it & 1u) * kMaxBN;
-                const float *bias_s = p.has_bias ? scale_s + (2u + (it & 1u)) * kMaxBN : nullptr;
-                nboxes = epilogue_tile_stream<kDebugAcc>(p, &tmY, tmem_row, m_row0, n_tile * p.BN, dxr, staging, dw_s,
-                                                         bias_s, nboxes, lane, col_half * kEpiStepCols, 2 * kEpiStepCols, zr, two_boxes);
-            } else {
-                nboxes = epilogue_tile<kDebugAcc, false, kStreamBox64>(p, &tmY, tmem_row, m_row0, n_tile * p.BN, dxr,
-                                                                       staging, nboxes, lane, col_half, zr);
-            }
+            const float *dw_s = scale_s + (it & 1u) * kMaxBN;
+            const float *bias_s = p.has_bias ? scale_s + (2u + (it & 1u)) * kMaxBN : nullptr;
+            nboxes = epilogue_tile_stream<kDebugAcc>(p, &tmY, tmem_row, m_row0, n_tile * p.BN, dxr, staging, dw_s,
+                                                     bias_s, nboxes, lane, col_half * kEpiStepCols, 2 * kEpiStepCols, zr, two_boxes);
             tc_fence_before_sync();
             __syncwarp();
             if (lane == 0) mbar_arrive(tempty_bar(buf));
@@ -733,7 +777,7 @@ ptq_gemm_dequant_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
             if (buf == 0u) bphase ^= 1u;
             // the next tile's scales go to the other buffer: every warp is past its reads of that buffer,
             // because it has passed this tile's wait on scale_bar, which needed every warp's arrival
-            if (p.use_tma_store) publish_scales((it + 1u) & 1u);
+            publish_scales((it + 1u) & 1u);
         }
         if (lane == 0) bulk_wait_group<0>();         // all of this thread's stores have completed
     }

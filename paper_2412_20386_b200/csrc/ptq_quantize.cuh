@@ -219,7 +219,9 @@ struct QuantParams {
     int q_pitch;         // bytes between rows of q
     int B;               // images (M = B * T)
     int imgs_per_iter;   // vector kernel: images between consecutive chunks of one thread
-    FastDiv fd_cpi, fd_cpr;   // vector kernel: divisors T * K / 8 (chunks per image) and K / 8 (chunks per row)
+    FastDiv fd_cpi, fd_cpr;   // divisors: chunks per image and chunks per row
+    int ld_bytes;        // ragged kernel: bytes per load (8, 4 or 2: alignment of the rows of x)
+    int st_bytes;        // ragged kernel: 8 (codes row-aligned to 8 bytes, the pitch covers whole chunks) or 1
 };
 
 #ifndef PTQ_QUANT_CTAS_PER_SM
@@ -268,10 +270,45 @@ __device__ __forceinline__ uint2 quantize8(const uint4 &v, const float (&c8)[8],
     return out;
 }
 
-// Vector path: K % 8 == 0, x 16-byte aligned, q 8-byte aligned, q_pitch % 8 == 0.
+template <int kBytes>
+__device__ __forceinline__ void cp_async_small(void *smem_dst, const void *gmem_src)
+{
+    const unsigned d = static_cast<unsigned>(__cvta_generic_to_shared(smem_dst));
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(d), "l"(gmem_src), "n"(kBytes) : "memory");
+}
+
+// A chunk whose row is not 16-byte aligned, or of which only `left` < 8 channels exist, into its 16-byte slot:
+// asynchronous copies of 8 or 4 bytes (x and 2*K multiples of that), plain loads where only 2-byte alignment is given.
+// What lies behind `left` channels in the slot is undefined.
+__device__ __forceinline__ void load_chunk_ragged(uint4 *slot, const __half *src, int left, int ld_bytes)
+{
+    char *d = reinterpret_cast<char *>(slot);
+    if (ld_bytes == 8) {
+        cp_async_small<8>(d, src);
+        if (left > 4) cp_async_small<8>(d + 8, src + 4);
+    } else if (ld_bytes == 4) {
+#pragma unroll
+        for (int j = 0; j < 8; j += 2)
+            if (left > j) cp_async_small<4>(d + 2 * j, src + j);
+    } else {
+        uint32_t w[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const uint32_t e0 = left > 2 * j ? __half_as_ushort(src[2 * j]) : 0u;
+            const uint32_t e1 = left > 2 * j + 1 ? __half_as_ushort(src[2 * j + 1]) : 0u;
+            w[j] = e0 | (e1 << 16);
+        }
+        *slot = make_uint4(w[0], w[1], w[2], w[3]);
+    }
+}
+
+// kRagged = false: K % 8 == 0, x 16-byte aligned, q 8-byte aligned, q_pitch % 8 == 0.  kRagged = true: any K, pitch and
+// alignment; the last chunk of a row may be partial.
 // A "chunk" is 8 consecutive channels of one token row: one 16-byte load, one 8-byte store.
 // Thread g of the grid owns chunk (g mod chunks-per-image) of images b0, b0+S, b0+2S, ... with
-// b0 = g / chunks-per-image; the grid's thread count is S * chunks-per-image.  A thread therefore
+// b0 = g / chunks-per-image < S (the threads that round the grid up to whole blocks have b0 = S and do nothing; a
+// kernel that instead demanded S * chunks-per-image to be a multiple of the block size sent odd T * K / 8 to an
+// element-wise kernel: 11229 x 520 took 24 us).  A thread therefore
 // sees ONE token position and ONE group of 8 channels for the whole launch -- that is what "static"
 // per-token steps buy: the 8 combined reciprocals RN(1/s[k]) * RN(1/dx[t]) are formed once and kept
 // in registers, and the per-element work is convert, multiply, round, tie test.  Consecutive lanes
@@ -280,18 +317,19 @@ __device__ __forceinline__ uint2 quantize8(const uint4 &v, const float (&c8)[8],
 // slots, kQuantRingDepth images ahead.  A thread reads back only the slots it filled itself, so no
 // barrier is involved: cp.async.wait_group orders the thread's own copies.  Loads in flight hold no
 // registers, and their number does not depend on how far the arithmetic of the current chunk has got.
-template <bool kFast, int kMode = kCodeS8>
+template <bool kFast, int kMode = kCodeS8, bool kRagged = false>
 __global__ void __launch_bounds__(256, kQuantCtasPerSm) ptq_quantize_vec8_kernel(QuantParams p)
 {
     constexpr int D = kQuantRingDepth;
     __shared__ uint4 ring[D][256];
-    const int cpr = p.K >> 3;                                        // chunks per row
+    const int cpr = kRagged ? (p.K + 7) >> 3 : p.K >> 3;             // chunks per row
     const int cpi = p.T * cpr;                                       // chunks per image
-    // the grid is at most four resident waves, so the global thread index fits 32 bits; no runtime divisions
+    // the grid has at most S * cpi <= 2^30 + one wave of threads, so the thread index fits 32 bits; no runtime divisions
     // in front of the parameter loads below (a CTA that starts late runs this prologue on the critical path)
     const unsigned gtid = blockIdx.x * blockDim.x + threadIdx.x;
     int b = static_cast<int>(fd_div(gtid, p.fd_cpi));
     const int c = static_cast<int>(gtid) - b * cpi;
+    if (b >= p.imgs_per_iter) b = p.B;                                // rounding-up thread: no image
     const int t = static_cast<int>(fd_div(static_cast<unsigned>(c), p.fd_cpr));
     const int kc = c - t * cpr;
     const int S = p.imgs_per_iter;
@@ -320,10 +358,17 @@ __global__ void __launch_bounds__(256, kQuantCtasPerSm) ptq_quantize_vec8_kernel
     griddep_launch_dependents();
 
     const uint64_t pol_x = l2_policy_evict_first();
+    const int left = kRagged ? min(8, p.K - kc * 8) : 8;
+    auto load = [&](int slot, const __half *src) {
+        if (kRagged)
+            load_chunk_ragged(&ring[slot][threadIdx.x], src, left, p.ld_bytes);
+        else
+            cp_async_16_hint(&ring[slot][threadIdx.x], src, pol_x);
+    };
     // fill the ring: slot i holds image b + i*S (one commit group per slot, empty past the last image)
 #pragma unroll
     for (int i = 0; i < D; ++i) {
-        if (b + i * S < p.B) cp_async_16_hint(&ring[i][threadIdx.x], xp + i * x_step, pol_x);
+        if (b + i * S < p.B) load(i, xp + i * x_step);
         cp_async_commit();
     }
     float c8[8];
@@ -334,10 +379,23 @@ __global__ void __launch_bounds__(256, kQuantCtasPerSm) ptq_quantize_vec8_kernel
     int slot = 0;
     while (b < p.B) {
         cp_async_wait<D - 1>();                                   // the oldest group, i.e. this slot, has landed
-        const uint4 v = ring[slot][threadIdx.x];
-        *reinterpret_cast<uint2 *>(qp) = quantize8<kFast, kMode>(v, c8, s8, rs8, d.x, d.y, z);
+        uint4 v = ring[slot][threadIdx.x];
+        if (kRagged && left < 8) {                                // channels beyond K: zero
+            v.x &= left > 1 ? 0xffffffffu : 0xffffu;
+            v.y &= left > 3 ? 0xffffffffu : left > 2 ? 0xffffu : 0u;
+            v.z &= left > 5 ? 0xffffffffu : left > 4 ? 0xffffu : 0u;
+            v.w &= left > 6 ? 0xffffu : 0u;
+        }
+        const uint2 o = quantize8<kFast, kMode>(v, c8, s8, rs8, d.x, d.y, z);
+        if (!kRagged || p.st_bytes == 8) {
+            *reinterpret_cast<uint2 *>(qp) = o;
+        } else {
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+                if (i < left) qp[i] = static_cast<int8_t>((i < 4 ? o.x : o.y) >> (8 * (i & 3)));
+        }
         // refill the slot just consumed (its value has been used above) with the image D*S further on
-        if (b + D * S < p.B) cp_async_16_hint(&ring[slot][threadIdx.x], xp + D * x_step, pol_x);
+        if (b + D * S < p.B) load(slot, xp + D * x_step);
         cp_async_commit();
         slot = (slot + 1 == D) ? 0 : slot + 1;
         b += S;
@@ -345,31 +403,6 @@ __global__ void __launch_bounds__(256, kQuantCtasPerSm) ptq_quantize_vec8_kernel
         qp += q_step;
     }
     cp_async_wait<0>();
-}
-
-// Generic path: any K, any alignment; one element per thread per step.
-template <bool kFast, int kMode = kCodeS8>
-__global__ void __launch_bounds__(256) ptq_quantize_scalar_kernel(QuantParams p)
-{
-    griddep_wait();
-    griddep_launch_dependents();
-    const long long total = p.M * p.K;
-    const long long stride = static_cast<long long>(gridDim.x) * blockDim.x;
-    for (long long i = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x; i < total; i += stride) {
-        const long long m = i / p.K;
-        const int k = static_cast<int>(i - m * p.K);
-        const int t = static_cast<int>(m % p.T);
-        const __half h = p.x[i];
-        const float xf = __half2float(h);
-        const unsigned short bits = __half_as_ushort(h);
-        const int z = kMode == kCodeU8 ? __ldg(p.zp + t) : 0;
-        int c;
-        if (kFast && (bits & 0x7c00u) != 0x7c00u)
-            c = quantize_fast<kMode>(xf, __ldg(p.s + k), __ldg(p.rs + k), __ldg(p.dx + t), __ldg(p.rdx + t), z);
-        else
-            c = quantize_ieee<kMode>(xf, __ldg(p.s + k), __ldg(p.dx + t), z);
-        p.q[m * p.q_pitch + k] = static_cast<int8_t>(c);
-    }
 }
 
 // Two adjacent 4-bit codes (held one per byte, row pitch `pitch`) into one byte, low nibble = even
