@@ -3,8 +3,10 @@
 Argument marshalling only: every step of the path (quantize, integer GEMM,
 dequantize, calibration reductions) runs in the library's CUDA kernels.  torch
 tensors are used for device memory and streams; their ``data_ptr()`` crosses
-the boundary as a plain pointer.  There is no fallback: if the library is
-missing, loading raises.
+the boundary as a plain pointer.  The forward calls on the current stream go
+through the extension module ``_ptq_torch`` (``csrc/ptq_torch.cpp``), which does
+the marshalling natively; everything else uses ctypes.  There is no fallback: if
+the library or the extension is missing, loading raises.
 """
 from __future__ import annotations
 
@@ -112,6 +114,26 @@ def load_library() -> ctypes.CDLL:
     return L
 
 
+_native = None
+
+
+def _load_native():
+    """The extension module of the forward calls, with the library's entry points handed over."""
+    global _native
+    if _native is None:
+        import torch  # noqa: F401  (its libraries must be loaded first)
+        L = load_library()
+        try:
+            from . import _ptq_torch
+        except ImportError as e:
+            raise ImportError("%s: build it with `python -m paper_2412_20386_b200.build`. There is no fallback." % e) from e
+        _ptq_torch.bind(*(ctypes.cast(f, ctypes.c_void_p).value for f in (
+            L.ptq_linear_forward, L.ptq_linear_forward_static, L.ptq_linear_forward_dynamic,
+            L.ptq_linear_workspace_bytes, L.ptq_linear_workspace_bytes_dynamic)))
+        _native = _ptq_torch
+    return _native
+
+
 def _check(status: int):
     if status != 0:
         raise PtqError(status, load_library().ptq_last_error().decode("utf-8", "replace"))
@@ -201,11 +223,14 @@ class PtqLinear:
                                        _hp(smooth), _hp(act_step), _hp(bias), flags))
         self._h = h
         self._L = L
+        self._native = _load_native()
+        self._call = (h.value, self.T, self.K, self.N)
 
     def close(self):
         if getattr(self, "_h", None):
             self._L.ptq_linear_destroy(self._h)
             self._h = None
+            self._call = (0, self.T, self.K, self.N)
 
     def __del__(self):
         try:
@@ -245,6 +270,11 @@ class PtqLinear:
 
     def forward(self, x, y=None, workspace=None, flags: int = 0, stream=None):
         """``ptq_linear_forward``: x fp16 [B,T,K] -> y fp16 [B,T,N] (both on the device)."""
+        if stream is None and flags == 0:
+            r = self._native.forward(*self._call, x, y, workspace)
+            if r.__class__ is int:
+                _check(r)
+            return r
         import torch
         B = self._batch(x)
         if y is None:
@@ -267,6 +297,11 @@ class PtqLinear:
         The caller passes both x and y; the int8 codes go to the scratch array built into the
         library (at most ``STATIC_SCRATCH_BYTES``), which all calls on a device share.
         """
+        if stream is None:
+            r = self._native.forward_static(*self._call, x, y, None)
+            if r.__class__ is int:
+                _check(r)
+            return r
         B = self._batch(x)
         if tuple(y.shape) != (B, self.T, self.N) or y.dtype != x.dtype or not y.is_contiguous() or not y.is_cuda:
             raise ValueError("y must be a contiguous CUDA float16 tensor [B,T,N]")
@@ -278,6 +313,11 @@ class PtqLinear:
 
     def forward_dynamic(self, x, y=None, workspace=None, stream=None):
         """``ptq_linear_forward_dynamic``: the per-token dynamic comparator (row steps measured at run time)."""
+        if stream is None:
+            r = self._native.forward_dynamic(*self._call, x, y, workspace)
+            if r.__class__ is int:
+                _check(r)
+            return r
         import torch
         B = self._batch(x)
         if y is None:

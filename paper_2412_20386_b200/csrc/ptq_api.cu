@@ -131,10 +131,11 @@ struct ptq_linear {
     bool fast_div = false;     // all scales inside the range where the reciprocal route is exact
     int device = -1;
     int num_sms = 0;
+    unsigned char *d_all = nullptr;   // the one allocation that holds all of the following
     int8_t *d_w = nullptr;     // [n_tiles*BN, Kpad], zero padded
     float *d_dw = nullptr, *d_bias = nullptr;            // [n_tiles*BN rounded up to 64, +64], zero padded
     float *d_s = nullptr, *d_rs = nullptr;               // [round_up(K,16)]
-    float *d_dx = nullptr, *d_rdx = nullptr;             // [T]
+    float *d_dx = nullptr;                               // [T]
     float2 *d_dx2 = nullptr;                             // [T] {dx, 1/dx}
     int *d_zp = nullptr;                                 // [T] zero offsets (asymmetric layers only)
     int *d_wsum = nullptr;                               // row sums of Wq, padded like d_dw (asymmetric only)
@@ -153,14 +154,6 @@ struct ptq_linear {
 };
 
 namespace {
-
-ptq_status_t upload(void **dst, const void *src, size_t bytes, size_t alloc_bytes)
-{
-    PTQ_CUDA(cudaMalloc(dst, alloc_bytes));
-    PTQ_CUDA(cudaMemset(*dst, 0, alloc_bytes));
-    if (bytes) PTQ_CUDA(cudaMemcpy(*dst, src, bytes, cudaMemcpyHostToDevice));
-    return PTQ_OK;
-}
 
 ptq_status_t check_device(const ptq_linear *h)
 {
@@ -277,8 +270,6 @@ ptq_status_t launch_quantize(const ptq_linear *h, const void *x, long long M, vo
     p.q = static_cast<int8_t *>(q);
     p.s = h->d_s;
     p.rs = h->d_rs;
-    p.dx = h->d_dx;
-    p.rdx = h->d_rdx;
     p.dx2 = h->d_dx2;
     p.zp = h->d_zp;
     p.M = M;
@@ -706,17 +697,7 @@ unsigned long long ptq_kernel_launch_count(void) { return g_launches.load(std::m
 void ptq_linear_destroy(ptq_linear_t *h)
 {
     if (!h) return;
-    cudaFree(h->d_w);
-    cudaFree(h->d_dw);
-    cudaFree(h->d_bias);
-    cudaFree(h->d_s);
-    cudaFree(h->d_rs);
-    cudaFree(h->d_dx);
-    cudaFree(h->d_rdx);
-    cudaFree(h->d_dx2);
-    cudaFree(h->d_zp);
-    cudaFree(h->d_wsum);
-    cudaFree(h->d_status);
+    cudaFree(h->d_all);
     delete h;
 }
 
@@ -753,17 +734,17 @@ static ptq_status_t create_impl(ptq_linear_t **out, int K, int N, int T, const i
     for (int t = 0; act_zero && t < T; ++t)
         if (act_zero[t] < 0 || act_zero[t] > 255)
             return fail(PTQ_ERR_VALUE, "act_zero[%d] = %d is outside [0,255]", t, act_zero[t]);
-    for (long long i = 0; i < static_cast<long long>(N) * K; ++i)
-        if (w_q[i] == -128)
-            return fail(PTQ_ERR_VALUE, "w_q[%lld] = -128 is outside the symmetric range [-127,127]", i);
+    if (const void *bad = std::memchr(w_q, 0x80, static_cast<size_t>(N) * K))
+        return fail(PTQ_ERR_VALUE, "w_q[%lld] = -128 is outside the symmetric range [-127,127]",
+                    static_cast<long long>(static_cast<const int8_t *>(bad) - w_q));
 
-    int dev = -1;
+    int dev = -1, major = 0, minor = 0, sms = 0;
     PTQ_CUDA(cudaGetDevice(&dev));
-    cudaDeviceProp prop;
-    PTQ_CUDA(cudaGetDeviceProperties(&prop, dev));
-    if (prop.major != 10 || prop.minor != 0)
-        return fail(PTQ_ERR_ARCH, "device %d is compute capability %d.%d; this library needs 10.0 (sm_100a)", dev,
-                    prop.major, prop.minor);
+    PTQ_CUDA(cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev));
+    PTQ_CUDA(cudaDeviceGetAttribute(&minor, cudaDevAttrComputeCapabilityMinor, dev));
+    PTQ_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    if (major != 10 || minor != 0)
+        return fail(PTQ_ERR_ARCH, "device %d is compute capability %d.%d; this library needs 10.0 (sm_100a)", dev, major, minor);
 
     ptq_linear *h = new (std::nothrow) ptq_linear();
     if (!h) return fail(PTQ_ERR_NOMEM, "host allocation failed");
@@ -772,7 +753,7 @@ static ptq_status_t create_impl(ptq_linear_t **out, int K, int N, int T, const i
     h->T = T;
     h->Kpad = round_up(K, 16);
     h->device = dev;
-    h->num_sms = prop.multiProcessorCount;
+    h->num_sms = sms;
     h->fast_div = fast;
     h->n_tiles = (N + ptq::kMaxBN - 1) / ptq::kMaxBN;
     if (h->n_tiles == 1)
@@ -791,41 +772,64 @@ static ptq_status_t create_impl(ptq_linear_t **out, int K, int N, int T, const i
     if (h->as_ok && h->as_n_tiles * h->as_BN > Npad) Npad = h->as_n_tiles * h->as_BN;
     const int Nvec = round_up(Npad, 64) + 64;
     const int Kvec = round_up(K, 16);
-    std::vector<int8_t> wpad(static_cast<size_t>(Npad) * h->Kpad, 0);
-    for (int n = 0; n < N; ++n) std::memcpy(&wpad[static_cast<size_t>(n) * h->Kpad], w_q + static_cast<size_t>(n) * K, K);
-    std::vector<float> rs(Kvec, 1.0f), sp(Kvec, 1.0f), rdx(T);
-    for (int k = 0; k < K; ++k) {
-        sp[k] = smooth[k];
-        rs[k] = 1.0f / smooth[k];
+    // One host image of all parameters, one allocation and one copy: a device allocation costs more than the copy does.
+    size_t total = 0;
+    auto place = [&](size_t bytes) {
+        const size_t at = total;
+        total += (bytes + 255) / 256 * 256;
+        return at;
+    };
+    const size_t o_w = place(static_cast<size_t>(Npad) * h->Kpad), o_dw = place(sizeof(float) * Nvec),
+                 o_bias = place(sizeof(float) * Nvec), o_s = place(sizeof(float) * Kvec), o_rs = place(sizeof(float) * Kvec),
+                 o_dx = place(sizeof(float) * T), o_dx2 = place(sizeof(float2) * T),
+                 o_zp = place(h->asym ? sizeof(int) * T : 0), o_wsum = place(h->asym ? sizeof(int) * Nvec : 0),
+                 o_status = place(sizeof(unsigned));
+    std::vector<unsigned char> image(total, 0);
+    int8_t *wpad = reinterpret_cast<int8_t *>(&image[o_w]);
+    for (int n = 0; n < N; ++n) std::memcpy(wpad + static_cast<size_t>(n) * h->Kpad, w_q + static_cast<size_t>(n) * K, K);
+    std::memcpy(&image[o_dw], w_step, sizeof(float) * N);
+    if (bias) std::memcpy(&image[o_bias], bias, sizeof(float) * N);
+    float *sp = reinterpret_cast<float *>(&image[o_s]), *rs = reinterpret_cast<float *>(&image[o_rs]);
+    for (int k = 0; k < Kvec; ++k) {
+        sp[k] = k < K ? smooth[k] : 1.0f;
+        rs[k] = 1.0f / sp[k];
     }
-    std::vector<float> dx2(2 * static_cast<size_t>(T));
+    std::memcpy(&image[o_dx], act_step, sizeof(float) * T);
+    float *dx2 = reinterpret_cast<float *>(&image[o_dx2]);
     for (int t = 0; t < T; ++t) {
-        rdx[t] = 1.0f / act_step[t];
         dx2[2 * t] = act_step[t];
-        dx2[2 * t + 1] = rdx[t];
+        dx2[2 * t + 1] = 1.0f / act_step[t];
+    }
+    if (h->asym) {
+        std::memcpy(&image[o_zp], act_zero, sizeof(int) * T);
+        int *wsum = reinterpret_cast<int *>(&image[o_wsum]);
+        for (int n = 0; n < N; ++n) {
+            int acc = 0;
+            for (int k = 0; k < K; ++k) acc += w_q[static_cast<size_t>(n) * K + k];
+            wsum[n] = acc;
+        }
     }
 
     ptq_status_t st = PTQ_OK;
+    auto move_in = [&]() -> ptq_status_t {
+        PTQ_CUDA(cudaMalloc(reinterpret_cast<void **>(&h->d_all), total));
+        PTQ_CUDA(cudaMemcpy(h->d_all, image.data(), total, cudaMemcpyHostToDevice));
+        return PTQ_OK;
+    };
     do {
-        if ((st = upload(reinterpret_cast<void **>(&h->d_w), wpad.data(), wpad.size(), wpad.size())) != PTQ_OK) break;
-        if ((st = upload(reinterpret_cast<void **>(&h->d_dw), w_step, sizeof(float) * N, sizeof(float) * Nvec)) != PTQ_OK) break;
-        if ((st = upload(reinterpret_cast<void **>(&h->d_bias), bias, bias ? sizeof(float) * N : 0, sizeof(float) * Nvec)) != PTQ_OK) break;
-        if ((st = upload(reinterpret_cast<void **>(&h->d_s), sp.data(), sizeof(float) * Kvec, sizeof(float) * Kvec)) != PTQ_OK) break;
-        if ((st = upload(reinterpret_cast<void **>(&h->d_rs), rs.data(), sizeof(float) * Kvec, sizeof(float) * Kvec)) != PTQ_OK) break;
-        if ((st = upload(reinterpret_cast<void **>(&h->d_dx), act_step, sizeof(float) * T, sizeof(float) * T)) != PTQ_OK) break;
-        if ((st = upload(reinterpret_cast<void **>(&h->d_rdx), rdx.data(), sizeof(float) * T, sizeof(float) * T)) != PTQ_OK) break;
-        if ((st = upload(reinterpret_cast<void **>(&h->d_dx2), dx2.data(), sizeof(float) * 2 * T, sizeof(float) * 2 * T)) != PTQ_OK) break;
-        if ((st = upload(reinterpret_cast<void **>(&h->d_status), nullptr, 0, sizeof(unsigned))) != PTQ_OK) break;
+        if ((st = move_in()) != PTQ_OK) break;
+        h->d_w = reinterpret_cast<int8_t *>(h->d_all + o_w);
+        h->d_dw = reinterpret_cast<float *>(h->d_all + o_dw);
+        h->d_bias = reinterpret_cast<float *>(h->d_all + o_bias);
+        h->d_s = reinterpret_cast<float *>(h->d_all + o_s);
+        h->d_rs = reinterpret_cast<float *>(h->d_all + o_rs);
+        h->d_dx = reinterpret_cast<float *>(h->d_all + o_dx);
+        h->d_dx2 = reinterpret_cast<float2 *>(h->d_all + o_dx2);
         if (h->asym) {
-            std::vector<int> wsum(Nvec, 0);
-            for (int n = 0; n < N; ++n) {
-                int acc = 0;
-                for (int k = 0; k < K; ++k) acc += w_q[static_cast<size_t>(n) * K + k];
-                wsum[n] = acc;
-            }
-            if ((st = upload(reinterpret_cast<void **>(&h->d_zp), act_zero, sizeof(int) * T, sizeof(int) * T)) != PTQ_OK) break;
-            if ((st = upload(reinterpret_cast<void **>(&h->d_wsum), wsum.data(), sizeof(int) * Nvec, sizeof(int) * Nvec)) != PTQ_OK) break;
+            h->d_zp = reinterpret_cast<int *>(h->d_all + o_zp);
+            h->d_wsum = reinterpret_cast<int *>(h->d_all + o_wsum);
         }
+        h->d_status = reinterpret_cast<unsigned *>(h->d_all + o_status);
         st = make_map_2d(&h->tmW, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, h->d_w, static_cast<unsigned long long>(K),
                          static_cast<unsigned long long>(Npad), static_cast<unsigned long long>(h->Kpad), ptq::kBK,
                          static_cast<unsigned>(h->BN));

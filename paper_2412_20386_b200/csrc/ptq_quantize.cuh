@@ -209,8 +209,6 @@ struct QuantParams {
     int8_t *q;           // [M, q_pitch]
     const float *s;      // [K]
     const float *rs;     // [K]  RN(1/s)
-    const float *dx;     // [T]
-    const float *rdx;    // [T]  RN(1/dx)
     const float2 *dx2;   // [T]  {dx, RN(1/dx)} interleaved (one 8-byte load)
     const int *zp;       // [T]  zero offsets (asymmetric layers), else nullptr
     long long M;
