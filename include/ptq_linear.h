@@ -128,7 +128,8 @@ size_t ptq_linear_workspace_bytes(const ptq_linear_t *h, int B, unsigned flags);
  *   workspace  device, at least ptq_linear_workspace_bytes(h,B,flags) bytes, 16-byte aligned;
  *              contents are scratch.  May be NULL with PTQ_FLAG_FUSED_PROLOGUE.
  *   flags      PTQ_FLAG_NONE: quantize kernel, then GEMM+dequant kernel (one of three variants chosen from
- *              the shape, all with the same bits: see ptq_linear_gemm_variant).
+ *              the shape, all with the same bits: see ptq_linear_gemm_variant); few rows take one kernel for
+ *              both, which leaves the workspace untouched (same bits).
  *              PTQ_FLAG_FUSED_PROLOGUE: one kernel; same results bit for bit.  Layers whose shape the
  *              fused kernel does not cover fall back to the two-kernel path and then need the workspace
  *              (ptq_linear_fused_supported tells which).
@@ -211,8 +212,8 @@ ptq_status_t ptq_linear_gemm_dequant(const ptq_linear_t *h, const void *q_int8, 
 int ptq_linear_code_pitch(const ptq_linear_t *h);
 
 /*
- * Which G1 + E1 kernel (Sec. 5.1; Appendix B.1, parts 3-4) a forward pass over B images takes on the
- * default path, assuming a 16-byte aligned y with N % 8 == 0 (otherwise always the first):
+ * Which G1 + E1 kernel (Sec. 5.1; Appendix B.1, parts 3-4) ptq_linear_gemm_dequant, and a forward pass that
+ * runs it, takes for B images, assuming a 16-byte aligned y with N % 8 == 0 (otherwise always the first):
  *   0  ptq_gemm_dequant_kernel          operand stages streamed per tile, eight epilogue warps per tile
  *   1  ptq_gemm_dequant_kernel, teams   same, the epilogue warps in two teams, one per accumulator
  *                                       (K <= 384 and at least three tiles per SM)

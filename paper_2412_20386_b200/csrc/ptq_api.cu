@@ -23,6 +23,7 @@
 #include "ptq_probe.cuh"
 #include "ptq_quantize.cuh"
 #include "ptq_quantize_dynamic.cuh"
+#include "ptq_small.cuh"
 
 namespace {
 
@@ -150,6 +151,7 @@ struct ptq_linear {
     bool as_ok = false;
     int as_BN = 0, as_n_tiles = 0, as_w_stages = 0, as_w_stage_bytes = 0, as_staging = 0, as_smem = 0;
     CUtensorMap tmWas;
+    CUtensorMap tmWsmall;      // box of 128 rows: the one-kernel path for few rows
     mutable MapCache codes_maps, y_maps;   // tensor maps of caller buffers seen so far
 };
 
@@ -617,6 +619,88 @@ ptq_status_t launch_fused(const ptq_linear *h, const void *x, long long M, void 
                : launch_fused_kernel<ptq::ptq_fused_linear_kernel<false, false>>(h, tmY, fp, grid, stream);
 }
 
+// The one-kernel path for few rows: taken where its CTAs (128 output channels x `tn` tokens) are all resident at once.
+struct SmallPlan {
+    int tn, grid, min_ctas;
+};
+
+// 16 tokens per CTA while that makes at most one CTA per SM, then 32 (the weights of a CTA are loaded half as often), then
+// the same two with two CTAs per SM where shared memory allows.  Beyond that a CTA waits for another to leave and the
+// quantization repeated per 128 output channels shows: the two kernels are faster.  us, one kernel against two:
+//   rows x K -> N     197 x 384 -> 1536  (156 CTAs, two per SM)  4.2 / 6.8     788 x 768 -> 384  (75 CTAs)   6.3 / 8.0
+//                     788 x 192 -> 768   (150, two per SM)       4.2 / 6.6    3152 x 384 -> 192  (198)       6.1 / 7.7
+//   not taken:        788 x 384 -> 1536  (300)                   8.4 / 7.4   12608 x 384 -> 44   (394)      11.4 / 9.4
+bool plan_small(const ptq_linear *h, long long M, SmallPlan &pl)
+{
+    if (h->k_blocks > ptq::kSmallMaxKBlocks) return false;
+    const long long n_tiles = (h->N + ptq::kSmallRows - 1) / ptq::kSmallRows;
+    for (int per_sm = 1; per_sm <= 2; ++per_sm)
+        for (int tn = 16; tn <= 32; tn += 16) {
+            const long long grid = (M + tn - 1) / tn * n_tiles;
+            const int smem = ptq::small_smem_bytes(tn, h->k_blocks, h->K);
+            if (grid > static_cast<long long>(per_sm) * h->num_sms || per_sm * (smem + 1024) > ptq::kSmallSmemPerSm ||
+                smem > ptq::kSmallSmemLimit)
+                continue;
+            pl.tn = tn;
+            pl.grid = static_cast<int>(grid);
+            pl.min_ctas = per_sm;
+            return true;
+        }
+    return false;
+}
+
+template <int kMode, int kTN, int kMinCtas>
+ptq_status_t launch_small_kernel(const ptq_linear *h, const ptq::SmallParams &p, int grid, cudaStream_t stream)
+{
+    const ptq_status_t st = ensure_smem<ptq::ptq_small_kernel<kMode, kTN, kMinCtas>>(h->device, ptq::kSmallSmemLimit);
+    if (st != PTQ_OK) return st;
+    PTQ_CUDA(launch_pdl(ptq::ptq_small_kernel<kMode, kTN, kMinCtas>, grid, ptq::kSmallThreads,
+                        ptq::small_smem_bytes(kTN, h->k_blocks, h->K), stream, h->tmWsmall, p));
+    g_launches.fetch_add(1, std::memory_order_relaxed);
+    PTQ_CUDA(cudaGetLastError());
+    return PTQ_OK;
+}
+
+ptq_status_t launch_small(const ptq_linear *h, const SmallPlan &pl, const void *x, long long M, void *y, void *acc_out, cudaStream_t stream)
+{
+    ptq::SmallParams p;
+    p.x = static_cast<const __half *>(x);
+    p.s = h->d_s;
+    p.rs = h->d_rs;
+    p.dx2 = h->d_dx2;
+    p.zp = h->d_zp;
+    p.wsum = h->d_wsum;
+    p.dw = h->d_dw;
+    p.bias = h->d_bias;
+    p.y = static_cast<__half *>(y);
+    p.acc_out = static_cast<int32_t *>(acc_out);
+    p.status = h->d_status;
+    p.M = static_cast<int>(M);
+    p.N = h->N;
+    p.K = h->K;
+    p.T = h->T;
+    p.k_blocks = h->k_blocks;
+    p.last_mmas = h->last_mmas;
+    p.n_tiles = (h->N + ptq::kSmallRows - 1) / ptq::kSmallRows;
+    const uintptr_t x_align = reinterpret_cast<uintptr_t>(x) | static_cast<uintptr_t>(2 * h->K);
+    p.ld_bytes = x_align % 16 == 0 ? 16 : x_align % 8 == 0 ? 8 : 2;
+    p.fast = h->fast_div ? 1 : 0;
+    p.fd_T = ptq::make_fastdiv(static_cast<unsigned>(h->T));
+    p.fd_cpr = ptq::make_fastdiv(static_cast<unsigned>((h->K + 7) / 8));
+    p.fd_n_tiles = ptq::make_fastdiv(static_cast<unsigned>(p.n_tiles));
+    auto go = [&](auto mode) {
+        constexpr int kMode = decltype(mode)::value;
+        if (pl.min_ctas == 1)
+            return pl.tn == 16 ? launch_small_kernel<kMode, 16, 1>(h, p, pl.grid, stream)
+                               : launch_small_kernel<kMode, 32, 1>(h, p, pl.grid, stream);
+        return pl.tn == 16 ? launch_small_kernel<kMode, 16, 2>(h, p, pl.grid, stream)
+                           : launch_small_kernel<kMode, 32, 2>(h, p, pl.grid, stream);
+    };
+    if (h->act_bits == 4) return go(std::integral_constant<int, ptq::kCodeS4>());
+    if (h->asym) return go(std::integral_constant<int, ptq::kCodeU8>());
+    return go(std::integral_constant<int, ptq::kCodeS8>());
+}
+
 bool fused_usable(const ptq_linear *h) { return h->as_ok && h->K % 16 == 0; }
 
 // Scratch for ptq_linear_forward_static: lives in the library image on every device that loads it.
@@ -845,6 +929,10 @@ static ptq_status_t create_impl(ptq_linear_t **out, int K, int N, int T, const i
                              ptq::kBK, static_cast<unsigned>(h->as_BN));
         else
             h->tmWas = h->tmW;
+        if (st != PTQ_OK) break;
+        st = make_map_2d(&h->tmWsmall, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, h->d_w, static_cast<unsigned long long>(K),
+                         static_cast<unsigned long long>(Npad), static_cast<unsigned long long>(h->Kpad), ptq::kBK,
+                         ptq::kSmallRows);
     } while (0);
     if (st != PTQ_OK) {
         char keep[sizeof(g_err)];
@@ -970,6 +1058,13 @@ ptq_status_t ptq_linear_forward_debug(const ptq_linear_t *h, const void *x_fp16,
     if (ranges_overlap(workspace, need, y_fp16, static_cast<size_t>(M) * h->N * 2) ||
         ranges_overlap(workspace, need, x_fp16, static_cast<size_t>(M) * h->K * 2))
         return fail(PTQ_ERR_VALUE, "workspace overlaps x or y");
+    SmallPlan pl;
+    if (!(flags & PTQ_FLAG_CTA_PAIR) && plan_small(h, M, pl)) {
+        // one kernel; the codes never exist in memory: a requested tap is produced by the quantize kernel on its own
+        if ((st = launch_small(h, pl, x_fp16, M, y_fp16, acc_int32_out, s)) != PTQ_OK) return st;
+        if (q_int8_out) return launch_quantize(h, x_fp16, M, q_int8_out, h->K, s);
+        return PTQ_OK;
+    }
     if ((st = launch_quantize(h, x_fp16, M, workspace, h->Kpad, s)) != PTQ_OK) return st;
     if ((st = launch_gemm(h, workspace, M, y_fp16, acc_int32_out, s, (flags & PTQ_FLAG_CTA_PAIR) != 0)) != PTQ_OK)
         return st;
@@ -997,9 +1092,11 @@ ptq_status_t ptq_linear_forward_static(const ptq_linear_t *h, const void *x_fp16
                     "B*T*pitch = %llu bytes of codes exceed the built-in scratch of %u bytes; "
                     "split the batch or use ptq_linear_forward with a caller workspace",
                     need, PTQ_STATIC_SCRATCH_BYTES);
+    cudaStream_t s = static_cast<cudaStream_t>(stream);
+    SmallPlan pl;
+    if (plan_small(h, M, pl)) return launch_small(h, pl, x_fp16, M, y_fp16, nullptr, s);
     void *scratch = nullptr;
     if ((st = static_scratch_address(h->device, &scratch)) != PTQ_OK) return st;
-    cudaStream_t s = static_cast<cudaStream_t>(stream);
     if ((st = launch_quantize(h, x_fp16, M, scratch, h->Kpad, s)) != PTQ_OK) return st;
     return launch_gemm(h, scratch, M, y_fp16, nullptr, s);
 }

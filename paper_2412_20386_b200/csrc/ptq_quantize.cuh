@@ -182,7 +182,7 @@ __device__ __forceinline__ bool quantize8_magic(uint32_t x0, uint32_t x1, uint32
 }
 
 // Exact route for the same 8 channels: two correctly rounded divisions per element.  s8 / rs8 point
-// at the channels' s and RN(1/s) in global memory.
+// at the channels' s and RN(1/s), in global or shared memory.
 template <bool kFast, int kMode = kCodeS8>
 __device__ __noinline__ void quantize8_exact(uint32_t x0, uint32_t x1, uint32_t x2, uint32_t x3, const float *s8,
                                              const float *rs8, float dx, float rdx, uint32_t &lo, uint32_t &hi,
@@ -194,9 +194,9 @@ __device__ __noinline__ void quantize8_exact(uint32_t x0, uint32_t x1, uint32_t 
     for (int i = 0; i < 8; ++i) {
         const __half hv = __ushort_as_half(static_cast<unsigned short>(xw[i >> 1] >> ((i & 1) * 16)));
         const float f = __half2float(hv);
-        const float sv = __ldg(s8 + i);
+        const float sv = s8[i];
         if (kFast && fabsf(f) <= 65504.0f)
-            c[i] = quantize_fast<kMode>(f, sv, __ldg(rs8 + i), dx, rdx, z);
+            c[i] = quantize_fast<kMode>(f, sv, rs8[i], dx, rdx, z);
         else
             c[i] = quantize_ieee<kMode>(f, sv, dx, z);
     }
