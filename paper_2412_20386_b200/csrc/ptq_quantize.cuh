@@ -83,14 +83,18 @@ __device__ __forceinline__ uint32_t pack4(int a, int b, int c, int d)
     return __byte_perm(ab, cd, 0x5410);
 }
 
-// Screening threshold of the fast route below.  v' = x * (RN(1/s) * RN(1/dx)) differs from the
-// defined value v = RN(RN(x/s)/dx) by six roundings: |v' - v| <= 6 * 2^-24 * (1 + tiny) * |v|, which is
-// below 4.6e-5 for |v| <= 127.5, the largest magnitude at which a rounding tie still changes the
-// clamped code.  If v' is farther than 6e-5 from every half-integer, rint(v') = rint(v).
-constexpr float kScreenThreshold = 0.49994f;
-// Asymmetric codes: rint(v) ranges over [-255, 255] before the offset, so ties matter up to |v| = 255.5,
-// where six roundings amount to 9.2e-5; the band is widened to 1.2e-4 accordingly.
-constexpr float kScreenThresholdAsym = 0.49988f;
+// Tie band of the fast routes below.  v' = x * (RN(1/s) * RN(1/dx)) differs from the defined value
+// v = RN(RN(x/s)/dx) by six roundings: |v' - v| <= 6 * 2^-24 * (1 + tiny) * |v| < 3.6e-7 * |v|.  If no v' of a chunk is larger
+// than `big` and none lies within 4e-7 * big + 1e-7 of a half-integer, rint(v') = rint(v) for all of them.  The band grows
+// with the chunk's largest magnitude and not with the largest possible one: a chunk of 8 typical values needs a fifth
+// of the 6e-5 that |v| = 127.5 does, and the exact route behind the band stalls its warp for a microsecond.  A constant
+// 6e-5 cost 8 - 13 % of the kernel: 50432 x 768 22.0 -> 20.2 us, 50432 x 1536 41.2 -> 39.0, 12608 x 384 5.8 -> 5.0.
+// Beyond kTieLimit no tie changes the clamped code any more (|v| = 127.5, or 255.5 before the offset).
+constexpr float kTieSlope = 4.0e-7f, kTieEdge = 0.4999999f, kTieLimit = 256.0f;
+__device__ __forceinline__ bool clear_of_ties(float worst, float big)
+{
+    return __fmaf_rn(big, kTieSlope, worst) <= kTieEdge;
+}
 constexpr float kRoundMagic = 12582912.0f;   // 1.5 * 2^23: (v + magic) - magic = rint(v) for |v| < 2^22
 
 // |v - rint(v)| for |v| < 2^22; NaN for NaN and infinite v; meaningless (but finite or NaN) beyond.
@@ -98,39 +102,6 @@ __device__ __forceinline__ float dist_to_integer(float v)
 {
     const float r = __fadd_rn(__fadd_rn(v, kRoundMagic), -kRoundMagic);
     return fabsf(__fadd_rn(v, -r));
-}
-
-// Fast route for 8 consecutive channels held as 4 packed half2 words: one multiply by the combined
-// reciprocal c = RN(RN(1/s) * RN(1/dx)), the saturating round-to-nearest-even conversion, and a
-// distance-to-tie test.  Returns true when one of the 8 values sits within the error bound of a
-// rounding tie, in which case the caller recomputes the 8 codes with the two exact divisions.
-// Values beyond +-127.5 clamp to the same code whichever way a tie falls, NaN converts to 0 and
-// infinities saturate on both routes, so whether such values pass the test or not only costs time:
-// the final codes are always those of the definition.
-// Valid only when every scale lies in [2^-30, 2^30] (no under/overflow in c or x * c).
-// Unsigned codes: clip(rint(v') + z, 0, 255); ties of v' are still the only place where v' and v
-// can disagree, with the wider band of kScreenThresholdAsym.
-template <int kMode = kCodeS8>
-__device__ __forceinline__ bool quantize8_screen(uint32_t x0, uint32_t x1, uint32_t x2, uint32_t x3,
-                                                 const float (&c8)[8], uint32_t &lo, uint32_t &hi, int z = 0)
-{
-    const uint32_t xw[4] = {x0, x1, x2, x3};
-    int c[8];
-    float worst = 0.0f;   // largest distance to an integer; fmaxf drops the NaN that NaN / inf inputs produce,
-                          // which is fine: their codes (0, +-saturation) are the same on both routes
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        __half2 h = *reinterpret_cast<const __half2 *>(&xw[i]);
-        const float2 f = __half22float2(h);
-        const float v0 = __fmul_rn(f.x, c8[2 * i]);
-        const float v1 = __fmul_rn(f.y, c8[2 * i + 1]);
-        c[2 * i] = code_of<kMode>(v0, z);
-        c[2 * i + 1] = code_of<kMode>(v1, z);
-        worst = fmaxf(worst, fmaxf(dist_to_integer(v0), dist_to_integer(v1)));
-    }
-    lo = pack4(c[0], c[1], c[2], c[3]);
-    hi = pack4(c[4], c[5], c[6], c[7]);
-    return worst > (kMode == kCodeU8 ? kScreenThresholdAsym : kScreenThreshold);
 }
 
 // max(a, |b|, |c|) in one instruction (three-input max of sm_100); NaN operands are dropped like fmaxf does.
@@ -147,6 +118,38 @@ __device__ __forceinline__ float max3_abs_nan(float a, float b, float c)
     float r;
     asm("max.NaN.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(fabsf(b)), "f"(fabsf(c)));
     return r;
+}
+
+// Fast route for 8 consecutive channels held as 4 packed half2 words: one multiply by the combined
+// reciprocal c = RN(RN(1/s) * RN(1/dx)), the saturating round-to-nearest-even conversion, and a
+// distance-to-tie test.  Returns true when one of the 8 values sits within the tie band, in which case the caller recomputes the 8 codes with the two exact divisions.
+// Values beyond +-127.5 clamp to the same code whichever way a tie falls, NaN converts to 0 and
+// infinities saturate on both routes, so whether such values pass the test or not only costs time:
+// the final codes are always those of the definition.
+// Valid only when every scale lies in [2^-30, 2^30] (no under/overflow in c or x * c).
+// Unsigned codes: clip(rint(v') + z, 0, 255); ties of v' are still the only place where v' and v can disagree.
+template <int kMode = kCodeS8>
+__device__ __forceinline__ bool quantize8_screen(uint32_t x0, uint32_t x1, uint32_t x2, uint32_t x3,
+                                                 const float (&c8)[8], uint32_t &lo, uint32_t &hi, int z = 0)
+{
+    const uint32_t xw[4] = {x0, x1, x2, x3};
+    int c[8];
+    float worst = 0.0f, big = 0.0f;   // largest distance to an integer and magnitude; fmaxf drops the NaN that NaN / inf
+                                      // inputs produce, which is fine: their codes (0, +-saturation) are the same on both routes
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        __half2 h = *reinterpret_cast<const __half2 *>(&xw[i]);
+        const float2 f = __half22float2(h);
+        const float v0 = __fmul_rn(f.x, c8[2 * i]);
+        const float v1 = __fmul_rn(f.y, c8[2 * i + 1]);
+        c[2 * i] = code_of<kMode>(v0, z);
+        c[2 * i + 1] = code_of<kMode>(v1, z);
+        worst = fmaxf(worst, fmaxf(dist_to_integer(v0), dist_to_integer(v1)));
+        big = max3_abs(big, v0, v1);
+    }
+    lo = pack4(c[0], c[1], c[2], c[3]);
+    hi = pack4(c[4], c[5], c[6], c[7]);
+    return !clear_of_ties(worst, fminf(big, kTieLimit));
 }
 
 // First-level route for signed codes, without any float-to-integer conversion instruction (those run
@@ -178,7 +181,7 @@ __device__ __forceinline__ bool quantize8_magic(uint32_t x0, uint32_t x1, uint32
     }
     lo = pack4(static_cast<int>(tb[0]), static_cast<int>(tb[1]), static_cast<int>(tb[2]), static_cast<int>(tb[3]));
     hi = pack4(static_cast<int>(tb[4]), static_cast<int>(tb[5]), static_cast<int>(tb[6]), static_cast<int>(tb[7]));
-    return !(worst <= kScreenThreshold && big <= (kMode == kCodeS4 ? 7.25f : 127.25f));
+    return !(clear_of_ties(worst, big) && big <= (kMode == kCodeS4 ? 7.25f : 127.25f));
 }
 
 // Exact route for the same 8 channels: two correctly rounded divisions per element.  s8 / rs8 point
@@ -252,8 +255,10 @@ template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
 // The three routes for one chunk of 8 channels, cheapest first; every route that returns codes returns
-// the codes of the definition.
-template <bool kFast, int kMode>
+// the codes of the definition.  c8 = RN(RN(1/s) * RN(1/dx)).  kExactRecip = false decides the last route with IEEE
+// divisions instead of reciprocals: more instructions but no 1/s to fetch, for kernels that keep s in shared memory and
+// nothing else at hand (a fetch from L2 stalls one warp for about a microsecond, and a CTA waits for its slowest warp).
+template <bool kFast, int kMode, bool kExactRecip = kFast>
 __device__ __forceinline__ uint2 quantize8(const uint4 &v, const float (&c8)[8], const float *s8, const float *rs8,
                                            float dx, float rdx, int z)
 {
@@ -264,7 +269,7 @@ __device__ __forceinline__ uint2 quantize8(const uint4 &v, const float (&c8)[8],
         if (kMode != kCodeU8) slow = quantize8_magic<kMode>(v.x, v.y, v.z, v.w, c8, out.x, out.y);
         exact = slow && quantize8_screen<kMode>(v.x, v.y, v.z, v.w, c8, out.x, out.y, z);
     }
-    if (exact) quantize8_exact<kFast, kMode>(v.x, v.y, v.z, v.w, s8, rs8, dx, rdx, out.x, out.y, z);
+    if (exact) quantize8_exact<kExactRecip, kMode>(v.x, v.y, v.z, v.w, s8, rs8, dx, rdx, out.x, out.y, z);
     return out;
 }
 

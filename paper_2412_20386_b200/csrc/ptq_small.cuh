@@ -38,7 +38,7 @@ constexpr int kSmallSmemPerSm = 233472;                       // 228 KB per SM, 
 
 struct SmallParams {
     const __half *x;
-    const float *s, *rs;      // [round_up(K,16)], padded with ones
+    const float *s, *rs;      // [round_up(K,16)] s and 1/s, padded with ones
     const float2 *dx2;        // [T] {dx, RN(1/dx)}
     const int *zp, *wsum;     // asymmetric layers
     const float *dw, *bias;   // zero padded
@@ -186,10 +186,10 @@ ptq_small_kernel(const __grid_constant__ CUtensorMap tmW, const SmallParams p)
                     const float2 c0 = __fmul2_rn(make_float2(q0.x, q0.y), rd2), c1 = __fmul2_rn(make_float2(q0.z, q0.w), rd2);
                     const float2 c2 = __fmul2_rn(make_float2(q1.x, q1.y), rd2), c3 = __fmul2_rn(make_float2(q1.z, q1.w), rd2);
                     const float c8[8] = {c0.x, c0.y, c1.x, c1.y, c2.x, c2.y, c3.x, c3.y};
-                    o = quantize8<true, kMode>(v[j], c8, s_s + kc * 8, p.rs + kc * 8, dx, rdx, z);
+                    o = quantize8<true, kMode, false>(v[j], c8, s_s + kc * 8, nullptr, dx, rdx, z);
                 } else {
                     const float none[8] = {};
-                    o = quantize8<false, kMode>(v[j], none, s_s + kc * 8, p.rs + kc * 8, dx, rdx, z);
+                    o = quantize8<false, kMode>(v[j], none, s_s + kc * 8, nullptr, dx, rdx, z);
                 }
                 const uint32_t dst = code_col + static_cast<uint32_t>(row) * 128u +
                                      (((static_cast<uint32_t>(kc & 15) >> 1) ^ static_cast<uint32_t>(row & 7)) << 4);
