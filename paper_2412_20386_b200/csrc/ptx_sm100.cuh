@@ -152,6 +152,16 @@ __device__ __forceinline__ void fence_proxy_async_smem()
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }
 
+// ---------------------------------------------------------------- L2 prefetch
+// Ask for `bytes` contiguous bytes (16-byte aligned address and size) to be brought to L2.  A hint: nothing waits for it
+// and nothing is read, so it may be issued before griddep_wait() even for data the kernel in front still writes (L2 is
+// where those writes become visible).  Kernels issue it for their activations as soon as they start: the dependency is
+// released about 2 us after the last CTA of the kernel in front ends, and the memory latency passes meanwhile.
+__device__ __forceinline__ void l2_prefetch(const void *p, uint32_t bytes)
+{
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
+}
+
 // ---------------------------------------------------------------- TMA
 __device__ __forceinline__ void prefetch_tensormap(const CUtensorMap *m)
 {
