@@ -152,6 +152,7 @@ struct ptq_linear {
     int as_BN = 0, as_n_tiles = 0, as_w_stages = 0, as_w_stage_bytes = 0, as_staging = 0, as_smem = 0;
     CUtensorMap tmWas;
     CUtensorMap tmWsmall;      // box of 128 rows: the one-kernel path for few rows
+    CUtensorMap tmWbn[4];      // boxes of 64, 128, 192 and 256 rows: tile widths chosen per call (choose_bn)
     mutable MapCache codes_maps, y_maps;   // tensor maps of caller buffers seen so far
 };
 
@@ -399,6 +400,52 @@ bool gemm_teams(const ptq_linear *h, const ptq::GemmParams &p, bool tma_store, b
     return PTQ_GEMM_TEAMS && tma_store && short_k && tiles >= static_cast<long long>(PTQ_GEMM_TEAM_MIN_ROUNDS) * h->num_sms;
 }
 
+// Cycles of the busiest CTA of the streaming kernel with tiles of `bn` columns, as measured on the workloads: an MMA of
+// K = 32 takes 57 + 0.54 bn, the eight epilogue warps take 550 per tile and 700 per pair of 64-column steps, the hand-overs
+// 300 per tile.
+double gemm_cycles(const ptq_linear *h, const ptq::GemmParams &p, int bn)
+{
+    const long long tiles = static_cast<long long>(p.m_tiles) * ((h->N + bn - 1) / bn);
+    const double rounds = static_cast<double>((tiles + h->num_sms - 1) / h->num_sms);
+    const int steps = (bn + 63) / 64;
+    const double mma = (h->K + 31) / 32 * (57.0 + 0.54 * bn);
+    const double epi = 550.0 + 700.0 * ((steps + 1) / 2);
+    return mma + (rounds - 1.0) * (mma > epi ? mma : epi) + epi + 300.0 * rounds;
+}
+
+// Tile width of the streaming kernel for this many rows: the layer's own (as few N tiles as possible), unless another
+// leaves the busiest CTA clearly less to do: idle SMs in a single round, or a last round that is nearly empty.  Layer,
+// both kernels, us: 1568 x 1536 -> 768 (256 -> 128 columns) 10.6 -> 9.7, 2793 x 1536 -> 768 (256 -> 192) 11.7 -> 10.8,
+// 12544 x 768 -> 384 (192 -> 128) 14.6 -> 14.1, 6304 x 384 -> 1536 (256 -> 192) 11.4 -> 11.0.  The margin keeps what the model cannot
+// tell apart: 11229 x 520 -> 600 (predicted -7 %) measured +1 %.  Widths that make the epilogue run in teams are not
+// compared: with several rounds and a short main loop the widths are within 3 % of one another either way.
+int choose_bn(const ptq_linear *h, const ptq::GemmParams &p)
+{
+    auto teams = [&](int bn) {
+        return h->k_blocks <= PTQ_GEMM_SHORT_K_BLOCKS && static_cast<long long>(p.m_tiles) * ((h->N + bn - 1) / bn) >=
+                                                            static_cast<long long>(PTQ_GEMM_TEAM_MIN_ROUNDS) * h->num_sms;
+    };
+    int best = h->BN;
+    if (teams(best)) return best;
+    double best_cost = 0.93 * gemm_cycles(h, p, best);
+    for (int bn = 64; bn <= ptq::kMaxBN && bn < h->N + 64; bn += 64) {
+        if (teams(bn)) continue;
+        const double cost = gemm_cycles(h, p, bn);
+        if (cost < best_cost) {
+            best = bn;
+            best_cost = cost;
+        }
+    }
+    return best;
+}
+
+void set_bn(const ptq_linear *h, ptq::GemmParams &p, int bn)
+{
+    p.BN = bn;
+    p.n_tiles = (h->N + bn - 1) / bn;
+    p.fd_n_tiles = ptq::make_fastdiv(static_cast<unsigned>(p.n_tiles));
+}
+
 // G1+E1 launch on codes [M, Kpad] at `codes`.
 // dx_rows != nullptr: the steps are per ROW (dynamic comparator), i.e. dx = dx_rows and T = M.
 ptq_status_t launch_gemm(const ptq_linear *h, const void *codes, long long M, void *y, void *acc_out,
@@ -482,10 +529,6 @@ ptq_status_t launch_gemm(const ptq_linear *h, const void *codes, long long M, vo
         PTQ_CUDA(cudaGetLastError());
         return PTQ_OK;
     }
-    const long long tiles = static_cast<long long>(p.m_tiles) * p.n_tiles;
-    // Short main loop (K <= 384) and several tiles per CTA: the epilogue sets the pace and runs in two teams of
-    // four warps, one per accumulator; otherwise all eight warps share every tile (shorter latency of a tile).
-    const bool teams = gemm_teams(h, p, tma_store, short_k);
     const bool dbg = acc_out != nullptr;
     if (plan_panel(h, p, tma_store)) {
         // several N tiles and 512 <= K <= 768: the codes of a row panel stay in shared memory for `group` tiles
@@ -503,9 +546,16 @@ ptq_status_t launch_gemm(const ptq_linear *h, const void *codes, long long M, vo
         PTQ_CUDA(cudaGetLastError());
         return PTQ_OK;
     }
+    const int bn = choose_bn(h, p);
+    if (bn != h->BN) set_bn(h, p, bn);
+    const CUtensorMap &tmW = bn != h->BN ? h->tmWbn[bn / 64 - 1] : h->tmW;
+    const long long tiles = static_cast<long long>(p.m_tiles) * p.n_tiles;
+    // Short main loop (K <= 384) and several tiles per CTA: the epilogue sets the pace and runs in two teams of
+    // four warps, one per accumulator; otherwise all eight warps share every tile (shorter latency of a tile).
+    const bool teams = gemm_teams(h, p, tma_store, short_k);
     const int grid = static_cast<int>(tiles < h->num_sms ? tiles : h->num_sms);
     auto go = [&](auto kern) -> ptq_status_t {
-        PTQ_CUDA(launch_pdl(kern, grid, ptq::kGemmThreads, gemm_smem, stream, tmA, h->tmW, tmY, p));
+        PTQ_CUDA(launch_pdl(kern, grid, ptq::kGemmThreads, gemm_smem, stream, tmA, tmW, tmY, p));
         return PTQ_OK;
     };
     ptq_status_t gs;
@@ -854,7 +904,7 @@ static ptq_status_t create_impl(ptq_linear_t **out, int K, int N, int T, const i
     if (h->asym || act_bits != 8) h->as_ok = false;   // these layers run the quantize kernel + single-CTA GEMM kernel only
     int Npad = h->n_tiles * h->BN;
     if (h->as_ok && h->as_n_tiles * h->as_BN > Npad) Npad = h->as_n_tiles * h->as_BN;
-    const int Nvec = round_up(Npad, 64) + 64;
+    const int Nvec = round_up(Npad, 64) + 256;      // the last tile of any width reads at most 255 beyond N, a step 64
     const int Kvec = round_up(K, 16);
     // One host image of all parameters, one allocation and one copy: a device allocation costs more than the copy does.
     size_t total = 0;
@@ -933,6 +983,10 @@ static ptq_status_t create_impl(ptq_linear_t **out, int K, int N, int T, const i
         st = make_map_2d(&h->tmWsmall, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, h->d_w, static_cast<unsigned long long>(K),
                          static_cast<unsigned long long>(Npad), static_cast<unsigned long long>(h->Kpad), ptq::kBK,
                          ptq::kSmallRows);
+        for (int i = 0; i < 4 && st == PTQ_OK; ++i)
+            st = make_map_2d(&h->tmWbn[i], CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, h->d_w, static_cast<unsigned long long>(K),
+                             static_cast<unsigned long long>(Npad), static_cast<unsigned long long>(h->Kpad), ptq::kBK,
+                             static_cast<unsigned>(64 * (i + 1)));
     } while (0);
     if (st != PTQ_OK) {
         char keep[sizeof(g_err)];
@@ -1017,6 +1071,7 @@ int ptq_linear_gemm_variant(const ptq_linear_t *h, int B)
     const bool short_k = h->k_blocks <= PTQ_GEMM_SHORT_K_BLOCKS;
     p.boxes = short_k ? 2 : 1;
     if (plan_panel(h, p, true)) return 2;
+    set_bn(h, p, choose_bn(h, p));
     return gemm_teams(h, p, true, short_k) ? 1 : 0;
 }
 
