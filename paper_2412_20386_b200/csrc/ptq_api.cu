@@ -126,14 +126,15 @@ struct MapCache {
 
 struct ptq_linear {
     int K = 0, N = 0, T = 0;
-    int Kpad = 0;              // pitch of the codes workspace and of the padded weight: K rounded up to 16
+    int Kpad = 0;              // pitch of the codes workspace: K rounded up to 16
+    int w_pitch = 0;           // pitch of the padded weight
     int BN = 0, n_tiles = 0;   // GEMM tiling along N
     int k_blocks = 0, last_mmas = 0;
     bool fast_div = false;     // all scales inside the range where the reciprocal route is exact
     int device = -1;
     int num_sms = 0;
     unsigned char *d_all = nullptr;   // the one allocation that holds all of the following
-    int8_t *d_w = nullptr;     // [n_tiles*BN, Kpad], zero padded
+    int8_t *d_w = nullptr;     // [n_tiles*BN, w_pitch], zero padded
     float *d_dw = nullptr, *d_bias = nullptr;            // [n_tiles*BN rounded up to 64, +64], zero padded
     float *d_s = nullptr, *d_rs = nullptr;               // [round_up(K,16)]
     float *d_dx = nullptr;                               // [T]
@@ -886,6 +887,12 @@ static ptq_status_t create_impl(ptq_linear_t **out, int K, int N, int T, const i
     h->N = N;
     h->T = T;
     h->Kpad = round_up(K, 16);
+    // Whole 128-byte lines per weight row: a TMA box is one 128-byte k-block of up to 256 rows, loaded by every CTA for every
+    // tile, and a row that straddles two lines is two requests to L2 (and the 16-byte rows of a narrow layer send all
+    // CTAs to a handful of lines).  Layers, both kernels: 200704 x 96 -> 384 51.3 -> 43.8 us, 200704 x 192 -> 96 36.5 -> 32.6,
+    // 12608 x 12 -> 384 9.9 -> 8.6, 3940 x 1455 -> 784 18.9 -> 17.2.  The codes keep 16-byte rounding: whole lines there cost
+    // more footprint than they save requests (200704 x 192 -> 96 32.6 -> 35.0).
+    h->w_pitch = round_up(K, 128);
     h->device = dev;
     h->num_sms = sms;
     h->fast_div = fast;
@@ -913,14 +920,14 @@ static ptq_status_t create_impl(ptq_linear_t **out, int K, int N, int T, const i
         total += (bytes + 255) / 256 * 256;
         return at;
     };
-    const size_t o_w = place(static_cast<size_t>(Npad) * h->Kpad), o_dw = place(sizeof(float) * Nvec),
+    const size_t o_w = place(static_cast<size_t>(Npad) * h->w_pitch), o_dw = place(sizeof(float) * Nvec),
                  o_bias = place(sizeof(float) * Nvec), o_s = place(sizeof(float) * Kvec), o_rs = place(sizeof(float) * Kvec),
                  o_dx = place(sizeof(float) * T), o_dx2 = place(sizeof(float2) * T),
                  o_zp = place(h->asym ? sizeof(int) * T : 0), o_wsum = place(h->asym ? sizeof(int) * Nvec : 0),
                  o_status = place(sizeof(unsigned));
     std::vector<unsigned char> image(total, 0);
     int8_t *wpad = reinterpret_cast<int8_t *>(&image[o_w]);
-    for (int n = 0; n < N; ++n) std::memcpy(wpad + static_cast<size_t>(n) * h->Kpad, w_q + static_cast<size_t>(n) * K, K);
+    for (int n = 0; n < N; ++n) std::memcpy(wpad + static_cast<size_t>(n) * h->w_pitch, w_q + static_cast<size_t>(n) * K, K);
     std::memcpy(&image[o_dw], w_step, sizeof(float) * N);
     if (bias) std::memcpy(&image[o_bias], bias, sizeof(float) * N);
     float *sp = reinterpret_cast<float *>(&image[o_s]), *rs = reinterpret_cast<float *>(&image[o_rs]);
@@ -965,27 +972,27 @@ static ptq_status_t create_impl(ptq_linear_t **out, int K, int N, int T, const i
         }
         h->d_status = reinterpret_cast<unsigned *>(h->d_all + o_status);
         st = make_map_2d(&h->tmW, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, h->d_w, static_cast<unsigned long long>(K),
-                         static_cast<unsigned long long>(Npad), static_cast<unsigned long long>(h->Kpad), ptq::kBK,
+                         static_cast<unsigned long long>(Npad), static_cast<unsigned long long>(h->w_pitch), ptq::kBK,
                          static_cast<unsigned>(h->BN));
         if (st != PTQ_OK) break;
         st = make_map_2d(&h->tmWh, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, h->d_w, static_cast<unsigned long long>(K),
-                         static_cast<unsigned long long>(Npad), static_cast<unsigned long long>(h->Kpad), ptq::kBK,
+                         static_cast<unsigned long long>(Npad), static_cast<unsigned long long>(h->w_pitch), ptq::kBK,
                          static_cast<unsigned>(h->BN / 2));
         if (st != PTQ_OK) break;
         h->max_pairs = h->asym ? 0 : query_max_pairs(dev);
         if (h->as_ok)
             st = make_map_2d(&h->tmWas, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, h->d_w, static_cast<unsigned long long>(K),
-                             static_cast<unsigned long long>(Npad), static_cast<unsigned long long>(h->Kpad),
+                             static_cast<unsigned long long>(Npad), static_cast<unsigned long long>(h->w_pitch),
                              ptq::kBK, static_cast<unsigned>(h->as_BN));
         else
             h->tmWas = h->tmW;
         if (st != PTQ_OK) break;
         st = make_map_2d(&h->tmWsmall, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, h->d_w, static_cast<unsigned long long>(K),
-                         static_cast<unsigned long long>(Npad), static_cast<unsigned long long>(h->Kpad), ptq::kBK,
+                         static_cast<unsigned long long>(Npad), static_cast<unsigned long long>(h->w_pitch), ptq::kBK,
                          ptq::kSmallRows);
         for (int i = 0; i < 4 && st == PTQ_OK; ++i)
             st = make_map_2d(&h->tmWbn[i], CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, h->d_w, static_cast<unsigned long long>(K),
-                             static_cast<unsigned long long>(Npad), static_cast<unsigned long long>(h->Kpad), ptq::kBK,
+                             static_cast<unsigned long long>(Npad), static_cast<unsigned long long>(h->w_pitch), ptq::kBK,
                              static_cast<unsigned>(64 * (i + 1)));
     } while (0);
     if (st != PTQ_OK) {
