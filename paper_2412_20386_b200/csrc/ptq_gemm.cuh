@@ -86,6 +86,7 @@ struct GemmParams {
     int use_tma_store; // y is written by TMA (needs N % 8 == 0 and a 16-byte aligned y)
     int y_vec2;        // plain-store path may use 4-byte stores (N even, y 4-byte aligned)
     int y_vec8;        // plain-store path may use 16-byte stores (N % 8 == 0, y 16-byte aligned)
+    int y_evict_first; // TMA stores of y carry the evict-first L2 policy (streaming and panel kernels)
     int y_copy_bytes;  // streaming kernel without TMA stores: bytes per lane of a row copy (8, 4 or 2: alignment of y's rows)
     // Asymmetric layers (zero offset per token position): the codes are unsigned, the tensor core
     // accumulates sum_k c * Wq, and the epilogue subtracts z[t] * sum_k Wq[n,k] to obtain the offset-free
@@ -439,8 +440,12 @@ __device__ __forceinline__ uint32_t epilogue_tile_stream(const GemmParams &p, co
             fence_proxy_async_smem();
             __syncwarp();
             if (lane == 0) {
-                if (n_first < p.N && m_row0 < p.M)
-                    tma_store_2d(tmY, n_first, static_cast<int>(m_row0), box);   // clipped at N and M
+                if (n_first < p.N && m_row0 < p.M) {           // clipped at N and M
+                    if (p.y_evict_first)
+                        tma_store_2d_evict_first(tmY, n_first, static_cast<int>(m_row0), box);
+                    else
+                        tma_store_2d(tmY, n_first, static_cast<int>(m_row0), box);
+                }
                 bulk_commit_group();
             }
         } else {

@@ -186,6 +186,16 @@ __device__ __forceinline__ void tma_store_2d(const CUtensorMap *m, int c0, int c
                  : "memory");
 }
 
+// The same with the evict-first L2 policy, for outputs that L2 cannot hold anyway.
+__device__ __forceinline__ void tma_store_2d_evict_first(const CUtensorMap *m, int c0, int c1, uint32_t smem_src)
+{
+    uint64_t pol;
+    asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol));
+    asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.tile.bulk_group.L2::cache_hint [%0, {%1, %2}], [%3], %4;"
+                 ::"l"(reinterpret_cast<uint64_t>(m)), "r"(c0), "r"(c1), "r"(smem_src), "l"(pol)
+                 : "memory");
+}
+
 __device__ __forceinline__ void bulk_commit_group()
 {
     asm volatile("cp.async.bulk.commit_group;" ::: "memory");
