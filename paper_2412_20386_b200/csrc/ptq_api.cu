@@ -1246,6 +1246,7 @@ ptq_status_t ptq_search_act_step_in(int K, int T, const void *xcal_fp16, int Bc,
     p.K = K;
     p.n_grid = n_grid;
     p.j_lo = j_lo;
+    p.fd_K = ptq::make_fastdiv(static_cast<unsigned>(K));
     const dim3 grid(static_cast<unsigned>(T), static_cast<unsigned>((C + ptq::kSearchCandPerBlock - 1) / ptq::kSearchCandPerBlock));
     ptq::ptq_search_loss_kernel<<<grid, ptq::kSearchThreads, 0, s>>>(p);
     ptq::ptq_search_pick_kernel<<<(T + 127) / 128, 128, 0, s>>>(d_loss, d_base, T, n_grid, j_lo, d_best, d_dx);

@@ -13,6 +13,8 @@
 #include <cuda_fp16.h>
 #include <stdint.h>
 
+#include "ptx_sm100.cuh"
+
 namespace ptq {
 
 constexpr float kCalibFloor = 1e-5f;
@@ -254,6 +256,7 @@ struct SearchParams {
     double *loss;        // [T, n_grid - j_lo + 1]
     int Bc, T, K;
     int n_grid, j_lo;
+    FastDiv fd_K;
 };
 
 __device__ __forceinline__ float search_candidate_step(float base, int j, int n_grid)
@@ -261,33 +264,56 @@ __device__ __forceinline__ float search_candidate_step(float base, int j, int n_
     return __fmul_rn(base, __fdiv_rn(static_cast<float>(j), static_cast<float>(n_grid)));
 }
 
+// Bound by issue: 49 M (element, candidate) pairs at 8 x 197 x 384 x 81.  The integer r = rne(u / Delta) is taken from one FMA,
+// t = RN(u * RN(1/Delta) + 1.5*2^23), whose low mantissa bits hold it; u * RN(1/Delta) is within 1.2e-7 |v| of the defined
+// quotient v, and beyond |v| = 128 every r clamps alike, so r can only be wrong where the distance to r exceeds 0.49998:
+// those elements (3 in 10^4) take the IEEE divisions, which were the whole cost before (an IEEE division, a rounding
+// instruction at an eighth of the rate, and two conversions per pair).
 __global__ void __launch_bounds__(kSearchThreads) ptq_search_loss_kernel(SearchParams p)
 {
     constexpr int C = kSearchCandPerBlock;
+    constexpr float kMagic = 12582912.0f;
     __shared__ double partial[kSearchThreads / 32][C];
     const int t = blockIdx.x;
     const int j0 = p.j_lo + static_cast<int>(blockIdx.y) * C;
     const int ncand = min(C, p.n_grid - j0 + 1);
     const float base = __ldg(p.base + t);
-    float delta[C];
+    float delta[C], rdelta[C];
     double acc[C];
+    bool fast = true;
 #pragma unroll
     for (int c = 0; c < C; ++c) {
         delta[c] = search_candidate_step(base, min(j0 + c, p.n_grid), p.n_grid);
+        rdelta[c] = __fdiv_rn(1.0f, delta[c]);
+        fast = fast && delta[c] >= 9.313225746154785e-10f && delta[c] <= 1073741824.0f;      // 2^-30 .. 2^30
         acc[c] = 0.0;
     }
     const int per_pos = p.Bc * p.K;
+#pragma unroll 2
     for (int i = threadIdx.x; i < per_pos; i += kSearchThreads) {
-        const int b = i / p.K;
+        const int b = static_cast<int>(fd_div(static_cast<unsigned>(i), p.fd_K));
         const int k = i - b * p.K;
-        const float xf = __half2float(p.x[(static_cast<long long>(b) * p.T + t) * p.K + k]);
+        const float xf = __half2float(__ldg(p.x + (static_cast<long long>(b) * p.T + t) * p.K + k));
         const float u = __fdiv_rn(xf, __ldg(p.s + k));
         if (!(fabsf(u) <= 3.402823466e38f)) continue;          // inf and NaN do not enter the loss
+        float r[C], worst = 0.0f;
 #pragma unroll
         for (int c = 0; c < C; ++c) {
-            float r = rintf(__fdiv_rn(u, delta[c]));
-            r = fminf(fmaxf(r, -128.0f), 127.0f);
-            const double e = static_cast<double>(__fmaf_rn(-delta[c], r, u));
+            r[c] = __fadd_rn(__fmaf_rn(u, rdelta[c], kMagic), -kMagic);
+            worst = fmaxf(worst, fabsf(__fmaf_rn(u, rdelta[c], -r[c])));
+        }
+        if (!fast || worst > 0.49998f) {
+#pragma unroll 1
+            for (int c = 0; c < C; ++c) {
+                const float exact = rintf(__fdiv_rn(u, search_candidate_step(base, min(j0 + c, p.n_grid), p.n_grid)));
+#pragma unroll
+                for (int q = 0; q < C; ++q)
+                    if (q == c) r[q] = exact;
+            }
+        }
+#pragma unroll
+        for (int c = 0; c < C; ++c) {
+            const double e = static_cast<double>(__fmaf_rn(-delta[c], fminf(fmaxf(r[c], -128.0f), 127.0f), u));
             acc[c] = fma(e, e, acc[c]);
         }
     }
