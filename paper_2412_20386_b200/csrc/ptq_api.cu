@@ -39,12 +39,12 @@ ptq_status_t fail(ptq_status_t st, const char *fmt, ...)
     return st;
 }
 
-#define PTQ_CUDA(call)                                                                         \
+#define PTQ_CUDA(...)                                                                          \
     do {                                                                                       \
-        cudaError_t e_ = (call);                                                               \
+        cudaError_t e_ = (__VA_ARGS__);                                                        \
         if (e_ != cudaSuccess)                                                                 \
             return fail(e_ == cudaErrorMemoryAllocation ? PTQ_ERR_NOMEM : PTQ_ERR_CUDA,        \
-                        "%s failed: %s", #call, cudaGetErrorString(e_));                       \
+                        "%s failed: %s", #__VA_ARGS__, cudaGetErrorString(e_));                \
     } while (0)
 
 // cuTensorMapEncodeTiled is reached through the runtime's driver entry point query, so the
@@ -334,12 +334,35 @@ ptq_status_t launch_quantize_dynamic(const ptq_linear *h, const void *x, long lo
     p.q_pitch = q_pitch;
     const bool vec = (h->K % 8 == 0) && (reinterpret_cast<uintptr_t>(x) % 16 == 0) &&
                      (reinterpret_cast<uintptr_t>(q) % 8 == 0) && (q_pitch % 8 == 0);
-    const long long rows_per_cta = vec ? 8 * ptq::kDynRowsPerWarp : 8;
+    const int chunks = (h->K / 8 + 31) / 32;                   // per lane, one row per warp
+    const bool row = vec && h->fast_div && chunks <= 6;
+    const int lanes = chunks > 1 || h->K > 128 ? 32 : h->K > 64 ? 16 : 8;
+    const long long rows_per_cta = row ? 256 / lanes : vec ? 8 * ptq::kDynRowsPerWarp : 8;
     long long want = (M + rows_per_cta - 1) / rows_per_cta;
-    const long long cap = static_cast<long long>(h->num_sms) * 8;
+    const long long cap = static_cast<long long>(h->num_sms) * (row ? ptq::dyn_row_ctas_per_sm(chunks) : 8);
     if (want > cap) want = cap;
     if (want < 1) want = 1;
-    if (!vec)
+    if (row) {
+        auto go = [&](auto n, auto l) {
+            return launch_pdl(ptq::ptq_quantize_dynamic_row_kernel<decltype(n)::value, decltype(l)::value>, static_cast<int>(want), 256, 0, stream, p);
+        };
+        const std::integral_constant<int, 32> warp;
+        switch (chunks) {
+            case 1:
+                if (lanes == 8)
+                    PTQ_CUDA(go(std::integral_constant<int, 1>(), std::integral_constant<int, 8>()));
+                else if (lanes == 16)
+                    PTQ_CUDA(go(std::integral_constant<int, 1>(), std::integral_constant<int, 16>()));
+                else
+                    PTQ_CUDA(go(std::integral_constant<int, 1>(), warp));
+                break;
+            case 2: PTQ_CUDA(go(std::integral_constant<int, 2>(), warp)); break;
+            case 3: PTQ_CUDA(go(std::integral_constant<int, 3>(), warp)); break;
+            case 4: PTQ_CUDA(go(std::integral_constant<int, 4>(), warp)); break;
+            case 5: PTQ_CUDA(go(std::integral_constant<int, 5>(), warp)); break;
+            default: PTQ_CUDA(go(std::integral_constant<int, 6>(), warp)); break;
+        }
+    } else if (!vec)
         PTQ_CUDA(launch_pdl(ptq::ptq_quantize_dynamic_scalar_kernel, static_cast<int>(want), 256, 0, stream, p));
     else if (h->fast_div)
         PTQ_CUDA(launch_pdl(ptq::ptq_quantize_dynamic_vec8_kernel<true>, static_cast<int>(want), 256, 0, stream, p));
