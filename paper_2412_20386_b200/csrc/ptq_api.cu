@@ -383,6 +383,13 @@ ptq_status_t launch_quantize_dynamic(const ptq_linear *h, const void *x, long lo
 #define PTQ_GEMM_TEAM_MIN_ROUNDS 3
 #endif
 
+// Per-channel vectors a GEMM kernel keeps in shared memory: weight steps, bias, and (short main loops) row sums.
+void set_vectors(const ptq_linear *h, ptq::GemmParams &p)
+{
+    p.ws_copy = h->asym && h->k_blocks <= PTQ_GEMM_SHORT_K_BLOCKS ? 1 : 0;
+    p.vectors = 1 + p.has_bias + p.ws_copy;
+}
+
 // Whether this launch takes the panel kernel (the codes of a row panel resident in shared memory for a
 // group of N tiles), and with which tiling: fills p.group, p.groups, p.b_stages, p.b_stage_bytes.
 // It pays on large compute-bound layers only (measured: 2-3 % of the Vim-B step, nothing or a loss on
@@ -397,7 +404,7 @@ bool plan_panel(const ptq_linear *h, ptq::GemmParams &p, bool tma_store)
         tiles < 8ll * h->num_sms)
         return false;
     const int stage_bytes = p.BN * ptq::kBK;
-    const int fixed = ptq::panel_smem_bytes(p.k_blocks, 0, 0, p.boxes, p.has_bias);
+    const int fixed = ptq::panel_smem_bytes(p.k_blocks, 0, 0, p.boxes, p.vectors);
     int stages = (ptq::kPanelSmemLimit - fixed) / stage_bytes;
     if (stages < 3) return false;
     if (stages > ptq::kPanelMaxBStages) stages = ptq::kPanelMaxBStages;
@@ -511,12 +518,13 @@ ptq_status_t launch_gemm(const ptq_linear *h, const void *codes, long long M, vo
     p.dw = h->d_dw;
     p.bias = h->d_bias;
     p.has_bias = h->has_bias ? 1 : 0;
+    set_vectors(h, p);
     // Short main loops (up to three k-blocks per tile, K <= 384) leave the epilogue little time: three stages and two
     // staging boxes per warp; longer ones keep four stages.  Layers with a bias hold two more scale copies.
     const bool short_k = h->k_blocks <= PTQ_GEMM_SHORT_K_BLOCKS;
     p.stages = (short_k || h->has_bias) ? ptq::kStages - 1 : ptq::kStages;
     p.boxes = short_k ? 2 : 1;
-    const int gemm_smem = ptq::gemm_smem_bytes(p.stages, p.boxes, p.has_bias);
+    const int gemm_smem = ptq::gemm_smem_bytes(p.stages, p.boxes, p.vectors);
     p.y = static_cast<__half *>(y);
     p.acc_out = static_cast<int32_t *>(acc_out);
     p.status = h->d_status;
@@ -560,16 +568,19 @@ ptq_status_t launch_gemm(const ptq_linear *h, const void *codes, long long M, vo
     const bool dbg = acc_out != nullptr;
     if (plan_panel(h, p, tma_store)) {
         // several N tiles and 512 <= K <= 768: the codes of a row panel stay in shared memory for `group` tiles
-        const int psmem = ptq::panel_smem_bytes(p.k_blocks, p.b_stages, p.b_stage_bytes, p.boxes, p.has_bias);
+        const int psmem = ptq::panel_smem_bytes(p.k_blocks, p.b_stages, p.b_stage_bytes, p.boxes, p.vectors);
         const long long units = static_cast<long long>(p.m_tiles) * p.groups;
         const int pgrid = static_cast<int>(units < h->num_sms ? units : h->num_sms);
-        ptq_status_t ps = dbg ? ensure_smem<ptq::ptq_gemm_dequant_panel_kernel<true>>(h->device, ptq::kPanelSmemLimit)
-                              : ensure_smem<ptq::ptq_gemm_dequant_panel_kernel<false>>(h->device, ptq::kPanelSmemLimit);
+        auto panel = [&](auto debug, auto asym) -> ptq_status_t {
+            constexpr auto kKern = ptq::ptq_gemm_dequant_panel_kernel<decltype(debug)::value, decltype(asym)::value>;
+            const ptq_status_t es = ensure_smem<kKern>(h->device, ptq::kPanelSmemLimit);
+            if (es != PTQ_OK) return es;
+            PTQ_CUDA(launch_pdl(kKern, pgrid, ptq::kGemmThreads, psmem, stream, tmA, h->tmW, tmY, p));
+            return PTQ_OK;
+        };
+        const ptq_status_t ps = h->asym ? (dbg ? panel(std::true_type(), std::true_type()) : panel(std::false_type(), std::true_type()))
+                                        : (dbg ? panel(std::true_type(), std::false_type()) : panel(std::false_type(), std::false_type()));
         if (ps != PTQ_OK) return ps;
-        if (dbg)
-            PTQ_CUDA(launch_pdl(ptq::ptq_gemm_dequant_panel_kernel<true>, pgrid, ptq::kGemmThreads, psmem, stream, tmA, h->tmW, tmY, p));
-        else
-            PTQ_CUDA(launch_pdl(ptq::ptq_gemm_dequant_panel_kernel<false>, pgrid, ptq::kGemmThreads, psmem, stream, tmA, h->tmW, tmY, p));
         g_launches.fetch_add(1, std::memory_order_relaxed);
         PTQ_CUDA(cudaGetLastError());
         return PTQ_OK;
@@ -582,20 +593,16 @@ ptq_status_t launch_gemm(const ptq_linear *h, const void *codes, long long M, vo
     // four warps, one per accumulator; otherwise all eight warps share every tile (shorter latency of a tile).
     const bool teams = gemm_teams(h, p, tma_store, short_k);
     const int grid = static_cast<int>(tiles < h->num_sms ? tiles : h->num_sms);
-    auto go = [&](auto kern) -> ptq_status_t {
-        PTQ_CUDA(launch_pdl(kern, grid, ptq::kGemmThreads, gemm_smem, stream, tmA, tmW, tmY, p));
+    auto go = [&](auto debug, auto team, auto asym) -> ptq_status_t {
+        constexpr auto kKern = ptq::ptq_gemm_dequant_kernel<decltype(debug)::value, decltype(team)::value, decltype(asym)::value>;
+        const ptq_status_t es = ensure_smem<kKern>(h->device, ptq::kGemmSmemBytes);
+        if (es != PTQ_OK) return es;
+        PTQ_CUDA(launch_pdl(kKern, grid, ptq::kGemmThreads, gemm_smem, stream, tmA, tmW, tmY, p));
         return PTQ_OK;
     };
-    ptq_status_t gs;
-    if (teams) {
-        gs = dbg ? ensure_smem<ptq::ptq_gemm_dequant_kernel<true, true>>(h->device, ptq::kGemmSmemBytes)
-                 : ensure_smem<ptq::ptq_gemm_dequant_kernel<false, true>>(h->device, ptq::kGemmSmemBytes);
-        if (gs == PTQ_OK) gs = dbg ? go(ptq::ptq_gemm_dequant_kernel<true, true>) : go(ptq::ptq_gemm_dequant_kernel<false, true>);
-    } else {
-        gs = dbg ? ensure_smem<ptq::ptq_gemm_dequant_kernel<true, false>>(h->device, ptq::kGemmSmemBytes)
-                 : ensure_smem<ptq::ptq_gemm_dequant_kernel<false, false>>(h->device, ptq::kGemmSmemBytes);
-        if (gs == PTQ_OK) gs = dbg ? go(ptq::ptq_gemm_dequant_kernel<true, false>) : go(ptq::ptq_gemm_dequant_kernel<false, false>);
-    }
+    auto pick = [&](auto team, auto asym) { return dbg ? go(std::true_type(), team, asym) : go(std::false_type(), team, asym); };
+    const ptq_status_t gs = h->asym ? (teams ? pick(std::true_type(), std::true_type()) : pick(std::false_type(), std::true_type()))
+                                    : (teams ? pick(std::true_type(), std::false_type()) : pick(std::false_type(), std::false_type()));
     if (gs != PTQ_OK) return gs;
     g_launches.fetch_add(1, std::memory_order_relaxed);
     PTQ_CUDA(cudaGetLastError());
@@ -672,6 +679,8 @@ ptq_status_t launch_fused(const ptq_linear *h, const void *x, long long M, void 
     p.dw = h->d_dw;
     p.bias = h->d_bias;
     p.has_bias = h->has_bias ? 1 : 0;
+    p.vectors = 1;
+    p.ws_copy = 0;
     p.y = static_cast<__half *>(y);
     p.acc_out = static_cast<int32_t *>(acc_out);
     p.status = h->d_status;
@@ -1105,6 +1114,7 @@ int ptq_linear_gemm_variant(const ptq_linear_t *h, int B)
     p.m_tiles = static_cast<int>((M + ptq::kBM - 1) / ptq::kBM);
     p.k_blocks = h->k_blocks;
     p.has_bias = h->has_bias ? 1 : 0;
+    set_vectors(h, p);
     const bool short_k = h->k_blocks <= PTQ_GEMM_SHORT_K_BLOCKS;
     p.boxes = short_k ? 2 : 1;
     if (plan_panel(h, p, true)) return 2;

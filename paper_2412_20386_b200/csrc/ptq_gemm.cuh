@@ -51,20 +51,22 @@ constexpr int kStreamBoxCols = kStreamBox64 ? 64 : kStoreBoxCols;
 constexpr int kStreamStagingPerWarp = kStreamBox64 ? 32 * 128 : kStagingBytesPerWarp;
 // Streaming kernel: per-tile copies of the weight steps (and of the bias, for layers that have one) in
 // shared memory, double buffered by tile parity, so that the conversion loop reads them with broadcast
-// shared-memory loads instead of global loads.  Layers with a bias run three stages to make room.
+// shared-memory loads instead of global loads; asymmetric layers with a short main loop keep the row sums of their
+// weights the same way (6304 x 384 -> 1536, both kernels: 13.9 -> 12.6 us; a long main loop needs the stage more: 50432 x 768 -> 3072
+// 140 us with the sums in global memory, 150 with a stage less).  Layers with a bias run three stages to make room.
 constexpr int kScaleBufBytes = kMaxBN * 4;                // one vector of one tile
 constexpr int kGemmNumBarriers = kNumBarriers + 1;        // + the barrier that publishes the scale copies
 // Two shapes of the shared memory: four stages and one staging box per epilogue warp, or three stages
 // and two boxes per warp (a step then never waits for the store before it; chosen where the main loop
 // of a tile is short, so that the epilogue is what must keep up).
-__host__ __device__ constexpr int gemm_smem_bytes(int stages, int boxes, int has_bias)
+__host__ __device__ constexpr int gemm_smem_bytes(int stages, int boxes, int vectors)
 {
     // no slack for alignment: the dynamic shared memory array is declared 1024-byte aligned (checked at run time)
-    return stages * kStageBytes + boxes * kNumEpiWarps * kStreamStagingPerWarp + (has_bias ? 4 : 2) * kScaleBufBytes +
+    return stages * kStageBytes + boxes * kNumEpiWarps * kStreamStagingPerWarp + 2 * vectors * kScaleBufBytes +
            kGemmNumBarriers * 8 + 16;
 }
-constexpr int kGemmSmemBytes = gemm_smem_bytes(kStages, 1, 0);
-static_assert(kGemmSmemBytes <= 232448 && gemm_smem_bytes(kStages - 1, 2, 1) <= kGemmSmemBytes,
+constexpr int kGemmSmemBytes = gemm_smem_bytes(kStages, 1, 1);
+static_assert(kGemmSmemBytes <= 232448 && gemm_smem_bytes(kStages - 1, 2, 3) <= kGemmSmemBytes,
               "streaming GEMM kernel exceeds the shared memory of one CTA");
 
 struct GemmParams {
@@ -78,6 +80,8 @@ struct GemmParams {
     const float *dw;   // [>= n_tiles*BN + 64], zero padded
     const float *bias; // same length, zeros when the layer has no bias
     int has_bias;      // 0: bias is all zeros and need not be read
+    int vectors;       // scale vectors kept in shared memory: steps, bias where the layer has one, row sums if ws_copy
+    int ws_copy;       // asymmetric layers: 1 = the row sums are read from their shared-memory copy, 0 = from global memory
     int stages;        // streaming kernel: shared-memory stages (3 or 4) ...
     int boxes;         // ... and staging boxes per epilogue warp (2 with three stages, 1 with four)
     __half *y;         // [M,N]
@@ -387,10 +391,10 @@ __device__ __noinline__ void copy_box_rows(__half *y, long long M, int N, int co
     }
 }
 
-template <bool kDebugAcc>
+template <bool kDebugAcc, bool kAsym>
 __device__ __forceinline__ uint32_t epilogue_tile_stream(const GemmParams &p, const CUtensorMap *tmY, uint32_t tmem_row,
                                                          long long m_row0, int n0, float dxr, uint32_t staging,
-                                                         const float *dw_s, const float *bias_s, uint32_t nboxes,
+                                                         const float *dw_s, const float *bias_s, const int *ws_s, uint32_t nboxes,
                                                          int lane, int c_begin, int c_stride, int zr, bool two_boxes)
 {
     const long long m = m_row0 + lane;
@@ -401,12 +405,12 @@ __device__ __forceinline__ uint32_t epilogue_tile_stream(const GemmParams &p, co
         tmem_ld_32x32(tmem_row + c0, v0);
         tmem_ld_32x32(tmem_row + c0 + 32, v1);
         tmem_ld_wait();
-        if (p.zp != nullptr) {
+        if (kAsym) {
             // offset-free accumulator: acc - z[t] * sum_k Wq[n,k]
 #pragma unroll
             for (int i4 = 0; i4 < 8; ++i4) {
-                const int4 wa = __ldg(reinterpret_cast<const int4 *>(p.wsum + n_first) + i4);
-                const int4 wb = __ldg(reinterpret_cast<const int4 *>(p.wsum + n_first + 32) + i4);
+                const int4 wa = reinterpret_cast<const int4 *>(ws_s + c0)[i4];
+                const int4 wb = reinterpret_cast<const int4 *>(ws_s + c0 + 32)[i4];
                 v0[4 * i4 + 0] -= static_cast<uint32_t>(zr * wa.x);
                 v0[4 * i4 + 1] -= static_cast<uint32_t>(zr * wa.y);
                 v0[4 * i4 + 2] -= static_cast<uint32_t>(zr * wa.z);
@@ -465,6 +469,7 @@ struct RowStep {
     float dx;
     int z;
 };
+template <bool kAsym>
 __device__ __forceinline__ RowStep load_row_step(const GemmParams &p, int m_tile, int quarter, int lane)
 {
     // Unconditional loads from clamped indices: a load under a condition is followed by a select that waits for
@@ -476,7 +481,7 @@ __device__ __forceinline__ RowStep load_row_step(const GemmParams &p, int m_tile
     const unsigned mu = static_cast<unsigned>(m);
     const unsigned t = mu - fd_div(mu, p.fd_T) * p.fd_T.d;
     r.dx = __ldg(p.dx + t);
-    if (p.zp != nullptr) r.z = __ldg(p.zp + t);
+    if (kAsym) r.z = __ldg(p.zp + t);
     return r;
 }
 
@@ -525,7 +530,7 @@ struct StreamCursor {
     __device__ int n_tile() const { return tile - m_tile() * n_tiles; }
 };
 
-template <bool kDebugAcc, class Cursor>
+template <bool kDebugAcc, bool kAsym, class Cursor>
 __device__ __forceinline__ void epilogue_team_loop(const GemmParams &p, const CUtensorMap *tmY, Cursor cur, uint32_t tmem_base,
                                                    uint32_t tfull_bar0, uint32_t tempty_bar0, float *scale_s,
                                                    uint32_t staging, bool two_boxes, volatile uint32_t *abort_flag,
@@ -536,9 +541,11 @@ __device__ __forceinline__ void epilogue_team_loop(const GemmParams &p, const CU
     const int tt = static_cast<int>(threadIdx.x) - 64 - team * 128;   // 0 .. 127 inside the team
     float *dw_buf = scale_s + team * kMaxBN;
     float *bias_buf = scale_s + (2 + team) * kMaxBN;
+    int *ws_buf = reinterpret_cast<int *>(scale_s + (2 * p.vectors - 2 + team) * kMaxBN);   // the last vector
     const uint32_t tfull = tfull_bar0 + 8u * team, tempty = tempty_bar0 + 8u * team;
     if (team == 1 && cur.valid()) cur.advance();        // team 1 starts at the CTA's second tile
     float dw_next[2] = {0.0f, 0.0f}, bias_next[2] = {0.0f, 0.0f};
+    int ws_next[2] = {0, 0};
     auto fetch_scales = [&](const Cursor &c) {
         // unconditional loads from clamped indices (see load_row_step); past the last tile the values are not used
         const int n0 = c.valid() ? c.n_tile() * p.BN : 0;
@@ -547,11 +554,12 @@ __device__ __forceinline__ void epilogue_team_loop(const GemmParams &p, const CU
             const int col = min(tt + 128 * h, p.BN - 1);
             dw_next[h] = __ldg(p.dw + n0 + col);
             if (p.has_bias) bias_next[h] = __ldg(p.bias + n0 + col);
+            if (kAsym && p.ws_copy) ws_next[h] = __ldg(p.wsum + n0 + col);
         }
     };
     fetch_scales(cur);
     RowStep rs_next = {0.0f, 0};
-    if (cur.valid()) rs_next = load_row_step(p, cur.m_tile(), quarter, lane);
+    if (cur.valid()) rs_next = load_row_step<kAsym>(p, cur.m_tile(), quarter, lane);
     uint32_t tphase = 0, nboxes = 0;
     while (cur.valid()) {                               // the same for every thread of the team
 #pragma unroll
@@ -560,6 +568,7 @@ __device__ __forceinline__ void epilogue_team_loop(const GemmParams &p, const CU
             if (col < p.BN) {
                 dw_buf[col] = dw_next[h];
                 if (p.has_bias) bias_buf[col] = bias_next[h];
+                if (kAsym && p.ws_copy) ws_buf[col] = ws_next[h];
             }
         }
         const int m_tile = cur.m_tile(), n_tile = cur.n_tile();
@@ -569,14 +578,15 @@ __device__ __forceinline__ void epilogue_team_loop(const GemmParams &p, const CU
         const long long m_row0 = static_cast<long long>(m_tile) * kBM + quarter * 32;
         const float dxr = rs_next.dx;
         const int zr = rs_next.z;
-        if (cur.valid()) rs_next = load_row_step(p, cur.m_tile(), quarter, lane);
+        if (cur.valid()) rs_next = load_row_step<kAsym>(p, cur.m_tile(), quarter, lane);
         bool got = mbar_wait(tfull, tphase, abort_flag, p.status);
         got = team_all(got, team);                      // also: the team's scale copies are complete and visible
         if (!got) break;
         tc_fence_after_sync();
         const uint32_t tmem_row = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) + static_cast<uint32_t>(team) * kMaxBN;
-        nboxes = epilogue_tile_stream<kDebugAcc>(p, tmY, tmem_row, m_row0, n_tile * p.BN, dxr, staging, dw_buf,
-                                                 p.has_bias ? bias_buf : nullptr, nboxes, lane, 0, kEpiStepCols, zr, two_boxes);
+        nboxes = epilogue_tile_stream<kDebugAcc, kAsym>(p, tmY, tmem_row, m_row0, n_tile * p.BN, dxr, staging, dw_buf,
+                                                 p.has_bias ? bias_buf : nullptr, !kAsym ? nullptr : p.ws_copy ? ws_buf : p.wsum + n_tile * p.BN, nboxes,
+                                                 lane, 0, kEpiStepCols, zr, two_boxes);
         tc_fence_before_sync();
         __syncwarp();
         if (lane == 0) mbar_arrive(tempty);
@@ -588,7 +598,7 @@ __device__ __forceinline__ void epilogue_team_loop(const GemmParams &p, const CU
 
 // --- the kernel ---------------------------------------------------------------------------------
 
-template <bool kDebugAcc, bool kTeams = false>
+template <bool kDebugAcc, bool kTeams, bool kAsym>
 __global__ void __launch_bounds__(kGemmThreads, 1)
 ptq_gemm_dequant_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmW,
                         const __grid_constant__ CUtensorMap tmY, const GemmParams p)
@@ -604,7 +614,7 @@ ptq_gemm_dequant_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
     const bool two_boxes = p.boxes == 2;
     const uint32_t staging_off = nstages * kStageBytes;
     const uint32_t scale_off = staging_off + static_cast<uint32_t>(p.boxes) * kNumEpiWarps * kStreamStagingPerWarp;
-    const uint32_t bar_off = scale_off + (p.has_bias ? 4 : 2) * kScaleBufBytes;
+    const uint32_t bar_off = scale_off + 2 * p.vectors * kScaleBufBytes;
     const uint32_t staging_base = base + staging_off;
     const uint32_t bar_base = base + bar_off;
     auto full_bar = [&](uint32_t s) { return bar_base + 8u * s; };
@@ -701,7 +711,7 @@ ptq_gemm_dequant_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
     } else if (warp == 1) {
         // ------------------------------------------------------------------ MMA issuer
         if (lane == 0) {
-            const uint32_t idesc = make_idesc_s8(kBM, p.BN, p.zp != nullptr);   // unsigned codes on asymmetric layers
+            const uint32_t idesc = make_idesc_s8(kBM, p.BN, kAsym);   // unsigned codes on asymmetric layers
             uint32_t stage = 0, phase = 0, buf = 0, bphase = 0;
             bool ok = true;
             for (int tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x) {
@@ -735,7 +745,7 @@ ptq_gemm_dequant_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
         // ------------------------------------------------------------------ epilogue warps, two teams (TMA stores only)
         griddep_wait();
         const StreamCursor cur{static_cast<int>(blockIdx.x), total_tiles, static_cast<int>(gridDim.x), p.n_tiles, p.fd_n_tiles};
-        epilogue_team_loop<kDebugAcc>(p, &tmY, cur, tmem_base, tfull_bar(0), tempty_bar(0),
+        epilogue_team_loop<kDebugAcc, kAsym>(p, &tmY, cur, tmem_base, tfull_bar(0), tempty_bar(0),
                                       reinterpret_cast<float *>(smem_raw + scale_off),
                                       staging_base + static_cast<uint32_t>(warp - 2) * static_cast<uint32_t>(p.boxes) * kStreamStagingPerWarp,
                                       two_boxes, abort_flag, warp, lane);
@@ -749,18 +759,21 @@ ptq_gemm_dequant_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
         float *scale_s = reinterpret_cast<float *>(smem_raw + scale_off);   // [2][BN] steps, then [2][BN] bias
         // The weight step (and bias) of one column of tile `tile`: fetched into registers one tile ahead ...
         float dw_next = 0.0f, bias_next = 0.0f;
+        int ws_next = 0;
         auto fetch_scales = [&](int tile) {
             // unconditional loads from clamped indices (see load_row_step); past the last tile the values are not used
             const unsigned tl = tile < total_tiles ? static_cast<unsigned>(tile) : 0u;
             const int n = static_cast<int>(tl - fd_div(tl, p.fd_n_tiles) * p.fd_n_tiles.d) * p.BN + min(et, p.BN - 1);
             dw_next = __ldg(p.dw + n);
             if (p.has_bias) bias_next = __ldg(p.bias + n);
+            if (kAsym && p.ws_copy) ws_next = __ldg(p.wsum + n);
         };
         // ... and published in buffer `b` once every warp is done with the tile that used that buffer last
         auto publish_scales = [&](uint32_t b) {
             if (et < p.BN) {
                 scale_s[b * kMaxBN + et] = dw_next;
                 if (p.has_bias) scale_s[(2 + b) * kMaxBN + et] = bias_next;
+                if (kAsym && p.ws_copy) reinterpret_cast<int *>(scale_s)[(2 * p.vectors - 2 + b) * kMaxBN + et] = ws_next;
             }
             __syncwarp();
             if (lane == 0) mbar_arrive(scale_bar);
@@ -768,7 +781,7 @@ ptq_gemm_dequant_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
         uint32_t buf = 0, bphase = 0, nboxes = 0, it = 0;
         fetch_scales(blockIdx.x);
         publish_scales(0u);
-        RowStep rs_next = load_row_step(p, static_cast<int>(fd_div(blockIdx.x, p.fd_n_tiles)), quarter, lane);
+        RowStep rs_next = load_row_step<kAsym>(p, static_cast<int>(fd_div(blockIdx.x, p.fd_n_tiles)), quarter, lane);
         for (int tile = blockIdx.x; tile < total_tiles; tile += gridDim.x, ++it) {
             const int tile_next = tile + static_cast<int>(gridDim.x);
             fetch_scales(tile_next);                            // in flight during this tile
@@ -778,7 +791,7 @@ ptq_gemm_dequant_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
             const float dxr = rs_next.dx;
             const int zr = rs_next.z;
             if (tile_next < total_tiles)
-                rs_next = load_row_step(p, static_cast<int>(fd_div(static_cast<unsigned>(tile_next), p.fd_n_tiles)), quarter, lane);
+                rs_next = load_row_step<kAsym>(p, static_cast<int>(fd_div(static_cast<unsigned>(tile_next), p.fd_n_tiles)), quarter, lane);
             // every epilogue warp has written its share of this tile's scale copies (arrival `it` of the barrier)
             bool got = mbar_wait(scale_bar, it & 1u, abort_flag, p.status);
             got = got && mbar_wait(tfull_bar(buf), bphase, abort_flag, p.status);
@@ -788,8 +801,11 @@ ptq_gemm_dequant_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
             const uint32_t tmem_row = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) + buf * kMaxBN;
             const float *dw_s = scale_s + (it & 1u) * kMaxBN;
             const float *bias_s = p.has_bias ? scale_s + (2u + (it & 1u)) * kMaxBN : nullptr;
-            nboxes = epilogue_tile_stream<kDebugAcc>(p, &tmY, tmem_row, m_row0, n_tile * p.BN, dxr, staging, dw_s,
-                                                     bias_s, nboxes, lane, col_half * kEpiStepCols, 2 * kEpiStepCols, zr, two_boxes);
+            const int *ws_s = !kAsym ? nullptr
+                              : p.ws_copy ? reinterpret_cast<const int *>(scale_s) + (2u * p.vectors - 2u + (it & 1u)) * kMaxBN
+                                          : p.wsum + n_tile * p.BN;
+            nboxes = epilogue_tile_stream<kDebugAcc, kAsym>(p, &tmY, tmem_row, m_row0, n_tile * p.BN, dxr, staging, dw_s,
+                                                     bias_s, ws_s, nboxes, lane, col_half * kEpiStepCols, 2 * kEpiStepCols, zr, two_boxes);
             tc_fence_before_sync();
             __syncwarp();
             if (lane == 0) mbar_arrive(tempty_bar(buf));
@@ -829,13 +845,13 @@ constexpr int kPanelMaxKBlocks = 6;                       // panel of at most 96
 constexpr int kPanelMaxBStages = 6;
 constexpr int kPanelNumBarriers = 2 * kPanelMaxKBlocks + 2 * kPanelMaxBStages + 4 + 1;
 constexpr int kPanelSmemLimit = 232448;                   // 227 KB opt-in maximum per CTA
-__host__ __device__ constexpr int panel_smem_bytes(int k_blocks, int b_stages, int b_stage_bytes, int boxes, int has_bias)
+__host__ __device__ constexpr int panel_smem_bytes(int k_blocks, int b_stages, int b_stage_bytes, int boxes, int vectors)
 {
     return k_blocks * kATileBytes + b_stages * b_stage_bytes + boxes * kNumEpiWarps * kStreamStagingPerWarp +
-           (has_bias ? 4 : 2) * kScaleBufBytes + kPanelNumBarriers * 8 + 16;
+           2 * vectors * kScaleBufBytes + kPanelNumBarriers * 8 + 16;
 }
 
-template <bool kDebugAcc>
+template <bool kDebugAcc, bool kAsym>
 __global__ void __launch_bounds__(kGemmThreads, 1)
 ptq_gemm_dequant_panel_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmW,
                               const __grid_constant__ CUtensorMap tmY, const GemmParams p)
@@ -852,7 +868,7 @@ ptq_gemm_dequant_panel_kernel(const __grid_constant__ CUtensorMap tmA, const __g
     const uint32_t b_off = static_cast<uint32_t>(p.k_blocks) * kATileBytes;
     const uint32_t staging_off = b_off + nb * b_bytes;
     const uint32_t scale_off = staging_off + static_cast<uint32_t>(p.boxes) * kNumEpiWarps * kStreamStagingPerWarp;
-    const uint32_t bar_off = scale_off + (p.has_bias ? 4 : 2) * kScaleBufBytes;
+    const uint32_t bar_off = scale_off + 2 * p.vectors * kScaleBufBytes;
     const uint32_t bar_base = base + bar_off;
     auto afull_bar = [&](uint32_t kb) { return bar_base + 8u * kb; };
     auto aempty_bar = [&](uint32_t kb) { return bar_base + 8u * (kPanelMaxKBlocks + kb); };
@@ -976,7 +992,7 @@ ptq_gemm_dequant_panel_kernel(const __grid_constant__ CUtensorMap tmA, const __g
     } else if (warp == 1) {
         // ------------------------------------------------------------------ MMA issuer
         if (lane == 0) {
-            const uint32_t idesc = make_idesc_s8(kBM, p.BN, p.zp != nullptr);
+            const uint32_t idesc = make_idesc_s8(kBM, p.BN, kAsym);
             uint32_t stage = 0, sphase = 0, uph = 0, buf = 0, bphase = 0;
             bool ok = true;
             for (int unit = blockIdx.x; unit < units && ok; unit += gridDim.x, uph ^= 1u) {
@@ -1025,15 +1041,18 @@ ptq_gemm_dequant_panel_kernel(const __grid_constant__ CUtensorMap tmA, const __g
         const uint32_t staging = base + staging_off + static_cast<uint32_t>(warp - 2) * static_cast<uint32_t>(p.boxes) * kStreamStagingPerWarp;
         float *scale_s = reinterpret_cast<float *>(smem_raw + scale_off);   // [2][BN] steps, then [2][BN] bias
         float dw_next = 0.0f, bias_next = 0.0f;
+        int ws_next = 0;
         auto fetch_scales = [&](int n_tile) {
             const int n = n_tile * p.BN + min(et, p.BN - 1);      // unconditional, clamped (see load_row_step)
             dw_next = __ldg(p.dw + n);
             if (p.has_bias) bias_next = __ldg(p.bias + n);
+            if (kAsym && p.ws_copy) ws_next = __ldg(p.wsum + n);
         };
         auto publish_scales = [&](uint32_t b) {
             if (et < p.BN) {
                 scale_s[b * kMaxBN + et] = dw_next;
                 if (p.has_bias) scale_s[(2 + b) * kMaxBN + et] = bias_next;
+                if (kAsym && p.ws_copy) reinterpret_cast<int *>(scale_s)[(2 * p.vectors - 2 + b) * kMaxBN + et] = ws_next;
             }
             __syncwarp();
             if (lane == 0) mbar_arrive(scale_bar);
@@ -1042,7 +1061,7 @@ ptq_gemm_dequant_panel_kernel(const __grid_constant__ CUtensorMap tmA, const __g
         int unit = blockIdx.x, j = 0;
         fetch_scales(unit < units ? unit_first(unit) : 0);
         publish_scales(0u);
-        RowStep rs_next = load_row_step(p, unit < units ? unit_panel(unit) : 0, quarter, lane);
+        RowStep rs_next = load_row_step<kAsym>(p, unit < units ? unit_panel(unit) : 0, quarter, lane);
         while (unit < units) {
             // the tile after this one: its scales are fetched now and stay in flight during this tile
             int next_unit = unit, next_j = j + 1;
@@ -1056,7 +1075,7 @@ ptq_gemm_dequant_panel_kernel(const __grid_constant__ CUtensorMap tmA, const __g
             const long long m_row0 = static_cast<long long>(m_tile) * kBM + quarter * 32;
             const float dxr = rs_next.dx;
             const int zr = rs_next.z;
-            if (next_unit != unit && next_unit < units) rs_next = load_row_step(p, unit_panel(next_unit), quarter, lane);
+            if (next_unit != unit && next_unit < units) rs_next = load_row_step<kAsym>(p, unit_panel(next_unit), quarter, lane);
             bool got = mbar_wait(scale_bar, it & 1u, abort_flag, p.status);
             got = got && mbar_wait(tfull_bar(buf), bphase, abort_flag, p.status);
             got = __all_sync(0xffffffffu, got);
@@ -1065,8 +1084,11 @@ ptq_gemm_dequant_panel_kernel(const __grid_constant__ CUtensorMap tmA, const __g
             const uint32_t tmem_row = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) + buf * kMaxBN;
             const float *dw_s = scale_s + (it & 1u) * kMaxBN;
             const float *bias_s = p.has_bias ? scale_s + (2u + (it & 1u)) * kMaxBN : nullptr;
-            nboxes = epilogue_tile_stream<kDebugAcc>(p, &tmY, tmem_row, m_row0, n_tile * p.BN, dxr, staging, dw_s, bias_s,
-                                                     nboxes, lane, col_half * kEpiStepCols, 2 * kEpiStepCols, zr, two_boxes);
+            const int *ws_s = !kAsym ? nullptr
+                              : p.ws_copy ? reinterpret_cast<const int *>(scale_s) + (2u * p.vectors - 2u + (it & 1u)) * kMaxBN
+                                          : p.wsum + n_tile * p.BN;
+            nboxes = epilogue_tile_stream<kDebugAcc, kAsym>(p, &tmY, tmem_row, m_row0, n_tile * p.BN, dxr, staging, dw_s, bias_s,
+                                                     ws_s, nboxes, lane, col_half * kEpiStepCols, 2 * kEpiStepCols, zr, two_boxes);
             tc_fence_before_sync();
             __syncwarp();
             if (lane == 0) mbar_arrive(tempty_bar(buf));
@@ -1284,8 +1306,8 @@ ptq_gemm_dequant_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __gr
             tc_fence_after_sync();
             const uint32_t tmem_row = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) + buf * kMaxBN;
             if (p.use_tma_store)
-                nboxes = epilogue_tile_stream<kDebugAcc>(p, &tmY, tmem_row, m_row0, n_tile * p.BN, dxr, staging,
-                                                         scale_s + (it & 1u) * kMaxBN, nullptr, nboxes, lane,
+                nboxes = epilogue_tile_stream<kDebugAcc, false>(p, &tmY, tmem_row, m_row0, n_tile * p.BN, dxr, staging,
+                                                         scale_s + (it & 1u) * kMaxBN, nullptr, nullptr, nboxes, lane,
                                                          col_half * kEpiStepCols, 2 * kEpiStepCols, 0, false);
             else
                 nboxes = epilogue_tile<kDebugAcc, false, kStreamBox64>(p, &tmY, tmem_row, m_row0, n_tile * p.BN, dxr, staging,
