@@ -813,22 +813,6 @@ ptq_status_t static_scratch_address(int device, void **out)
     return PTQ_OK;
 }
 
-template <int kVec>
-void launch_calib_rowrange(bool asym, const __half *x, int Bc, int K, int T, int sms, const float *s, unsigned *hi,
-                           unsigned *nlo, cudaStream_t stream)
-{
-    // two blocks per SM where there are few positions, but at least eight images per block
-    int splits = (2 * sms + T - 1) / T;
-    const int most = (Bc + 7) / 8;
-    if (splits > most) splits = most;
-    const int per = (Bc + splits - 1) / splits;
-    const dim3 grid(static_cast<unsigned>(T), static_cast<unsigned>((Bc + per - 1) / per));
-    if (asym)
-        ptq::ptq_calib_rowrange_kernel<kVec, true><<<grid, 128, 0, stream>>>(x, Bc, per, K, T, s, hi, nlo);
-    else
-        ptq::ptq_calib_rowrange_kernel<kVec, false><<<grid, 128, 0, stream>>>(x, Bc, per, K, T, s, hi, nlo);
-}
-
 ptq_status_t validate_forward(const ptq_linear *h, const void *x, int B, const void *y)
 {
     if (!h || !x || !y) return fail(PTQ_ERR_NULL, "handle, x and y must not be NULL");
@@ -1282,7 +1266,7 @@ ptq_status_t ptq_search_act_step_in(int K, int T, const void *xcal_fp16, int Bc,
     p.fd_K = ptq::make_fastdiv(static_cast<unsigned>(K));
     const dim3 grid(static_cast<unsigned>(T), static_cast<unsigned>((C + ptq::kSearchCandPerBlock - 1) / ptq::kSearchCandPerBlock));
     ptq::ptq_search_loss_kernel<<<grid, ptq::kSearchThreads, 0, s>>>(p);
-    ptq::ptq_search_pick_kernel<<<(T + 127) / 128, 128, 0, s>>>(d_loss, d_base, T, n_grid, j_lo, d_best, d_dx);
+    ptq::ptq_search_pick_kernel<<<(T + 3) / 4, 128, 0, s>>>(d_loss, d_base, T, n_grid, j_lo, d_best, d_dx);
     g_launches.fetch_add(2, std::memory_order_relaxed);
     PTQ_CUDA(cudaGetLastError());
     PTQ_CUDA(cudaMemcpyAsync(out.data(), d_dx, sizeof(float) * out.size(), cudaMemcpyDeviceToHost, s));
@@ -1549,10 +1533,12 @@ ptq_status_t ptq_calibrate_in(int scheme, int K, int N, int T, const void *xcal_
     PTQ_CUDA(cudaMemsetAsync(d_xbits, 0, sizeof(unsigned) * (2 * static_cast<size_t>(K) + 2 * static_cast<size_t>(T)), s));
     const bool vec = K % 8 == 0 && reinterpret_cast<uintptr_t>(x) % 16 == 0;
     const int cpr = vec ? K / 8 : K;
-    const long long rp = 256 / (cpr < 256 ? cpr : 256);
-    long long rpb = (M + 2 * sms - 1) / (2 * sms);
+    const int cgroups = (cpr + ptq::kCalibGroup - 1) / ptq::kCalibGroup;
+    const long long rp = 256 / (cpr < ptq::kCalibGroup ? cpr : ptq::kCalibGroup);
+    long long rpb = (M * cgroups + 2 * sms - 1) / (2 * sms);              // about two blocks per SM, four rows per thread at least
     if (rpb < 4 * rp) rpb = 4 * rp;
-    const int cgrid = static_cast<int>((M + rpb - 1) / rpb);
+    const long long shares = (M + rpb - 1) / rpb;
+    const dim3 cgrid(static_cast<unsigned>(cgroups), static_cast<unsigned>(shares));
     if (vec)
         ptq::ptq_calib_colmax_kernel<8><<<cgrid, 256, 0, s>>>(x, M, K, static_cast<int>(rpb), d_xbits);
     else
@@ -1561,28 +1547,49 @@ ptq_status_t ptq_calibrate_in(int scheme, int K, int N, int T, const void *xcal_
     PTQ_CUDA(cudaMemcpyAsync(d_w, w_q, static_cast<size_t>(N) * row_bytes, cudaMemcpyHostToDevice, s));
     const bool w4 = row_bytes % 4 == 0;
     const int groups = w4 ? row_bytes / 4 : row_bytes;
-    const dim3 wgrid(static_cast<unsigned>((groups + 127) / 128),
-                     static_cast<unsigned>((N + ptq::kCalibRowsPerBlock - 1) / ptq::kCalibRowsPerBlock));
+    const int wcols = (groups + 127) / 128;
+    int wrows = (N * wcols + 2 * sms - 1) / (2 * sms);                    // about two blocks per SM, 16 rows at least
+    if (wrows < 16) wrows = 16;
+    const dim3 wgrid(static_cast<unsigned>(wcols), static_cast<unsigned>((N + wrows - 1) / wrows));
     if (packed && w4)
-        ptq::ptq_calib_wmax_kernel<4, true><<<wgrid, 128, 0, s>>>(d_w, d_dw, N, K, d_wbits);
+        ptq::ptq_calib_wmax_kernel<4, true><<<wgrid, 128, 0, s>>>(d_w, d_dw, N, K, wrows, d_wbits);
     else if (packed)
-        ptq::ptq_calib_wmax_kernel<1, true><<<wgrid, 128, 0, s>>>(d_w, d_dw, N, K, d_wbits);
+        ptq::ptq_calib_wmax_kernel<1, true><<<wgrid, 128, 0, s>>>(d_w, d_dw, N, K, wrows, d_wbits);
     else if (w4)
-        ptq::ptq_calib_wmax_kernel<4, false><<<wgrid, 128, 0, s>>>(d_w, d_dw, N, K, d_wbits);
+        ptq::ptq_calib_wmax_kernel<4, false><<<wgrid, 128, 0, s>>>(d_w, d_dw, N, K, wrows, d_wbits);
     else
-        ptq::ptq_calib_wmax_kernel<1, false><<<wgrid, 128, 0, s>>>(d_w, d_dw, N, K, d_wbits);
-    ptq::ptq_calib_smooth_kernel<<<(K + 127) / 128, 128, 0, s>>>(d_xbits, d_wbits, K, d_s);
-    if (vec)
-        launch_calib_rowrange<8>(asym, x, Bc, K, T, sms, d_s, d_hi, d_nlo, s);
-    else
-        launch_calib_rowrange<1>(asym, x, Bc, K, T, sms, d_s, d_hi, d_nlo, s);
+        ptq::ptq_calib_wmax_kernel<1, false><<<wgrid, 128, 0, s>>>(d_w, d_dw, N, K, wrows, d_wbits);
+    // image shares per position: two blocks per SM where there are few positions, but at least eight images each
+    int splits = (2 * sms + T - 1) / T;
+    const int most = (Bc + 7) / 8;
+    if (splits > most) splits = most;
+    ptq::CalibRange r;
+    r.x = x;
+    r.max_x_bits = d_xbits;
+    r.max_w_bits = d_wbits;
+    r.hi_bits = d_hi;
+    r.nlo_bits = d_nlo;
+    r.s = d_s;
+    r.dx = d_dx;
+    r.z = d_z;
+    r.Bc = Bc;
+    r.imgs_per_block = (Bc + splits - 1) / splits;
+    r.K = K;
+    r.T = T;
+    r.qmax = packed ? 7.0f : 127.0f;
+    const dim3 rgrid(static_cast<unsigned>(T), static_cast<unsigned>((Bc + r.imgs_per_block - 1) / r.imgs_per_block));
+    r.final = rgrid.y == 1 && scheme != PTQ_CALIB_PER_TENSOR ? 1 : 0;
     if (asym)
-        ptq::ptq_calib_step_asym_kernel<<<(T + 127) / 128, 128, 0, s>>>(d_hi, d_nlo, T, d_dx, d_z);
-    else if (scheme == PTQ_CALIB_PER_TENSOR)
-        ptq::ptq_calib_step_tensor_kernel<<<1, 256, 0, s>>>(d_hi, T, d_dx, 127.0f);
+        vec ? ptq::ptq_calib_rowrange_kernel<8, true><<<rgrid, 128, 0, s>>>(r) : ptq::ptq_calib_rowrange_kernel<1, true><<<rgrid, 128, 0, s>>>(r);
     else
-        ptq::ptq_calib_step_kernel<<<(T + 127) / 128, 128, 0, s>>>(d_hi, T, d_dx, packed ? 7.0f : 127.0f);
-    g_launches.fetch_add(5, std::memory_order_relaxed);
+        vec ? ptq::ptq_calib_rowrange_kernel<8, false><<<rgrid, 128, 0, s>>>(r) : ptq::ptq_calib_rowrange_kernel<1, false><<<rgrid, 128, 0, s>>>(r);
+    if (scheme == PTQ_CALIB_PER_TENSOR)
+        ptq::ptq_calib_step_tensor_kernel<<<1, 256, 0, s>>>(d_hi, T, d_dx, 127.0f);
+    else if (!r.final && asym)
+        ptq::ptq_calib_step_asym_kernel<<<(T + 127) / 128, 128, 0, s>>>(d_hi, d_nlo, T, d_dx, d_z);
+    else if (!r.final)
+        ptq::ptq_calib_step_kernel<<<(T + 127) / 128, 128, 0, s>>>(d_hi, T, d_dx, r.qmax);
+    g_launches.fetch_add(r.final ? 3 : 4, std::memory_order_relaxed);
     PTQ_CUDA(cudaGetLastError());
     // one copy back: s, dx and (asymmetric) z are adjacent
     const size_t words = static_cast<size_t>(K) + static_cast<size_t>(T) * (asym ? 2 : 1);

@@ -50,73 +50,63 @@ __device__ __forceinline__ float calib_channel(const CalibChunk<kVec> &c, int i)
     return (i & 1) ? __high2float(c.h[kVec == 8 ? i >> 1 : 0]) : __low2float(c.h[kVec == 8 ? i >> 1 : 0]);
 }
 
-// maxX[k].  A block takes `rows_per_block` consecutive rows; a thread keeps one group of kVec channels in binary16
-// registers (max.f16x2 drops NaN, and a maximum of binary16 values is exact in binary16) over every rp-th of those
-// rows, the block merges its rp row lanes in shared memory and issues one global atomicMax per channel.
-// Bound: memory latency at calibration sizes (8 images: 0.6 - 4.8 MB, a few loads deep per thread).
+// maxX[k].  Grid (channel groups, row shares): a block takes up to kCalibGroup chunks of kVec channels of `rows_per_block`
+// consecutive rows; a thread keeps one chunk in binary16 registers (max.f16x2 drops NaN, and a maximum of binary16 values
+// is exact in binary16) over every rp-th of those rows, the block merges its rp row lanes in shared memory and issues one
+// global atomicMax per channel.  Bound: memory latency at calibration sizes (8 images: 0.6 - 4.8 MB, a few loads deep per
+// thread).  1576 x 1536: 25 us with whole rows per block (one row lane, 400 thousand atomics), 4.4 so.
+constexpr int kCalibGroup = 32;
+
 template <int kVec>
 __global__ void __launch_bounds__(256) ptq_calib_colmax_kernel(const __half *x, long long M, int K, int rows_per_block,
                                                                unsigned *max_x_bits)
 {
-    __shared__ unsigned best[256 * kVec];
-    const int cpr = K / kVec;
-    const int tpr = min(cpr, 256);                       // threads along a row
+    __shared__ unsigned best[kCalibGroup * kVec];
+    const int c0 = blockIdx.x * kCalibGroup;
+    const int tpr = min(K / kVec - c0, kCalibGroup);     // threads along a row
     const int rp = 256 / tpr;                            // rows side by side
     const int r = static_cast<int>(threadIdx.x) / tpr;
     const int c = static_cast<int>(threadIdx.x) - r * tpr;
-    const long long m0 = static_cast<long long>(blockIdx.x) * rows_per_block;
+    const long long m0 = static_cast<long long>(blockIdx.y) * rows_per_block;
     const int rows = static_cast<int>(M - m0 < rows_per_block ? M - m0 : rows_per_block);
-    for (int c0 = 0; c0 < cpr; c0 += tpr) {
-        const bool on = r < rp && c0 + c < cpr;
-        CalibChunk<kVec> mx;
+    if (threadIdx.x < kCalibGroup) {
 #pragma unroll
-        for (int i = 0; i < (kVec == 8 ? 4 : 1); ++i) mx.h[i] = __float2half2_rn(0.0f);
-        if (on) {
-            const __half *p = x + (m0 + r) * K + static_cast<long long>(c0 + c) * kVec;
-#pragma unroll 4
-            for (int m = r; m < rows; m += rp, p += static_cast<long long>(rp) * K) {
-                const CalibChunk<kVec> v = calib_load<kVec>(p);
-#pragma unroll
-                for (int i = 0; i < (kVec == 8 ? 4 : 1); ++i) mx.h[i] = __hmax2(mx.h[i], __habs2(v.h[i]));
-            }
-        }
-        if (rp > 1) {
-            __syncthreads();
-#pragma unroll
-            for (int i = 0; i < kVec; ++i) best[threadIdx.x * kVec + i] = 0u;
-            __syncthreads();
-            if (on) {
-#pragma unroll
-                for (int i = 0; i < kVec; ++i) atomicMax(&best[c * kVec + i], __float_as_uint(calib_channel<kVec>(mx, i)));
-            }
-            __syncthreads();
-            for (int k = threadIdx.x; k < tpr * kVec && c0 * kVec + k < K; k += 256)
-                if (best[k] != 0u) atomicMax(max_x_bits + c0 * kVec + k, best[k]);
-        } else if (on) {
-#pragma unroll
-            for (int i = 0; i < kVec; ++i) {
-                const unsigned bits = __float_as_uint(calib_channel<kVec>(mx, i));
-                if (bits != 0u) atomicMax(max_x_bits + (c0 + c) * kVec + i, bits);
-            }
-        }
+        for (int i = 0; i < kVec; ++i) best[threadIdx.x * kVec + i] = 0u;
     }
+    __syncthreads();
+    CalibChunk<kVec> mx;
+#pragma unroll
+    for (int i = 0; i < (kVec == 8 ? 4 : 1); ++i) mx.h[i] = __float2half2_rn(0.0f);
+    if (r < rp) {
+        const __half *p = x + (m0 + r) * K + static_cast<long long>(c0 + c) * kVec;
+#pragma unroll 4
+        for (int m = r; m < rows; m += rp, p += static_cast<long long>(rp) * K) {
+            const CalibChunk<kVec> v = calib_load<kVec>(p);
+#pragma unroll
+            for (int i = 0; i < (kVec == 8 ? 4 : 1); ++i) mx.h[i] = __hmax2(mx.h[i], __habs2(v.h[i]));
+        }
+#pragma unroll
+        for (int i = 0; i < kVec; ++i) atomicMax(&best[c * kVec + i], __float_as_uint(calib_channel<kVec>(mx, i)));
+    }
+    __syncthreads();
+    for (int k = threadIdx.x; k < tpr * kVec; k += 256)
+        if (best[k] != 0u) atomicMax(max_x_bits + c0 * kVec + k, best[k]);
 }
 
-// maxW[k] = max_n |Wq[n,k]| * dw[n]: grid (byte-group blocks, row blocks); a thread scans kCalibRowsPerBlock weight rows
+// maxW[k] = max_n |Wq[n,k]| * dw[n]: grid (byte-group blocks, row blocks); a thread scans `rows_per_block` weight rows
 // of kBytes adjacent bytes (coalesced across the block) and merges with one atomicMax per channel.  kPacked: two
 // signed 4-bit weights per byte, low nibble = even channel, rows of (K+1)/2 bytes.
-constexpr int kCalibRowsPerBlock = 32;
 
 template <int kBytes, bool kPacked>
-__global__ void __launch_bounds__(128) ptq_calib_wmax_kernel(const uint8_t *wq, const float *dw, int N, int K,
+__global__ void __launch_bounds__(128) ptq_calib_wmax_kernel(const uint8_t *wq, const float *dw, int N, int K, int rows_per_block,
                                                              unsigned *max_w_bits)
 {
     constexpr int kChan = kPacked ? 2 * kBytes : kBytes;
     const int row_bytes = kPacked ? (K + 1) / 2 : K;
     const int j = (blockIdx.x * blockDim.x + threadIdx.x) * kBytes;
     if (j >= row_bytes) return;
-    const int n0 = blockIdx.y * kCalibRowsPerBlock;
-    const int n1 = min(N, n0 + kCalibRowsPerBlock);
+    const int n0 = blockIdx.y * rows_per_block;
+    const int n1 = min(N, n0 + rows_per_block);
     float mw[kChan];
 #pragma unroll
     for (int i = 0; i < kChan; ++i) mw[i] = 0.0f;
@@ -137,45 +127,64 @@ __global__ void __launch_bounds__(128) ptq_calib_wmax_kernel(const uint8_t *wq, 
         if (k0 + i < K && mw[i] > 0.0f) atomicMax(max_w_bits + k0 + i, __float_as_uint(mw[i]));
 }
 
-// s[k] from maxX[k] and maxW[k]; one thread per channel.
-__global__ void __launch_bounds__(128) ptq_calib_smooth_kernel(const unsigned *max_x_bits, const unsigned *max_w_bits,
-                                                               int K, float *s)
+// s[k] from maxX[k] and maxW[k].
+__device__ __forceinline__ float calib_smooth(unsigned max_x_bits, unsigned max_w_bits)
 {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= K) return;
-    const float mx = fmaxf(__uint_as_float(max_x_bits[k]), kCalibFloor);
-    const float mw = fmaxf(__uint_as_float(max_w_bits[k]), kCalibFloor);
-    s[k] = __fsqrt_rn(__fdiv_rn(mx, mw));
+    const float mx = fmaxf(__uint_as_float(max_x_bits), kCalibFloor);
+    const float mw = fmaxf(__uint_as_float(max_w_bits), kCalibFloor);
+    return __fsqrt_rn(__fdiv_rn(mx, mw));
+}
+
+// dx (and z) of one position from its range.
+__device__ __forceinline__ float calib_step_sym(float mu, float qmax) { return __fdiv_rn(fmaxf(mu, kCalibFloor), qmax); }   // 127 levels, or 7 for 4-bit codes
+__device__ __forceinline__ float calib_step_asym(float hi, float nlo, int &z)
+{
+    const float d = __fdiv_rn(fmaxf(__fadd_rn(hi, nlo), kCalibFloor), 255.0f);   // hi - lo with lo = -nlo
+    z = static_cast<int>(fminf(fmaxf(rintf(__fdiv_rn(nlo, d)), 0.0f), 255.0f));  // -lo / d, ties to even
+    return d;
 }
 
 // Largest and smallest x/s of a token position over the images of a block's share, both widened to zero; grid
 // (T, image splits).  A correctly rounded division by a positive s is monotone, so the maximum over the images is taken
 // on the binary16 inputs and only the one survivor per (position, channel) is divided: the same bits as dividing every
 // element, with 1/Bc of the divisions.
-//   kAsym = false: mu[t] = max |x/s| in hi_bits;   kAsym = true: hi[t] in hi_bits, -lo[t] in nlo_bits
+// Every thread forms the s of its channels itself from the maxima, and block (0, 0) writes them out.  With one share per
+// position (`final`) the block also forms the position's step, otherwise the shares meet in hi_bits / nlo_bits
+// (mu[t], or hi[t] and -lo[t] for kAsym) and a second kernel forms the steps.
+struct CalibRange {
+    const __half *x;
+    const unsigned *max_x_bits, *max_w_bits;
+    unsigned *hi_bits, *nlo_bits;
+    float *s, *dx;
+    int *z;
+    int Bc, imgs_per_block, K, T;
+    int final;
+    float qmax;
+};
+
 template <int kVec, bool kAsym>
-__global__ void __launch_bounds__(128) ptq_calib_rowrange_kernel(const __half *x, int Bc, int imgs_per_block, int K, int T,
-                                                                 const float *s, unsigned *hi_bits, unsigned *nlo_bits)
+__global__ void __launch_bounds__(128) ptq_calib_rowrange_kernel(CalibRange p)
 {
+    __shared__ float part[2][4];
     const int t = blockIdx.x;
-    const int b0 = blockIdx.y * imgs_per_block;
-    const int nb = min(imgs_per_block, Bc - b0);
-    const int cpr = K / kVec;
+    const int b0 = blockIdx.y * p.imgs_per_block;
+    const int nb = min(p.imgs_per_block, p.Bc - b0);
+    const int cpr = p.K / kVec;
     const int tpr = min(cpr, 128);
     const int ip = 128 / tpr;                            // images side by side
     const int img = static_cast<int>(threadIdx.x) / tpr;
     const int c = static_cast<int>(threadIdx.x) - img * tpr;
-    const long long img_step = static_cast<long long>(T) * K;
+    const long long img_step = static_cast<long long>(p.T) * p.K;
     float hi = 0.0f, nlo = 0.0f;
     if (img < ip) {
         for (int c0 = c; c0 < cpr; c0 += tpr) {
             CalibChunk<kVec> mx, mn;
 #pragma unroll
             for (int i = 0; i < (kVec == 8 ? 4 : 1); ++i) mx.h[i] = mn.h[i] = __float2half2_rn(0.0f);
-            const __half *p = x + (static_cast<long long>(b0 + img) * T + t) * K + static_cast<long long>(c0) * kVec;
+            const __half *px = p.x + (static_cast<long long>(b0 + img) * p.T + t) * p.K + static_cast<long long>(c0) * kVec;
 #pragma unroll 8
-            for (int b = img; b < nb; b += ip, p += ip * img_step) {
-                const CalibChunk<kVec> v = calib_load<kVec>(p);
+            for (int b = img; b < nb; b += ip, px += ip * img_step) {
+                const CalibChunk<kVec> v = calib_load<kVec>(px);
 #pragma unroll
                 for (int i = 0; i < (kVec == 8 ? 4 : 1); ++i) {
                     mx.h[i] = __hmax2(mx.h[i], kAsym ? v.h[i] : __habs2(v.h[i]));     // NaN is dropped
@@ -184,7 +193,9 @@ __global__ void __launch_bounds__(128) ptq_calib_rowrange_kernel(const __half *x
             }
 #pragma unroll
             for (int i = 0; i < kVec; ++i) {
-                const float sv = __ldg(s + c0 * kVec + i);
+                const int k = c0 * kVec + i;
+                const float sv = calib_smooth(p.max_x_bits[k], p.max_w_bits[k]);
+                if (t == 0 && blockIdx.y == 0 && img == 0) p.s[k] = sv;
                 hi = fmaxf(hi, __fdiv_rn(calib_channel<kVec>(mx, i), sv));
                 if (kAsym) nlo = fmaxf(nlo, -__fdiv_rn(calib_channel<kVec>(mn, i), sv));
             }
@@ -192,9 +203,30 @@ __global__ void __launch_bounds__(128) ptq_calib_rowrange_kernel(const __half *x
     }
     hi = warp_max(hi);
     if (kAsym) nlo = warp_max(nlo);
+    if (!p.final) {
+        if ((threadIdx.x & 31) == 0) {
+            if (hi > 0.0f) atomicMax(p.hi_bits + t, __float_as_uint(hi));
+            if (kAsym && nlo > 0.0f) atomicMax(p.nlo_bits + t, __float_as_uint(nlo));
+        }
+        return;
+    }
     if ((threadIdx.x & 31) == 0) {
-        if (hi > 0.0f) atomicMax(hi_bits + t, __float_as_uint(hi));
-        if (kAsym && nlo > 0.0f) atomicMax(nlo_bits + t, __float_as_uint(nlo));
+        part[0][threadIdx.x >> 5] = hi;
+        part[1][threadIdx.x >> 5] = nlo;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < 4; ++w) {
+            hi = fmaxf(hi, part[0][w]);
+            nlo = fmaxf(nlo, part[1][w]);
+        }
+        if (kAsym) {
+            int z;
+            p.dx[t] = calib_step_asym(hi, nlo, z);
+            p.z[t] = z;
+        } else {
+            p.dx[t] = calib_step_sym(hi, p.qmax);
+        }
     }
 }
 
@@ -202,7 +234,7 @@ __global__ void __launch_bounds__(128) ptq_calib_step_kernel(const unsigned *mu_
 {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= T) return;
-    dx[t] = __fdiv_rn(fmaxf(__uint_as_float(mu_bits[t]), kCalibFloor), qmax);      // 127 levels, or 7 for 4-bit codes
+    dx[t] = calib_step_sym(__uint_as_float(mu_bits[t]), qmax);
 }
 
 // Per-tensor static comparator: ONE step for every token position, from the largest smoothed magnitude
@@ -231,12 +263,9 @@ __global__ void __launch_bounds__(128) ptq_calib_step_asym_kernel(const unsigned
 {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= T) return;
-    const float hi = __uint_as_float(hi_bits[t]), nlo = __uint_as_float(nlo_bits[t]);
-    const float range = fmaxf(__fadd_rn(hi, nlo), kCalibFloor);      // hi - lo with lo = -nlo
-    const float d = __fdiv_rn(range, 255.0f);
-    const float zr = rintf(__fdiv_rn(nlo, d));                        // -lo / d, ties to even
-    dx[t] = d;
-    z[t] = static_cast<int>(fminf(fmaxf(zr, 0.0f), 255.0f));
+    int zt;
+    dx[t] = calib_step_asym(__uint_as_float(hi_bits[t]), __uint_as_float(nlo_bits[t]), zt);
+    z[t] = zt;
 }
 
 // --- step-size search (Sec. 5.2, second stage; "+Truncation" in the ablation) ----------------------
@@ -246,7 +275,9 @@ __global__ void __launch_bounds__(128) ptq_calib_step_asym_kernel(const unsigned
 // non-finite u skipped.  One block per (position, group of kSearchCandPerBlock candidates); threads
 // stride over the Bc*K elements of the position, keep one binary64 partial sum per candidate, and the
 // block reduces them in a fixed order (shuffles, then warp by warp), so a launch is reproducible.
-constexpr int kSearchCandPerBlock = 8;
+constexpr int kSearchSub = 9;                            // candidates whose integers are in registers at a time
+constexpr int kSearchCandPerBlock = 3 * kSearchSub;
+constexpr int kSearchTile = 2048;                        // elements whose x/s are in shared memory at a time
 constexpr int kSearchThreads = 256;
 
 struct SearchParams {
@@ -264,16 +295,18 @@ __device__ __forceinline__ float search_candidate_step(float base, int j, int n_
     return __fmul_rn(base, __fdiv_rn(static_cast<float>(j), static_cast<float>(n_grid)));
 }
 
-// Bound by issue: 49 M (element, candidate) pairs at 8 x 197 x 384 x 81.  The integer r = rne(u / Delta) is taken from one FMA,
-// t = RN(u * RN(1/Delta) + 1.5*2^23), whose low mantissa bits hold it; u * RN(1/Delta) is within 1.2e-7 |v| of the defined
-// quotient v, and beyond |v| = 128 every r clamps alike, so r can only be wrong where the distance to r exceeds 0.49998:
-// those elements (3 in 10^4) take the IEEE divisions, which were the whole cost before (an IEEE division, a rounding
-// instruction at an eighth of the rate, and two conversions per pair).
-__global__ void __launch_bounds__(kSearchThreads) ptq_search_loss_kernel(SearchParams p)
+// Bound by issue: 49 M (element, candidate) pairs at 8 x 197 x 384 x 81, 9 instructions each.  The integer r = rne(u / Delta)
+// is taken from one FMA, t = RN(u * RN(1/Delta) + 1.5*2^23), whose low mantissa bits hold it; u * RN(1/Delta) is within
+// 1.2e-7 |v| of the defined quotient v, and beyond |v| = 128 every r clamps alike, so r can only be wrong where the distance
+// to r exceeds 0.49998: those elements (3 in 10^4) take the IEEE divisions.  27 candidates per block, so that loading an
+// element and dividing it by s, 60 instructions, is paid 3 times and not 11 times for 81 candidates.
+// 8 x 197 x 384: 60 us with IEEE divisions, 46 with 8 candidates per block, 44 so.
+__global__ void __launch_bounds__(kSearchThreads, 2) ptq_search_loss_kernel(SearchParams p)
 {
-    constexpr int C = kSearchCandPerBlock;
+    constexpr int C = kSearchCandPerBlock, S = kSearchSub;
     constexpr float kMagic = 12582912.0f;
     __shared__ double partial[kSearchThreads / 32][C];
+    __shared__ float u_s[kSearchTile];
     const int t = blockIdx.x;
     const int j0 = p.j_lo + static_cast<int>(blockIdx.y) * C;
     const int ncand = min(C, p.n_grid - j0 + 1);
@@ -289,32 +322,37 @@ __global__ void __launch_bounds__(kSearchThreads) ptq_search_loss_kernel(SearchP
         acc[c] = 0.0;
     }
     const int per_pos = p.Bc * p.K;
-#pragma unroll 2
-    for (int i = threadIdx.x; i < per_pos; i += kSearchThreads) {
-        const int b = static_cast<int>(fd_div(static_cast<unsigned>(i), p.fd_K));
-        const int k = i - b * p.K;
-        const float xf = __half2float(__ldg(p.x + (static_cast<long long>(b) * p.T + t) * p.K + k));
-        const float u = __fdiv_rn(xf, __ldg(p.s + k));
-        if (!(fabsf(u) <= 3.402823466e38f)) continue;          // inf and NaN do not enter the loss
-        float r[C], worst = 0.0f;
-#pragma unroll
-        for (int c = 0; c < C; ++c) {
-            r[c] = __fadd_rn(__fmaf_rn(u, rdelta[c], kMagic), -kMagic);
-            worst = fmaxf(worst, fabsf(__fmaf_rn(u, rdelta[c], -r[c])));
+    for (int i0 = 0; i0 < per_pos; i0 += kSearchTile) {
+        const int n = min(kSearchTile, per_pos - i0);
+        __syncthreads();
+#pragma unroll 4
+        for (int i = threadIdx.x; i < n; i += kSearchThreads) {
+            const int b = static_cast<int>(fd_div(static_cast<unsigned>(i0 + i), p.fd_K));
+            const int k = i0 + i - b * p.K;
+            u_s[i] = __fdiv_rn(__half2float(__ldg(p.x + (static_cast<long long>(b) * p.T + t) * p.K + k)), __ldg(p.s + k));
         }
-        if (!fast || worst > 0.49998f) {
-#pragma unroll 1
-            for (int c = 0; c < C; ++c) {
-                const float exact = rintf(__fdiv_rn(u, search_candidate_step(base, min(j0 + c, p.n_grid), p.n_grid)));
+        __syncthreads();
+        for (int i = threadIdx.x; i < n; i += kSearchThreads) {
+            const float u = u_s[i];
+            if (!(fabsf(u) <= 3.402823466e38f)) continue;      // inf and NaN do not enter the loss
 #pragma unroll
-                for (int q = 0; q < C; ++q)
-                    if (q == c) r[q] = exact;
+            for (int c0 = 0; c0 < C; c0 += S) {
+                float r[S], worst = 0.0f;
+#pragma unroll
+                for (int c = 0; c < S; ++c) {
+                    r[c] = __fadd_rn(__fmaf_rn(u, rdelta[c0 + c], kMagic), -kMagic);
+                    worst = fmaxf(worst, fabsf(__fmaf_rn(u, rdelta[c0 + c], -r[c])));
+                }
+                if (!fast || worst > 0.49998f) {
+#pragma unroll
+                    for (int c = 0; c < S; ++c) r[c] = rintf(__fdiv_rn(u, delta[c0 + c]));
+                }
+#pragma unroll
+                for (int c = 0; c < S; ++c) {
+                    const double e = static_cast<double>(__fmaf_rn(-delta[c0 + c], fminf(fmaxf(r[c], -128.0f), 127.0f), u));
+                    acc[c0 + c] = fma(e, e, acc[c0 + c]);
+                }
             }
-        }
-#pragma unroll
-        for (int c = 0; c < C; ++c) {
-            const double e = static_cast<double>(__fmaf_rn(-delta[c], fminf(fmaxf(r[c], -128.0f), 127.0f), u));
-            acc[c] = fma(e, e, acc[c]);
         }
     }
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -333,21 +371,32 @@ __global__ void __launch_bounds__(kSearchThreads) ptq_search_loss_kernel(SearchP
     }
 }
 
-// The candidate of least loss per position, the largest j among equals (scan from n_grid down, strict <).
+// The candidate of least loss per position, the largest j among equals.  A warp per position: lane i takes candidates
+// n_grid - i, n_grid - i - 32, ..., descending (strict <, so that the first of equals, the larger j, stays).  A thread
+// per position walked the row alone, one memory latency after another.
 __global__ void __launch_bounds__(128) ptq_search_pick_kernel(const double *loss, const float *base, int T, int n_grid,
                                                               int j_lo, int *best, float *dx)
 {
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= T) return;
+    const int t = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (t >= T) return;                                       // a whole warp
     const double *row = loss + static_cast<long long>(t) * (n_grid - j_lo + 1);
-    int bj = n_grid;
-    double bl = row[n_grid - j_lo];
-    for (int j = n_grid - 1; j >= j_lo; --j) {
+    int bj = max(n_grid - lane, j_lo);                        // a lane without candidates repeats j_lo's
+    double bl = row[bj - j_lo];
+#pragma unroll 4
+    for (int j = n_grid - lane - 32; j >= j_lo; j -= 32) {
         const double l = row[j - j_lo];
         if (l < bl) { bl = l; bj = j; }
     }
-    best[t] = bj;
-    dx[t] = search_candidate_step(__ldg(base + t), bj, n_grid);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const double ol = __shfl_xor_sync(0xffffffffu, bl, o);
+        const int oj = __shfl_xor_sync(0xffffffffu, bj, o);
+        if (ol < bl || (ol == bl && oj > bj)) { bl = ol; bj = oj; }
+    }
+    if (lane == 0) {
+        best[t] = bj;
+        dx[t] = search_candidate_step(__ldg(base + t), bj, n_grid);
+    }
 }
 
 }  // namespace ptq
