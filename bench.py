@@ -538,7 +538,7 @@ def run_ours(args, specs, rank, world, local_rank):
                 _, mn, med = event_times_ms(torch, gemm, iters)
                 avg = region_time_ms(torch, gemm, iters)
             gname = ("ptq_gemm_dequant_pair_kernel" if flags & ptq.FLAG_CTA_PAIR else
-                     ("ptq_gemm_dequant_kernel", "ptq_gemm_dequant_kernel<teams>", "ptq_gemm_dequant_panel_kernel")[layer.gemm_variant(sp.B)])
+                     ("ptq_gemm_dequant_kernel", "ptq_gemm_dequant_resident_kernel", "ptq_gemm_dequant_panel_kernel")[layer.gemm_variant(sp.B)])
             kernels.append(dict(kernel=gname, layer=tag, ms=avg, ms_single_median=med, ms_single_min=mn,
                                 ops=2.0 * M * K * N, bytes=1.0 * M * K + N * K + 2.0 * M * N))
             del qdense

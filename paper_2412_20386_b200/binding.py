@@ -369,7 +369,7 @@ class PtqLinear:
         return int(self._L.ptq_linear_code_pitch(self._h))
 
     def gemm_variant(self, B: int) -> int:
-        """``ptq_linear_gemm_variant``: 0 streaming kernel, 1 streaming with two epilogue teams, 2 panel kernel."""
+        """``ptq_linear_gemm_variant``: 0 streaming kernel, 1 resident weights, 2 resident panel of codes."""
         return int(self._L.ptq_linear_gemm_variant(self._h, int(B)))
 
     def gemm_dequant(self, q, B: int, y=None, stream=None):

@@ -425,7 +425,9 @@ bool plan_panel(const ptq_linear *h, ptq::GemmParams &p, bool tma_store)
     return true;
 }
 
-// Whether the streaming kernel runs its epilogue in two teams: short main loop (K <= 384) and several tiles per CTA.
+// Whether the kernel with resident weights (and its epilogue in two teams) is taken: short main loop (K <= 384) and three tiles
+// per CTA.  With two the streaming kernel's shorter latency of a tile wins: 12608 x 192 -> 768 10.5 us against 11.1, 6304 x 384 ->
+// 1536 11.0 against 12.2, 25088 x 384 -> 384 14.3 against 14.7; with four and more this one does (figures at the kernel).
 bool gemm_teams(const ptq_linear *h, const ptq::GemmParams &p, bool tma_store, bool short_k)
 {
     const long long tiles = static_cast<long long>(p.m_tiles) * p.n_tiles;
@@ -589,20 +591,27 @@ ptq_status_t launch_gemm(const ptq_linear *h, const void *codes, long long M, vo
     if (bn != h->BN) set_bn(h, p, bn);
     const CUtensorMap &tmW = bn != h->BN ? h->tmWbn[bn / 64 - 1] : h->tmW;
     const long long tiles = static_cast<long long>(p.m_tiles) * p.n_tiles;
-    // Short main loop (K <= 384) and several tiles per CTA: the epilogue sets the pace and runs in two teams of
-    // four warps, one per accumulator; otherwise all eight warps share every tile (shorter latency of a tile).
     const bool teams = gemm_teams(h, p, tma_store, short_k);
     const int grid = static_cast<int>(tiles < h->num_sms ? tiles : h->num_sms);
-    auto go = [&](auto debug, auto team, auto asym) -> ptq_status_t {
-        constexpr auto kKern = ptq::ptq_gemm_dequant_kernel<decltype(debug)::value, decltype(team)::value, decltype(asym)::value>;
-        const ptq_status_t es = ensure_smem<kKern>(h->device, ptq::kGemmSmemBytes);
-        if (es != PTQ_OK) return es;
-        PTQ_CUDA(launch_pdl(kKern, grid, ptq::kGemmThreads, gemm_smem, stream, tmA, tmW, tmY, p));
+    auto go = [&](auto debug, auto asym) -> ptq_status_t {
+        constexpr bool kDbg = decltype(debug)::value, kAsym = decltype(asym)::value;
+        if (teams) {
+            constexpr auto kKern = ptq::ptq_gemm_dequant_resident_kernel<kDbg, kAsym>;
+            p.fd_n_tiles = ptq::make_fastdiv(static_cast<unsigned>(p.m_tiles));
+            const ptq_status_t es = ensure_smem<kKern>(h->device, ptq::kResSmemMax);
+            if (es != PTQ_OK) return es;
+            const int smem = ptq::res_smem_bytes(p.k_blocks, p.BN, p.vectors);
+            PTQ_CUDA(launch_pdl(kKern, grid, ptq::kGemmThreads, smem, stream, tmA, tmW, tmY, p));
+        } else {
+            constexpr auto kKern = ptq::ptq_gemm_dequant_kernel<kDbg, kAsym>;
+            const ptq_status_t es = ensure_smem<kKern>(h->device, ptq::kGemmSmemBytes);
+            if (es != PTQ_OK) return es;
+            PTQ_CUDA(launch_pdl(kKern, grid, ptq::kGemmThreads, gemm_smem, stream, tmA, tmW, tmY, p));
+        }
         return PTQ_OK;
     };
-    auto pick = [&](auto team, auto asym) { return dbg ? go(std::true_type(), team, asym) : go(std::false_type(), team, asym); };
-    const ptq_status_t gs = h->asym ? (teams ? pick(std::true_type(), std::true_type()) : pick(std::false_type(), std::true_type()))
-                                    : (teams ? pick(std::true_type(), std::false_type()) : pick(std::false_type(), std::false_type()));
+    const ptq_status_t gs = h->asym ? (dbg ? go(std::true_type(), std::true_type()) : go(std::false_type(), std::true_type()))
+                                    : (dbg ? go(std::true_type(), std::false_type()) : go(std::false_type(), std::false_type()));
     if (gs != PTQ_OK) return gs;
     g_launches.fetch_add(1, std::memory_order_relaxed);
     PTQ_CUDA(cudaGetLastError());

@@ -101,7 +101,7 @@ struct GemmParams {
     // units cover a panel; the weight ring has `b_stages` slots of `b_stage_bytes` (= BN * 128) each.
     int group, groups;
     int b_stages, b_stage_bytes;
-    FastDiv fd_T, fd_n_tiles, fd_groups;   // divisors T, n_tiles, groups (the GEMM kernels' loops)
+    FastDiv fd_T, fd_n_tiles, fd_groups;   // divisors T, n_tiles (resident kernel: m_tiles), groups
 };
 
 // --- epilogue helpers -------------------------------------------------------------------------
@@ -495,9 +495,8 @@ __device__ __forceinline__ RowStep load_row_step(const GemmParams &p, int m_tile
 // the accumulator.  In team mode the eight warps form two teams of four (one warp per TMEM lane quarter
 // and per scheduler); team b drains accumulator b, i.e. every second tile of the CTA, all 64-column
 // steps of it.  A tile's epilogue takes longer, but it has two main loops' time to finish, and one
-// team's waits are filled by the other team's arithmetic.  Used when a CTA has several tiles and the
-// main loop of a tile is short (K <= 384), i.e. where the epilogue sets the pace: 7-8 % on such layers
-// with many rows; layers with a long main loop are bounded elsewhere and gain nothing.
+// team's waits are filled by the other team's arithmetic.  Used by the kernel with resident weights, i.e. where the epilogue
+// sets the pace: 7-8 % on such layers with many rows; layers with a long main loop are bounded elsewhere and gain nothing.
 //
 // The team's copy of the tile's weight steps (and bias) lives in scale buffer b; a named barrier over
 // the team's 128 threads publishes it (together with the vote on the bounded waits, so that the four
@@ -520,21 +519,22 @@ __device__ __forceinline__ bool team_all(bool pred, int team)
 }
 __device__ __forceinline__ void team_sync(int team) { asm volatile("bar.sync %0, 128;" ::"r"(1 + team) : "memory"); }
 
-// The CTA's tiles in the order the MMA thread produces them.
-struct StreamCursor {
-    int tile, total, step, n_tiles;
-    FastDiv fd;
-    __device__ bool valid() const { return tile < total; }
+// The CTA's tiles in the order the MMA thread produces them.  Tiles are numbered with the row tiles of an N tile adjacent;
+// with several N tiles a CTA takes a contiguous share, so that its weights change at most once or twice, with a single one it
+// strides over them, so that the CTAs read and write neighbouring rows at a time (200704 x 384 -> 96: 60.0 -> 58.5 us).
+struct TileCursor {
+    int tile, end, step, m_tiles;
+    FastDiv fd_m;
+    __device__ bool valid() const { return tile < end; }
     __device__ void advance() { tile += step; }
-    __device__ int m_tile() const { return static_cast<int>(fd_div(static_cast<unsigned>(tile), fd)); }
-    __device__ int n_tile() const { return tile - m_tile() * n_tiles; }
+    __device__ int n_tile() const { return static_cast<int>(fd_div(static_cast<unsigned>(tile), fd_m)); }
+    __device__ int m_tile() const { return tile - n_tile() * m_tiles; }
 };
 
-template <bool kDebugAcc, bool kAsym, class Cursor>
-__device__ __forceinline__ void epilogue_team_loop(const GemmParams &p, const CUtensorMap *tmY, Cursor cur, uint32_t tmem_base,
+template <bool kDebugAcc, bool kAsym>
+__device__ __forceinline__ void epilogue_team_loop(const GemmParams &p, const CUtensorMap *tmY, TileCursor cur, uint32_t tmem_base,
                                                    uint32_t tfull_bar0, uint32_t tempty_bar0, float *scale_s,
-                                                   uint32_t staging, bool two_boxes, volatile uint32_t *abort_flag,
-                                                   int warp, int lane)
+                                                   uint32_t staging, volatile uint32_t *abort_flag, int warp, int lane)
 {
     const int quarter = warp & 3;                       // TMEM lanes [32*quarter, 32*quarter+32)
     const int team = (warp - 2) >> 2;                   // = the accumulator buffer this team drains
@@ -546,7 +546,7 @@ __device__ __forceinline__ void epilogue_team_loop(const GemmParams &p, const CU
     if (team == 1 && cur.valid()) cur.advance();        // team 1 starts at the CTA's second tile
     float dw_next[2] = {0.0f, 0.0f}, bias_next[2] = {0.0f, 0.0f};
     int ws_next[2] = {0, 0};
-    auto fetch_scales = [&](const Cursor &c) {
+    auto fetch_scales = [&](const TileCursor &c) {
         // unconditional loads from clamped indices (see load_row_step); past the last tile the values are not used
         const int n0 = c.valid() ? c.n_tile() * p.BN : 0;
 #pragma unroll
@@ -586,7 +586,7 @@ __device__ __forceinline__ void epilogue_team_loop(const GemmParams &p, const CU
         const uint32_t tmem_row = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) + static_cast<uint32_t>(team) * kMaxBN;
         nboxes = epilogue_tile_stream<kDebugAcc, kAsym>(p, tmY, tmem_row, m_row0, n_tile * p.BN, dxr, staging, dw_buf,
                                                  p.has_bias ? bias_buf : nullptr, !kAsym ? nullptr : p.ws_copy ? ws_buf : p.wsum + n_tile * p.BN, nboxes,
-                                                 lane, 0, kEpiStepCols, zr, two_boxes);
+                                                 lane, 0, kEpiStepCols, zr, true);
         tc_fence_before_sync();
         __syncwarp();
         if (lane == 0) mbar_arrive(tempty);
@@ -598,7 +598,7 @@ __device__ __forceinline__ void epilogue_team_loop(const GemmParams &p, const CU
 
 // --- the kernel ---------------------------------------------------------------------------------
 
-template <bool kDebugAcc, bool kTeams, bool kAsym>
+template <bool kDebugAcc, bool kAsym>
 __global__ void __launch_bounds__(kGemmThreads, 1)
 ptq_gemm_dequant_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmW,
                         const __grid_constant__ CUtensorMap tmY, const GemmParams p)
@@ -635,7 +635,7 @@ ptq_gemm_dequant_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
         }
         for (uint32_t b = 0; b < 2; ++b) {
             mbar_init(tfull_bar(b), 1);
-            mbar_init(tempty_bar(b), kTeams ? kNumEpiWarps / 2 : kNumEpiWarps);   // in team mode one team drains a buffer
+            mbar_init(tempty_bar(b), kNumEpiWarps);
         }
         mbar_init(scale_bar, kNumEpiWarps);
         *abort_flag = 0u;
@@ -741,14 +741,6 @@ ptq_gemm_dequant_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
                 if (buf == 0u) bphase ^= 1u;
             }
         }
-    } else if (kTeams) {
-        // ------------------------------------------------------------------ epilogue warps, two teams (TMA stores only)
-        griddep_wait();
-        const StreamCursor cur{static_cast<int>(blockIdx.x), total_tiles, static_cast<int>(gridDim.x), p.n_tiles, p.fd_n_tiles};
-        epilogue_team_loop<kDebugAcc, kAsym>(p, &tmY, cur, tmem_base, tfull_bar(0), tempty_bar(0),
-                                      reinterpret_cast<float *>(smem_raw + scale_off),
-                                      staging_base + static_cast<uint32_t>(warp - 2) * static_cast<uint32_t>(p.boxes) * kStreamStagingPerWarp,
-                                      two_boxes, abort_flag, warp, lane);
     } else {
         // ------------------------------------------------------------------ epilogue warps
         griddep_wait();
@@ -1100,6 +1092,204 @@ ptq_gemm_dequant_panel_kernel(const __grid_constant__ CUtensorMap tmA, const __g
             ++it;
         }
         if (lane == 0) bulk_wait_group<0>();         // all of this thread's stores have completed
+    }
+
+    __syncthreads();
+    if (warp == 1) {
+        __syncwarp();
+        tc_fence_after_sync();
+        tmem_dealloc(tmem_base, kTmemCols);
+    }
+}
+
+// --- weights resident ---------------------------------------------------------------------------
+//
+// Same computation for layers with a short main loop (K <= 384) and several tiles per CTA.  Such a layer is bound by its
+// output: the SM moves 2 x BN bytes of y per row against K bytes of codes, and the loads share its TMA unit and the way to L2
+// with the stores.  The weights of one N tile (at most 96 KB) therefore stay in shared memory and only the codes stream:
+// 128 x K bytes per output tile instead of (128 + BN) x K, a third at BN = 256.  Whole forward, streamed weights -> resident:
+// 200704 x 96 -> 384: 43.2 -> 41.3 us; 200704 x 192 -> 384: 53.8 -> 52.2; 50176 x 192 -> 768: 24.2 -> 23.5; 25216 x 384 -> 1536:
+// 26.5 -> 26.1; 200704 x 64 -> 256: 33.5 -> 29-31.  The narrowest outputs gain nothing: 200704 x 192 -> 96: 32.8 -> 32.9.
+//
+// Three stages of codes: two cost 2 to 10 % (200704 x 384 -> 96: 65 us, not 58.5), and with eight the loads run so far ahead
+// of the stores that 200704 x 192 -> 96 takes 34.0 us, not 33.0; the other shapes cannot tell three from eight.
+//
+// Barriers: full/empty per stage of codes, wfull/wempty for the weights (the MMA thread frees them with a commit behind the
+// last tile that uses them), tfull/tempty per accumulator.  The epilogue runs in two teams.
+constexpr int kResMaxKBlocks = 3;
+constexpr int kResStages = 3;
+constexpr int kResNumBarriers = 2 * kResStages + 2 + 4;
+__host__ __device__ constexpr int res_smem_bytes(int k_blocks, int bn, int vectors)
+{
+    return k_blocks * bn * kBK + kResStages * kATileBytes + 2 * kNumEpiWarps * kStreamStagingPerWarp + 2 * vectors * kScaleBufBytes +
+           kResNumBarriers * 8 + 16;
+}
+constexpr int kResSmemMax = res_smem_bytes(kResMaxKBlocks, kMaxBN, 3);
+static_assert(kResSmemMax <= 232448, "resident kernel exceeds the shared memory of one CTA");
+
+template <bool kDebugAcc, bool kAsym>
+__global__ void __launch_bounds__(kGemmThreads, 1)
+ptq_gemm_dequant_resident_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmW,
+                                 const __grid_constant__ CUtensorMap tmY, const GemmParams p)
+{
+    extern __shared__ __align__(1024) uint8_t smem_raw[];
+    const uint32_t base = smem_u32(smem_raw);
+    if ((base & 1023u) != 0u) {
+        if (threadIdx.x == 0) atomicOr(p.status, PTQ_DEV_SMEM_ALIGN);
+        return;
+    }
+    constexpr uint32_t nstages = kResStages;
+    const uint32_t w_bytes = static_cast<uint32_t>(p.BN) * kBK;                   // one k-block of weights
+    const uint32_t a_off = static_cast<uint32_t>(p.k_blocks) * w_bytes;
+    const uint32_t staging_off = a_off + nstages * kATileBytes;
+    const uint32_t scale_off = staging_off + 2 * kNumEpiWarps * kStreamStagingPerWarp;
+    const uint32_t bar_off = scale_off + 2 * p.vectors * kScaleBufBytes;
+    const uint32_t bar_base = base + bar_off;
+    auto full_bar = [&](uint32_t s) { return bar_base + 8u * s; };
+    auto empty_bar = [&](uint32_t s) { return bar_base + 8u * (kResStages + s); };
+    const uint32_t wfull_bar = bar_base + 8u * (2 * kResStages), wempty_bar = wfull_bar + 8u;
+    auto tfull_bar = [&](uint32_t b) { return bar_base + 8u * (2 * kResStages + 2 + b); };
+    auto tempty_bar = [&](uint32_t b) { return bar_base + 8u * (2 * kResStages + 4 + b); };
+    volatile uint32_t *tmem_holder = reinterpret_cast<volatile uint32_t *>(smem_raw + bar_off + kResNumBarriers * 8);
+    volatile uint32_t *abort_flag = tmem_holder + 1;
+
+    const int warp = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31;
+
+    if (threadIdx.x == 0) {
+        for (uint32_t s = 0; s < nstages; ++s) {
+            mbar_init(full_bar(s), 1);
+            mbar_init(empty_bar(s), 1);
+        }
+        mbar_init(wfull_bar, 1);
+        mbar_init(wempty_bar, 1);
+        for (uint32_t b = 0; b < 2; ++b) {
+            mbar_init(tfull_bar(b), 1);
+            mbar_init(tempty_bar(b), kNumEpiWarps / 2);                          // one team drains a buffer
+        }
+        *abort_flag = 0u;
+        fence_mbar_init();
+        prefetch_tensormap(&tmA);
+        prefetch_tensormap(&tmW);
+        prefetch_tensormap(&tmY);
+    }
+    if (warp == 1) {
+        tmem_alloc(smem_u32(const_cast<uint32_t *>(tmem_holder)), kTmemCols);
+        tmem_relinquish_alloc_permit();
+    }
+    tc_fence_before_sync();
+    __syncthreads();
+    tc_fence_after_sync();
+    const uint32_t tmem_base = *tmem_holder;
+    griddep_launch_dependents();         // the codes (and row steps) of the kernel before are read behind griddep_wait() only
+
+    const int total = p.m_tiles * p.n_tiles, grid = static_cast<int>(gridDim.x), cta = static_cast<int>(blockIdx.x);
+    const int share = total / grid, extra = total - share * grid;
+    TileCursor cur;
+    const bool strided = p.n_tiles == 1;
+    cur.tile = strided ? cta : cta * share + min(cta, extra);
+    cur.end = strided ? total : cur.tile + share + (cta < extra ? 1 : 0);
+    cur.step = strided ? grid : 1;
+    cur.m_tiles = p.m_tiles;
+    cur.fd_m = p.fd_n_tiles;
+
+    if (warp == 0) {
+        // ------------------------------------------------------------------ TMA producer
+        if (lane == 0 && cur.valid()) {
+            uint32_t stage = 0, phase = 0, issued = 0, w_loads = 0;
+            int w_tile = -1;
+            auto load_weights = [&](int n_tile) {
+                mbar_arrive_expect_tx(wfull_bar, static_cast<uint32_t>(p.k_blocks) * w_bytes);
+                for (int kb = 0; kb < p.k_blocks; ++kb)
+                    tma_load_2d(base + static_cast<uint32_t>(kb) * w_bytes, &tmW, kb * kBK, n_tile * p.BN, wfull_bar);
+                w_tile = n_tile;
+                ++w_loads;
+            };
+            load_weights(cur.n_tile());                                          // parameters: before the dependency wait
+            griddep_wait();
+            bool ok = true;
+            for (; cur.valid() && ok; cur.advance()) {
+                const int n_tile = cur.n_tile(), m_tile = cur.m_tile();
+                if (n_tile != w_tile) {
+                    if (!mbar_wait(wempty_bar, (w_loads - 1u) & 1u, abort_flag, p.status)) {
+                        ok = false;
+                        break;
+                    }
+                    load_weights(n_tile);
+                }
+                for (int kb = 0; kb < p.k_blocks; ++kb) {
+                    if (!mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag, p.status)) {
+                        ok = false;
+                        break;
+                    }
+                    mbar_arrive_expect_tx(full_bar(stage), kATileBytes);
+                    tma_load_2d(base + a_off + stage * kATileBytes, &tmA, kb * kBK, m_tile * kBM, full_bar(stage));
+                    ++issued;
+                    if (++stage == nstages) {
+                        stage = 0;
+                        phase ^= 1u;
+                    }
+                }
+            }
+            if (!ok) {
+                // Error path only: let this thread's own loads land before the CTA gives up its shared memory (bounded).
+                for (uint32_t s = 0; s < nstages; ++s) {
+                    const uint32_t uses = (issued + nstages - 1u - s) / nstages;
+                    if (uses == 0u) continue;
+                    for (int i = 0; i < 200000 && !mbar_try_wait(full_bar(s), (uses - 1u) & 1u); ++i) {
+                    }
+                }
+                for (int i = 0; i < 200000 && !mbar_try_wait(wfull_bar, (w_loads - 1u) & 1u); ++i) {
+                }
+            }
+        }
+    } else if (warp == 1) {
+        // ------------------------------------------------------------------ MMA issuer
+        if (lane == 0) {
+            const uint32_t idesc = make_idesc_s8(kBM, p.BN, kAsym);
+            uint32_t stage = 0, phase = 0, buf = 0, bphase = 0, w_uses = 0;
+            int w_tile = -1;
+            bool ok = true;
+            while (cur.valid() && ok) {
+                const int n_tile = cur.n_tile();
+                if (n_tile != w_tile) {
+                    if (!mbar_wait(wfull_bar, w_uses & 1u, abort_flag, p.status)) break;
+                    w_tile = n_tile;
+                    ++w_uses;
+                }
+                if (!mbar_wait(tempty_bar(buf), bphase ^ 1u, abort_flag, p.status)) break;
+                tc_fence_after_sync();
+                const uint32_t d_tmem = tmem_base + buf * kMaxBN;
+                for (int kb = 0; kb < p.k_blocks; ++kb) {
+                    if (!mbar_wait(full_bar(stage), phase, abort_flag, p.status)) {
+                        ok = false;
+                        break;
+                    }
+                    tc_fence_after_sync();
+                    mma_i8_ss_kblock(d_tmem, make_smem_desc_sw128(base + a_off + stage * kATileBytes),
+                                     make_smem_desc_sw128(base + static_cast<uint32_t>(kb) * w_bytes), idesc, kb != 0 ? 1u : 0u,
+                                     kb == p.k_blocks - 1 ? p.last_mmas : kBK / 32);
+                    mma_commit(empty_bar(stage));
+                    if (++stage == nstages) {
+                        stage = 0;
+                        phase ^= 1u;
+                    }
+                }
+                if (!ok) break;
+                mma_commit(tfull_bar(buf));          // accumulator complete
+                buf ^= 1u;
+                if (buf == 0u) bphase ^= 1u;
+                cur.advance();
+                if (cur.valid() && cur.n_tile() != w_tile) mma_commit(wempty_bar);   // the weights have been read for the last time
+            }
+        }
+    } else {
+        // ------------------------------------------------------------------ epilogue warps, two teams
+        griddep_wait();
+        epilogue_team_loop<kDebugAcc, kAsym>(p, &tmY, cur, tmem_base, tfull_bar(0), tempty_bar(0),
+                                             reinterpret_cast<float *>(smem_raw + scale_off),
+                                             base + staging_off + static_cast<uint32_t>(warp - 2) * 2u * kStreamStagingPerWarp,
+                                             abort_flag, warp, lane);
     }
 
     __syncthreads();

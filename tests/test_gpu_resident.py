@@ -1,0 +1,62 @@
+"""The GEMM kernel that keeps its weights in shared memory (K <= 384, three tiles and more per CTA), where its tile order and
+its weight reloads can go wrong: a single N tile (CTAs stride over the rows), shares that run over one and over several N
+tiles, one to three k-blocks with ragged K, ragged N, asymmetric layers and layers with a bias.  Oracle: the integer
+accumulators computed on the host from the codes and weights, every element, and the scaled output within the repository's bound
+max(2^-10 |y|, 1e-3)."""
+import numpy as np
+import pytest
+
+from paper_2412_20386_b200 import workloads as wl
+from parity_util import assert_y_close, layer_inputs
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def env():
+    import torch
+    assert torch.cuda.is_available(), "GPU tests need a CUDA device"
+    import __graft_entry__ as entry
+    entry.build()
+    import paper_2412_20386_b200 as ptq
+    torch.cuda.set_device(0)
+    return ptq, torch
+
+
+@pytest.mark.parametrize("K,N,T,B,bias,asym", [
+    (96, 96, 784, 80, False, False),       # one N tile, strided
+    (384, 200, 197, 300, True, True),      # one N tile, three k-blocks
+    (200, 600, 197, 110, True, False),     # a share crosses one N tile; K and N ragged
+    (40, 60000, 67, 3, False, False),      # two row tiles: a share crosses several N tiles
+    (384, 58000, 64, 4, False, True),
+    (256, 16, 7, 8121, False, False),      # a single 16-column step per tile
+])
+def test_resident_weights(env, K, N, T, B, bias, asym):
+    ptq, torch = env
+    spec = wl.LinearSpec(13, K % 89, N % 7, "resident", B, T, K, N, bias=bias)
+    x, wq, dw, b, s, dx = layer_inputs(spec, B=1)
+    z = (np.arange(T) * 37 % 256).astype(np.int32) if asym else None
+    layer = ptq.PtqLinear(wq, dw, s, dx, b, act_zero=z) if asym else ptq.PtqLinear(wq, dw, s, dx, b)
+    assert layer.gemm_variant(B) == 1
+    g = torch.Generator(device="cuda").manual_seed(K + N)
+    xd = torch.randn(B, T, K, device="cuda", generator=g).half() * torch.from_numpy(s).cuda().half()
+    y, codes, acc = layer.forward_debug(xd)
+    y2 = layer.forward(xd)
+    torch.cuda.synchronize()
+    layer.device_status()
+    assert torch.equal(y, y2)
+    M = B * T
+    c = codes.reshape(M, K).double()
+    if asym:
+        c = c - torch.from_numpy(z).cuda().double().repeat(B)[:, None]
+    w = torch.from_numpy(wq).cuda().double()
+    acc, y = acc.reshape(M, N), y.reshape(M, N)
+    dxr = torch.from_numpy(dx).cuda().double().repeat(B)[:, None]
+    for m0 in range(0, M, 8192):                                     # |acc| < 2^53: the products and sums are exact in binary64
+        ref = c[m0:m0 + 8192] @ w.T
+        assert torch.equal(acc[m0:m0 + 8192].double(), ref), "accumulators differ in rows from %d" % m0
+        ref = ref * dxr[m0:m0 + 8192] * torch.from_numpy(dw).cuda().double()
+        if b is not None:
+            ref = ref + torch.from_numpy(b).cuda().double()
+        assert_y_close(y[m0:m0 + 8192].cpu().numpy(), ref.cpu().numpy(), "rows from %d" % m0)
+    layer.close()
