@@ -164,13 +164,35 @@ __device__ __forceinline__ float group_max(float v)
     return v;
 }
 
+// max RN(|x|/s) over the channels of a chunk with RN(|x| * RN(1/s)) >= edge.  Rare: unrolled into every chunk of
+// the kernel below its divisions cost more instruction-cache misses than calls (50432 x 1536: 79 -> 71 us for this and for
+// leaving the saturating route out of the second pass); with a single chunk the call costs more (50176 x 192: 22.4 -> 22.9).
+__device__ __forceinline__ float divided_max_inline(uint4 v, const float4 *ra, const float4 *rb, const float *s8, float edge)
+{
+    const uint32_t xw[4] = {v.x, v.y, v.z, v.w};
+    float mu = 0.0f;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const float f = fabsf(__half2float(__ushort_as_half(static_cast<unsigned short>(xw[i >> 1] >> ((i & 1) * 16)))));
+        const float r = reinterpret_cast<const float *>(i < 4 ? ra : rb)[i & 3];
+        if (__fmul_rn(f, r) >= edge) mu = fmaxf(mu, __fdiv_rn(f, s8[i]));
+    }
+    return mu;
+}
+__device__ __noinline__ float divided_max_call(uint4 v, const float4 *ra, const float4 *rb, const float *s8, float edge)
+{
+    return divided_max_inline(v, ra, rb, s8, edge);
+}
+
 // Row path: K <= 1536, K % 8 == 0, x 16-byte aligned, q 8-byte aligned, scales in the reciprocal range.  A warp holds one row
 // of x in registers (kChunks chunks of 8 channels per lane), so that x is read once; s and 1/s sit in shared memory.
 // The row maximum of RN(|x|/s) needs no division per element: a = RN(|x| * RN(1/s)) is within 2^-23 of the quotient,
 // so only elements with a >= (1 - 2^-21) * max a can hold the maximum, and only those (one or two a row) are divided.
-// Bound by issue (10 instructions an element) and, with few rows, by its chain of latencies: load, two warp reductions,
-// store.  6304 x 768: quantize + GEMM to 3072 channels 28.5 -> 24.9 us, 6304 x 1536 -> 768 29.8 -> 23.1, 50432 x 768 -> 8 58.0 -> 42.4, against the two-pass
-// kernel above.
+// Each lane copies its part of the warp's next row into shared memory (cp.async) while it works on this one: in registers the
+// second row spilled and lost (6304 x 1536 -> 768: 25.4 us), without it that layer took 23.1 us and 50432 x 1536 -> 8 86.5.
+// Bound by issue (15 instructions an element, 64 % of the issue slots taken) and, with few rows, by its chain of latencies: load,
+// two warp reductions, store.  Quantize + GEMM, against the two-pass kernel above: 6304 x 768 -> 3072 28.5 -> 24.4 us, 6304 x 1536 ->
+// 768 29.8 -> 21.2, 50432 x 768 -> 8 58.0 -> 39.4.
 constexpr int dyn_row_ctas_per_sm(int chunks) { return chunks <= 3 ? 4 : 3; }
 // kLanes lanes share a row: 32, or 16 / 8 where a row has no more chunks (kChunks = 1).
 template <int kChunks, int kLanes = 32>
@@ -181,6 +203,7 @@ __global__ void __launch_bounds__(256, dyn_row_ctas_per_sm(kChunks)) ptq_quantiz
     const int lane = threadIdx.x & (kLanes - 1);
     const int cpr = p.K >> 3;
     __shared__ float4 r_s[2][kChunks * kLanes];                    // 1/s of a chunk's channels 0-3 and 4-7: conflict-free reads
+    __shared__ uint4 x_s[kChunks][256];
     for (int k = threadIdx.x; k < p.K; k += 256) s_s[k] = __ldg(p.s + k);
     for (int i = threadIdx.x; i < 2 * cpr; i += 256) r_s[i & 1][i >> 1] = __ldg(reinterpret_cast<const float4 *>(p.rs) + i);
     {
@@ -193,16 +216,26 @@ __global__ void __launch_bounds__(256, dyn_row_ctas_per_sm(kChunks)) ptq_quantiz
     griddep_wait();
     griddep_launch_dependents();
 
-    for (long long m0 = static_cast<long long>(blockIdx.x) * kRows; m0 < p.M; m0 += static_cast<long long>(gridDim.x) * kRows) {
+    // Each lane copies its chunks of the next row into its own slots while it works on this one, and reads nobody else's.
+    const uint64_t once = l2_policy_evict_first();
+    const auto fetch = [&](long long m) {
+        if (m < p.M) {
+            const uint4 *xrow = reinterpret_cast<const uint4 *>(p.x + m * p.K);
+#pragma unroll
+            for (int j = 0; j < kChunks; ++j)
+                if (lane + kLanes * j < cpr) cp_async_16_hint(&x_s[j][threadIdx.x], xrow + lane + kLanes * j, once);
+        }
+        cp_async_commit();
+    };
+    long long m0 = static_cast<long long>(blockIdx.x) * kRows;
+    fetch(m0 + threadIdx.x / kLanes);
+    for (; m0 < p.M; m0 += static_cast<long long>(gridDim.x) * kRows) {
         const long long m = m0 + threadIdx.x / kLanes;
         const bool row_ok = m < p.M;                           // (whole warps run every round: the shuffles below need all lanes)
-        const uint4 *xrow = reinterpret_cast<const uint4 *>(p.x + m * p.K);
         uint4 v[kChunks];
+        cp_async_wait<0>();
 #pragma unroll
-        for (int j = 0; j < kChunks; ++j) {
-            v[j] = make_uint4(0u, 0u, 0u, 0u);
-            if (row_ok && lane + kLanes * j < cpr) v[j] = __ldg(xrow + lane + kLanes * j);
-        }
+        for (int j = 0; j < kChunks; ++j) v[j] = row_ok && lane + kLanes * j < cpr ? x_s[j][threadIdx.x] : make_uint4(0u, 0u, 0u, 0u);
         float cm[kChunks], top = 0.0f;
 #pragma unroll
         for (int j = 0; j < kChunks; ++j) {
@@ -220,18 +253,15 @@ __global__ void __launch_bounds__(256, dyn_row_ctas_per_sm(kChunks)) ptq_quantiz
             }
         }
         top = group_max<kLanes>(top);
+        fetch(m + static_cast<long long>(gridDim.x) * kRows);  // every chunk of this row has been read: its slots are free
         const float edge = __fmul_rn(top, 0.9999995f);         // below 1 - 2^-21
         float mu = 0.0f;
 #pragma unroll
         for (int j = 0; j < kChunks; ++j) {
             if (top > 0.0f && cm[j] >= edge) {
-                const uint32_t xw[4] = {v[j].x, v[j].y, v[j].z, v[j].w};
-#pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    const float f = fabsf(__half2float(__ushort_as_half(static_cast<unsigned short>(xw[i >> 1] >> ((i & 1) * 16)))));
-                    const float r = reinterpret_cast<const float *>(&r_s[i >> 2][lane + kLanes * j])[i & 3];
-                    if (__fmul_rn(f, r) >= edge) mu = fmaxf(mu, __fdiv_rn(f, s_s[8 * (lane + kLanes * j) + i]));
-                }
+                const int c = lane + kLanes * j;
+                mu = fmaxf(mu, kChunks == 1 ? divided_max_inline(v[j], &r_s[0][c], &r_s[1][c], s_s + 8 * c, edge)
+                                            : divided_max_call(v[j], &r_s[0][c], &r_s[1][c], s_s + 8 * c, edge));
             }
         }
         mu = group_max<kLanes>(mu);
@@ -246,16 +276,15 @@ __global__ void __launch_bounds__(256, dyn_row_ctas_per_sm(kChunks)) ptq_quantiz
             const int c = lane + kLanes * j;
             if (!row_ok || c >= cpr) break;
             uint2 out;
+            bool exact = true;
             if (fast) {
                 const float4 ra = r_s[0][c], rb = r_s[1][c];
                 const float2 c0 = __fmul2_rn(make_float2(ra.x, ra.y), rd2), c1 = __fmul2_rn(make_float2(ra.z, ra.w), rd2);
                 const float2 c2 = __fmul2_rn(make_float2(rb.x, rb.y), rd2), c3 = __fmul2_rn(make_float2(rb.z, rb.w), rd2);
                 const float c8[8] = {c0.x, c0.y, c1.x, c1.y, c2.x, c2.y, c3.x, c3.y};
-                out = quantize8<true, kCodeS8, false>(v[j], c8, s_s + 8 * c, nullptr, dx, rdx, 0);
-            } else {
-                const float none[8] = {};
-                out = quantize8<false, kCodeS8>(v[j], none, s_s + 8 * c, nullptr, dx, rdx, 0);
+                exact = quantize8_magic<kCodeS8>(v[j].x, v[j].y, v[j].z, v[j].w, c8, out.x, out.y);   // |v'| <= 127: no saturation
             }
+            if (exact) quantize8_exact<false, kCodeS8>(v[j].x, v[j].y, v[j].z, v[j].w, s_s + 8 * c, nullptr, dx, rdx, out.x, out.y);
             *reinterpret_cast<uint2 *>(qrow + 8 * c) = out;
         }
     }

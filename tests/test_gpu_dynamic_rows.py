@@ -42,3 +42,22 @@ def test_row_steps_and_codes_match_oracle(env, K, M):
     assert np.array_equal(step.cpu().numpy().view(np.uint32), step_ref.view(np.uint32))
     assert np.array_equal(q.cpu().numpy().reshape(M, K), q_ref)
     layer.close()
+
+
+@pytest.mark.parametrize("K,M", [(8, 47000), (128, 23003), (264, 12001), (768, 11003), (1536, 9007)])
+def test_rows_of_later_rounds(env, K, M):
+    """More rows than the chip takes at once: a warp's second and third row come from the copies it made ahead, with rows
+    missing in the last round and an infinite and an all-zero row among them."""
+    ptq, torch = env
+    rng = np.random.default_rng(K)
+    x = (rng.standard_normal((M, K)) * np.exp(rng.normal(0, 2, (M, 1)))).astype(np.float16)
+    x[M // 2, K // 2], x[M - 2] = np.inf, 0.0
+    s = np.exp(rng.uniform(-3, 3, K)).astype(np.float32)
+    layer = ptq.PtqLinear(np.ones((8, K), np.int8), np.ones(8, np.float32), s, np.ones(1, np.float32))
+    _, q, _, step = layer.forward_dynamic_debug(torch.from_numpy(x.reshape(M, 1, K)).cuda())
+    torch.cuda.synchronize()
+    layer.device_status()
+    q_ref, step_ref = oracle.quantize_dynamic(x, s)
+    assert np.array_equal(step.cpu().numpy().view(np.uint32), step_ref.view(np.uint32))
+    assert np.array_equal(q.cpu().numpy().reshape(M, K), q_ref)
+    layer.close()
