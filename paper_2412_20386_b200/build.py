@@ -20,7 +20,7 @@ _HERE = os.path.dirname(os.path.abspath(__file__))
 _CSRC = os.path.join(_HERE, "csrc")
 _SO = os.path.join(_HERE, "libptq_linear.so")
 _SOURCES = ["ptq_api.cu"]
-_DEPS = ["ptq_api.cu", "ptq_gemm.cuh", "ptq_fused.cuh", "ptq_small.cuh", "ptq_quantize.cuh", "ptq_quantize_dynamic.cuh",
+_DEPS = ["ptq_api.cu", "ptq_gemm.cuh", "ptq_fused.cuh", "ptq_small.cuh", "ptq_short_k.cuh", "ptq_quantize.cuh", "ptq_quantize_dynamic.cuh",
          "ptq_calibrate.cuh", "ptq_probe.cuh", "ptx_sm100.cuh",
          os.path.join("..", "..", "include", "ptq_linear.h")]
 

@@ -23,6 +23,7 @@
 #include "ptq_probe.cuh"
 #include "ptq_quantize.cuh"
 #include "ptq_quantize_dynamic.cuh"
+#include "ptq_short_k.cuh"
 #include "ptq_small.cuh"
 
 namespace {
@@ -480,6 +481,46 @@ void set_bn(const ptq_linear *h, ptq::GemmParams &p, int bn)
     p.fd_n_tiles = ptq::make_fastdiv(static_cast<unsigned>(p.n_tiles));
 }
 
+// Parameters of the GEMM kernels at the layer's own tile width.
+void set_gemm_params(const ptq_linear *h, ptq::GemmParams &p, long long M, void *y, void *acc_out, bool tma_store, const float *dx_rows)
+{
+    p.M = M;
+    p.N = h->N;
+    p.K = h->K;
+    p.T = dx_rows ? static_cast<int>(M) : h->T;
+    p.BN = h->BN;
+    p.n_tiles = h->n_tiles;
+    p.m_tiles = static_cast<int>((M + ptq::kBM - 1) / ptq::kBM);
+    p.k_blocks = h->k_blocks;
+    p.last_mmas = h->last_mmas;
+    p.dx = dx_rows ? dx_rows : h->d_dx;
+    p.dw = h->d_dw;
+    p.bias = h->d_bias;
+    p.has_bias = h->has_bias ? 1 : 0;
+    set_vectors(h, p);
+    // Short main loops (up to three k-blocks per tile, K <= 384) leave the epilogue little time: three stages and two
+    // staging boxes per warp; longer ones keep four stages.  Layers with a bias hold two more scale copies.
+    const bool short_k = h->k_blocks <= PTQ_GEMM_SHORT_K_BLOCKS;
+    p.stages = (short_k || h->has_bias) ? ptq::kStages - 1 : ptq::kStages;
+    p.boxes = short_k ? 2 : 1;
+    p.y = static_cast<__half *>(y);
+    p.acc_out = static_cast<int32_t *>(acc_out);
+    p.status = h->d_status;
+    p.use_tma_store = tma_store ? 1 : 0;
+    p.y_vec2 = (h->N % 2 == 0 && reinterpret_cast<uintptr_t>(y) % 4 == 0) ? 1 : 0;
+    p.y_vec8 = 0;   // this kernel always has a staging buffer; 16-byte alignment means TMA stores
+    // An output of more than half of L2 is gone before its consumer reads it all: marked evict-first it does not push out the
+    // codes, which this kernel is still reading (50432 x 768 -> 3072, both kernels: 132.7 -> 129.2 us).
+    p.y_evict_first = static_cast<long long>(M) * h->N * 2 > h->l2_bytes / 2;
+    const uintptr_t y_align = reinterpret_cast<uintptr_t>(y) | static_cast<uintptr_t>(2 * h->N);
+    p.y_copy_bytes = y_align % 8 == 0 ? 8 : y_align % 4 == 0 ? 4 : 2;
+    p.zp = h->d_zp;
+    p.wsum = h->d_wsum;
+    p.fd_T = ptq::make_fastdiv(static_cast<unsigned>(p.T));
+    p.fd_n_tiles = ptq::make_fastdiv(static_cast<unsigned>(p.n_tiles));
+    p.fd_groups = ptq::make_fastdiv(1u);
+}
+
 // G1+E1 launch on codes [M, Kpad] at `codes`.
 // dx_rows != nullptr: the steps are per ROW (dynamic comparator), i.e. dx = dx_rows and T = M.
 ptq_status_t launch_gemm(const ptq_linear *h, const void *codes, long long M, void *y, void *acc_out,
@@ -507,42 +548,9 @@ ptq_status_t launch_gemm(const ptq_linear *h, const void *codes, long long M, vo
     }
 
     ptq::GemmParams p;
-    p.M = M;
-    p.N = h->N;
-    p.K = h->K;
-    p.T = dx_rows ? static_cast<int>(M) : h->T;
-    p.BN = h->BN;
-    p.n_tiles = h->n_tiles;
-    p.m_tiles = static_cast<int>((M + ptq::kBM - 1) / ptq::kBM);
-    p.k_blocks = h->k_blocks;
-    p.last_mmas = h->last_mmas;
-    p.dx = dx_rows ? dx_rows : h->d_dx;
-    p.dw = h->d_dw;
-    p.bias = h->d_bias;
-    p.has_bias = h->has_bias ? 1 : 0;
-    set_vectors(h, p);
-    // Short main loops (up to three k-blocks per tile, K <= 384) leave the epilogue little time: three stages and two
-    // staging boxes per warp; longer ones keep four stages.  Layers with a bias hold two more scale copies.
+    set_gemm_params(h, p, M, y, acc_out, tma_store, dx_rows);
     const bool short_k = h->k_blocks <= PTQ_GEMM_SHORT_K_BLOCKS;
-    p.stages = (short_k || h->has_bias) ? ptq::kStages - 1 : ptq::kStages;
-    p.boxes = short_k ? 2 : 1;
     const int gemm_smem = ptq::gemm_smem_bytes(p.stages, p.boxes, p.vectors);
-    p.y = static_cast<__half *>(y);
-    p.acc_out = static_cast<int32_t *>(acc_out);
-    p.status = h->d_status;
-    p.use_tma_store = tma_store ? 1 : 0;
-    p.y_vec2 = (h->N % 2 == 0 && reinterpret_cast<uintptr_t>(y) % 4 == 0) ? 1 : 0;
-    p.y_vec8 = 0;   // this kernel always has a staging buffer; 16-byte alignment means TMA stores
-    // An output of more than half of L2 is gone before its consumer reads it all: marked evict-first it does not push out the
-    // codes, which this kernel is still reading (50432 x 768 -> 3072, both kernels: 132.7 -> 129.2 us).
-    p.y_evict_first = static_cast<long long>(M) * h->N * 2 > h->l2_bytes / 2;
-    const uintptr_t y_align = reinterpret_cast<uintptr_t>(y) | static_cast<uintptr_t>(2 * h->N);
-    p.y_copy_bytes = y_align % 8 == 0 ? 8 : y_align % 4 == 0 ? 4 : 2;
-    p.zp = h->d_zp;
-    p.wsum = h->d_wsum;
-    p.fd_T = ptq::make_fastdiv(static_cast<unsigned>(p.T));
-    p.fd_n_tiles = ptq::make_fastdiv(static_cast<unsigned>(p.n_tiles));
-    p.fd_groups = ptq::make_fastdiv(1u);
 
     if (use_pair) {
         // enough 256-row tiles to occupy every CTA pair: cta_group::2 kernel (half the weight bytes per CTA)
@@ -796,6 +804,66 @@ ptq_status_t launch_small(const ptq_linear *h, const SmallPlan &pl, const void *
     if (h->act_bits == 4) return go(std::integral_constant<int, ptq::kCodeS4>());
     if (h->asym) return go(std::integral_constant<int, ptq::kCodeU8>());
     return go(std::integral_constant<int, ptq::kCodeS8>());
+}
+
+// The one-kernel path for layers of a few channels: up to 32, and eight outputs or more per channel, so that the four quantizer
+// warps are not what a CTA waits for.  us, two kernels -> one: 3152 x 12 -> 384 5.6 -> 4.9, 25216 x 12 -> 384 10.4 -> 8.2, 12608 x 17 ->
+// 200 7.6 -> 6.5, 50432 x 24 -> 768 17.9 -> 17.6, 200704 x 8 -> 64 13.7 -> 13.8; not taken: 200704 x 16 -> 64 14.5 -> 15.6, 200704 x 32 -> 128
+// 19.1 -> 22.5, 12608 x 48 -> 1536 13.6 -> 15.9, 50176 x 64 -> 256 11.7 -> 14.0.
+bool plan_short_k(const ptq_linear *h, const void *y)
+{
+    return h->K <= ptq::kShortKMaxK && h->N >= 8 * h->K && !h->asym && h->fast_div && h->N % 8 == 0 &&
+           reinterpret_cast<uintptr_t>(y) % 16 == 0;
+}
+
+ptq_status_t launch_short_k(const ptq_linear *h, const void *x, long long M, void *y, void *acc_out, cudaStream_t stream)
+{
+    CUtensorMap tmY;
+    ptq_status_t st = cached_map_2d(h->y_maps, &tmY, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, y, static_cast<unsigned long long>(h->N),
+                                    static_cast<unsigned long long>(M), static_cast<unsigned long long>(h->N) * 2, ptq::kStreamBoxCols, 32);
+    if (st != PTQ_OK) return st;
+    ptq::ShortKParams sp;
+    ptq::GemmParams &p = sp.g;
+    set_gemm_params(h, p, M, y, acc_out, true, nullptr);
+    // N tiles per unit: the number that leaves the busiest CTA the fewest tiles; the larger one (rows quantized less often) if equal
+    long long fewest = 0;
+    for (int group = 1; group <= p.n_tiles && group <= ptq::kShortKMaxGroup; ++group) {
+        const int groups = (p.n_tiles + group - 1) / group;
+        const long long tiles = (static_cast<long long>(p.m_tiles) * groups + h->num_sms - 1) / h->num_sms * group;
+        if (group == 1 || tiles <= fewest) {
+            fewest = tiles;
+            p.group = group;
+            p.groups = groups;
+        }
+    }
+    p.fd_n_tiles = ptq::make_fastdiv(static_cast<unsigned>(p.m_tiles));
+    sp.x = static_cast<const __half *>(x);
+    sp.s = h->d_s;
+    sp.rs = h->d_rs;
+    sp.dx2 = h->d_dx2;
+    const uintptr_t x_align = reinterpret_cast<uintptr_t>(x) | static_cast<uintptr_t>(2 * h->K);
+    sp.ld_bytes = x_align % 16 == 0 ? 16 : x_align % 8 == 0 ? 8 : 2;
+    const long long units = static_cast<long long>(p.m_tiles) * p.groups;
+    const int grid = static_cast<int>(units < h->num_sms ? units : h->num_sms);
+    const int smem = ptq::short_k_smem_bytes(p.group * p.BN * ptq::kBK, p.vectors);
+    auto go = [&](auto chunks, auto mode, auto debug) -> ptq_status_t {
+        constexpr auto kKern = ptq::ptq_short_k_kernel<decltype(chunks)::value, decltype(mode)::value, decltype(debug)::value>;
+        const ptq_status_t es = ensure_smem<kKern>(h->device, ptq::kShortKSmemMax);
+        if (es != PTQ_OK) return es;
+        PTQ_CUDA(launch_pdl(kKern, grid, ptq::kShortKThreads, smem, stream, h->tmW, tmY, sp));
+        return PTQ_OK;
+    };
+    auto mode = [&](auto chunks) {
+        const std::integral_constant<int, ptq::kCodeS4> s4;
+        const std::integral_constant<int, ptq::kCodeS8> s8;
+        return h->act_bits == 4 ? (acc_out ? go(chunks, s4, std::true_type()) : go(chunks, s4, std::false_type()))
+                                : (acc_out ? go(chunks, s8, std::true_type()) : go(chunks, s8, std::false_type()));
+    };
+    st = h->K <= 16 ? mode(std::integral_constant<int, 2>()) : mode(std::integral_constant<int, 4>());
+    if (st != PTQ_OK) return st;
+    g_launches.fetch_add(1, std::memory_order_relaxed);
+    PTQ_CUDA(cudaGetLastError());
+    return PTQ_OK;
 }
 
 bool fused_usable(const ptq_linear *h) { return h->as_ok && h->K % 16 == 0; }
@@ -1160,6 +1228,11 @@ ptq_status_t ptq_linear_forward_debug(const ptq_linear_t *h, const void *x_fp16,
         if (q_int8_out) return launch_quantize(h, x_fp16, M, q_int8_out, h->K, s);
         return PTQ_OK;
     }
+    if (!(flags & PTQ_FLAG_CTA_PAIR) && plan_short_k(h, y_fp16)) {
+        if ((st = launch_short_k(h, x_fp16, M, y_fp16, acc_int32_out, s)) != PTQ_OK) return st;
+        if (q_int8_out) return launch_quantize(h, x_fp16, M, q_int8_out, h->K, s);
+        return PTQ_OK;
+    }
     if ((st = launch_quantize(h, x_fp16, M, workspace, h->Kpad, s)) != PTQ_OK) return st;
     if ((st = launch_gemm(h, workspace, M, y_fp16, acc_int32_out, s, (flags & PTQ_FLAG_CTA_PAIR) != 0)) != PTQ_OK)
         return st;
@@ -1190,6 +1263,7 @@ ptq_status_t ptq_linear_forward_static(const ptq_linear_t *h, const void *x_fp16
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     SmallPlan pl;
     if (plan_small(h, M, pl)) return launch_small(h, pl, x_fp16, M, y_fp16, nullptr, s);
+    if (plan_short_k(h, y_fp16)) return launch_short_k(h, x_fp16, M, y_fp16, nullptr, s);
     void *scratch = nullptr;
     if ((st = static_scratch_address(h->device, &scratch)) != PTQ_OK) return st;
     if ((st = launch_quantize(h, x_fp16, M, scratch, h->Kpad, s)) != PTQ_OK) return st;

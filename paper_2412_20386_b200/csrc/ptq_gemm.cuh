@@ -531,8 +531,8 @@ struct TileCursor {
     __device__ int m_tile() const { return tile - n_tile() * m_tiles; }
 };
 
-template <bool kDebugAcc, bool kAsym>
-__device__ __forceinline__ void epilogue_team_loop(const GemmParams &p, const CUtensorMap *tmY, TileCursor cur, uint32_t tmem_base,
+template <bool kDebugAcc, bool kAsym, class Cursor>
+__device__ __forceinline__ void epilogue_team_loop(const GemmParams &p, const CUtensorMap *tmY, Cursor cur, uint32_t tmem_base,
                                                    uint32_t tfull_bar0, uint32_t tempty_bar0, float *scale_s,
                                                    uint32_t staging, volatile uint32_t *abort_flag, int warp, int lane)
 {
@@ -546,7 +546,7 @@ __device__ __forceinline__ void epilogue_team_loop(const GemmParams &p, const CU
     if (team == 1 && cur.valid()) cur.advance();        // team 1 starts at the CTA's second tile
     float dw_next[2] = {0.0f, 0.0f}, bias_next[2] = {0.0f, 0.0f};
     int ws_next[2] = {0, 0};
-    auto fetch_scales = [&](const TileCursor &c) {
+    auto fetch_scales = [&](const Cursor &c) {
         // unconditional loads from clamped indices (see load_row_step); past the last tile the values are not used
         const int n0 = c.valid() ? c.n_tile() * p.BN : 0;
 #pragma unroll
