@@ -122,7 +122,6 @@ ptq_small_kernel(const __grid_constant__ CUtensorMap tmW, const SmallParams p)
     const int m_tile = static_cast<int>(fd_div(blockIdx.x, p.fd_n_tiles));
     const int n0 = (static_cast<int>(blockIdx.x) - m_tile * p.n_tiles) * kSmallRows;
     const int m0 = m_tile * kTN;
-    griddep_launch_dependents();
 
     if (tid == 0) {
         mbar_init(wbar, 1);
@@ -165,6 +164,7 @@ ptq_small_kernel(const __grid_constant__ CUtensorMap tmW, const SmallParams p)
     __syncthreads();
     tc_fence_after_sync();
     const uint32_t tmem_base = *tmem_holder;
+    griddep_launch_dependents();                               // behind the allocation: see griddep_launch_dependents()
     griddep_wait();                                            // everything above read only the layer's own parameters
 
     // ---- quantize ------------------------------------------------------------------------------------

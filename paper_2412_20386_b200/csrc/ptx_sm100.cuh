@@ -59,6 +59,9 @@ __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count)
 // calling thread until every prerequisite grid has completed and its memory operations are visible
 // (a no-op when the launch carried no such dependency).  griddep_launch_dependents() lets the NEXT
 // kernel's CTAs be scheduled as soon as resources free up instead of at this grid's very end.
+// A kernel that allocates tensor memory calls it only once its own allocation has been granted (behind the barrier that
+// publishes the address): a dependent CTA on the same SM that got all 512 columns first would hold them while it waits
+// for this grid, whose CTA would wait in tcgen05.alloc for those columns.
 __device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void griddep_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
