@@ -267,9 +267,8 @@ cudaError_t launch_pdl(void (*kern)(KArgs...), int grid, int block, size_t smem,
     return cudaLaunchKernelEx(&cfg, kern, std::forward<Args>(args)...);
 }
 
-// Q1 launch: codes to `q` with `q_pitch` bytes between rows.
-ptq_status_t launch_quantize(const ptq_linear *h, const void *x, long long M, void *q, int q_pitch,
-                             cudaStream_t stream)
+// Q1 launch for `images` <= kQuantMaxImages images.
+ptq_status_t launch_quantize_images(const ptq_linear *h, const void *x, int images, void *q, int q_pitch, cudaStream_t stream)
 {
     ptq::QuantParams p;
     p.x = static_cast<const __half *>(x);
@@ -278,23 +277,16 @@ ptq_status_t launch_quantize(const ptq_linear *h, const void *x, long long M, vo
     p.rs = h->d_rs;
     p.dx2 = h->d_dx2;
     p.zp = h->d_zp;
-    p.M = M;
+    p.M = static_cast<long long>(images) * h->T;
     p.K = h->K;
     p.T = h->T;
     p.q_pitch = q_pitch;
-    const long long B = M / h->T;
-    // Thread count = S * (chunks per image), S images apart between a thread's chunks: the smallest S that needs no more
-    // rounds than one resident wave of threads does (at least one image at a time, however large).
     const bool vec = (h->K % 8 == 0) && (reinterpret_cast<uintptr_t>(x) % 16 == 0) &&
                      (reinterpret_cast<uintptr_t>(q) % 8 == 0) && (q_pitch % 8 == 0);
     const int cpr = (h->K + 7) / 8;
     const long long cpi = static_cast<long long>(h->T) * cpr;
-    const long long wave = static_cast<long long>(h->num_sms) * ptq::kQuantCtasPerSm * 256;
-    long long S = wave / cpi;
-    if (S < 1) S = 1;
-    const long long rounds = (B + S - 1) / S;
-    S = (B + rounds - 1) / rounds;
-    p.B = static_cast<int>(B);
+    const long long S = ptq::quant_image_step(images, cpi, h->num_sms);     // threads: S * (chunks per image)
+    p.B = images;
     p.imgs_per_iter = static_cast<int>(S);
     p.fd_cpi = ptq::make_fastdiv(static_cast<unsigned>(cpi));
     p.fd_cpr = ptq::make_fastdiv(static_cast<unsigned>(cpr));
@@ -317,6 +309,19 @@ ptq_status_t launch_quantize(const ptq_linear *h, const void *x, long long M, vo
         PTQ_CUDA(pick(std::integral_constant<int, ptq::kCodeS8>()));
     g_launches.fetch_add(1, std::memory_order_relaxed);
     PTQ_CUDA(cudaGetLastError());
+    return PTQ_OK;
+}
+
+// Q1: codes of M rows to `q` with `q_pitch` bytes between rows.
+ptq_status_t launch_quantize(const ptq_linear *h, const void *x, long long M, void *q, int q_pitch, cudaStream_t stream)
+{
+    const long long B = M / h->T;
+    for (long long b = 0; b < B; b += ptq::kQuantMaxImages) {
+        const int images = static_cast<int>(B - b < ptq::kQuantMaxImages ? B - b : ptq::kQuantMaxImages);
+        const ptq_status_t st = launch_quantize_images(h, static_cast<const __half *>(x) + b * h->T * h->K, images,
+                                                       static_cast<int8_t *>(q) + b * h->T * q_pitch, q_pitch, stream);
+        if (st != PTQ_OK) return st;
+    }
     return PTQ_OK;
 }
 

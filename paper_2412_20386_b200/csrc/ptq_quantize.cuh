@@ -254,6 +254,20 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
+// Images of one launch.  A thread steps through the images in 32 bits and looks kQuantRingDepth steps ahead, so that the
+// sums must stay below 2^31; a larger batch is launched in parts.  (Wider counters in the kernel cost 1 - 2 % of a model.)
+constexpr int kQuantMaxImages = 1 << 30;
+
+// Images between two of a thread: the smallest number that needs no more rounds than one resident wave of threads does (at
+// least one image at a time, however large).
+__host__ __device__ inline int quant_image_step(int images, long long chunks_per_image, int sms)
+{
+    long long S = static_cast<long long>(sms) * kQuantCtasPerSm * 256 / chunks_per_image;
+    if (S < 1) S = 1;
+    const long long rounds = (images + S - 1) / S;
+    return static_cast<int>((images + rounds - 1) / rounds);
+}
+
 // The three routes for one chunk of 8 channels, cheapest first; every route that returns codes returns
 // the codes of the definition.  c8 = RN(RN(1/s) * RN(1/dx)).  kExactRecip = false decides the last route with IEEE
 // divisions instead of reciprocals: more instructions but no 1/s to fetch, for kernels that keep s in shared memory and

@@ -1,0 +1,59 @@
+"""The kernels' loop and launch arithmetic at the top of the ranges that the entry points accept, on the host: the helpers are
+compiled from the kernel headers into a small program (no GPU is needed), and their walks are compared with Python's integers."""
+import os
+import subprocess
+
+import pytest
+
+from paper_2412_20386_b200 import build as lib_build
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2412_20386_b200", "csrc")
+INT_MAX = 2 ** 31 - 1
+
+PROGRAM = r"""
+#include <cstdio>
+#include <cstdlib>
+#include <cstring>
+#include "ptq_quantize.cuh"
+
+// quant images chunks_per_image sms: images between two of a thread, ring depth, images of one launch
+static int quant(char **a)
+{
+    printf("%d %d %d\n", ptq::quant_image_step(atoi(a[0]), atoll(a[1]), atoi(a[2])), ptq::kQuantRingDepth, ptq::kQuantMaxImages);
+    return 0;
+}
+
+int main(int argc, char **argv)
+{
+    if (argc > 1 && !strcmp(argv[1], "quant")) return quant(argv + 2);
+    return 2;
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def program(tmp_path_factory):
+    d = tmp_path_factory.mktemp("index")
+    (d / "index.cu").write_text(PROGRAM)
+    exe = str(d / "index")
+    subprocess.run([lib_build.nvcc_path(), "-gencode", "arch=compute_100a,code=sm_100a", "-std=c++17", "-I", CSRC, "-o", exe,
+                    str(d / "index.cu")], check=True, stdout=subprocess.PIPE, stderr=subprocess.STDOUT)
+
+    def run(*args):
+        out = subprocess.run([exe] + [str(a) for a in args], check=True, stdout=subprocess.PIPE, text=True).stdout
+        return [int(v) for v in out.split()]
+    return run
+
+
+# one token position of 1 to 8 channels puts the most images between two of a thread
+@pytest.mark.parametrize("B,chunks,sms", [(1, 1, 148), (9, 197 * 48, 148), (2147483000, 1, 148), (INT_MAX, 1, 148), (INT_MAX, 3, 132),
+                                          (2 ** 30 + 1, 1, 160), (257, 2 ** 30, 148)])
+def test_quantize_image_counters_stay_in_32_bits(program, B, chunks, sms):
+    """Every thread's image index plus the loads it looks ahead (the index starts below the step and ends below the images plus one
+    step) fits an int in each part of the batch, and a part's threads together visit every image."""
+    most = program("quant", 1, 1, sms)[2]
+    for first in range(0, B, most):
+        images = min(most, B - first)
+        step, depth, _ = program("quant", images, chunks, sms)
+        assert 1 <= step <= images and images + depth * step <= INT_MAX
+        assert step * chunks <= max(chunks, sms * 4 * 256)          # the launch has at most one wave of threads, or one image
