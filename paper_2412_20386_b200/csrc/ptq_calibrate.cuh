@@ -290,6 +290,15 @@ struct SearchParams {
     FastDiv fd_K;
 };
 
+// A position's elements in tiles of kSearchTile.  Unsigned: there may be 2^31 - 1, and the start behind the last tile leaves int.
+struct SearchTiles {
+    unsigned at, end;
+    __host__ __device__ explicit SearchTiles(int elements) : at(0u), end(static_cast<unsigned>(elements)) {}
+    __host__ __device__ bool valid() const { return at < end; }
+    __host__ __device__ int count() const { return end - at < kSearchTile ? static_cast<int>(end - at) : kSearchTile; }
+    __host__ __device__ void next() { at += kSearchTile; }
+};
+
 __device__ __forceinline__ float search_candidate_step(float base, int j, int n_grid)
 {
     return __fmul_rn(base, __fdiv_rn(static_cast<float>(j), static_cast<float>(n_grid)));
@@ -321,14 +330,13 @@ __global__ void __launch_bounds__(kSearchThreads, 2) ptq_search_loss_kernel(Sear
         fast = fast && delta[c] >= 9.313225746154785e-10f && delta[c] <= 1073741824.0f;      // 2^-30 .. 2^30
         acc[c] = 0.0;
     }
-    const int per_pos = p.Bc * p.K;
-    for (int i0 = 0; i0 < per_pos; i0 += kSearchTile) {
-        const int n = min(kSearchTile, per_pos - i0);
+    for (SearchTiles tile(p.Bc * p.K); tile.valid(); tile.next()) {
+        const int n = tile.count();
         __syncthreads();
 #pragma unroll 4
         for (int i = threadIdx.x; i < n; i += kSearchThreads) {
-            const int b = static_cast<int>(fd_div(static_cast<unsigned>(i0 + i), p.fd_K));
-            const int k = i0 + i - b * p.K;
+            const int b = static_cast<int>(fd_div(tile.at + i, p.fd_K));
+            const int k = static_cast<int>(tile.at + i) - b * p.K;
             u_s[i] = __fdiv_rn(__half2float(__ldg(p.x + (static_cast<long long>(b) * p.T + t) * p.K + k)), __ldg(p.s + k));
         }
         __syncthreads();

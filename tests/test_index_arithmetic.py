@@ -14,6 +14,7 @@ PROGRAM = r"""
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include "ptq_calibrate.cuh"
 #include "ptq_quantize.cuh"
 
 // quant images chunks_per_image sms: images between two of a thread, ring depth, images of one launch
@@ -23,9 +24,23 @@ static int quant(char **a)
     return 0;
 }
 
+// tiles elements: tiles visited, elements in them, start of the last one
+static int tiles(char **a)
+{
+    long long visited = 0, elements = 0, last = -1;
+    for (ptq::SearchTiles t(atoi(a[0])); t.valid() && visited < 4000000; t.next()) {
+        ++visited;
+        elements += t.count();
+        last = t.at;
+    }
+    printf("%lld %lld %lld\n", visited, elements, last);
+    return 0;
+}
+
 int main(int argc, char **argv)
 {
     if (argc > 1 && !strcmp(argv[1], "quant")) return quant(argv + 2);
+    if (argc > 1 && !strcmp(argv[1], "tiles")) return tiles(argv + 2);
     return 2;
 }
 """
@@ -57,3 +72,9 @@ def test_quantize_image_counters_stay_in_32_bits(program, B, chunks, sms):
         step, depth, _ = program("quant", images, chunks, sms)
         assert 1 <= step <= images and images + depth * step <= INT_MAX
         assert step * chunks <= max(chunks, sms * 4 * 256)          # the launch has at most one wave of threads, or one image
+
+
+@pytest.mark.parametrize("elements", [1, 2047, 2048, 2049, 2147481600, 2147481601, INT_MAX])
+def test_search_tiles_cover_every_element(program, elements):
+    starts = range(0, elements, 2048)
+    assert program("tiles", elements) == [len(starts), elements, starts[-1]]
