@@ -1647,10 +1647,7 @@ ptq_status_t ptq_calibrate_in(int scheme, int K, int N, int T, const void *xcal_
         ptq::ptq_calib_wmax_kernel<4, false><<<wgrid, 128, 0, s>>>(d_w, d_dw, N, K, wrows, d_wbits);
     else
         ptq::ptq_calib_wmax_kernel<1, false><<<wgrid, 128, 0, s>>>(d_w, d_dw, N, K, wrows, d_wbits);
-    // image shares per position: two blocks per SM where there are few positions, but at least eight images each
-    int splits = (2 * sms + T - 1) / T;
-    const int most = (Bc + 7) / 8;
-    if (splits > most) splits = most;
+    const ptq::CalibShares shares_of_position = ptq::calib_shares(Bc, T, sms);
     ptq::CalibRange r;
     r.x = x;
     r.max_x_bits = d_xbits;
@@ -1661,11 +1658,11 @@ ptq_status_t ptq_calibrate_in(int scheme, int K, int N, int T, const void *xcal_
     r.dx = d_dx;
     r.z = d_z;
     r.Bc = Bc;
-    r.imgs_per_block = (Bc + splits - 1) / splits;
+    r.imgs_per_block = shares_of_position.images;
     r.K = K;
     r.T = T;
     r.qmax = packed ? 7.0f : 127.0f;
-    const dim3 rgrid(static_cast<unsigned>(T), static_cast<unsigned>((Bc + r.imgs_per_block - 1) / r.imgs_per_block));
+    const dim3 rgrid(static_cast<unsigned>(T), static_cast<unsigned>(shares_of_position.blocks));
     r.final = rgrid.y == 1 && scheme != PTQ_CALIB_PER_TENSOR ? 1 : 0;
     if (asym)
         vec ? ptq::ptq_calib_rowrange_kernel<8, true><<<rgrid, 128, 0, s>>>(r) : ptq::ptq_calib_rowrange_kernel<1, true><<<rgrid, 128, 0, s>>>(r);

@@ -151,6 +151,20 @@ __device__ __forceinline__ float calib_step_asym(float hi, float nlo, int &z)
 // Every thread forms the s of its channels itself from the maxima, and block (0, 0) writes them out.  With one share per
 // position (`final`) the block also forms the position's step, otherwise the shares meet in hi_bits / nlo_bits
 // (mu[t], or hi[t] and -lo[t] for kAsym) and a second kernel forms the steps.
+struct CalibShares {
+    int images, blocks;   // images of a block, blocks per position
+};
+// Two blocks per SM where there are few positions, but no more than one per eight images (or part of them).  In 64 bits: Bc may be
+// 2^31 - 1.
+__host__ __device__ inline CalibShares calib_shares(int Bc, int T, int sms)
+{
+    long long splits = (2ll * sms + T - 1) / T;
+    const long long most = (Bc + 7ll) / 8;
+    if (splits > most) splits = most;
+    const long long images = (Bc + splits - 1) / splits;
+    return {static_cast<int>(images), static_cast<int>((Bc + images - 1) / images)};
+}
+
 struct CalibRange {
     const __half *x;
     const unsigned *max_x_bits, *max_w_bits;

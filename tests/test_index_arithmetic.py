@@ -37,10 +37,19 @@ static int tiles(char **a)
     return 0;
 }
 
+// shares Bc T sms: images of a block, blocks per position
+static int shares(char **a)
+{
+    const ptq::CalibShares s = ptq::calib_shares(atoi(a[0]), atoi(a[1]), atoi(a[2]));
+    printf("%d %d\n", s.images, s.blocks);
+    return 0;
+}
+
 int main(int argc, char **argv)
 {
     if (argc > 1 && !strcmp(argv[1], "quant")) return quant(argv + 2);
     if (argc > 1 && !strcmp(argv[1], "tiles")) return tiles(argv + 2);
+    if (argc > 1 && !strcmp(argv[1], "shares")) return shares(argv + 2);
     return 2;
 }
 """
@@ -78,3 +87,11 @@ def test_quantize_image_counters_stay_in_32_bits(program, B, chunks, sms):
 def test_search_tiles_cover_every_element(program, elements):
     starts = range(0, elements, 2048)
     assert program("tiles", elements) == [len(starts), elements, starts[-1]]
+
+
+@pytest.mark.parametrize("Bc,T", [(1, 1), (8, 197), (9, 2), (700, 2), (2147483352, 1), (2147483353, 1), (2147483641, 1), (INT_MAX, 1),
+                                  (INT_MAX, 40)])
+def test_calibration_shares_cover_every_image(program, Bc, T):
+    images, blocks = program("shares", Bc, T, 148)
+    assert 1 <= blocks <= min(-(-2 * 148 // T), -(-Bc // 8))
+    assert (blocks - 1) * images < Bc <= blocks * images
