@@ -7,6 +7,7 @@
 
 #include <ATen/cuda/EmptyTensor.h>
 #include <c10/cuda/CUDAStream.h>
+#include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
 
 #include "../../include/ptq_linear.h"
@@ -83,15 +84,13 @@ void make_ws(Call &c, size_t bytes)
         c.ws = at::Tensor(at::detail::empty_cuda({static_cast<int64_t>(bytes < 16 ? 16 : bytes)}, at::kByte, c.x->device(), std::nullopt));
 }
 
+// C++ exceptions become the classes that torch's own calls raise: torch.OutOfMemoryError where an allocation fails.
 template <class Fn>
 PyObject *guarded(Fn fn)
 {
-    try {
-        return fn();
-    } catch (const std::exception &e) {
-        PyErr_SetString(PyExc_RuntimeError, e.what());
-        return nullptr;
-    }
+    HANDLE_TH_ERRORS
+    return fn();
+    END_HANDLE_TH_ERRORS
 }
 
 // y on success (the caller's object where one was passed), the status as an int otherwise.

@@ -1,0 +1,45 @@
+"""Error classes of the forward calls: what the extension module refuses by itself (no GPU needed), and a failed allocation,
+which raises the class that torch's own allocations raise, so that a caller can catch it and shrink its batch."""
+import numpy as np
+import pytest
+
+import __graft_entry__ as entry
+
+
+@pytest.fixture(scope="module")
+def native():
+    entry.build()
+    from paper_2412_20386_b200 import binding
+    return binding._load_native()
+
+
+@pytest.mark.parametrize("call", ["forward", "forward_static", "forward_dynamic"])
+def test_bad_arguments_are_refused_before_the_library_is_called(native, call):
+    import torch
+    f = getattr(native, call)
+    with pytest.raises(TypeError):
+        f(0, 1, 1, 1)
+    with pytest.raises(TypeError):
+        f(0, 1, 1, 1, np.zeros((1, 1, 1), np.float16), None, None)
+    for x in (torch.zeros(1, 1, 1), torch.zeros(1, 1, 1, dtype=torch.float16)):      # wrong type, not on the device
+        with pytest.raises(ValueError):
+            f(0, 1, 1, 1, x, None, None)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("call", ["forward", "forward_dynamic"])
+def test_an_output_that_does_not_fit_raises_torchs_out_of_memory(call):
+    import torch
+    entry.build()
+    import paper_2412_20386_b200 as ptq
+    torch.cuda.set_device(0)
+    N = 65536
+    layer = ptq.PtqLinear(np.ones((N, 1), np.int8), np.ones(N, np.float32), np.ones(1, np.float32), np.ones(1, np.float32))
+    x = torch.zeros((1 << 21, 1, 1), dtype=torch.float16, device="cuda")             # 4 MB in, 256 GiB out
+    with pytest.raises(torch.OutOfMemoryError):
+        getattr(layer, call)(x)
+    y = getattr(layer, call)(x[:3])                                                  # a smaller batch goes on
+    torch.cuda.synchronize()
+    layer.device_status()
+    assert tuple(y.shape) == (3, 1, N) and float(y.float().abs().max()) == 0.0
+    layer.close()
