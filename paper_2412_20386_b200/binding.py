@@ -160,14 +160,14 @@ def _stream_ptr(stream) -> Optional[int]:
 
 
 def _scratch(nbytes: int, device, stream):
-    """A temporary device buffer for one call.  The kernels run on `stream`, which need not be the
-    stream torch's allocator associates the block with: recording the use keeps the block from being
-    handed out again while the kernels still read it."""
+    """A temporary device buffer for one call on `stream` (None: the current stream).  It is allocated with that
+    stream current: torch's allocator reuses a block in the order of the stream it belongs to, so neither work queued
+    before on another stream nor the next owner of the block can meet this call's kernels."""
     import torch
-    buf = torch.empty(max(int(nbytes), 16), dtype=torch.uint8, device=device)
     if stream is not None:
-        buf.record_stream(stream)
-    return buf
+        with torch.cuda.stream(stream):
+            return _scratch(nbytes, device, None)
+    return torch.empty(max(int(nbytes), 16), dtype=torch.uint8, device=device)
 
 
 def kernel_launch_count() -> int:
