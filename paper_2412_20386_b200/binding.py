@@ -170,6 +170,15 @@ def _scratch(nbytes: int, device, stream):
     return torch.empty(max(int(nbytes), 16), dtype=torch.uint8, device=device)
 
 
+def _offline_workspace(nbytes: int, device, stream):
+    """`_scratch` for the offline steps, whose callers see a failed allocation as the library's PTQ_ERR_NOMEM."""
+    import torch
+    try:
+        return _scratch(nbytes, device, stream)
+    except torch.OutOfMemoryError as e:
+        raise PtqError(7, str(e)) from e
+
+
 def kernel_launch_count() -> int:
     return int(load_library().ptq_kernel_launch_count())
 
@@ -430,7 +439,7 @@ def _calibrate(scheme, xcal, w, w_step, stream, packed_K=None):
     s = np.empty(K, np.float32)
     dx = np.empty(T, np.float32)
     z = np.empty(T, np.int32) if scheme == CALIB_ASYM else None
-    ws = _scratch(L.ptq_calibrate_workspace_bytes(K, N, T), xcal.device, stream)
+    ws = _offline_workspace(L.ptq_calibrate_workspace_bytes(K, N, T), xcal.device, stream)
     _check(L.ptq_calibrate_in(scheme, K, N, T, xcal.data_ptr(), Bc, _hp(w), _hp(w_step), _hp(s), _hp(dx), _hp(z),
                               ws.data_ptr(), ws.numel(), _stream_ptr(stream)))
     return (s, dx) if z is None else (s, dx, z)
@@ -456,7 +465,7 @@ def search_act_step(xcal, smooth, base_step, n_grid: int = 100, j_lo: int = 20, 
     dx = np.empty(T, np.float32)
     best = np.empty(T, np.int32)
     loss = np.empty((T, max(n_grid - j_lo + 1, 1)), np.float64) if want_loss else None
-    ws = _scratch(L.ptq_search_workspace_bytes(K, T, n_grid, j_lo), xcal.device, stream)
+    ws = _offline_workspace(L.ptq_search_workspace_bytes(K, T, n_grid, j_lo), xcal.device, stream)
     _check(L.ptq_search_act_step_in(K, T, xcal.data_ptr(), Bc, _hp(smooth), _hp(base_step), n_grid, j_lo, _hp(dx),
                                     _hp(best), _hp(loss), ws.data_ptr(), ws.numel(), _stream_ptr(stream)))
     return dx, best, loss

@@ -26,6 +26,26 @@ def test_bad_arguments_are_refused_before_the_library_is_called(native, call):
             f(0, 1, 1, 1, x, None, None)
 
 
+def test_offline_steps_report_a_failed_allocation_as_the_librarys_error(native, monkeypatch):
+    import torch
+    import paper_2412_20386_b200 as ptq
+
+    class DeviceTensor:                                      # as far as the offline calls look before they allocate
+        dtype, is_cuda, shape, device = torch.float16, True, (2, 3, 8), "cuda"
+        is_contiguous, dim, data_ptr = (lambda self: True), (lambda self: 3), (lambda self: 16)
+
+    def no_memory(*args, **kwargs):
+        raise torch.OutOfMemoryError("no memory")
+    monkeypatch.setattr(ptq.binding, "_scratch", no_memory)
+    x, w, dw = DeviceTensor(), np.ones((4, 8), np.int8), np.ones(4, np.float32)
+    for call in (lambda: ptq.calibrate(x, w, dw), lambda: ptq.calibrate(x, w, dw, per_tensor=True), lambda: ptq.calibrate_asym(x, w, dw),
+                 lambda: ptq.calibrate_w4a4(x, np.ones((4, 4), np.uint8), 8, dw),
+                 lambda: ptq.search_act_step(x, np.ones(8, np.float32), np.ones(3, np.float32))):
+        with pytest.raises(ptq.PtqError) as e:
+            call()
+        assert e.value.status == 7                           # PTQ_ERR_NOMEM
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("call", ["forward", "forward_dynamic"])
 def test_an_output_that_does_not_fit_raises_torchs_out_of_memory(call):
