@@ -11,6 +11,7 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <memory>
 #include <mutex>
 #include <new>
 #include <type_traits>
@@ -47,6 +48,17 @@ ptq_status_t fail(ptq_status_t st, const char *fmt, ...)
             return fail(e_ == cudaErrorMemoryAllocation ? PTQ_ERR_NOMEM : PTQ_ERR_CUDA,        \
                         "%s failed: %s", #__VA_ARGS__, cudaGetErrorString(e_));                \
     } while (0)
+
+// The body of an entry point that allocates host memory: no exception may leave a C function.
+template <class Fn>
+ptq_status_t no_throw(Fn fn)
+{
+    try {
+        return fn();
+    } catch (const std::exception &) {      // std::bad_alloc is all that these bodies raise
+        return fail(PTQ_ERR_NOMEM, "host allocation failed");
+    }
+}
 
 // cuTensorMapEncodeTiled is reached through the runtime's driver entry point query, so the
 // library has no link-time dependency on libcuda and loads on machines without a driver.
@@ -985,8 +997,8 @@ static ptq_status_t create_impl(ptq_linear_t **out, int K, int N, int T, const i
     if (major != 10 || minor != 0)
         return fail(PTQ_ERR_ARCH, "device %d is compute capability %d.%d; this library needs 10.0 (sm_100a)", dev, major, minor);
 
-    ptq_linear *h = new (std::nothrow) ptq_linear();
-    if (!h) return fail(PTQ_ERR_NOMEM, "host allocation failed");
+    std::unique_ptr<ptq_linear, decltype(&ptq_linear_destroy)> owner(new ptq_linear(), ptq_linear_destroy);
+    ptq_linear *h = owner.get();
     h->K = K;
     h->N = N;
     h->T = T;
@@ -1100,21 +1112,15 @@ static ptq_status_t create_impl(ptq_linear_t **out, int K, int N, int T, const i
                              static_cast<unsigned long long>(Npad), static_cast<unsigned long long>(h->w_pitch), ptq::kBK,
                              static_cast<unsigned>(64 * (i + 1)));
     } while (0);
-    if (st != PTQ_OK) {
-        char keep[sizeof(g_err)];
-        std::memcpy(keep, g_err, sizeof(keep));
-        ptq_linear_destroy(h);
-        std::memcpy(g_err, keep, sizeof(keep));
-        return st;
-    }
-    *out = h;
+    if (st != PTQ_OK) return st;
+    *out = owner.release();
     return PTQ_OK;
 }
 
 ptq_status_t ptq_linear_create(ptq_linear_t **out, int K, int N, int T, const int8_t *w_q, const float *w_step,
                                const float *smooth, const float *act_step, const float *bias, unsigned flags)
 {
-    return create_impl(out, K, N, T, w_q, w_step, smooth, act_step, nullptr, bias, flags);
+    return no_throw([&] { return create_impl(out, K, N, T, w_q, w_step, smooth, act_step, nullptr, bias, flags); });
 }
 
 ptq_status_t ptq_linear_create_asym(ptq_linear_t **out, int K, int N, int T, const int8_t *w_q, const float *w_step,
@@ -1123,7 +1129,7 @@ ptq_status_t ptq_linear_create_asym(ptq_linear_t **out, int K, int N, int T, con
 {
     if (out) *out = nullptr;
     if (!act_zero) return fail(PTQ_ERR_NULL, "act_zero must not be NULL");
-    return create_impl(out, K, N, T, w_q, w_step, smooth, act_step, act_zero, bias, flags);
+    return no_throw([&] { return create_impl(out, K, N, T, w_q, w_step, smooth, act_step, act_zero, bias, flags); });
 }
 
 size_t ptq_linear_workspace_bytes(const ptq_linear_t *h, int B, unsigned flags)
@@ -1318,10 +1324,9 @@ static ptq_status_t search_check(int K, int T, const void *xcal_fp16, int Bc, co
     return PTQ_OK;
 }
 
-ptq_status_t ptq_search_act_step_in(int K, int T, const void *xcal_fp16, int Bc, const float *smooth,
-                                    const float *base_step, int n_grid, int j_lo, float *act_step_out,
-                                    int32_t *best_out, double *loss_out, void *workspace, size_t workspace_bytes,
-                                    void *stream)
+static ptq_status_t search_impl(int K, int T, const void *xcal_fp16, int Bc, const float *smooth, const float *base_step,
+                                int n_grid, int j_lo, float *act_step_out, int32_t *best_out, double *loss_out, void *workspace,
+                                size_t workspace_bytes, void *stream)
 {
     const ptq_status_t st = search_check(K, T, xcal_fp16, Bc, smooth, base_step, n_grid, j_lo, act_step_out);
     if (st != PTQ_OK) return st;
@@ -1364,6 +1369,17 @@ ptq_status_t ptq_search_act_step_in(int K, int T, const void *xcal_fp16, int Bc,
     std::memcpy(act_step_out, out.data(), sizeof(float) * T);
     if (best_out) std::memcpy(best_out, out.data() + T, sizeof(int32_t) * T);
     return PTQ_OK;
+}
+
+ptq_status_t ptq_search_act_step_in(int K, int T, const void *xcal_fp16, int Bc, const float *smooth,
+                                    const float *base_step, int n_grid, int j_lo, float *act_step_out,
+                                    int32_t *best_out, double *loss_out, void *workspace, size_t workspace_bytes,
+                                    void *stream)
+{
+    return no_throw([&] {
+        return search_impl(K, T, xcal_fp16, Bc, smooth, base_step, n_grid, j_lo, act_step_out, best_out, loss_out, workspace,
+                           workspace_bytes, stream);
+    });
 }
 
 ptq_status_t ptq_search_act_step(int K, int T, const void *xcal_fp16, int Bc, const float *smooth,
@@ -1588,9 +1604,9 @@ size_t ptq_calibrate_workspace_bytes(int K, int N, int T)
     return calib_layout(K, N, T).total;
 }
 
-ptq_status_t ptq_calibrate_in(int scheme, int K, int N, int T, const void *xcal_fp16, int Bc, const void *w_q,
-                              const float *w_step, float *smooth_out, float *act_step_out, int32_t *act_zero_out,
-                              void *workspace, size_t workspace_bytes, void *stream)
+static ptq_status_t calibrate_impl(int scheme, int K, int N, int T, const void *xcal_fp16, int Bc, const void *w_q,
+                                   const float *w_step, float *smooth_out, float *act_step_out, int32_t *act_zero_out,
+                                   void *workspace, size_t workspace_bytes, void *stream)
 {
     const bool asym = scheme == PTQ_CALIB_ASYM, packed = scheme == PTQ_CALIB_W4A4;
     if (scheme < PTQ_CALIB_PTS || scheme > PTQ_CALIB_W4A4) return fail(PTQ_ERR_VALUE, "calibrate: unknown scheme %d", scheme);
@@ -1604,9 +1620,6 @@ ptq_status_t ptq_calibrate_in(int scheme, int K, int N, int T, const void *xcal_
         return fail(PTQ_ERR_SHAPE, "calibrate: workspace has %zu bytes, %zu needed", workspace_bytes, l.total);
     if (reinterpret_cast<uintptr_t>(workspace) % 256) return fail(PTQ_ERR_ALIGN, "calibrate: workspace must be 256-byte aligned");
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    int dev = -1, sms = 0;
-    PTQ_CUDA(cudaGetDevice(&dev));
-    PTQ_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     const long long M = static_cast<long long>(Bc) * T;
     const __half *x = static_cast<const __half *>(xcal_fp16);
     unsigned char *base = static_cast<unsigned char *>(workspace);
@@ -1616,6 +1629,13 @@ ptq_status_t ptq_calibrate_in(int scheme, int K, int N, int T, const void *xcal_
     float *d_dw = reinterpret_cast<float *>(base + l.dw);
     uint8_t *d_w = base + l.w;
     const int row_bytes = packed ? (K + 1) / 2 : K;
+    // one copy back: s, dx and (asymmetric) z are adjacent
+    const size_t words = static_cast<size_t>(K) + static_cast<size_t>(T) * (asym ? 2 : 1);
+    std::vector<float> got(words);
+
+    int dev = -1, sms = 0;
+    PTQ_CUDA(cudaGetDevice(&dev));
+    PTQ_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
 
     // The activations' column maxima first: they run while the weights are on their way from the host.
     PTQ_CUDA(cudaMemsetAsync(d_xbits, 0, sizeof(unsigned) * (2 * static_cast<size_t>(K) + 2 * static_cast<size_t>(T)), s));
@@ -1676,15 +1696,22 @@ ptq_status_t ptq_calibrate_in(int scheme, int K, int N, int T, const void *xcal_
         ptq::ptq_calib_step_kernel<<<(T + 127) / 128, 128, 0, s>>>(d_hi, T, d_dx, r.qmax);
     g_launches.fetch_add(r.final ? 3 : 4, std::memory_order_relaxed);
     PTQ_CUDA(cudaGetLastError());
-    // one copy back: s, dx and (asymmetric) z are adjacent
-    const size_t words = static_cast<size_t>(K) + static_cast<size_t>(T) * (asym ? 2 : 1);
-    std::vector<float> got(words);
     PTQ_CUDA(cudaMemcpyAsync(got.data(), d_s, sizeof(float) * words, cudaMemcpyDeviceToHost, s));
     PTQ_CUDA(cudaStreamSynchronize(s));
     std::memcpy(smooth_out, got.data(), sizeof(float) * K);
     std::memcpy(act_step_out, got.data() + K, sizeof(float) * T);
     if (asym) std::memcpy(act_zero_out, got.data() + K + T, sizeof(int32_t) * T);
     return PTQ_OK;
+}
+
+ptq_status_t ptq_calibrate_in(int scheme, int K, int N, int T, const void *xcal_fp16, int Bc, const void *w_q,
+                              const float *w_step, float *smooth_out, float *act_step_out, int32_t *act_zero_out,
+                              void *workspace, size_t workspace_bytes, void *stream)
+{
+    return no_throw([&] {
+        return calibrate_impl(scheme, K, N, T, xcal_fp16, Bc, w_q, w_step, smooth_out, act_step_out, act_zero_out, workspace,
+                              workspace_bytes, stream);
+    });
 }
 
 // The entry points without a caller workspace: one temporary device allocation around ptq_calibrate_in.
@@ -1751,9 +1778,11 @@ ptq_status_t ptq_linear_create_w4a4(ptq_linear_t **out, int K, int N, int T, con
     if (!w_q_packed) return fail(PTQ_ERR_NULL, "w_q_packed must not be NULL");
     if (K < 1 || K > PTQ_MAX_K || N < 1 || N > PTQ_MAX_N)
         return fail(PTQ_ERR_SHAPE, "K, N out of range (K=%d N=%d)", K, N);
-    std::vector<int8_t> w;
-    unpack_int4_host(w_q_packed, N, K, w);
-    return create_impl(out, K, N, T, w.data(), w_step, smooth, act_step, nullptr, bias, flags, 4);
+    return no_throw([&] {
+        std::vector<int8_t> w;
+        unpack_int4_host(w_q_packed, N, K, w);
+        return create_impl(out, K, N, T, w.data(), w_step, smooth, act_step, nullptr, bias, flags, 4);
+    });
 }
 
 ptq_status_t ptq_quantize_packed4(const ptq_linear_t *h, const void *x_fp16, int B, void *q_packed, void *workspace,

@@ -3,6 +3,8 @@ include/ptq_linear.h declares, and its argument validation returns error codes (
 import ctypes
 import os
 import re
+import subprocess
+import sys
 
 import numpy as np
 import pytest
@@ -95,3 +97,35 @@ def test_without_a_device_create_fails_with_an_error_code(lib):
     st, h = _create(lib, K, N, T, np.ones((N, K), np.int8), np.full(N, 0.01, np.float32),
                     np.ones(K, np.float32), np.ones(T, np.float32))
     assert st in (5, 6) and not h.value        # PTQ_ERR_ARCH / PTQ_ERR_CUDA: loud, no fallback
+
+
+NO_MEMORY = r"""
+import ctypes, resource, sys
+import numpy as np
+from paper_2412_20386_b200 import binding
+lib = binding.load_library()
+p = lambda a: a.ctypes.data_as(ctypes.c_void_p)
+T = 1 << 20
+step, one, w = np.ones(T, np.float32), np.ones(8192, np.float32), np.ones(65536, np.float32)
+codes, out = np.ones((1, 8192), np.uint8), np.ones(2 * T, np.float32)
+h, device = ctypes.c_void_p(), ctypes.c_void_p(256)                  # a device address that no host code looks at
+calls = {
+    "search": lambda: lib.ptq_search_act_step_in(1, T, device, 1, p(one), p(step), 20, 20, p(out), None, None, device, 1 << 40, None),
+    "calibrate": lambda: lib.ptq_calibrate_in(2, 1, 1, T, device, 1, p(codes), p(one), p(out), p(out), p(out), device, 1 << 40, None),
+    "create_w4a4": lambda: lib.ptq_linear_create_w4a4(ctypes.byref(h), 8192, 65536, 1, p(codes), p(w), p(one), p(step), None, 0),
+}
+used = int(open("/proc/self/statm").read().split()[0]) * resource.getpagesize()
+resource.setrlimit(resource.RLIMIT_AS, (used + (1 << 20), resource.RLIM_INFINITY))
+st = calls[sys.argv[1]]()
+resource.setrlimit(resource.RLIMIT_AS, (resource.RLIM_INFINITY, resource.RLIM_INFINITY))
+print(st, bool(h.value), lib.ptq_last_error().decode())
+"""
+
+
+@pytest.mark.parametrize("call", ["search", "calibrate", "create_w4a4"])
+def test_host_memory_that_cannot_be_had_is_an_error_code(lib, call):
+    """Under an address-space limit the entry point's host buffers cannot be allocated: no C++ exception may leave it."""
+    r = subprocess.run([sys.executable, "-c", NO_MEMORY, call], cwd=ROOT, capture_output=True, text=True, timeout=120,
+                       env=dict(os.environ, MALLOC_MMAP_THRESHOLD_="65536"))
+    assert r.returncode == 0, r.stderr
+    assert r.stdout.split()[:2] == ["7", "False"], r.stdout          # PTQ_ERR_NOMEM
