@@ -82,7 +82,8 @@ typedef enum {
  *   act_step     host, [T] fp32, Delta_X per token position, finite and > 0
  *   bias         host, [N] fp32 or NULL (added after the scaling, before the fp16 rounding)
  *   flags        reserved, pass PTQ_FLAG_NONE
- * The handle is bound to the device that is current at the time of the call.
+ * The handle is bound to the device that is current at the time of the call, and its parameters are on that device when the
+ * call returns: any stream may use it at once.
  */
 ptq_status_t ptq_linear_create(ptq_linear_t **out, int K, int N, int T,
                                const int8_t *w_q, const float *w_step,

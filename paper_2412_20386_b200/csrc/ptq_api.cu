@@ -1072,6 +1072,9 @@ static ptq_status_t create_impl(ptq_linear_t **out, int K, int N, int T, const i
     auto move_in = [&]() -> ptq_status_t {
         PTQ_CUDA(cudaMalloc(reinterpret_cast<void **>(&h->d_all), total));
         PTQ_CUDA(cudaMemcpy(h->d_all, image.data(), total, cudaMemcpyHostToDevice));
+        // A copy from pageable memory returns once the last part is staged, and streams that do not synchronise with the
+        // default stream, on which a forward call may follow at once, are not ordered behind it.
+        PTQ_CUDA(cudaStreamSynchronize(cudaStreamLegacy));
         return PTQ_OK;
     };
     do {

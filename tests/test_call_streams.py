@@ -7,6 +7,7 @@ import pytest
 
 import oracle
 from paper_2412_20386_b200 import binding
+from parity_util import assert_y_close
 
 
 def test_scratch_is_allocated_on_the_stream_that_uses_it(monkeypatch):
@@ -64,3 +65,30 @@ def test_offline_steps_on_another_stream_while_freed_memory_is_still_written():
         torch.cuda.synchronize()
         for g, r in zip(got, ref):
             assert np.array_equal(g, np.asarray(r))
+
+
+@pytest.mark.gpu
+def test_a_new_layer_can_be_used_at_once_on_any_stream():
+    """Create returns with the parameters on the device: a call on a stream that is not ordered behind the upload sees them all."""
+    import torch
+    import __graft_entry__ as entry
+    entry.build()
+    import paper_2412_20386_b200 as ptq
+    torch.cuda.set_device(0)
+    rng = np.random.default_rng(6)
+    K, N, T = 8192, 2048, 16
+    wq, dw = rng.integers(-127, 128, (N, K)).astype(np.int8), rng.uniform(1e-3, 1e-2, N).astype(np.float32)
+    s, dx = np.ones(K, np.float32), np.full(T, 0.05, np.float32)
+    x = rng.standard_normal((1, T, K)).astype(np.float16)
+    y_ref = oracle.linear_forward(x.reshape(T, K), T, wq, dw, s, dx)
+    xd, y = torch.from_numpy(x).cuda(), torch.empty((1, T, N), dtype=torch.float16, device="cuda")
+    ws = torch.empty(T * K, dtype=torch.uint8, device="cuda")
+    side = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    for _ in range(5):
+        layer = ptq.PtqLinear(wq, dw, s, dx)
+        layer.forward(xd, y=y, workspace=ws, stream=side)
+        side.synchronize()
+        assert_y_close(y.cpu().numpy().reshape(T, N), y_ref, "new layer")
+        layer.device_status()
+        layer.close()
