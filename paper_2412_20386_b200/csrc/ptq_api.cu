@@ -1348,6 +1348,9 @@ static ptq_status_t search_impl(int K, int T, const void *xcal_fp16, int Bc, con
     std::vector<float> in(static_cast<size_t>(K) + T), out(2 * static_cast<size_t>(T));   // one copy each way
     std::memcpy(in.data(), smooth, sizeof(float) * K);
     std::memcpy(in.data() + K, base_step, sizeof(float) * T);
+    int dev = -1, sms = 0;
+    PTQ_CUDA(cudaGetDevice(&dev));
+    PTQ_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     PTQ_CUDA(cudaMemcpyAsync(d_s, in.data(), sizeof(float) * in.size(), cudaMemcpyHostToDevice, s));
     ptq::SearchParams p;
     p.x = static_cast<const __half *>(xcal_fp16);
@@ -1360,8 +1363,12 @@ static ptq_status_t search_impl(int K, int T, const void *xcal_fp16, int Bc, con
     p.n_grid = n_grid;
     p.j_lo = j_lo;
     p.fd_K = ptq::make_fastdiv(static_cast<unsigned>(K));
-    const dim3 grid(static_cast<unsigned>(T), static_cast<unsigned>((C + ptq::kSearchCandPerBlock - 1) / ptq::kSearchCandPerBlock));
-    ptq::ptq_search_loss_kernel<<<grid, ptq::kSearchThreads, 0, s>>>(p);
+    const ptq::SearchPlan plan = ptq::search_plan(Bc * K, T, C, sms);
+    const dim3 grid(static_cast<unsigned>(T), static_cast<unsigned>((C + plan.candidates - 1) / plan.candidates));
+    if (plan.candidates == ptq::kSearchMany)
+        ptq::ptq_search_loss_kernel<ptq::kSearchMany><<<grid, plan.threads, 0, s>>>(p);
+    else
+        ptq::ptq_search_loss_kernel<ptq::kSearchFew><<<grid, plan.threads, 0, s>>>(p);
     ptq::ptq_search_pick_kernel<<<(T + 3) / 4, 128, 0, s>>>(d_loss, d_base, T, n_grid, j_lo, d_best, d_dx);
     g_launches.fetch_add(2, std::memory_order_relaxed);
     PTQ_CUDA(cudaGetLastError());

@@ -286,13 +286,14 @@ __global__ void __launch_bounds__(128) ptq_calib_step_asym_kernel(const unsigned
 // Per token position t and candidate j (j_lo <= j <= n_grid):
 //   Delta = RN(base[t] * RN(j / n_grid)),  u = RN(x / s[k]),  q = clip(rne(RN(u / Delta)), -128, 127)
 //   e = RN(u - Delta * q)  (one fused multiply-add),  loss[t,j] = sum_{b,k} e^2 in binary64,
-// non-finite u skipped.  One block per (position, group of kSearchCandPerBlock candidates); threads
+// non-finite u skipped.  One block per (position, group of candidates); threads
 // stride over the Bc*K elements of the position, keep one binary64 partial sum per candidate, and the
 // block reduces them in a fixed order (shuffles, then warp by warp), so a launch is reproducible.
 constexpr int kSearchSub = 9;                            // candidates whose integers are in registers at a time
-constexpr int kSearchCandPerBlock = 3 * kSearchSub;
+constexpr int kSearchFew = kSearchSub, kSearchMany = 3 * kSearchSub;   // candidates per block, the two kernels
 constexpr int kSearchTile = 2048;                        // elements whose x/s are in shared memory at a time
-constexpr int kSearchThreads = 256;
+constexpr int kSearchThreads = 256;                      // per block, at most
+constexpr int kSearchBlocksFew = 3, kSearchBlocksMany = 2;   // blocks of so many threads that an SM's registers hold
 
 struct SearchParams {
     const __half *x;     // [Bc,T,K]
@@ -318,15 +319,37 @@ __device__ __forceinline__ float search_candidate_step(float base, int j, int n_
     return __fmul_rn(base, __fdiv_rn(static_cast<float>(j), static_cast<float>(n_grid)));
 }
 
+// Candidates per block and threads of a launch.  A block's threads each form the candidates' steps and, at the end, reduce
+// their sums: about as much work as 10 elements, so a block has as few threads as still fill the chip (256 threads where
+// blocks are few, 64 where they are many).  27 candidates share the loading and dividing of an element, 60 instructions, but
+// hold 128 registers: taken with three blocks per SM or more and at most an eighth of the candidates idle, else 9.
+// Kernel, us, with 9 candidates and 64 / 128 / 256 threads, with 27 and the same:
+//   8 x 197 x 384    8 candidates  24.6 / 15.2 / 11.0   42.6 / 27.4 / 21.8      81   40.0 / 41.4 / 48.0   47.8 / 35.1 / 40.6
+//   4 x 3136 x 96    8             14.2 / 17.3 / 28.2   35.0 / 47.0 / 75.1      81   95.7 / 128 / 222     93.4 / 127 / 213
+//   16 x 49 x 1536   8             168 / 88.7 / 53.9    290 / 155 / 96.7        81   190 / 109 / 79.7     296 / 158 / 96.9
+struct SearchPlan {
+    int candidates, threads;
+};
+__host__ __device__ inline SearchPlan search_plan(int elements, int T, int C, int sms)
+{
+    const long long many = (C + kSearchMany - 1) / kSearchMany, few = (C + kSearchFew - 1) / kSearchFew;
+    const bool wide = T * many >= 3ll * sms && 8 * (many * kSearchMany - C) <= many * kSearchMany;
+    const long long blocks = T * (wide ? many : few);
+    const long long resident = static_cast<long long>(sms) * kSearchThreads * (wide ? kSearchBlocksMany : kSearchBlocksFew);
+    int threads = kSearchThreads;
+    while (threads > 64 && (blocks * threads > resident || elements <= threads / 2)) threads /= 2;
+    return {wide ? kSearchMany : kSearchFew, threads};
+}
+
 // Bound by issue: 49 M (element, candidate) pairs at 8 x 197 x 384 x 81, 9 instructions each.  The integer r = rne(u / Delta)
 // is taken from one FMA, t = RN(u * RN(1/Delta) + 1.5*2^23), whose low mantissa bits hold it; u * RN(1/Delta) is within
 // 1.2e-7 |v| of the defined quotient v, and beyond |v| = 128 every r clamps alike, so r can only be wrong where the distance
-// to r exceeds 0.49998: those elements (3 in 10^4) take the IEEE divisions.  27 candidates per block, so that loading an
-// element and dividing it by s, 60 instructions, is paid 3 times and not 11 times for 81 candidates.
-// 8 x 197 x 384: 60 us with IEEE divisions, 46 with 8 candidates per block, 44 so.
-__global__ void __launch_bounds__(kSearchThreads, 2) ptq_search_loss_kernel(SearchParams p)
+// to r exceeds 0.49998: those elements (3 in 10^4) take the IEEE divisions.
+// 8 x 197 x 384 x 81: 71 us with IEEE divisions and 8 candidates per block, 40.6 with 27 and 256 threads, 35.1 so.
+template <int C>
+__global__ void __launch_bounds__(kSearchThreads, C == kSearchFew ? kSearchBlocksFew : kSearchBlocksMany) ptq_search_loss_kernel(SearchParams p)
 {
-    constexpr int C = kSearchCandPerBlock, S = kSearchSub;
+    constexpr int S = kSearchSub;
     constexpr float kMagic = 12582912.0f;
     __shared__ double partial[kSearchThreads / 32][C];
     __shared__ float u_s[kSearchTile];
@@ -348,13 +371,13 @@ __global__ void __launch_bounds__(kSearchThreads, 2) ptq_search_loss_kernel(Sear
         const int n = tile.count();
         __syncthreads();
 #pragma unroll 4
-        for (int i = threadIdx.x; i < n; i += kSearchThreads) {
+        for (int i = threadIdx.x; i < n; i += blockDim.x) {
             const int b = static_cast<int>(fd_div(tile.at + i, p.fd_K));
             const int k = static_cast<int>(tile.at + i) - b * p.K;
             u_s[i] = __fdiv_rn(__half2float(__ldg(p.x + (static_cast<long long>(b) * p.T + t) * p.K + k)), __ldg(p.s + k));
         }
         __syncthreads();
-        for (int i = threadIdx.x; i < n; i += kSearchThreads) {
+        for (int i = threadIdx.x; i < n; i += blockDim.x) {
             const float u = u_s[i];
             if (!(fabsf(u) <= 3.402823466e38f)) continue;      // inf and NaN do not enter the loss
 #pragma unroll
@@ -388,7 +411,7 @@ __global__ void __launch_bounds__(kSearchThreads, 2) ptq_search_loss_kernel(Sear
     __syncthreads();
     if (threadIdx.x < ncand) {
         double v = 0.0;
-        for (int w = 0; w < kSearchThreads / 32; ++w) v += partial[w][threadIdx.x];
+        for (int w = 0; w < static_cast<int>(blockDim.x) / 32; ++w) v += partial[w][threadIdx.x];
         p.loss[static_cast<long long>(t) * (p.n_grid - p.j_lo + 1) + (j0 - p.j_lo) + threadIdx.x] = v;
     }
 }

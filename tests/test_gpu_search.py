@@ -80,6 +80,17 @@ def test_search_small_grids_ties_and_specials(env):
         check_search(ptq, torch, x, s, base, n_grid, j_lo)
 
 
+@pytest.mark.parametrize("K,T,Bc,C", [(8, 2000, 2, 5), (40, 900, 4, 10), (683, 3, 3, 19), (8, 500, 3, 27), (100, 500, 3, 54),
+                                      (129, 150, 16, 79), (1, 445, 1, 24)])
+def test_search_block_shapes(env, K, T, Bc, C):
+    """9 and 27 candidates per block, 64, 128 and 256 threads, groups and tiles that are not full."""
+    ptq, torch = env
+    rng = np.random.default_rng(K * 31 + C)
+    x = (rng.standard_t(3, (Bc, T, K)) * 0.7).astype(np.float16)
+    s = np.exp(rng.uniform(-1, 1, K)).astype(F32)
+    check_search(ptq, torch, x, s, rng.uniform(0.02, 0.06, T).astype(F32), 100, 101 - C)
+
+
 def test_search_argument_errors(env):
     ptq, torch = env
     x = torch.zeros((2, 3, 8), dtype=torch.float16, device="cuda")

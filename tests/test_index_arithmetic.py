@@ -45,11 +45,20 @@ static int shares(char **a)
     return 0;
 }
 
+// plan elements T C sms: candidates per block, threads
+static int plan(char **a)
+{
+    const ptq::SearchPlan p = ptq::search_plan(atoi(a[0]), atoi(a[1]), atoi(a[2]), atoi(a[3]));
+    printf("%d %d\n", p.candidates, p.threads);
+    return 0;
+}
+
 int main(int argc, char **argv)
 {
     if (argc > 1 && !strcmp(argv[1], "quant")) return quant(argv + 2);
     if (argc > 1 && !strcmp(argv[1], "tiles")) return tiles(argv + 2);
     if (argc > 1 && !strcmp(argv[1], "shares")) return shares(argv + 2);
+    if (argc > 1 && !strcmp(argv[1], "plan")) return plan(argv + 2);
     return 2;
 }
 """
@@ -95,3 +104,11 @@ def test_calibration_shares_cover_every_image(program, Bc, T):
     images, blocks = program("shares", Bc, T, 148)
     assert 1 <= blocks <= min(-(-2 * 148 // T), -(-Bc // 8))
     assert (blocks - 1) * images < Bc <= blocks * images
+
+
+@pytest.mark.parametrize("elements,T,C,want", [
+    (3072, 197, 8, [9, 256]), (3072, 197, 20, [9, 128]), (3072, 197, 54, [9, 64]), (3072, 197, 81, [27, 128]), (3072, 197, 100, [27, 64]),
+    (384, 3136, 1, [9, 64]), (384, 3136, 28, [9, 64]), (384, 3136, 81, [27, 64]), (24576, 49, 81, [9, 256]), (96, 197, 1, [9, 128]),
+    (1, 1, 1, [9, 64]), (INT_MAX, 1, 4096, [9, 128]), (INT_MAX, 1048576, 4096, [27, 64])])
+def test_search_blocks_fill_the_chip_and_no_more(program, elements, T, C, want):
+    assert program("plan", elements, T, C, 148) == want
