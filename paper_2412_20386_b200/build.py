@@ -9,6 +9,7 @@ loads (and exports its symbols) on machines that have no NVIDIA driver.  It does
 """
 from __future__ import annotations
 
+import importlib.metadata
 import os
 import shutil
 import subprocess
@@ -33,6 +34,7 @@ def nvcc_path() -> str:
 
 
 _EXT = os.path.join(_HERE, "_ptq_torch.so")
+_EXT_STAMP = os.path.join(_HERE, "_build", "_ptq_torch.versions")     # what the extension was compiled against
 _EXT_DEPS = ["ptq_torch.cpp", os.path.join("..", "..", "include", "ptq_linear.h")]
 
 
@@ -41,6 +43,18 @@ def up_to_date(target: str = _SO, deps=_DEPS) -> bool:
         return False
     t = os.path.getmtime(target)
     return all(os.path.getmtime(os.path.join(_CSRC, d)) <= t for d in deps)
+
+
+def _ext_versions() -> str:
+    """The extension uses torch's C++ classes and Python's C API: another version of either is another layout."""
+    return "torch %s, python %s" % (importlib.metadata.version("torch"), sys.version.split()[0])
+
+
+def extension_up_to_date() -> bool:
+    if not up_to_date(_EXT, _EXT_DEPS) or not os.path.exists(_EXT_STAMP):
+        return False
+    with open(_EXT_STAMP) as f:
+        return f.read() == _ext_versions()
 
 
 def _run(cmd, target: str, verbose: bool) -> None:
@@ -75,13 +89,16 @@ def _build_extension(verbose: bool) -> None:
            "-Wl,-rpath," + os.path.join(root, "lib"),
            "-ltorch_python", "-ltorch_cuda", "-ltorch_cpu", "-lc10_cuda", "-lc10"]
     _run(cmd, _EXT, verbose)
+    os.makedirs(os.path.dirname(_EXT_STAMP), exist_ok=True)
+    with open(_EXT_STAMP, "w") as f:
+        f.write(_ext_versions())
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
     jobs = []
     if force or not up_to_date():
         jobs.append(_build_library)
-    if force or not up_to_date(_EXT, _EXT_DEPS):
+    if force or not extension_up_to_date():
         jobs.append(_build_extension)
     with ThreadPoolExecutor(2) as pool:
         for f in [pool.submit(j, verbose) for j in jobs]:
