@@ -107,9 +107,9 @@ ptq_status_t make_map_2d(CUtensorMap *map, CUtensorMapDataType dt, int elem_byte
     return PTQ_OK;
 }
 
-#ifndef PTQ_GEMM_SHORT_K_BLOCKS
-#define PTQ_GEMM_SHORT_K_BLOCKS 3
-#endif
+// Up to so many k-blocks (K <= 384) the main loop of a tile is short against its epilogue.
+constexpr int kShortMainLoop = 3;
+static_assert(kShortMainLoop <= ptq::kResMaxKBlocks, "the resident kernel takes every short main loop");
 
 inline int round_up(int v, int m) { return (v + m - 1) / m * m; }
 
@@ -391,20 +391,10 @@ ptq_status_t launch_quantize_dynamic(const ptq_linear *h, const void *x, long lo
     return PTQ_OK;
 }
 
-#ifndef PTQ_GEMM_PANEL
-#define PTQ_GEMM_PANEL 1
-#endif
-#ifndef PTQ_GEMM_TEAMS
-#define PTQ_GEMM_TEAMS 1
-#endif
-#ifndef PTQ_GEMM_TEAM_MIN_ROUNDS
-#define PTQ_GEMM_TEAM_MIN_ROUNDS 3
-#endif
-
 // Per-channel vectors a GEMM kernel keeps in shared memory: weight steps, bias, and (short main loops) row sums.
 void set_vectors(const ptq_linear *h, ptq::GemmParams &p)
 {
-    p.ws_copy = h->asym && h->k_blocks <= PTQ_GEMM_SHORT_K_BLOCKS ? 1 : 0;
+    p.ws_copy = h->asym && h->k_blocks <= kShortMainLoop ? 1 : 0;
     p.vectors = 1 + p.has_bias + p.ws_copy;
 }
 
@@ -418,7 +408,7 @@ bool plan_panel(const ptq_linear *h, ptq::GemmParams &p, bool tma_store)
 {
     p.group = p.groups = p.b_stages = p.b_stage_bytes = 0;
     const long long tiles = static_cast<long long>(p.m_tiles) * p.n_tiles;
-    if (!PTQ_GEMM_PANEL || !tma_store || p.n_tiles < 2 || p.k_blocks < 4 || p.k_blocks > ptq::kPanelMaxKBlocks ||
+    if (!tma_store || p.n_tiles < 2 || p.k_blocks < 4 || p.k_blocks > ptq::kPanelMaxKBlocks ||
         tiles < 8ll * h->num_sms)
         return false;
     const int stage_bytes = p.BN * ptq::kBK;
@@ -444,12 +434,12 @@ bool plan_panel(const ptq_linear *h, ptq::GemmParams &p, bool tma_store)
 }
 
 // Whether the kernel with resident weights (and its epilogue in two teams) is taken: short main loop (K <= 384) and three tiles
-// per CTA.  With two the streaming kernel's shorter latency of a tile wins: 12608 x 192 -> 768 10.5 us against 11.1, 6304 x 384 ->
+// per CTA (and TMA stores).  With two the streaming kernel's shorter latency of a tile wins: 12608 x 192 -> 768 10.5 us against 11.1, 6304 x 384 ->
 // 1536 11.0 against 12.2, 25088 x 384 -> 384 14.3 against 14.7; with four and more this one does (figures at the kernel).
-bool gemm_teams(const ptq_linear *h, const ptq::GemmParams &p, bool tma_store, bool short_k)
+constexpr long long kResidentMinRounds = 3;
+bool takes_resident(const ptq_linear *h, int m_tiles, int n_tiles)
 {
-    const long long tiles = static_cast<long long>(p.m_tiles) * p.n_tiles;
-    return PTQ_GEMM_TEAMS && tma_store && short_k && tiles >= static_cast<long long>(PTQ_GEMM_TEAM_MIN_ROUNDS) * h->num_sms;
+    return h->k_blocks <= kShortMainLoop && static_cast<long long>(m_tiles) * n_tiles >= kResidentMinRounds * h->num_sms;
 }
 
 // Cycles of the busiest CTA of the streaming kernel with tiles of `bn` columns, as measured on the workloads: an MMA of
@@ -469,19 +459,16 @@ double gemm_cycles(const ptq_linear *h, const ptq::GemmParams &p, int bn)
 // leaves the busiest CTA clearly less to do: idle SMs in a single round, or a last round that is nearly empty.  Layer,
 // both kernels, us: 1568 x 1536 -> 768 (256 -> 128 columns) 10.6 -> 9.7, 2793 x 1536 -> 768 (256 -> 192) 11.7 -> 10.8,
 // 12544 x 768 -> 384 (192 -> 128) 14.6 -> 14.1, 6304 x 384 -> 1536 (256 -> 192) 11.4 -> 11.0.  The margin keeps what the model cannot
-// tell apart: 11229 x 520 -> 600 (predicted -7 %) measured +1 %.  Widths that make the epilogue run in teams are not
+// tell apart: 11229 x 520 -> 600 (predicted -7 %) measured +1 %.  Widths that lead to the resident kernel are not
 // compared: with several rounds and a short main loop the widths are within 3 % of one another either way.
 int choose_bn(const ptq_linear *h, const ptq::GemmParams &p)
 {
-    auto teams = [&](int bn) {
-        return h->k_blocks <= PTQ_GEMM_SHORT_K_BLOCKS && static_cast<long long>(p.m_tiles) * ((h->N + bn - 1) / bn) >=
-                                                            static_cast<long long>(PTQ_GEMM_TEAM_MIN_ROUNDS) * h->num_sms;
-    };
+    auto resident = [&](int bn) { return takes_resident(h, p.m_tiles, (h->N + bn - 1) / bn); };
     int best = h->BN;
-    if (teams(best)) return best;
+    if (resident(best)) return best;
     double best_cost = 0.93 * gemm_cycles(h, p, best);
     for (int bn = 64; bn <= ptq::kMaxBN && bn < h->N + 64; bn += 64) {
-        if (teams(bn)) continue;
+        if (resident(bn)) continue;
         const double cost = gemm_cycles(h, p, bn);
         if (cost < best_cost) {
             best = bn;
@@ -517,7 +504,7 @@ void set_gemm_params(const ptq_linear *h, ptq::GemmParams &p, long long M, void 
     set_vectors(h, p);
     // Short main loops (up to three k-blocks per tile, K <= 384) leave the epilogue little time: three stages and two
     // staging boxes per warp; longer ones keep four stages.  Layers with a bias hold two more scale copies.
-    const bool short_k = h->k_blocks <= PTQ_GEMM_SHORT_K_BLOCKS;
+    const bool short_k = h->k_blocks <= kShortMainLoop;
     p.stages = (short_k || h->has_bias) ? ptq::kStages - 1 : ptq::kStages;
     p.boxes = short_k ? 2 : 1;
     p.y = static_cast<__half *>(y);
@@ -550,9 +537,6 @@ ptq_status_t launch_gemm(const ptq_linear *h, const void *codes, long long M, vo
     if (st != PTQ_OK) return st;
     const bool tma_store = (h->N % 8 == 0) && (reinterpret_cast<uintptr_t>(y) % 16 == 0);
     const int m_tiles_ = static_cast<int>((M + ptq::kBM - 1) / ptq::kBM);
-#ifdef PTQ_EXP_FORCE_PAIR
-    want_pair = true;
-#endif
     const bool use_pair = want_pair && h->max_pairs > 0 && !h->has_bias &&
                           static_cast<long long>((m_tiles_ + 1) / 2) * h->n_tiles >= h->max_pairs;
     if (tma_store) {
@@ -566,7 +550,6 @@ ptq_status_t launch_gemm(const ptq_linear *h, const void *codes, long long M, vo
 
     ptq::GemmParams p;
     set_gemm_params(h, p, M, y, acc_out, tma_store, dx_rows);
-    const bool short_k = h->k_blocks <= PTQ_GEMM_SHORT_K_BLOCKS;
     const int gemm_smem = ptq::gemm_smem_bytes(p.stages, p.boxes, p.vectors);
 
     if (use_pair) {
@@ -616,11 +599,11 @@ ptq_status_t launch_gemm(const ptq_linear *h, const void *codes, long long M, vo
     if (bn != h->BN) set_bn(h, p, bn);
     const CUtensorMap &tmW = bn != h->BN ? h->tmWbn[bn / 64 - 1] : h->tmW;
     const long long tiles = static_cast<long long>(p.m_tiles) * p.n_tiles;
-    const bool teams = gemm_teams(h, p, tma_store, short_k);
+    const bool resident = tma_store && takes_resident(h, p.m_tiles, p.n_tiles);
     const int grid = static_cast<int>(tiles < h->num_sms ? tiles : h->num_sms);
     auto go = [&](auto debug, auto asym) -> ptq_status_t {
         constexpr bool kDbg = decltype(debug)::value, kAsym = decltype(asym)::value;
-        if (teams) {
+        if (resident) {
             constexpr auto kKern = ptq::ptq_gemm_dequant_resident_kernel<kDbg, kAsym>;
             p.fd_n_tiles = ptq::make_fastdiv(static_cast<unsigned>(p.m_tiles));
             const ptq_status_t es = ensure_smem<kKern>(h->device, ptq::kResSmemMax);
@@ -1190,11 +1173,11 @@ int ptq_linear_gemm_variant(const ptq_linear_t *h, int B)
     p.k_blocks = h->k_blocks;
     p.has_bias = h->has_bias ? 1 : 0;
     set_vectors(h, p);
-    const bool short_k = h->k_blocks <= PTQ_GEMM_SHORT_K_BLOCKS;
+    const bool short_k = h->k_blocks <= kShortMainLoop;
     p.boxes = short_k ? 2 : 1;
     if (plan_panel(h, p, true)) return 2;
     set_bn(h, p, choose_bn(h, p));
-    return gemm_teams(h, p, true, short_k) ? 1 : 0;
+    return takes_resident(h, p.m_tiles, p.n_tiles) ? 1 : 0;
 }
 
 ptq_status_t ptq_linear_gemm_dequant(const ptq_linear_t *h, const void *q_int8, int B, void *y_fp16, void *stream)
