@@ -66,3 +66,11 @@ def check_layer(ptq, torch, spec, B=None, flags_list=(0, 1, 2), seed=0):
             assert_y_close(y[m0:m1], y_ref, "%s rows %d:%d" % (what, m0, m1))
     layer.close()
     return clip
+
+
+def launches(ptq, call):
+    """Kernels that the library launches during call(): the path a test is meant for, so that a later rule that sends its sizes
+    elsewhere is noticed."""
+    n0 = ptq.binding.kernel_launch_count()
+    call()
+    return ptq.binding.kernel_launch_count() - n0

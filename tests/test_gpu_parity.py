@@ -6,7 +6,7 @@ import pytest
 
 import oracle
 from paper_2412_20386_b200 import workloads as wl
-from parity_util import assert_y_close, check_layer, layer_inputs
+from parity_util import assert_y_close, check_layer, launches, layer_inputs
 
 pytestmark = pytest.mark.gpu
 
@@ -251,7 +251,8 @@ def test_two_host_threads_share_one_handle(env):
 
 
 def test_seeded_random_shapes(env):
-    """Sixteen seeded random (K, N, T, B): every kernel variant the shape and alignment select, every flag."""
+    """Sixteen seeded random (K, N, T, B), every flag.  Without a flag nearly all have few enough rows for the one-kernel path; the
+    pair flag, whose kernel needs more rows, sends the same shapes through the quantize and the streaming GEMM kernel."""
     ptq, torch = env
     rng = np.random.default_rng(20241228)
     for i in range(16):
@@ -322,22 +323,23 @@ def test_fused_flag_is_reported_and_needs_no_workspace(env):
             assert layer.workspace_bytes(2, ptq.FLAG_FUSED_PROLOGUE) == layer.workspace_bytes(2, 0) > 0
 
 
-def test_unaligned_pointers_take_the_generic_paths(env):
+@pytest.mark.parametrize("B,kernels", [(2, 1), (25, 2)])             # few rows: one kernel; more: quantize and GEMM
+def test_unaligned_pointers_take_the_generic_paths(env, B, kernels):
     ptq, torch = env
     spec = CFG[0][0]
-    x, wq, dw, bias, s, dx = layer_inputs(spec, B=2)
-    M = 2 * spec.T
+    x, wq, dw, bias, s, dx = layer_inputs(spec, B=B)
+    M = B * spec.T
     layer = ptq.PtqLinear(wq, dw, s, dx, bias)
     xbuf = torch.zeros(x.size + 8, dtype=torch.float16, device="cuda")
     ybuf = torch.zeros(M * spec.N + 8, dtype=torch.float16, device="cuda")
-    xv = xbuf[1:1 + x.size].view(2, spec.T, spec.K)          # 2-byte aligned only
-    yv = ybuf[1:1 + M * spec.N].view(2, spec.T, spec.N)
+    xv = xbuf[1:1 + x.size].view(B, spec.T, spec.K)          # 2-byte aligned only
+    yv = ybuf[1:1 + M * spec.N].view(B, spec.T, spec.N)
     xv.copy_(torch.from_numpy(x).cuda())
     y_ref = oracle.linear_forward(x.reshape(M, spec.K), spec.T, wq, dw, s, dx, bias)
     for flags in (0, ptq.FLAG_FUSED_PROLOGUE):       # the fused flag falls back: x is not 16-byte aligned
         yv.zero_()
-        layer.forward(xv, y=yv, workspace=torch.empty(layer.workspace_bytes(2), dtype=torch.uint8, device="cuda"),
-                      flags=flags)
+        ws = torch.empty(layer.workspace_bytes(B), dtype=torch.uint8, device="cuda")
+        assert launches(ptq, lambda: layer.forward(xv, y=yv, workspace=ws, flags=flags)) == kernels
         torch.cuda.synchronize()
         layer.device_status()
         assert_y_close(yv.cpu().numpy().reshape(M, spec.N), y_ref, "unaligned flags=%d" % flags)

@@ -1,12 +1,13 @@
 """Sizes that fill no chunk, no vector store and no tile: the quantize kernel's partial chunks at every load width (row
 alignment 16, 8, 4 and 2 bytes; dense and padded code rows) and the GEMM's row copies at every store width (N a multiple
-of 4, of 2, odd; y offset by one element), against the oracle."""
+of 4, of 2, odd; y offset by 1, 2 and 4 elements), against the oracle.  The sizes come with few rows, which one kernel takes, and
+with rows for the quantize and the GEMM kernel; the number of launches tells which ran."""
 import numpy as np
 import pytest
 
 import oracle
 from paper_2412_20386_b200 import workloads as wl
-from parity_util import assert_y_close, check_layer, layer_inputs
+from parity_util import assert_y_close, check_layer, launches, layer_inputs
 
 pytestmark = pytest.mark.gpu
 
@@ -29,11 +30,23 @@ def test_ragged_layers_match_oracle(env, K, N, T, B):
     check_layer(ptq, torch, wl.LinearSpec(11, K % 89, N % 7, "ragged", B, T, K, N, bias=bool(K & 1)), flags_list=(0,))
 
 
+# as above, with rows beyond the one-kernel path
+@pytest.mark.parametrize("K,N,T,B", [(1, 1, 1, 9500), (7, 9, 3, 3200), (9, 65, 5, 1901), (12, 44, 197, 49), (129, 257, 5, 640),
+                                     (250, 130, 13, 365), (31, 1028, 1, 1100), (33, 1026, 1, 1100)])
+def test_ragged_layers_in_two_kernels_match_oracle(env, K, N, T, B):
+    ptq, torch = env
+    check_layer(ptq, torch, wl.LinearSpec(11, K % 89, N % 7, "ragged", B, T, K, N, bias=bool(K & 1)), flags_list=(0,))
+    layer = ptq.PtqLinear(np.ones((N, K), np.int8), np.ones(N, np.float32), np.ones(K, np.float32), np.ones(T, np.float32))
+    assert launches(ptq, lambda: layer.forward(torch.zeros((B, T, K), dtype=torch.float16, device="cuda"))) == 2
+    layer.close()
+
+
 @pytest.mark.parametrize("K", [4, 6, 13, 24, 520])
 @pytest.mark.parametrize("x_off,y_off", [(0, 0), (1, 1), (2, 2), (4, 4)])
-def test_ragged_alignments(env, K, x_off, y_off):
+@pytest.mark.parametrize("B", [37, 870])
+def test_ragged_alignments(env, K, x_off, y_off, B):
     ptq, torch = env
-    spec = wl.LinearSpec(12, K, 1, "align", 37, 11, K, 40, bias=False)
+    spec = wl.LinearSpec(12, K, 1, "align", B, 11, K, 40, bias=False)
     x, wq, dw, bias, s, dx = layer_inputs(spec)
     M = spec.M
     layer = ptq.PtqLinear(wq, dw, s, dx, bias)
@@ -45,7 +58,8 @@ def test_ragged_alignments(env, K, x_off, y_off):
     y_ref, q_ref, _ = oracle.linear_forward(x.reshape(M, K), spec.T, wq, dw, s, dx, bias, taps=True)
     qb = torch.full((M * K + 8,), 99, dtype=torch.int8, device="cuda")
     layer.quantize(xv, q=qb[x_off:x_off + M * K])
-    layer.forward(xv, y=yv)
+    one_kernel = B == 37 or (K == 4 and y_off == 0)          # few rows; few channels, for which y has to be aligned
+    assert launches(ptq, lambda: layer.forward(xv, y=yv)) == (1 if one_kernel else 2)
     torch.cuda.synchronize()
     layer.device_status()
     q = qb.cpu().numpy()

@@ -7,7 +7,7 @@ import pytest
 
 import oracle
 from paper_2412_20386_b200 import workloads as wl
-from parity_util import assert_y_close, layer_inputs
+from parity_util import assert_y_close, launches, layer_inputs
 
 pytestmark = pytest.mark.gpu
 
@@ -21,13 +21,6 @@ def env():
     import paper_2412_20386_b200 as ptq
     torch.cuda.set_device(0)
     return ptq, torch
-
-
-def launches(ptq, torch, layer, x):
-    n0 = ptq.binding.kernel_launch_count()
-    layer.forward(x)
-    torch.cuda.synchronize()
-    return ptq.binding.kernel_launch_count() - n0
 
 
 @pytest.mark.parametrize("K,N,T,M,bias,off", [
@@ -45,7 +38,7 @@ def test_few_channels_match_oracle(env, K, N, T, M, bias, off):
     xb = torch.zeros(x.size + 8, dtype=torch.float16, device="cuda")
     xd = xb[off:off + x.size].view(spec.B, T, K)
     xd.copy_(torch.from_numpy(x.reshape(spec.B, T, K)).cuda())
-    assert launches(ptq, torch, layer, xd) == 1
+    assert launches(ptq, lambda: layer.forward(xd)) == 1
     y, q, acc = layer.forward_debug(xd)
     y2 = layer.forward(xd)
     torch.cuda.synchronize()
@@ -68,7 +61,7 @@ def test_few_channels_4bit(env):
     s, dx = oracle.calibrate4(xcal, w4, dw)
     layer = ptq.PtqLinear(oracle.pack_int4(w4), dw, s, dx, bias, packed4_K=K)
     xd = torch.from_numpy(x).cuda()
-    assert launches(ptq, torch, layer, xd) == 1
+    assert launches(ptq, lambda: layer.forward(xd)) == 1
     y, _, acc = layer.forward_debug(xd, want_q=False)
     torch.cuda.synchronize()
     layer.device_status()
@@ -83,5 +76,5 @@ def test_which_layers_take_one_kernel(env):
     for K, N, want in ((32, 256, 1), (33, 264, 2), (32, 248, 2), (12, 388, 2)):
         layer = ptq.PtqLinear(np.ones((N, K), np.int8), np.ones(N, np.float32), np.ones(K, np.float32), np.ones(9, np.float32))
         x = torch.zeros((1200, 9, K), dtype=torch.float16, device="cuda")
-        assert launches(ptq, torch, layer, x) == want, (K, N)
+        assert launches(ptq, lambda: layer.forward(x)) == want, (K, N)
         layer.close()
