@@ -29,10 +29,11 @@
  *     so concurrent forwards on different streams are allowed as long as they
  *     use different workspaces (each handle also carries one device status
  *     word that all its launches may set; see ptq_linear_device_status).
- *   - The quantize and GEMM kernels are launched with the programmatic-stream-serialization
- *     attribute: their set-up may run while the previous kernel on the stream drains, and each waits
- *     for that kernel's completion before it reads or writes any buffer.  Results and ordering are
- *     those of plain stream order.
+ *   - The kernels of a forward call without flags are launched with the
+ *     programmatic-stream-serialization attribute: their set-up, which reads the layer's own parameters,
+ *     may run while the previous kernel on the stream drains, and each waits for that kernel's
+ *     completion before it reads or writes any other buffer.  Results and ordering are those of plain
+ *     stream order.
  *   - Requires a device of compute capability 10.0 (sm_100a); create fails
  *     with PTQ_ERR_ARCH elsewhere.  There is no CPU or generic-GPU fallback.
  */
@@ -56,7 +57,7 @@ typedef enum {
     PTQ_ERR_ALIGN   = 4,   /* a device pointer is not aligned as required */
     PTQ_ERR_ARCH    = 5,   /* current device is not compute capability 10.0 */
     PTQ_ERR_CUDA    = 6,   /* a CUDA runtime / driver call failed; text in ptq_last_error() */
-    PTQ_ERR_NOMEM   = 7,   /* device or host allocation failed (create / calibrate only) */
+    PTQ_ERR_NOMEM   = 7,   /* device or host allocation failed (create, calibrate and search only) */
     PTQ_ERR_TIMEOUT = 8    /* a bounded device-side wait gave up (reported by ptq_linear_device_status) */
 } ptq_status_t;
 

@@ -810,6 +810,10 @@ ptq_status_t launch_small(const ptq_linear *h, const SmallPlan &pl, const void *
 // warps are not what a CTA waits for.  us, two kernels -> one: 3152 x 12 -> 384 5.6 -> 4.9, 25216 x 12 -> 384 10.4 -> 8.2, 12608 x 17 ->
 // 200 7.6 -> 6.5, 50432 x 24 -> 768 17.9 -> 17.6, 200704 x 8 -> 64 13.7 -> 13.8; not taken: 200704 x 16 -> 64 14.5 -> 15.6, 200704 x 32 -> 128
 // 19.1 -> 22.5, 12608 x 48 -> 1536 13.6 -> 15.9, 50176 x 64 -> 256 11.7 -> 14.0.
+// At the range's other end (with a bias, launches replayed from a graph): 12608 x 1 -> 32 5.8 -> 4.1, 201728 x 1 -> 32 14.4 -> 12.6, 50432 x
+// 2 -> 32 8.9 -> 5.9, 50432 x 6 -> 64 9.6 -> 6.0, 201728 x 6 -> 64 14.7 -> 13.2, 201728 x 8 -> 64 13.5 -> 12.0.  The nearest to a loss: 6304 x 32 ->
+// 256 5.8 -> 6.3, 100864 x 32 -> 768 33.2 -> 33.1.  A thread takes the slower routes of the quantizer for a whole row, so activations
+// far from the calibrated steps (every thirtieth code saturated or near a tie) cost this kernel more: 25216 x 24 -> 768 12.0 -> 13.8.
 bool plan_short_k(const ptq_linear *h, const void *y)
 {
     return h->K <= ptq::kShortKMaxK && h->N >= 8 * h->K && !h->asym && h->fast_div && h->N % 8 == 0 &&
