@@ -190,7 +190,7 @@ __device__ __noinline__ float divided_max_call(uint4 v, const float4 *ra, const 
 // so only elements with a >= (1 - 2^-21) * max a can hold the maximum, and only those (one or two a row) are divided.
 // Each lane copies its part of the warp's next row into shared memory (cp.async) while it works on this one: in registers the
 // second row spilled and lost (6304 x 1536 -> 768: 25.4 us), without it that layer took 23.1 us and 50432 x 1536 -> 8 86.5.
-// Bound by issue (15 instructions an element, 64 % of the issue slots taken) and, with few rows, by its chain of latencies: load,
+// Bound by issue (16 instructions an element at K = 1536, 20 at 768; 68 % of the issue slots taken) and, with few rows, by its chain of latencies: load,
 // two warp reductions, store.  Quantize + GEMM, against the two-pass kernel above: 6304 x 768 -> 3072 28.5 -> 24.4 us, 6304 x 1536 ->
 // 768 29.8 -> 21.2, 50432 x 768 -> 8 58.0 -> 39.4.
 constexpr int dyn_row_ctas_per_sm(int chunks) { return chunks <= 3 ? 4 : 3; }
