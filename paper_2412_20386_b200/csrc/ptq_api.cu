@@ -442,17 +442,36 @@ bool takes_resident(const ptq_linear *h, int m_tiles, int n_tiles)
     return h->k_blocks <= kShortMainLoop && static_cast<long long>(m_tiles) * n_tiles >= kResidentMinRounds * h->num_sms;
 }
 
-// Cycles of the busiest CTA of the streaming kernel with tiles of `bn` columns, as measured on the workloads: an MMA of
-// K = 32 takes 57 + 0.54 bn, the eight epilogue warps take 550 per tile and 700 per pair of 64-column steps, the hand-overs
-// 300 per tile.
+// Cycles of one tile of `cols` columns in the streaming kernel, as measured on the workloads: an MMA of K = 32 takes 57 + 0.54 cols;
+// the eight epilogue warps take 550 per tile and 700 per pair of 64-column steps.
+double mma_cycles(const ptq_linear *h, int cols) { return (h->K + 31) / 32 * (57.0 + 0.54 * cols); }
+double epilogue_cycles(int cols) { return 550.0 + 700.0 * (((cols + 63) / 64 + 1) / 2); }
+
+// Columns per piece of the streaming kernel's last round with tiles of `bn` columns, 0 where it is not cut: at least one full
+// round before it, SMs enough for all pieces at once (narrow ones first), and a long main loop: the epilogue gains little by
+// a narrower tile.  Layer, both kernels, us, whole and cut: 6304 x 1536 -> 768 (dynamic) 21.4 -> 19.7, 6304 x 768 -> 3072 (dynamic) 24.5 -> 24.0,
+// 1568 x 768 -> 3072 10.8 -> 9.8, 3136 x 768 -> 3072 13.9 -> 13.2; with K <= 384 25088 x 384 -> 192 11.6 -> 11.7, 12608 x 192 -> 768 10.3 -> 10.3,
+// and a pair of layers with 6304 x 384 -> 1536 24.75 -> 24.9.
+int cut_cols(const ptq_linear *h, const ptq::GemmParams &p, int bn)
+{
+    const long long tiles = static_cast<long long>(p.m_tiles) * ((h->N + bn - 1) / bn), last = tiles % h->num_sms;
+    if (tiles < h->num_sms || last == 0 || h->k_blocks <= kShortMainLoop) return 0;
+    for (int cols = 64; cols <= 128 && cols < bn; cols += 64)
+        if (last * ((bn + cols - 1) / cols) <= h->num_sms) return cols;
+    return 0;
+}
+
+// Cycles of the busiest CTA of the streaming kernel with tiles of `bn` columns; the hand-overs take 300 per tile.
 double gemm_cycles(const ptq_linear *h, const ptq::GemmParams &p, int bn)
 {
     const long long tiles = static_cast<long long>(p.m_tiles) * ((h->N + bn - 1) / bn);
     const double rounds = static_cast<double>((tiles + h->num_sms - 1) / h->num_sms);
-    const int steps = (bn + 63) / 64;
-    const double mma = (h->K + 31) / 32 * (57.0 + 0.54 * bn);
-    const double epi = 550.0 + 700.0 * ((steps + 1) / 2);
-    return mma + (rounds - 1.0) * (mma > epi ? mma : epi) + epi + 300.0 * rounds;
+    auto longer = [](double a, double b) { return a > b ? a : b; };
+    const int cut = cut_cols(h, p, bn), last = cut ? cut : bn;                // columns of the last round's tiles
+    double cycles = mma_cycles(h, rounds > 1.0 ? bn : last) + epilogue_cycles(last) + 300.0 * rounds;
+    if (rounds > 1.0)
+        cycles += (rounds - 2.0) * longer(mma_cycles(h, bn), epilogue_cycles(bn)) + longer(mma_cycles(h, last), epilogue_cycles(bn));
+    return cycles;
 }
 
 // Tile width of the streaming kernel for this many rows: the layer's own (as few N tiles as possible), unless another
@@ -600,6 +619,7 @@ ptq_status_t launch_gemm(const ptq_linear *h, const void *codes, long long M, vo
     const CUtensorMap &tmW = bn != h->BN ? h->tmWbn[bn / 64 - 1] : h->tmW;
     const long long tiles = static_cast<long long>(p.m_tiles) * p.n_tiles;
     const bool resident = tma_store && takes_resident(h, p.m_tiles, p.n_tiles);
+    const int cut = resident ? 0 : cut_cols(h, p, bn);
     const int grid = static_cast<int>(tiles < h->num_sms ? tiles : h->num_sms);
     auto go = [&](auto debug, auto asym) -> ptq_status_t {
         constexpr bool kDbg = decltype(debug)::value, kAsym = decltype(asym)::value;
@@ -610,8 +630,20 @@ ptq_status_t launch_gemm(const ptq_linear *h, const void *codes, long long M, vo
             if (es != PTQ_OK) return es;
             const int smem = ptq::res_smem_bytes(p.k_blocks, p.BN, p.vectors);
             PTQ_CUDA(launch_pdl(kKern, grid, ptq::kGemmThreads, smem, stream, tmA, tmW, tmY, p));
+        } else if (cut) {
+            constexpr auto kKern = ptq::ptq_gemm_dequant_kernel<kDbg, kAsym, ptq::GemmCutParams>;
+            ptq::GemmCutParams cp;
+            static_cast<ptq::GemmParams &>(cp) = p;
+            cp.tmWcut = h->tmWbn[cut / 64 - 1];
+            cp.full_tiles = static_cast<int>(tiles / h->num_sms) * h->num_sms;
+            cp.piece_cols = cut;
+            cp.pieces = (bn + cut - 1) / cut;
+            cp.fd_pieces = ptq::make_fastdiv(static_cast<unsigned>(cp.pieces));
+            const ptq_status_t es = ensure_smem<kKern>(h->device, ptq::kGemmSmemBytes);
+            if (es != PTQ_OK) return es;
+            PTQ_CUDA(launch_pdl(kKern, grid, ptq::kGemmThreads, gemm_smem, stream, tmA, tmW, tmY, cp));
         } else {
-            constexpr auto kKern = ptq::ptq_gemm_dequant_kernel<kDbg, kAsym>;
+            constexpr auto kKern = ptq::ptq_gemm_dequant_kernel<kDbg, kAsym, ptq::GemmParams>;
             const ptq_status_t es = ensure_smem<kKern>(h->device, ptq::kGemmSmemBytes);
             if (es != PTQ_OK) return es;
             PTQ_CUDA(launch_pdl(kKern, grid, ptq::kGemmThreads, gemm_smem, stream, tmA, tmW, tmY, p));

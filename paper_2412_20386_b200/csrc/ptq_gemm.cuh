@@ -21,6 +21,8 @@
 #include <cuda_fp16.h>
 #include <stdint.h>
 
+#include <type_traits>
+
 #include "ptx_sm100.cuh"
 
 namespace ptq {
@@ -395,11 +397,11 @@ template <bool kDebugAcc, bool kAsym>
 __device__ __forceinline__ uint32_t epilogue_tile_stream(const GemmParams &p, const CUtensorMap *tmY, uint32_t tmem_row,
                                                          long long m_row0, int n0, float dxr, uint32_t staging,
                                                          const float *dw_s, const float *bias_s, const int *ws_s, uint32_t nboxes,
-                                                         int lane, int c_begin, int c_stride, int zr, bool two_boxes)
+                                                         int lane, int c_begin, int c_stride, int cols, int zr, bool two_boxes)
 {
     const long long m = m_row0 + lane;
     const bool row_ok = m < p.M;
-    for (int c0 = c_begin; c0 < p.BN; c0 += c_stride) {
+    for (int c0 = c_begin; c0 < cols; c0 += c_stride) {
         const int n_first = n0 + c0;
         uint32_t v0[32], v1[32];
         tmem_ld_32x32(tmem_row + c0, v0);
@@ -586,7 +588,7 @@ __device__ __forceinline__ void epilogue_team_loop(const GemmParams &p, const CU
         const uint32_t tmem_row = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) + static_cast<uint32_t>(team) * kMaxBN;
         nboxes = epilogue_tile_stream<kDebugAcc, kAsym>(p, tmY, tmem_row, m_row0, n_tile * p.BN, dxr, staging, dw_buf,
                                                  p.has_bias ? bias_buf : nullptr, !kAsym ? nullptr : p.ws_copy ? ws_buf : p.wsum + n_tile * p.BN, nboxes,
-                                                 lane, 0, kEpiStepCols, zr, true);
+                                                 lane, 0, kEpiStepCols, p.BN, zr, true);
         tc_fence_before_sync();
         __syncwarp();
         if (lane == 0) mbar_arrive(tempty);
@@ -598,11 +600,44 @@ __device__ __forceinline__ void epilogue_team_loop(const GemmParams &p, const CU
 
 // --- the kernel ---------------------------------------------------------------------------------
 
-template <bool kDebugAcc, bool kAsym>
+// A last round that would leave most SMs without a tile is cut: its tiles become `pieces` narrower ones of `piece_cols` columns
+// each, so that the round takes the time of 64 or 128 columns and not of 256 (6304 x 1536 -> 768, 150 tiles on 148 SMs, both kernels:
+// 21.4 -> 19.7 us).  An instance of its own (one more tensor map, four more parameters): in one kernel all launches carried them, and
+// layers without such a round lost 1 %.
+struct GemmCutParams : GemmParams {
+    CUtensorMap tmWcut;    // the weights in boxes of piece_cols rows
+    int full_tiles;        // tiles before the last round
+    int pieces, piece_cols;
+    FastDiv fd_pieces;
+};
+
+// What a tile index stands for: rows kBM * m_tile .., columns n0 .. n0 + cols.
+struct TileAt {
+    int m_tile, n0, cols;
+};
+template <bool kCut, class P>
+__device__ __forceinline__ TileAt tile_at(const P &p, int tile)
+{
+    int sub = 0;
+    if constexpr (kCut) {
+        if (tile >= p.full_tiles) {
+            const unsigned q = static_cast<unsigned>(tile - p.full_tiles), t = fd_div(q, p.fd_pieces);
+            sub = static_cast<int>(q - t * p.fd_pieces.d) * p.piece_cols;
+            tile = p.full_tiles + static_cast<int>(t);
+            const int m_tile = static_cast<int>(fd_div(static_cast<unsigned>(tile), p.fd_n_tiles));
+            return {m_tile, (tile - m_tile * p.n_tiles) * p.BN + sub, min(p.piece_cols, p.BN - sub)};
+        }
+    }
+    const int m_tile = static_cast<int>(fd_div(static_cast<unsigned>(tile), p.fd_n_tiles));
+    return {m_tile, (tile - m_tile * p.n_tiles) * p.BN, p.BN};
+}
+
+template <bool kDebugAcc, bool kAsym, class P>
 __global__ void __launch_bounds__(kGemmThreads, 1)
 ptq_gemm_dequant_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmW,
-                        const __grid_constant__ CUtensorMap tmY, const GemmParams p)
+                        const __grid_constant__ CUtensorMap tmY, const __grid_constant__ P p)
 {
+    constexpr bool kCut = std::is_same<P, GemmCutParams>::value;
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     const uint32_t base = smem_u32(smem_raw);                        // swizzled tiles need 1024-byte alignment
     if ((base & 1023u) != 0u) {
@@ -659,7 +694,8 @@ ptq_gemm_dequant_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
     // 12 -> 384: 11.5 -> 9.9; 200704 x 96 -> 384: 53.4 -> 52.1).
     griddep_launch_dependents();
 
-    const int total_tiles = p.m_tiles * p.n_tiles;
+    int total_tiles = p.m_tiles * p.n_tiles;
+    if constexpr (kCut) total_tiles = p.full_tiles + (total_tiles - p.full_tiles) * p.pieces;
 
     if (warp == 0) {
         // ------------------------------------------------------------------ TMA producer
@@ -667,6 +703,12 @@ ptq_gemm_dequant_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
             uint32_t stage = 0, phase = 0, issued = 0;
             bool ok = true;
             const uint32_t tx = static_cast<uint32_t>(kATileBytes + p.BN * kBK);
+            uint32_t tx_piece = tx;
+            const CUtensorMap *tmPiece = &tmW;
+            if constexpr (kCut) {
+                tx_piece = static_cast<uint32_t>(kATileBytes + p.piece_cols * kBK);        // a box counts whole, also beyond N
+                tmPiece = &p.tmWcut;
+            }
             const int early = min(static_cast<int>(nstages), p.k_blocks);   // k-blocks of the first tile whose weights go first
             if (static_cast<int>(blockIdx.x) < total_tiles) {
                 const int n_tile = static_cast<int>(blockIdx.x - fd_div(blockIdx.x, p.fd_n_tiles) * p.fd_n_tiles.d);
@@ -677,8 +719,8 @@ ptq_gemm_dequant_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
             }
             griddep_wait();
             for (int tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x) {
-                const int m_tile = static_cast<int>(fd_div(static_cast<unsigned>(tile), p.fd_n_tiles));
-                const int n_tile = tile - m_tile * p.n_tiles;
+                const TileAt at = tile_at<kCut>(p, tile);
+                const bool piece = kCut && at.cols != p.BN;    // a whole tile among the pieces (never made) would load alike
                 for (int kb = 0; kb < p.k_blocks; ++kb) {
                     if (!mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag, p.status)) {
                         ok = false;
@@ -686,10 +728,10 @@ ptq_gemm_dequant_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
                     }
                     const uint32_t a_dst = base + stage * kStageBytes;
                     if (static_cast<int>(issued) >= early) {
-                        mbar_arrive_expect_tx(full_bar(stage), tx);
-                        tma_load_2d(a_dst + kATileBytes, &tmW, kb * kBK, n_tile * p.BN, full_bar(stage));
+                        mbar_arrive_expect_tx(full_bar(stage), piece ? tx_piece : tx);
+                        tma_load_2d(a_dst + kATileBytes, piece ? tmPiece : &tmW, kb * kBK, at.n0, full_bar(stage));
                     }
-                    tma_load_2d(a_dst, &tmA, kb * kBK, m_tile * kBM, full_bar(stage));
+                    tma_load_2d(a_dst, &tmA, kb * kBK, at.m_tile * kBM, full_bar(stage));
                     ++issued;
                     if (++stage == nstages) {
                         stage = 0;
@@ -711,12 +753,13 @@ ptq_gemm_dequant_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
     } else if (warp == 1) {
         // ------------------------------------------------------------------ MMA issuer
         if (lane == 0) {
-            const uint32_t idesc = make_idesc_s8(kBM, p.BN, kAsym);   // unsigned codes on asymmetric layers
+            uint32_t idesc = make_idesc_s8(kBM, p.BN, kAsym);   // unsigned codes on asymmetric layers
             uint32_t stage = 0, phase = 0, buf = 0, bphase = 0;
             bool ok = true;
             for (int tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x) {
                 if (!mbar_wait(tempty_bar(buf), bphase ^ 1u, abort_flag, p.status)) break;
                 tc_fence_after_sync();
+                if constexpr (kCut) idesc = make_idesc_s8(kBM, tile_at<kCut>(p, tile).cols, kAsym);
                 const uint32_t d_tmem = tmem_base + buf * kMaxBN;
                 for (int kb = 0; kb < p.k_blocks; ++kb) {
                     if (!mbar_wait(full_bar(stage), phase, abort_flag, p.status)) {
@@ -754,8 +797,8 @@ ptq_gemm_dequant_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
         int ws_next = 0;
         auto fetch_scales = [&](int tile) {
             // unconditional loads from clamped indices (see load_row_step); past the last tile the values are not used
-            const unsigned tl = tile < total_tiles ? static_cast<unsigned>(tile) : 0u;
-            const int n = static_cast<int>(tl - fd_div(tl, p.fd_n_tiles) * p.fd_n_tiles.d) * p.BN + min(et, p.BN - 1);
+            const TileAt at = tile_at<kCut>(p, tile < total_tiles ? tile : 0);
+            const int n = at.n0 + min(et, at.cols - 1);
             dw_next = __ldg(p.dw + n);
             if (p.has_bias) bias_next = __ldg(p.bias + n);
             if (kAsym && p.ws_copy) ws_next = __ldg(p.wsum + n);
@@ -777,13 +820,12 @@ ptq_gemm_dequant_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
         for (int tile = blockIdx.x; tile < total_tiles; tile += gridDim.x, ++it) {
             const int tile_next = tile + static_cast<int>(gridDim.x);
             fetch_scales(tile_next);                            // in flight during this tile
-            const int m_tile = static_cast<int>(fd_div(static_cast<unsigned>(tile), p.fd_n_tiles));
-            const int n_tile = tile - m_tile * p.n_tiles;
-            const long long m_row0 = static_cast<long long>(m_tile) * kBM + quarter * 32;
+            const TileAt at = tile_at<kCut>(p, tile);
+            const long long m_row0 = static_cast<long long>(at.m_tile) * kBM + quarter * 32;
             const float dxr = rs_next.dx;
             const int zr = rs_next.z;
             if (tile_next < total_tiles)
-                rs_next = load_row_step<kAsym>(p, static_cast<int>(fd_div(static_cast<unsigned>(tile_next), p.fd_n_tiles)), quarter, lane);
+                rs_next = load_row_step<kAsym>(p, tile_at<kCut>(p, tile_next).m_tile, quarter, lane);
             // every epilogue warp has written its share of this tile's scale copies (arrival `it` of the barrier)
             bool got = mbar_wait(scale_bar, it & 1u, abort_flag, p.status);
             got = got && mbar_wait(tfull_bar(buf), bphase, abort_flag, p.status);
@@ -795,9 +837,9 @@ ptq_gemm_dequant_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
             const float *bias_s = p.has_bias ? scale_s + (2u + (it & 1u)) * kMaxBN : nullptr;
             const int *ws_s = !kAsym ? nullptr
                               : p.ws_copy ? reinterpret_cast<const int *>(scale_s) + (2u * p.vectors - 2u + (it & 1u)) * kMaxBN
-                                          : p.wsum + n_tile * p.BN;
-            nboxes = epilogue_tile_stream<kDebugAcc, kAsym>(p, &tmY, tmem_row, m_row0, n_tile * p.BN, dxr, staging, dw_s,
-                                                     bias_s, ws_s, nboxes, lane, col_half * kEpiStepCols, 2 * kEpiStepCols, zr, two_boxes);
+                                          : p.wsum + at.n0;
+            nboxes = epilogue_tile_stream<kDebugAcc, kAsym>(p, &tmY, tmem_row, m_row0, at.n0, dxr, staging, dw_s,
+                                                     bias_s, ws_s, nboxes, lane, col_half * kEpiStepCols, 2 * kEpiStepCols, at.cols, zr, two_boxes);
             tc_fence_before_sync();
             __syncwarp();
             if (lane == 0) mbar_arrive(tempty_bar(buf));
@@ -1080,7 +1122,7 @@ ptq_gemm_dequant_panel_kernel(const __grid_constant__ CUtensorMap tmA, const __g
                               : p.ws_copy ? reinterpret_cast<const int *>(scale_s) + (2u * p.vectors - 2u + (it & 1u)) * kMaxBN
                                           : p.wsum + n_tile * p.BN;
             nboxes = epilogue_tile_stream<kDebugAcc, kAsym>(p, &tmY, tmem_row, m_row0, n_tile * p.BN, dxr, staging, dw_s, bias_s,
-                                                     ws_s, nboxes, lane, col_half * kEpiStepCols, 2 * kEpiStepCols, zr, two_boxes);
+                                                     ws_s, nboxes, lane, col_half * kEpiStepCols, 2 * kEpiStepCols, p.BN, zr, two_boxes);
             tc_fence_before_sync();
             __syncwarp();
             if (lane == 0) mbar_arrive(tempty_bar(buf));
@@ -1498,7 +1540,7 @@ ptq_gemm_dequant_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __gr
             if (p.use_tma_store)
                 nboxes = epilogue_tile_stream<kDebugAcc, false>(p, &tmY, tmem_row, m_row0, n_tile * p.BN, dxr, staging,
                                                          scale_s + (it & 1u) * kMaxBN, nullptr, nullptr, nboxes, lane,
-                                                         col_half * kEpiStepCols, 2 * kEpiStepCols, 0, false);
+                                                         col_half * kEpiStepCols, 2 * kEpiStepCols, p.BN, 0, false);
             else
                 nboxes = epilogue_tile<kDebugAcc, false, kStreamBox64>(p, &tmY, tmem_row, m_row0, n_tile * p.BN, dxr, staging,
                                                                        nboxes, lane, col_half);
