@@ -75,7 +75,7 @@ ptq_fused_linear_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_co
         reinterpret_cast<volatile uint32_t *>(base_ptr + bar_off + kFusedNumBarriers * 8);
     volatile uint32_t *abort_flag = tmem_holder + 1;
 
-    const int warp = threadIdx.x >> 5;
+    const int warp = uniform_warp();
     const int lane = threadIdx.x & 31;
 
     if (threadIdx.x == 0) {
@@ -103,7 +103,7 @@ ptq_fused_linear_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_co
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
-    const uint32_t tmem_base = *tmem_holder;
+    const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_holder, 0);
 
     if (warp == 0) {
         // ------------------------------------------------------------------ TMA producer
@@ -140,44 +140,42 @@ ptq_fused_linear_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_co
         }
     } else if (warp == 1) {
         // ------------------------------------------------------------------ MMA issuer
-        if (lane == 0) {
-            const uint32_t idesc = make_idesc_s8(kBM, p.BN);
-            uint32_t stage = 0, phase = 0, buf = 0, bphase = 0, it = 0;
-            bool ok = true;
-            for (int m_tile = blockIdx.x; m_tile < p.m_tiles && ok; m_tile += gridDim.x, ++it) {
-                for (int n_tile = 0; n_tile < p.n_tiles && ok; ++n_tile) {
-                    if (!mbar_wait(tempty_bar(buf), bphase ^ 1u, abort_flag, p.status)) {
+        const uint32_t idesc = make_idesc_s8(kBM, p.BN);
+        uint32_t stage = 0, phase = 0, buf = 0, bphase = 0, it = 0;
+        bool ok = true;
+        for (int m_tile = blockIdx.x; m_tile < p.m_tiles && ok; m_tile += gridDim.x, ++it) {
+            for (int n_tile = 0; n_tile < p.n_tiles && ok; ++n_tile) {
+                if (!mbar_wait_warp(tempty_bar(buf), bphase ^ 1u, abort_flag, p.status)) {
+                    ok = false;
+                    break;
+                }
+                tc_fence_after_sync();
+                const uint32_t d_tmem = tmem_base + buf * kMaxBN;
+                for (int kb = 0; kb < p.k_blocks; ++kb) {
+                    if (n_tile == 0 && !mbar_wait_warp(pfull_bar(kb), it & 1u, abort_flag, p.status)) {
+                        ok = false;
+                        break;
+                    }
+                    if (!mbar_wait_warp(wfull_bar(stage), phase, abort_flag, p.status)) {
                         ok = false;
                         break;
                     }
                     tc_fence_after_sync();
-                    const uint32_t d_tmem = tmem_base + buf * kMaxBN;
-                    for (int kb = 0; kb < p.k_blocks; ++kb) {
-                        if (n_tile == 0 && !mbar_wait(pfull_bar(kb), it & 1u, abort_flag, p.status)) {
-                            ok = false;
-                            break;
-                        }
-                        if (!mbar_wait(wfull_bar(stage), phase, abort_flag, p.status)) {
-                            ok = false;
-                            break;
-                        }
-                        tc_fence_after_sync();
-                        const uint64_t a_desc = make_smem_desc_sw128(panel_base + kb * kATileBytes);
-                        const uint64_t b_desc = make_smem_desc_sw128(w_base + stage * fp.w_stage_bytes);
-                        const int nmma = (kb == p.k_blocks - 1) ? p.last_mmas : (kBK / 32);
-                        mma_i8_ss_kblock(d_tmem, a_desc, b_desc, idesc, kb != 0 ? 1u : 0u, nmma);
-                        mma_commit(wempty_bar(stage));
-                        if (n_tile == p.n_tiles - 1) mma_commit(pempty_bar(kb));   // last reader of this panel block
-                        if (++stage == static_cast<uint32_t>(fp.w_stages)) {
-                            stage = 0;
-                            phase ^= 1u;
-                        }
+                    const uint64_t a_desc = make_smem_desc_sw128(panel_base + kb * kATileBytes);
+                    const uint64_t b_desc = make_smem_desc_sw128(w_base + stage * fp.w_stage_bytes);
+                    const int nmma = (kb == p.k_blocks - 1) ? p.last_mmas : (kBK / 32);
+                    mma_i8_ss_kblock(d_tmem, a_desc, b_desc, idesc, kb != 0 ? 1u : 0u, nmma);
+                    mma_commit(wempty_bar(stage));
+                    if (n_tile == p.n_tiles - 1) mma_commit(pempty_bar(kb));   // last reader of this panel block
+                    if (++stage == static_cast<uint32_t>(fp.w_stages)) {
+                        stage = 0;
+                        phase ^= 1u;
                     }
-                    if (!ok) break;
-                    mma_commit(tfull_bar(buf));
-                    buf ^= 1u;
-                    if (buf == 0u) bphase ^= 1u;
                 }
+                if (!ok) break;
+                mma_commit(tfull_bar(buf));
+                buf ^= 1u;
+                if (buf == 0u) bphase ^= 1u;
             }
         }
     } else if (warp < 2 + kNumEpiWarps) {

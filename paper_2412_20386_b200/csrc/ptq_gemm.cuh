@@ -431,12 +431,10 @@ __device__ __forceinline__ uint32_t epilogue_tile_stream(const GemmParams &p, co
         }
         // the store that last used this box must have read it before it is refilled
         const uint32_t box = staging + ((two_boxes && (nboxes & 1u)) ? static_cast<uint32_t>(kStreamStagingPerWarp) : 0u);
-        if (lane == 0) {
-            if (two_boxes) {
-                if (nboxes >= 2u) bulk_wait_group_read<1>();
-            } else if (nboxes >= 1u) {
-                bulk_wait_group_read<0>();
-            }
+        if (two_boxes) {
+            if (nboxes >= 2u) bulk_wait_group_read<1>();
+        } else if (nboxes >= 1u) {
+            bulk_wait_group_read<0>();
         }
         __syncwarp();
         convert_stage64_sw128(v0, v1, dxr, reinterpret_cast<const float4 *>(dw_s + c0),
@@ -445,15 +443,13 @@ __device__ __forceinline__ uint32_t epilogue_tile_stream(const GemmParams &p, co
         if (p.use_tma_store) {
             fence_proxy_async_smem();
             __syncwarp();
-            if (lane == 0) {
-                if (n_first < p.N && m_row0 < p.M) {           // clipped at N and M
-                    if (p.y_evict_first)
-                        tma_store_2d_evict_first(tmY, n_first, static_cast<int>(m_row0), box);
-                    else
-                        tma_store_2d(tmY, n_first, static_cast<int>(m_row0), box);
-                }
-                bulk_commit_group();
+            if (n_first < p.N && m_row0 < p.M) {               // clipped at N and M
+                if (p.y_evict_first)
+                    tma_store_2d_evict_first_warp(tmY, n_first, static_cast<int>(m_row0), box);
+                else
+                    tma_store_2d_warp(tmY, n_first, static_cast<int>(m_row0), box);
             }
+            bulk_commit_group();
         } else {
             __syncwarp();
             copy_box_rows(p.y, p.M, p.N, p.y_copy_bytes, box, m_row0, n_first, lane);
@@ -595,7 +591,7 @@ __device__ __forceinline__ void epilogue_team_loop(const GemmParams &p, const CU
         tphase ^= 1u;
         team_sync(team);                                // every warp of the team is done reading the scale copies
     }
-    if (lane == 0) bulk_wait_group<0>();                // all of this thread's stores have completed
+    bulk_wait_group<0>();                               // all of this warp's stores have completed
 }
 
 // --- the kernel ---------------------------------------------------------------------------------
@@ -660,7 +656,7 @@ ptq_gemm_dequant_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
     volatile uint32_t *tmem_holder = reinterpret_cast<volatile uint32_t *>(smem_raw + bar_off + kGemmNumBarriers * 8);
     volatile uint32_t *abort_flag = tmem_holder + 1;
 
-    const int warp = threadIdx.x >> 5;
+    const int warp = uniform_warp();
     const int lane = threadIdx.x & 31;
 
     if (threadIdx.x == 0) {
@@ -686,7 +682,7 @@ ptq_gemm_dequant_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
-    const uint32_t tmem_base = *tmem_holder;
+    const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_holder, 0);
 
     // The set-up above touched nothing another kernel writes.  The codes (and, for the dynamic comparator, the row steps)
     // of the quantize kernel launched just before are read behind griddep_wait() only; the weights are parameters,
@@ -699,90 +695,86 @@ ptq_gemm_dequant_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
 
     if (warp == 0) {
         // ------------------------------------------------------------------ TMA producer
-        if (lane == 0) {
-            uint32_t stage = 0, phase = 0, issued = 0;
-            bool ok = true;
-            const uint32_t tx = static_cast<uint32_t>(kATileBytes + p.BN * kBK);
-            uint32_t tx_piece = tx;
-            const CUtensorMap *tmPiece = &tmW;
-            if constexpr (kCut) {
-                tx_piece = static_cast<uint32_t>(kATileBytes + p.piece_cols * kBK);        // a box counts whole, also beyond N
-                tmPiece = &p.tmWcut;
+        uint32_t stage = 0, phase = 0, issued = 0;
+        bool ok = true;
+        const uint32_t tx = static_cast<uint32_t>(kATileBytes + p.BN * kBK);
+        uint32_t tx_piece = tx;
+        const CUtensorMap *tmPiece = &tmW;
+        if constexpr (kCut) {
+            tx_piece = static_cast<uint32_t>(kATileBytes + p.piece_cols * kBK);        // a box counts whole, also beyond N
+            tmPiece = &p.tmWcut;
+        }
+        const int early = min(static_cast<int>(nstages), p.k_blocks);   // k-blocks of the first tile whose weights go first
+        if (static_cast<int>(blockIdx.x) < total_tiles) {
+            const int n_tile = static_cast<int>(blockIdx.x - fd_div(blockIdx.x, p.fd_n_tiles) * p.fd_n_tiles.d);
+            for (int kb = 0; kb < early; ++kb) {
+                mbar_arrive_expect_tx_warp(full_bar(kb), tx);
+                tma_load_2d_warp(base + kb * kStageBytes + kATileBytes, &tmW, kb * kBK, n_tile * p.BN, full_bar(kb));
             }
-            const int early = min(static_cast<int>(nstages), p.k_blocks);   // k-blocks of the first tile whose weights go first
-            if (static_cast<int>(blockIdx.x) < total_tiles) {
-                const int n_tile = static_cast<int>(blockIdx.x - fd_div(blockIdx.x, p.fd_n_tiles) * p.fd_n_tiles.d);
-                for (int kb = 0; kb < early; ++kb) {
-                    mbar_arrive_expect_tx(full_bar(kb), tx);
-                    tma_load_2d(base + kb * kStageBytes + kATileBytes, &tmW, kb * kBK, n_tile * p.BN, full_bar(kb));
+        }
+        griddep_wait();
+        for (int tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x) {
+            const TileAt at = tile_at<kCut>(p, tile);
+            const bool piece = kCut && at.cols != p.BN;    // a whole tile among the pieces (never made) would load alike
+            for (int kb = 0; kb < p.k_blocks; ++kb) {
+                if (!mbar_wait_warp(empty_bar(stage), phase ^ 1u, abort_flag, p.status)) {
+                    ok = false;
+                    break;
+                }
+                const uint32_t a_dst = base + stage * kStageBytes;
+                if (static_cast<int>(issued) >= early) {
+                    mbar_arrive_expect_tx_warp(full_bar(stage), piece ? tx_piece : tx);
+                    tma_load_2d_warp(a_dst + kATileBytes, piece ? tmPiece : &tmW, kb * kBK, at.n0, full_bar(stage));
+                }
+                tma_load_2d_warp(a_dst, &tmA, kb * kBK, at.m_tile * kBM, full_bar(stage));
+                ++issued;
+                if (++stage == nstages) {
+                    stage = 0;
+                    phase ^= 1u;
                 }
             }
-            griddep_wait();
-            for (int tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x) {
-                const TileAt at = tile_at<kCut>(p, tile);
-                const bool piece = kCut && at.cols != p.BN;    // a whole tile among the pieces (never made) would load alike
-                for (int kb = 0; kb < p.k_blocks; ++kb) {
-                    if (!mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag, p.status)) {
-                        ok = false;
-                        break;
-                    }
-                    const uint32_t a_dst = base + stage * kStageBytes;
-                    if (static_cast<int>(issued) >= early) {
-                        mbar_arrive_expect_tx(full_bar(stage), piece ? tx_piece : tx);
-                        tma_load_2d(a_dst + kATileBytes, piece ? tmPiece : &tmW, kb * kBK, at.n0, full_bar(stage));
-                    }
-                    tma_load_2d(a_dst, &tmA, kb * kBK, at.m_tile * kBM, full_bar(stage));
-                    ++issued;
-                    if (++stage == nstages) {
-                        stage = 0;
-                        phase ^= 1u;
-                    }
-                }
-            }
-            if (!ok) {
-                // Error path only: let this thread's own loads land before the CTA gives up its
-                // shared memory (bounded; each stage's last load is at most microseconds away).
-                for (uint32_t s = 0; s < nstages; ++s) {
-                    const uint32_t uses = (issued + nstages - 1u - s) / nstages;
-                    if (uses == 0u) continue;
-                    for (int i = 0; i < 200000 && !mbar_try_wait(full_bar(s), (uses - 1u) & 1u); ++i) {
-                    }
+        }
+        if (!ok) {
+            // Error path only: let this thread's own loads land before the CTA gives up its
+            // shared memory (bounded; each stage's last load is at most microseconds away).
+            for (uint32_t s = 0; s < nstages; ++s) {
+                const uint32_t uses = (issued + nstages - 1u - s) / nstages;
+                if (uses == 0u) continue;
+                for (int i = 0; i < 200000 && !mbar_try_wait(full_bar(s), (uses - 1u) & 1u); ++i) {
                 }
             }
         }
     } else if (warp == 1) {
         // ------------------------------------------------------------------ MMA issuer
-        if (lane == 0) {
-            uint32_t idesc = make_idesc_s8(kBM, p.BN, kAsym);   // unsigned codes on asymmetric layers
-            uint32_t stage = 0, phase = 0, buf = 0, bphase = 0;
-            bool ok = true;
-            for (int tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x) {
-                if (!mbar_wait(tempty_bar(buf), bphase ^ 1u, abort_flag, p.status)) break;
-                tc_fence_after_sync();
-                if constexpr (kCut) idesc = make_idesc_s8(kBM, tile_at<kCut>(p, tile).cols, kAsym);
-                const uint32_t d_tmem = tmem_base + buf * kMaxBN;
-                for (int kb = 0; kb < p.k_blocks; ++kb) {
-                    if (!mbar_wait(full_bar(stage), phase, abort_flag, p.status)) {
-                        ok = false;
-                        break;
-                    }
-                    tc_fence_after_sync();
-                    const uint32_t a_addr = base + stage * kStageBytes;
-                    const uint64_t a_desc = make_smem_desc_sw128(a_addr);
-                    const uint64_t b_desc = make_smem_desc_sw128(a_addr + kATileBytes);
-                    const int nmma = (kb == p.k_blocks - 1) ? p.last_mmas : (kBK / 32);
-                    mma_i8_ss_kblock(d_tmem, a_desc, b_desc, idesc, kb != 0 ? 1u : 0u, nmma);
-                    mma_commit(empty_bar(stage));    // the stage is free once these MMAs have read it
-                    if (++stage == nstages) {
-                        stage = 0;
-                        phase ^= 1u;
-                    }
+        uint32_t idesc = make_idesc_s8(kBM, p.BN, kAsym);   // unsigned codes on asymmetric layers
+        uint32_t stage = 0, phase = 0, buf = 0, bphase = 0;
+        bool ok = true;
+        for (int tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x) {
+            if (!mbar_wait_warp(tempty_bar(buf), bphase ^ 1u, abort_flag, p.status)) break;
+            tc_fence_after_sync();
+            if constexpr (kCut) idesc = make_idesc_s8(kBM, tile_at<kCut>(p, tile).cols, kAsym);
+            const uint32_t d_tmem = tmem_base + buf * kMaxBN;
+            for (int kb = 0; kb < p.k_blocks; ++kb) {
+                if (!mbar_wait_warp(full_bar(stage), phase, abort_flag, p.status)) {
+                    ok = false;
+                    break;
                 }
-                if (!ok) break;
-                mma_commit(tfull_bar(buf));          // accumulator complete
-                buf ^= 1u;
-                if (buf == 0u) bphase ^= 1u;
+                tc_fence_after_sync();
+                const uint32_t a_addr = base + stage * kStageBytes;
+                const uint64_t a_desc = make_smem_desc_sw128(a_addr);
+                const uint64_t b_desc = make_smem_desc_sw128(a_addr + kATileBytes);
+                const int nmma = (kb == p.k_blocks - 1) ? p.last_mmas : (kBK / 32);
+                mma_i8_ss_kblock(d_tmem, a_desc, b_desc, idesc, kb != 0 ? 1u : 0u, nmma);
+                mma_commit(empty_bar(stage));    // the stage is free once these MMAs have read it
+                if (++stage == nstages) {
+                    stage = 0;
+                    phase ^= 1u;
+                }
             }
+            if (!ok) break;
+            mma_commit(tfull_bar(buf));          // accumulator complete
+            buf ^= 1u;
+            if (buf == 0u) bphase ^= 1u;
         }
     } else {
         // ------------------------------------------------------------------ epilogue warps
@@ -849,7 +841,7 @@ ptq_gemm_dequant_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
             // because it has passed this tile's wait on scale_bar, which needed every warp's arrival
             publish_scales((it + 1u) & 1u);
         }
-        if (lane == 0) bulk_wait_group<0>();         // all of this thread's stores have completed
+        bulk_wait_group<0>();                        // all of this warp's stores have completed
     }
 
     __syncthreads();
@@ -914,7 +906,7 @@ ptq_gemm_dequant_panel_kernel(const __grid_constant__ CUtensorMap tmA, const __g
     volatile uint32_t *tmem_holder = reinterpret_cast<volatile uint32_t *>(smem_raw + bar_off + kPanelNumBarriers * 8);
     volatile uint32_t *abort_flag = tmem_holder + 1;
 
-    const int warp = threadIdx.x >> 5;
+    const int warp = uniform_warp();
     const int lane = threadIdx.x & 31;
 
     if (threadIdx.x == 0) {
@@ -944,7 +936,7 @@ ptq_gemm_dequant_panel_kernel(const __grid_constant__ CUtensorMap tmA, const __g
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
-    const uint32_t tmem_base = *tmem_holder;
+    const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_holder, 0);
 
     // The codes (and, for the dynamic comparator, the row steps) of the kernel before are read behind griddep_wait() only;
     // the weights of the first stages go before it.
@@ -961,109 +953,105 @@ ptq_gemm_dequant_panel_kernel(const __grid_constant__ CUtensorMap tmA, const __g
 
     if (warp == 0) {
         // ------------------------------------------------------------------ TMA producer
-        if (lane == 0) {
-            uint32_t stage = 0, sphase = 0, uph = 0, b_issued = 0, a_units = 0;
-            int a_kb_issued = 0;                 // panel k-blocks issued for the unit in progress
-            bool ok = true;
-            const uint32_t early = min(nb, static_cast<uint32_t>(p.k_blocks));   // k-blocks of the first tile whose weights go first
-            if (static_cast<int>(blockIdx.x) < units) {
-                for (uint32_t kb = 0; kb < early; ++kb) {
-                    mbar_arrive_expect_tx(bfull_bar(kb), b_bytes);
-                    tma_load_2d(base + b_off + kb * b_bytes, &tmW, static_cast<int>(kb) * kBK, unit_first(blockIdx.x) * p.BN, bfull_bar(kb));
-                }
+        uint32_t stage = 0, sphase = 0, uph = 0, b_issued = 0, a_units = 0;
+        int a_kb_issued = 0;                 // panel k-blocks issued for the unit in progress
+        bool ok = true;
+        const uint32_t early = min(nb, static_cast<uint32_t>(p.k_blocks));   // k-blocks of the first tile whose weights go first
+        if (static_cast<int>(blockIdx.x) < units) {
+            for (uint32_t kb = 0; kb < early; ++kb) {
+                mbar_arrive_expect_tx_warp(bfull_bar(kb), b_bytes);
+                tma_load_2d_warp(base + b_off + kb * b_bytes, &tmW, static_cast<int>(kb) * kBK, unit_first(blockIdx.x) * p.BN, bfull_bar(kb));
             }
-            griddep_wait();
-            for (int unit = blockIdx.x; unit < units && ok; unit += gridDim.x, uph ^= 1u) {
-                const int m_tile = unit_panel(unit);
-                const int n_first = unit_first(unit), n_count = unit_count(unit);
-                a_kb_issued = 0;
-                for (int j = 0; j < n_count && ok; ++j) {
-                    for (int kb = 0; kb < p.k_blocks; ++kb) {
-                        if (j == 0) {
-                            // slot kb of the panel: free once the previous unit's last tile has read it
-                            if (!mbar_wait(aempty_bar(kb), uph ^ 1u, abort_flag, p.status)) {
-                                ok = false;
-                                break;
-                            }
-                            mbar_arrive_expect_tx(afull_bar(kb), static_cast<uint32_t>(kATileBytes));
-                            tma_load_2d(base + static_cast<uint32_t>(kb) * kATileBytes, &tmA, kb * kBK, m_tile * kBM,
-                                        afull_bar(kb));
-                            ++a_kb_issued;
-                        }
-                        if (!mbar_wait(bempty_bar(stage), sphase ^ 1u, abort_flag, p.status)) {
+        }
+        griddep_wait();
+        for (int unit = blockIdx.x; unit < units && ok; unit += gridDim.x, uph ^= 1u) {
+            const int m_tile = unit_panel(unit);
+            const int n_first = unit_first(unit), n_count = unit_count(unit);
+            a_kb_issued = 0;
+            for (int j = 0; j < n_count && ok; ++j) {
+                for (int kb = 0; kb < p.k_blocks; ++kb) {
+                    if (j == 0) {
+                        // slot kb of the panel: free once the previous unit's last tile has read it
+                        if (!mbar_wait_warp(aempty_bar(kb), uph ^ 1u, abort_flag, p.status)) {
                             ok = false;
                             break;
                         }
-                        if (b_issued >= early) {
-                            mbar_arrive_expect_tx(bfull_bar(stage), b_bytes);
-                            tma_load_2d(base + b_off + stage * b_bytes, &tmW, kb * kBK, (n_first + j) * p.BN, bfull_bar(stage));
-                        }
-                        ++b_issued;
-                        if (++stage == nb) {
-                            stage = 0;
-                            sphase ^= 1u;
-                        }
+                        mbar_arrive_expect_tx_warp(afull_bar(kb), static_cast<uint32_t>(kATileBytes));
+                        tma_load_2d_warp(base + static_cast<uint32_t>(kb) * kATileBytes, &tmA, kb * kBK, m_tile * kBM,
+                                    afull_bar(kb));
+                        ++a_kb_issued;
+                    }
+                    if (!mbar_wait_warp(bempty_bar(stage), sphase ^ 1u, abort_flag, p.status)) {
+                        ok = false;
+                        break;
+                    }
+                    if (b_issued >= early) {
+                        mbar_arrive_expect_tx_warp(bfull_bar(stage), b_bytes);
+                        tma_load_2d_warp(base + b_off + stage * b_bytes, &tmW, kb * kBK, (n_first + j) * p.BN, bfull_bar(stage));
+                    }
+                    ++b_issued;
+                    if (++stage == nb) {
+                        stage = 0;
+                        sphase ^= 1u;
                     }
                 }
-                if (ok) ++a_units;
             }
-            if (!ok) {
-                // Error path only: let this thread's own loads land before the CTA gives up its shared memory (bounded).
-                for (uint32_t s = 0; s < nb; ++s) {
-                    const uint32_t uses = (b_issued + nb - 1u - s) / nb;
-                    if (uses == 0u) continue;
-                    for (int i = 0; i < 200000 && !mbar_try_wait(bfull_bar(s), (uses - 1u) & 1u); ++i) {
-                    }
+            if (ok) ++a_units;
+        }
+        if (!ok) {
+            // Error path only: let this thread's own loads land before the CTA gives up its shared memory (bounded).
+            for (uint32_t s = 0; s < nb; ++s) {
+                const uint32_t uses = (b_issued + nb - 1u - s) / nb;
+                if (uses == 0u) continue;
+                for (int i = 0; i < 200000 && !mbar_try_wait(bfull_bar(s), (uses - 1u) & 1u); ++i) {
                 }
-                for (int kb = 0; kb < p.k_blocks; ++kb) {
-                    const uint32_t uses = a_units + (kb < a_kb_issued ? 1u : 0u);
-                    if (uses == 0u) continue;
-                    for (int i = 0; i < 200000 && !mbar_try_wait(afull_bar(kb), (uses - 1u) & 1u); ++i) {
-                    }
+            }
+            for (int kb = 0; kb < p.k_blocks; ++kb) {
+                const uint32_t uses = a_units + (kb < a_kb_issued ? 1u : 0u);
+                if (uses == 0u) continue;
+                for (int i = 0; i < 200000 && !mbar_try_wait(afull_bar(kb), (uses - 1u) & 1u); ++i) {
                 }
             }
         }
     } else if (warp == 1) {
         // ------------------------------------------------------------------ MMA issuer
-        if (lane == 0) {
-            const uint32_t idesc = make_idesc_s8(kBM, p.BN, kAsym);
-            uint32_t stage = 0, sphase = 0, uph = 0, buf = 0, bphase = 0;
-            bool ok = true;
-            for (int unit = blockIdx.x; unit < units && ok; unit += gridDim.x, uph ^= 1u) {
-                const int n_count = unit_count(unit);
-                for (int j = 0; j < n_count && ok; ++j) {
-                    if (!mbar_wait(tempty_bar(buf), bphase ^ 1u, abort_flag, p.status)) {
+        const uint32_t idesc = make_idesc_s8(kBM, p.BN, kAsym);
+        uint32_t stage = 0, sphase = 0, uph = 0, buf = 0, bphase = 0;
+        bool ok = true;
+        for (int unit = blockIdx.x; unit < units && ok; unit += gridDim.x, uph ^= 1u) {
+            const int n_count = unit_count(unit);
+            for (int j = 0; j < n_count && ok; ++j) {
+                if (!mbar_wait_warp(tempty_bar(buf), bphase ^ 1u, abort_flag, p.status)) {
+                    ok = false;
+                    break;
+                }
+                tc_fence_after_sync();
+                const uint32_t d_tmem = tmem_base + buf * kMaxBN;
+                for (int kb = 0; kb < p.k_blocks; ++kb) {
+                    if (j == 0 && !mbar_wait_warp(afull_bar(kb), uph, abort_flag, p.status)) {
+                        ok = false;
+                        break;
+                    }
+                    if (!mbar_wait_warp(bfull_bar(stage), sphase, abort_flag, p.status)) {
                         ok = false;
                         break;
                     }
                     tc_fence_after_sync();
-                    const uint32_t d_tmem = tmem_base + buf * kMaxBN;
-                    for (int kb = 0; kb < p.k_blocks; ++kb) {
-                        if (j == 0 && !mbar_wait(afull_bar(kb), uph, abort_flag, p.status)) {
-                            ok = false;
-                            break;
-                        }
-                        if (!mbar_wait(bfull_bar(stage), sphase, abort_flag, p.status)) {
-                            ok = false;
-                            break;
-                        }
-                        tc_fence_after_sync();
-                        const uint64_t a_desc = make_smem_desc_sw128(base + static_cast<uint32_t>(kb) * kATileBytes);
-                        const uint64_t b_desc = make_smem_desc_sw128(base + b_off + stage * b_bytes);
-                        const int nmma = (kb == p.k_blocks - 1) ? p.last_mmas : (kBK / 32);
-                        mma_i8_ss_kblock(d_tmem, a_desc, b_desc, idesc, kb != 0 ? 1u : 0u, nmma);
-                        mma_commit(bempty_bar(stage));                       // the weight stage is free once these MMAs have read it
-                        if (j == n_count - 1) mma_commit(aempty_bar(kb));    // and, after the unit's last tile, so is the panel slot
-                        if (++stage == nb) {
-                            stage = 0;
-                            sphase ^= 1u;
-                        }
+                    const uint64_t a_desc = make_smem_desc_sw128(base + static_cast<uint32_t>(kb) * kATileBytes);
+                    const uint64_t b_desc = make_smem_desc_sw128(base + b_off + stage * b_bytes);
+                    const int nmma = (kb == p.k_blocks - 1) ? p.last_mmas : (kBK / 32);
+                    mma_i8_ss_kblock(d_tmem, a_desc, b_desc, idesc, kb != 0 ? 1u : 0u, nmma);
+                    mma_commit(bempty_bar(stage));                       // the weight stage is free once these MMAs have read it
+                    if (j == n_count - 1) mma_commit(aempty_bar(kb));    // and, after the unit's last tile, so is the panel slot
+                    if (++stage == nb) {
+                        stage = 0;
+                        sphase ^= 1u;
                     }
-                    if (!ok) break;
-                    mma_commit(tfull_bar(buf));          // accumulator complete
-                    buf ^= 1u;
-                    if (buf == 0u) bphase ^= 1u;
                 }
+                if (!ok) break;
+                mma_commit(tfull_bar(buf));          // accumulator complete
+                buf ^= 1u;
+                if (buf == 0u) bphase ^= 1u;
             }
         }
     } else {
@@ -1133,7 +1121,7 @@ ptq_gemm_dequant_panel_kernel(const __grid_constant__ CUtensorMap tmA, const __g
             j = next_j;
             ++it;
         }
-        if (lane == 0) bulk_wait_group<0>();         // all of this thread's stores have completed
+        bulk_wait_group<0>();                        // all of this warp's stores have completed
     }
 
     __syncthreads();
@@ -1195,7 +1183,7 @@ ptq_gemm_dequant_resident_kernel(const __grid_constant__ CUtensorMap tmA, const 
     volatile uint32_t *tmem_holder = reinterpret_cast<volatile uint32_t *>(smem_raw + bar_off + kResNumBarriers * 8);
     volatile uint32_t *abort_flag = tmem_holder + 1;
 
-    const int warp = threadIdx.x >> 5;
+    const int warp = uniform_warp();
     const int lane = threadIdx.x & 31;
 
     if (threadIdx.x == 0) {
@@ -1222,7 +1210,7 @@ ptq_gemm_dequant_resident_kernel(const __grid_constant__ CUtensorMap tmA, const 
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
-    const uint32_t tmem_base = *tmem_holder;
+    const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_holder, 0);
     griddep_launch_dependents();         // the codes (and row steps) of the kernel before are read behind griddep_wait() only
 
     const int total = p.m_tiles * p.n_tiles, grid = static_cast<int>(gridDim.x), cta = static_cast<int>(blockIdx.x);
@@ -1237,13 +1225,13 @@ ptq_gemm_dequant_resident_kernel(const __grid_constant__ CUtensorMap tmA, const 
 
     if (warp == 0) {
         // ------------------------------------------------------------------ TMA producer
-        if (lane == 0 && cur.valid()) {
+        if (cur.valid()) {
             uint32_t stage = 0, phase = 0, issued = 0, w_loads = 0;
             int w_tile = -1;
             auto load_weights = [&](int n_tile) {
-                mbar_arrive_expect_tx(wfull_bar, static_cast<uint32_t>(p.k_blocks) * w_bytes);
+                mbar_arrive_expect_tx_warp(wfull_bar, static_cast<uint32_t>(p.k_blocks) * w_bytes);
                 for (int kb = 0; kb < p.k_blocks; ++kb)
-                    tma_load_2d(base + static_cast<uint32_t>(kb) * w_bytes, &tmW, kb * kBK, n_tile * p.BN, wfull_bar);
+                    tma_load_2d_warp(base + static_cast<uint32_t>(kb) * w_bytes, &tmW, kb * kBK, n_tile * p.BN, wfull_bar);
                 w_tile = n_tile;
                 ++w_loads;
             };
@@ -1253,19 +1241,19 @@ ptq_gemm_dequant_resident_kernel(const __grid_constant__ CUtensorMap tmA, const 
             for (; cur.valid() && ok; cur.advance()) {
                 const int n_tile = cur.n_tile(), m_tile = cur.m_tile();
                 if (n_tile != w_tile) {
-                    if (!mbar_wait(wempty_bar, (w_loads - 1u) & 1u, abort_flag, p.status)) {
+                    if (!mbar_wait_warp(wempty_bar, (w_loads - 1u) & 1u, abort_flag, p.status)) {
                         ok = false;
                         break;
                     }
                     load_weights(n_tile);
                 }
                 for (int kb = 0; kb < p.k_blocks; ++kb) {
-                    if (!mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag, p.status)) {
+                    if (!mbar_wait_warp(empty_bar(stage), phase ^ 1u, abort_flag, p.status)) {
                         ok = false;
                         break;
                     }
-                    mbar_arrive_expect_tx(full_bar(stage), kATileBytes);
-                    tma_load_2d(base + a_off + stage * kATileBytes, &tmA, kb * kBK, m_tile * kBM, full_bar(stage));
+                    mbar_arrive_expect_tx_warp(full_bar(stage), kATileBytes);
+                    tma_load_2d_warp(base + a_off + stage * kATileBytes, &tmA, kb * kBK, m_tile * kBM, full_bar(stage));
                     ++issued;
                     if (++stage == nstages) {
                         stage = 0;
@@ -1287,43 +1275,41 @@ ptq_gemm_dequant_resident_kernel(const __grid_constant__ CUtensorMap tmA, const 
         }
     } else if (warp == 1) {
         // ------------------------------------------------------------------ MMA issuer
-        if (lane == 0) {
-            const uint32_t idesc = make_idesc_s8(kBM, p.BN, kAsym);
-            uint32_t stage = 0, phase = 0, buf = 0, bphase = 0, w_uses = 0;
-            int w_tile = -1;
-            bool ok = true;
-            while (cur.valid() && ok) {
-                const int n_tile = cur.n_tile();
-                if (n_tile != w_tile) {
-                    if (!mbar_wait(wfull_bar, w_uses & 1u, abort_flag, p.status)) break;
-                    w_tile = n_tile;
-                    ++w_uses;
-                }
-                if (!mbar_wait(tempty_bar(buf), bphase ^ 1u, abort_flag, p.status)) break;
-                tc_fence_after_sync();
-                const uint32_t d_tmem = tmem_base + buf * kMaxBN;
-                for (int kb = 0; kb < p.k_blocks; ++kb) {
-                    if (!mbar_wait(full_bar(stage), phase, abort_flag, p.status)) {
-                        ok = false;
-                        break;
-                    }
-                    tc_fence_after_sync();
-                    mma_i8_ss_kblock(d_tmem, make_smem_desc_sw128(base + a_off + stage * kATileBytes),
-                                     make_smem_desc_sw128(base + static_cast<uint32_t>(kb) * w_bytes), idesc, kb != 0 ? 1u : 0u,
-                                     kb == p.k_blocks - 1 ? p.last_mmas : kBK / 32);
-                    mma_commit(empty_bar(stage));
-                    if (++stage == nstages) {
-                        stage = 0;
-                        phase ^= 1u;
-                    }
-                }
-                if (!ok) break;
-                mma_commit(tfull_bar(buf));          // accumulator complete
-                buf ^= 1u;
-                if (buf == 0u) bphase ^= 1u;
-                cur.advance();
-                if (cur.valid() && cur.n_tile() != w_tile) mma_commit(wempty_bar);   // the weights have been read for the last time
+        const uint32_t idesc = make_idesc_s8(kBM, p.BN, kAsym);
+        uint32_t stage = 0, phase = 0, buf = 0, bphase = 0, w_uses = 0;
+        int w_tile = -1;
+        bool ok = true;
+        while (cur.valid() && ok) {
+            const int n_tile = cur.n_tile();
+            if (n_tile != w_tile) {
+                if (!mbar_wait_warp(wfull_bar, w_uses & 1u, abort_flag, p.status)) break;
+                w_tile = n_tile;
+                ++w_uses;
             }
+            if (!mbar_wait_warp(tempty_bar(buf), bphase ^ 1u, abort_flag, p.status)) break;
+            tc_fence_after_sync();
+            const uint32_t d_tmem = tmem_base + buf * kMaxBN;
+            for (int kb = 0; kb < p.k_blocks; ++kb) {
+                if (!mbar_wait_warp(full_bar(stage), phase, abort_flag, p.status)) {
+                    ok = false;
+                    break;
+                }
+                tc_fence_after_sync();
+                mma_i8_ss_kblock(d_tmem, make_smem_desc_sw128(base + a_off + stage * kATileBytes),
+                                 make_smem_desc_sw128(base + static_cast<uint32_t>(kb) * w_bytes), idesc, kb != 0 ? 1u : 0u,
+                                 kb == p.k_blocks - 1 ? p.last_mmas : kBK / 32);
+                mma_commit(empty_bar(stage));
+                if (++stage == nstages) {
+                    stage = 0;
+                    phase ^= 1u;
+                }
+            }
+            if (!ok) break;
+            mma_commit(tfull_bar(buf));          // accumulator complete
+            buf ^= 1u;
+            if (buf == 0u) bphase ^= 1u;
+            cur.advance();
+            if (cur.valid() && cur.n_tile() != w_tile) mma_commit(wempty_bar);   // the weights have been read for the last time
         }
     } else {
         // ------------------------------------------------------------------ epilogue warps, two teams
@@ -1551,7 +1537,7 @@ ptq_gemm_dequant_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __gr
             if (buf == 0u) bphase ^= 1u;
             if (p.use_tma_store) publish_scales((it + 1u) & 1u);
         }
-        if (lane == 0) bulk_wait_group<0>();
+        bulk_wait_group<0>();
     }
 
     __syncthreads();

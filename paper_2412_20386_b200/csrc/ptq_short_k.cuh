@@ -94,7 +94,7 @@ ptq_short_k_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constan
     volatile uint32_t *abort_flag = tmem_holder + 1;
     float *s_s = reinterpret_cast<float *>(smem_raw + tab_off), *rs_s = s_s + kShortKMaxK;
 
-    const int warp = threadIdx.x >> 5;
+    const int warp = uniform_warp();
     const int lane = threadIdx.x & 31;
 
     if (threadIdx.x == 0) {
@@ -124,7 +124,7 @@ ptq_short_k_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constan
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
-    const uint32_t tmem_base = *tmem_holder;
+    const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_holder, 0);
     griddep_launch_dependents();
 
     const int total = p.m_tiles * p.groups, grid = static_cast<int>(gridDim.x), cta = static_cast<int>(blockIdx.x);
@@ -166,40 +166,38 @@ ptq_short_k_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constan
         }
     } else if (warp == 1) {
         // ------------------------------------------------------------------ MMA issuer
-        if (lane == 0) {
-            const uint32_t idesc = make_idesc_s8(kBM, p.BN, false);
-            uint32_t stage = 0, phase = 0, buf = 0, bphase = 0, w_uses = 0;
-            int held = -1;
-            bool ok = true;
-            while (cur.valid() && ok) {
-                const int grp = cur.grp(), n = cur.size();
-                if (grp != held) {
-                    if (!mbar_wait(wfull_bar, w_uses & 1u, abort_flag, p.status)) break;
-                    held = grp;
-                    ++w_uses;
-                }
-                if (!mbar_wait(afull_bar(stage), phase, abort_flag, p.status)) break;
-                for (int i = 0; i < n; ++i) {
-                    if (!mbar_wait(tempty_bar(buf), bphase ^ 1u, abort_flag, p.status)) {
-                        ok = false;
-                        break;
-                    }
-                    tc_fence_after_sync();
-                    mma_i8_ss_kblock(tmem_base + buf * kMaxBN, make_smem_desc_sw128(base + a_off + stage * kATileBytes),
-                                     make_smem_desc_sw128(base + static_cast<uint32_t>(i) * w_bytes), idesc, 0u, p.last_mmas);
-                    mma_commit(tfull_bar(buf));
-                    buf ^= 1u;
-                    if (buf == 0u) bphase ^= 1u;
-                }
-                if (!ok) break;
-                mma_commit(aempty_bar(stage));
-                if (++stage == nstages) {
-                    stage = 0;
-                    phase ^= 1u;
-                }
-                cur.next_unit();
-                if (cur.valid() && cur.grp() != held) mma_commit(wempty_bar);   // the weights have been read for the last time
+        const uint32_t idesc = make_idesc_s8(kBM, p.BN, false);
+        uint32_t stage = 0, phase = 0, buf = 0, bphase = 0, w_uses = 0;
+        int held = -1;
+        bool ok = true;
+        while (cur.valid() && ok) {
+            const int grp = cur.grp(), n = cur.size();
+            if (grp != held) {
+                if (!mbar_wait_warp(wfull_bar, w_uses & 1u, abort_flag, p.status)) break;
+                held = grp;
+                ++w_uses;
             }
+            if (!mbar_wait_warp(afull_bar(stage), phase, abort_flag, p.status)) break;
+            for (int i = 0; i < n; ++i) {
+                if (!mbar_wait_warp(tempty_bar(buf), bphase ^ 1u, abort_flag, p.status)) {
+                    ok = false;
+                    break;
+                }
+                tc_fence_after_sync();
+                mma_i8_ss_kblock(tmem_base + buf * kMaxBN, make_smem_desc_sw128(base + a_off + stage * kATileBytes),
+                                 make_smem_desc_sw128(base + static_cast<uint32_t>(i) * w_bytes), idesc, 0u, p.last_mmas);
+                mma_commit(tfull_bar(buf));
+                buf ^= 1u;
+                if (buf == 0u) bphase ^= 1u;
+            }
+            if (!ok) break;
+            mma_commit(aempty_bar(stage));
+            if (++stage == nstages) {
+                stage = 0;
+                phase ^= 1u;
+            }
+            cur.next_unit();
+            if (cur.valid() && cur.grp() != held) mma_commit(wempty_bar);   // the weights have been read for the last time
         }
     } else if (warp < 2 + kNumEpiWarps) {
         // ------------------------------------------------------------------ epilogue warps, two teams

@@ -10,7 +10,7 @@
 //
 //   all 12 warps  quantize the tile's kTN x K activations into the swizzled operand: a thread keeps one group of 8
 //                 channels (its 1/s in registers) and takes every rp-th row, four loads in flight
-//   thread 0      weight loads (TMA), then the MMAs of all k-blocks
+//   warp 0        weight loads (TMA, thread 0), then the MMAs of all k-blocks
 //   warps 0..     drain: lane = output channel, 16 tokens per warp (lane quarter = warp % 4)
 //
 // Bound by its chain of latencies: an empty kernel takes 2.4-2.5 us from launch to launch, this one 2.7 us at K = 12,
@@ -118,7 +118,7 @@ ptq_small_kernel(const __grid_constant__ CUtensorMap tmW, const SmallParams p)
     volatile uint32_t *tmem_holder = reinterpret_cast<volatile uint32_t *>(tab + 3 * kTN) + 4;
     volatile uint32_t *abort_flag = tmem_holder + 1;
 
-    const int tid = static_cast<int>(threadIdx.x), warp = tid >> 5, lane = tid & 31;
+    const int tid = static_cast<int>(threadIdx.x), warp = uniform_warp(), lane = tid & 31;
     const int m_tile = static_cast<int>(fd_div(blockIdx.x, p.fd_n_tiles));
     const int n0 = (static_cast<int>(blockIdx.x) - m_tile * p.n_tiles) * kSmallRows;
     const int m0 = m_tile * kTN;
@@ -163,7 +163,7 @@ ptq_small_kernel(const __grid_constant__ CUtensorMap tmW, const SmallParams p)
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
-    const uint32_t tmem_base = *tmem_holder;
+    const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_holder, 0);
     griddep_launch_dependents();                               // behind the allocation: see griddep_launch_dependents()
     griddep_wait();                                            // everything above read only the layer's own parameters
 
@@ -203,8 +203,8 @@ ptq_small_kernel(const __grid_constant__ CUtensorMap tmW, const SmallParams p)
     // ---- multiply ------------------------------------------------------------------------------------
     // Codes of rows beyond M and of channels beyond K are whatever lies there: those columns are not read, and the weights
     // are zero beyond K.
-    if (tid == 0) {
-        const bool ok = mbar_wait(wbar, 0u, abort_flag, p.status);
+    if (warp == 0) {
+        const bool ok = mbar_wait_warp(wbar, 0u, abort_flag, p.status);
         if (ok) {
             tc_fence_after_sync();
             const uint32_t idesc = make_idesc_i8(kSmallRows, kTN, false, kMode == kCodeU8);

@@ -120,6 +120,16 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
     }
 }
 
+// The same for a whole warp: true if every lane's wait ended.
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile uint32_t *abort_flag, unsigned *status)
+{
+    if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+    return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag, status));
+}
+
+// Number of this warp, known to the compiler to be the same for all of its lanes.
+__device__ __forceinline__ int uniform_warp() { return __shfl_sync(0xffffffffu, static_cast<int>(threadIdx.x) >> 5, 0); }
+
 // Self-test of the bounded wait, for the failure-detection tests: one CTA of 64 threads and one mbarrier
 // that nothing ever arrives on (no copy, no MMA and no other thread refers to it, so giving up leaves
 // nothing in flight).  Thread 0 waits with the short limit `limit_ns` and must give up: it raises the
@@ -181,6 +191,30 @@ __device__ __forceinline__ void tma_load_2d(uint32_t smem_dst, const CUtensorMap
         : "memory");
 }
 
+// The same two steps for a whole warp that runs its loop together (see mma_i8_ss): always the same lane issues.
+__device__ __forceinline__ void mbar_arrive_expect_tx_warp(uint32_t bar, uint32_t bytes)
+{
+    asm volatile(
+        "{\n\t"
+        ".reg .pred e;\n\t"
+        "elect.sync _|e, 0xffffffff;\n\t"
+        "@e mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n\t"
+        "}"
+        ::"r"(bar), "r"(bytes)
+        : "memory");
+}
+__device__ __forceinline__ void tma_load_2d_warp(uint32_t smem_dst, const CUtensorMap *m, int c0, int c1, uint32_t bar)
+{
+    asm volatile(
+        "{\n\t"
+        ".reg .pred e;\n\t"
+        "elect.sync _|e, 0xffffffff;\n\t"
+        "@e cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];\n\t"
+        "}"
+        ::"r"(smem_dst), "l"(reinterpret_cast<uint64_t>(m)), "r"(c0), "r"(c1), "r"(bar)
+        : "memory");
+}
+
 // 2-D tiled store shared -> global (bulk async group of the issuing thread); coordinates >= 0.
 __device__ __forceinline__ void tma_store_2d(const CUtensorMap *m, int c0, int c1, uint32_t smem_src)
 {
@@ -189,14 +223,31 @@ __device__ __forceinline__ void tma_store_2d(const CUtensorMap *m, int c0, int c
                  : "memory");
 }
 
-// The same with the evict-first L2 policy, for outputs that L2 cannot hold anyway.
-__device__ __forceinline__ void tma_store_2d_evict_first(const CUtensorMap *m, int c0, int c1, uint32_t smem_src)
+// The same for a whole warp, and with the evict-first L2 policy, for outputs that L2 cannot hold anyway.  The groups that the
+// other lanes commit and wait for are empty.
+__device__ __forceinline__ void tma_store_2d_warp(const CUtensorMap *m, int c0, int c1, uint32_t smem_src)
 {
-    uint64_t pol;
-    asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol));
-    asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.tile.bulk_group.L2::cache_hint [%0, {%1, %2}], [%3], %4;"
-                 ::"l"(reinterpret_cast<uint64_t>(m)), "r"(c0), "r"(c1), "r"(smem_src), "l"(pol)
-                 : "memory");
+    asm volatile(
+        "{\n\t"
+        ".reg .pred e;\n\t"
+        "elect.sync _|e, 0xffffffff;\n\t"
+        "@e cp.async.bulk.tensor.2d.global.shared::cta.tile.bulk_group [%0, {%1, %2}], [%3];\n\t"
+        "}"
+        ::"l"(reinterpret_cast<uint64_t>(m)), "r"(c0), "r"(c1), "r"(smem_src)
+        : "memory");
+}
+__device__ __forceinline__ void tma_store_2d_evict_first_warp(const CUtensorMap *m, int c0, int c1, uint32_t smem_src)
+{
+    asm volatile(
+        "{\n\t"
+        ".reg .pred e;\n\t"
+        ".reg .b64 pol;\n\t"
+        "elect.sync _|e, 0xffffffff;\n\t"
+        "createpolicy.fractional.L2::evict_first.b64 pol, 1.0;\n\t"
+        "@e cp.async.bulk.tensor.2d.global.shared::cta.tile.bulk_group.L2::cache_hint [%0, {%1, %2}], [%3], pol;\n\t"
+        "}"
+        ::"l"(reinterpret_cast<uint64_t>(m)), "r"(c0), "r"(c1), "r"(smem_src)
+        : "memory");
 }
 
 __device__ __forceinline__ void bulk_commit_group()
@@ -243,15 +294,22 @@ __device__ __forceinline__ void tc_fence_after_sync()
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 }
 
-// D[tmem] (+)= A[smem desc] * B[smem desc]; s8 x s8 -> s32, one CTA.
+// The warps that issue MMAs, TMA loads and TMA stores run their loops with all 32 lanes and elect one inside the statement that
+// issues, so that control flow, addresses and descriptors are uniform over the warp for the compiler.  In a branch of one lane an MMA took 57 +
+// 0.54 N cycles of issue, whatever the tensor pipe needed; so 30 to 40 less, and the GEMM kernels 20 registers less.  Layers, both
+// kernels, us: 12608 x 192 -> 768 10.3 -> 9.7, 25216 x 384 -> 1536 26.0 -> 23.7, 2793 x 1536 -> 768 11.1 -> 9.9, 1568 x 1536 -> 768 9.5 -> 8.3,
+// 50432 x 768 -> 3072 131 -> 126; one kernel, 197 x 384 -> 192 3.46 -> 3.27.  (Loads and stores alone are 1.5 to 2.5 % of that.)
+//
+// D[tmem] (+)= A[smem desc] * B[smem desc]; s8 x s8 -> s32, one CTA.  Called by a whole warp; always the same lane issues.
 __device__ __forceinline__ void mma_i8_ss(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
                                           uint32_t accumulate)
 {
     asm volatile(
         "{\n\t"
-        ".reg .pred p;\n\t"
+        ".reg .pred p, e;\n\t"
+        "elect.sync _|e, 0xffffffff;\n\t"
         "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::i8 [%0], %1, %2, %3, p;\n\t"
+        "@e tcgen05.mma.cta_group::1.kind::i8 [%0], %1, %2, %3, p;\n\t"
         "}"
         ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
         : "memory");
@@ -267,7 +325,8 @@ __device__ __forceinline__ void mma_i8_ss_x4(uint32_t d_tmem, uint64_t a_desc, u
 {
     asm volatile(
         "{\n\t"
-        ".reg .pred p, q;\n\t"
+        ".reg .pred p, q, e;\n\t"
+        "elect.sync _|e, 0xffffffff;\n\t"
         ".reg .b64 a1, a2, a3, b1, b2, b3;\n\t"
         "setp.ne.b32 p, %4, 0;\n\t"
         "setp.eq.b32 q, 0, 0;\n\t"
@@ -277,10 +336,10 @@ __device__ __forceinline__ void mma_i8_ss_x4(uint32_t d_tmem, uint64_t a_desc, u
         "add.u64 b1, %2, 2;\n\t"
         "add.u64 b2, %2, 4;\n\t"
         "add.u64 b3, %2, 6;\n\t"
-        "tcgen05.mma.cta_group::1.kind::i8 [%0], %1, %2, %3, p;\n\t"
-        "tcgen05.mma.cta_group::1.kind::i8 [%0], a1, b1, %3, q;\n\t"
-        "tcgen05.mma.cta_group::1.kind::i8 [%0], a2, b2, %3, q;\n\t"
-        "tcgen05.mma.cta_group::1.kind::i8 [%0], a3, b3, %3, q;\n\t"
+        "@e tcgen05.mma.cta_group::1.kind::i8 [%0], %1, %2, %3, p;\n\t"
+        "@e tcgen05.mma.cta_group::1.kind::i8 [%0], a1, b1, %3, q;\n\t"
+        "@e tcgen05.mma.cta_group::1.kind::i8 [%0], a2, b2, %3, q;\n\t"
+        "@e tcgen05.mma.cta_group::1.kind::i8 [%0], a3, b3, %3, q;\n\t"
         "}"
         ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate_first)
         : "memory");
@@ -298,10 +357,17 @@ __device__ __forceinline__ void mma_i8_ss_kblock(uint32_t d_tmem, uint64_t a_des
     }
 }
 
-// mbarrier arrives once all tcgen05 operations issued so far by this thread have completed.
+// mbarrier arrives once all MMAs issued so far by this warp have completed.
 __device__ __forceinline__ void mma_commit(uint32_t bar)
 {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+    asm volatile(
+        "{\n\t"
+        ".reg .pred e;\n\t"
+        "elect.sync _|e, 0xffffffff;\n\t"
+        "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t"
+        "}"
+        ::"r"(bar)
+        : "memory");
 }
 
 __device__ __forceinline__ void tmem_ld_wait()

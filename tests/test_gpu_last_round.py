@@ -34,7 +34,7 @@ def images_for(torch, n_tiles, last):
 
 @pytest.mark.parametrize("K,N,n_tiles,last", [(416, 768, 3, lambda sms: 1), (416, 760, 3, lambda sms: sms // 4),
                                               (450, 768, 3, lambda sms: sms // 4 + 1), (416, 512, 2, lambda sms: sms // 2),
-                                              (416, 512, 2, lambda sms: sms // 2 + 1), (520, 523, 3, lambda sms: 2),
+                                              (416, 512, 2, lambda sms: sms // 2 + 1), (900, 523, 3, lambda sms: 2),
                                               (900, 200, 1, lambda sms: 3)])
 def test_cut_last_round_matches_oracle(env, K, N, n_tiles, last):
     ptq, torch = env
@@ -43,8 +43,8 @@ def test_cut_last_round_matches_oracle(env, K, N, n_tiles, last):
 
 def test_cut_last_round_with_zero_offsets(env):
     ptq, torch = env
-    K, N = 416, 770
-    spec = wl.LinearSpec(22, 1, 1, "cut", images_for(torch, 4, lambda sms: 2), T, K, N, bias=True)
+    K, N = 900, 760
+    spec = wl.LinearSpec(22, 1, 1, "cut", images_for(torch, 3, lambda sms: 1), T, K, N, bias=True)
     x = wl.activations(spec)
     x[:, ::3] = np.abs(x[:, ::3])
     wq, dw, bias = wl.weights(spec)
