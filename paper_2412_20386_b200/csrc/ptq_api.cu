@@ -442,10 +442,10 @@ bool takes_resident(const ptq_linear *h, int m_tiles, int n_tiles)
     return h->k_blocks <= kShortMainLoop && static_cast<long long>(m_tiles) * n_tiles >= kResidentMinRounds * h->num_sms;
 }
 
-// Cycles of one tile of `cols` columns in the streaming kernel, as measured on the workloads: an MMA of K = 32 takes 57 + 0.54 cols;
-// the eight epilogue warps take 550 per tile and 700 per pair of 64-column steps.
-double mma_cycles(const ptq_linear *h, int cols) { return (h->K + 31) / 32 * (57.0 + 0.54 * cols); }
-double epilogue_cycles(int cols) { return 550.0 + 700.0 * (((cols + 63) / 64 + 1) / 2); }
+// Cycles of one tile of `cols` columns in the streaming kernel, as fitted to timings of 24 shapes at all widths: an MMA of K = 32
+// takes 35 + 0.52 cols; the eight epilogue warps take 360 per tile and 670 per pair of 64-column steps.
+double mma_cycles(const ptq_linear *h, int cols) { return (h->K + 31) / 32 * (35.0 + 0.52 * cols); }
+double epilogue_cycles(int cols) { return 360.0 + 670.0 * (((cols + 63) / 64 + 1) / 2); }
 
 // Columns per piece of the streaming kernel's last round with tiles of `bn` columns, 0 where it is not cut: at least one full
 // round before it, SMs enough for all pieces at once (narrow ones first), and a long main loop: the epilogue gains little by
@@ -461,31 +461,35 @@ int cut_cols(const ptq_linear *h, const ptq::GemmParams &p, int bn)
     return 0;
 }
 
-// Cycles of the busiest CTA of the streaming kernel with tiles of `bn` columns; the hand-overs take 300 per tile.
+// Cycles of the busiest CTA of the streaming kernel with tiles of `bn` columns; the hand-overs take 420 per tile.  Of what a cut
+// last round should save nine tenths are believed.
 double gemm_cycles(const ptq_linear *h, const ptq::GemmParams &p, int bn)
 {
     const long long tiles = static_cast<long long>(p.m_tiles) * ((h->N + bn - 1) / bn);
     const double rounds = static_cast<double>((tiles + h->num_sms - 1) / h->num_sms);
     auto longer = [](double a, double b) { return a > b ? a : b; };
-    const int cut = cut_cols(h, p, bn), last = cut ? cut : bn;                // columns of the last round's tiles
-    double cycles = mma_cycles(h, rounds > 1.0 ? bn : last) + epilogue_cycles(last) + 300.0 * rounds;
-    if (rounds > 1.0)
-        cycles += (rounds - 2.0) * longer(mma_cycles(h, bn), epilogue_cycles(bn)) + longer(mma_cycles(h, last), epilogue_cycles(bn));
-    return cycles;
+    auto busiest = [&](int last) {                                            // columns of the last round's tiles
+        if (rounds < 2.0) return mma_cycles(h, last) + epilogue_cycles(last) + 420.0;
+        return mma_cycles(h, bn) + (rounds - 2.0) * longer(mma_cycles(h, bn), epilogue_cycles(bn)) +
+               longer(mma_cycles(h, last), epilogue_cycles(bn)) + epilogue_cycles(last) + 420.0 * rounds;
+    };
+    const int cut = cut_cols(h, p, bn);
+    return cut ? 0.9 * busiest(cut) + 0.1 * busiest(bn) : busiest(bn);
 }
 
 // Tile width of the streaming kernel for this many rows: the layer's own (as few N tiles as possible), unless another
-// leaves the busiest CTA clearly less to do: idle SMs in a single round, or a last round that is nearly empty.  Layer,
-// both kernels, us: 1568 x 1536 -> 768 (256 -> 128 columns) 10.6 -> 9.7, 2793 x 1536 -> 768 (256 -> 192) 11.7 -> 10.8,
-// 12544 x 768 -> 384 (192 -> 128) 14.6 -> 14.1, 6304 x 384 -> 1536 (256 -> 192) 11.4 -> 11.0.  The margin keeps what the model cannot
-// tell apart: 11229 x 520 -> 600 (predicted -7 %) measured +1 %.  Widths that lead to the resident kernel are not
-// compared: with several rounds and a short main loop the widths are within 3 % of one another either way.
+// leaves the busiest CTA clearly less to do: idle SMs in a single round, or a last round that is nearly empty.  GEMM kernel alone,
+// us, own width -> the one chosen: 2793 x 1536 -> 768 (256 -> 128) 7.4 -> 5.3, 1568 x 1536 -> 768 (256 -> 128) 7.3 -> 4.9, 3152 x 768 -> 384 (192 -> 128)
+// 4.7 -> 3.8, 12544 x 768 -> 384 (192, cut -> 128) 6.6 -> 6.1, 11229 x 520 -> 600 (256 -> 128) 8.9 -> 8.6, 12608 x 192 -> 768 (256 -> 192) 6.6 -> 6.3.
+// The margin keeps what the model cannot tell apart: 25216 x 768 -> 384 (192 -> 128, predicted -1.6 %) 10.7 -> 10.9.  What it gets wrong: 6304 x 768 ->
+// 384 keeps 192 columns, 5.0, where 128 with a cut round take 4.5, and 6304 x 384 -> 192 takes 128, 3.4, where 64 take 3.1.  Widths that lead to the
+// resident kernel are not compared: with several rounds and a short main loop the widths are within 3 % of one another either way.
 int choose_bn(const ptq_linear *h, const ptq::GemmParams &p)
 {
     auto resident = [&](int bn) { return takes_resident(h, p.m_tiles, (h->N + bn - 1) / bn); };
     int best = h->BN;
     if (resident(best)) return best;
-    double best_cost = 0.93 * gemm_cycles(h, p, best);
+    double best_cost = 0.975 * gemm_cycles(h, p, best);
     for (int bn = 64; bn <= ptq::kMaxBN && bn < h->N + 64; bn += 64) {
         if (resident(bn)) continue;
         const double cost = gemm_cycles(h, p, bn);
