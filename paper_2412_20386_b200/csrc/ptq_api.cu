@@ -434,8 +434,10 @@ bool plan_panel(const ptq_linear *h, ptq::GemmParams &p, bool tma_store)
 }
 
 // Whether the kernel with resident weights (and its epilogue in two teams) is taken: short main loop (K <= 384) and three tiles
-// per CTA (and TMA stores).  With two the streaming kernel's shorter latency of a tile wins: 12608 x 192 -> 768 10.5 us against 11.1, 6304 x 384 ->
-// 1536 11.0 against 12.2, 25088 x 384 -> 384 14.3 against 14.7; with four and more this one does (figures at the kernel).
+// per CTA (and TMA stores).  GEMM kernel alone, us, streaming / resident.  Below three the streaming kernel's shorter latency of a tile wins
+// mostly: 25088 x 384 -> 192 (1.3 tiles per CTA) 5.3 / 5.4, 12608 x 192 -> 768 (2.0) 6.6 / 6.8, 6304 x 384 -> 1536 (2.0) 7.1 / 7.6; at 2.7 it
+// depends, 6304 x 384 -> 1536 in 192 columns 6.8 / 7.2, 50176 x 384 -> 192 8.7 / 8.4.  With four and more this one does: 12544 x 384 -> 1536 10.8 /
+// 10.4, 25088 x 192 -> 768 9.55 / 9.2, 25216 x 384 -> 1536 18.9 / 17.3.
 constexpr long long kResidentMinRounds = 3;
 bool takes_resident(const ptq_linear *h, int m_tiles, int n_tiles)
 {

@@ -160,13 +160,15 @@ __device__ __forceinline__ bool quantize8_screen(uint32_t x0, uint32_t x1, uint3
 // when the chunk has to go to the slower routes: a value within the tie band, a magnitude above
 // 127.25 (saturation is not handled here), or a NaN / infinity: the running magnitude maximum
 // propagates NaN, and an infinity exceeds the limit, so both fail the one comparison on `big`.
-template <int kMode = kCodeS8>
+// kBounded: the caller knows that no |v'| exceeds 127 and passes a bound of them as `big`; NaN is then caught in the maximum of
+// the tie distances, and the maximum of the magnitudes is saved.
+template <int kMode = kCodeS8, bool kBounded = false>
 __device__ __forceinline__ bool quantize8_magic(uint32_t x0, uint32_t x1, uint32_t x2, uint32_t x3,
-                                                const float (&c8)[8], uint32_t &lo, uint32_t &hi)
+                                                const float (&c8)[8], uint32_t &lo, uint32_t &hi, float big = 0.0f)
 {
     const uint32_t xw[4] = {x0, x1, x2, x3};
     uint32_t tb[8];
-    float worst = 0.0f, big = 0.0f;
+    float worst = 0.0f;
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
         const float2 f = __half22float2(*reinterpret_cast<const __half2 *>(&xw[i]));
@@ -174,14 +176,14 @@ __device__ __forceinline__ bool quantize8_magic(uint32_t x0, uint32_t x1, uint32
         const float2 t = __fadd2_rn(v, make_float2(kRoundMagic, kRoundMagic));
         const float2 r = __fadd2_rn(t, make_float2(-kRoundMagic, -kRoundMagic));
         const float2 d = __ffma2_rn(v, make_float2(-1.0f, -1.0f), r);      // rint(v) - v: exact, or NaN
-        worst = max3_abs(worst, d.x, d.y);
-        big = max3_abs_nan(big, v.x, v.y);
+        worst = kBounded ? max3_abs_nan(worst, d.x, d.y) : max3_abs(worst, d.x, d.y);
+        if (!kBounded) big = max3_abs_nan(big, v.x, v.y);
         tb[2 * i] = __float_as_uint(t.x);
         tb[2 * i + 1] = __float_as_uint(t.y);
     }
     lo = pack4(static_cast<int>(tb[0]), static_cast<int>(tb[1]), static_cast<int>(tb[2]), static_cast<int>(tb[3]));
     hi = pack4(static_cast<int>(tb[4]), static_cast<int>(tb[5]), static_cast<int>(tb[6]), static_cast<int>(tb[7]));
-    return !(clear_of_ties(worst, big) && big <= (kMode == kCodeS4 ? 7.25f : 127.25f));
+    return !(clear_of_ties(worst, big) && (kBounded || big <= (kMode == kCodeS4 ? 7.25f : 127.25f)));
 }
 
 // Exact route for the same 8 channels: two correctly rounded divisions per element.  s8 / rs8 point

@@ -190,7 +190,8 @@ __device__ __noinline__ float divided_max_call(uint4 v, const float4 *ra, const 
 // so only elements with a >= (1 - 2^-21) * max a can hold the maximum, and only those (one or two a row) are divided.
 // Each lane copies its part of the warp's next row into shared memory (cp.async) while it works on this one: in registers the
 // second row spilled and lost (6304 x 1536 -> 768: 25.4 us), without it that layer took 23.1 us and 50432 x 1536 -> 8 86.5.
-// Bound by issue (16 instructions an element at K = 1536, 20 at 768; 68 % of the issue slots taken) and, with few rows, by its chain of latencies: load,
+// The chunk maxima of the first pass scale the tie band of the second (50432 x 1536 -> 8 68.0 -> 66.9 us, 50432 x 768 -> 8 38.8 -> 38.2).
+// Bound by issue (15 to 20 instructions an element; 68 % of the issue slots taken) and, with few rows, by its chain of latencies: load,
 // two warp reductions, store.  Quantize + GEMM, against the two-pass kernel above: 6304 x 768 -> 3072 28.5 -> 24.4 us, 6304 x 1536 ->
 // 768 29.8 -> 21.2, 50432 x 768 -> 8 58.0 -> 39.4.
 constexpr int dyn_row_ctas_per_sm(int chunks) { return chunks <= 3 ? 4 : 3; }
@@ -282,7 +283,8 @@ __global__ void __launch_bounds__(256, dyn_row_ctas_per_sm(kChunks)) ptq_quantiz
                 const float2 c0 = __fmul2_rn(make_float2(ra.x, ra.y), rd2), c1 = __fmul2_rn(make_float2(ra.z, ra.w), rd2);
                 const float2 c2 = __fmul2_rn(make_float2(rb.x, rb.y), rd2), c3 = __fmul2_rn(make_float2(rb.z, rb.w), rd2);
                 const float c8[8] = {c0.x, c0.y, c1.x, c1.y, c2.x, c2.y, c3.x, c3.y};
-                exact = quantize8_magic<kCodeS8>(v[j].x, v[j].y, v[j].z, v[j].w, c8, out.x, out.y);   // |v'| <= 127: no saturation
+                // |v'| <= 127: no saturation; cm is within 2^-24 of the chunk's largest |x/s|, far inside the slack of the band's slope
+                exact = quantize8_magic<kCodeS8, true>(v[j].x, v[j].y, v[j].z, v[j].w, c8, out.x, out.y, __fmul_rn(cm[j], rdx));
             }
             if (exact) quantize8_exact<false, kCodeS8>(v[j].x, v[j].y, v[j].z, v[j].w, s_s + 8 * c, nullptr, dx, rdx, out.x, out.y);
             *reinterpret_cast<uint2 *>(qrow + 8 * c) = out;

@@ -4,7 +4,7 @@
 // release of the GEMM kernel behind it, about 2 us.  Here four warps of the GEMM CTA quantize, one row per thread: the work
 // unit is a row tile of 128 rows x a group of up to three N tiles, whose weights (at most 96 KB) stay in shared memory as in the
 // resident kernel.  A row tile is quantized once per group.  Bound by latency with one unit per CTA and by the output beyond;
-// whole forward, two kernels -> this one: 12608 x 12 -> 384 8.6 -> 5.9 us, 25216 x 24 -> 768 11.7 -> 11.1, 200704 x 16 -> 512 48.2 -> 37.7.
+// whole forward, two kernels -> this one: 12608 x 12 -> 384 8.6 -> 5.6 us, 25216 x 24 -> 768 11.7 -> 11.1, 200704 x 16 -> 512 48.2 -> 37.7.
 // Four quantizer warps keep up with the epilogue only while K is small against N (the rule is where the kernel is launched): a
 // form for K <= 128 with chunks spread over the threads took 58 us for 200704 x 96 -> 384 (two kernels 41), with eight quantizer
 // warps, for which the epilogue's registers spill, 48.

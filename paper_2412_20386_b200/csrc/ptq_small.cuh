@@ -13,8 +13,9 @@
 //   warp 0        weight loads (TMA, thread 0), then the MMAs of all k-blocks
 //   warps 0..     drain: lane = output channel, 16 tokens per warp (lane quarter = warp % 4)
 //
-// Bound by its chain of latencies: an empty kernel takes 2.4-2.5 us from launch to launch, this one 2.7 us at K = 12,
-// 3.4 at K = 192, 3.7 at K = 384 and 4.7 at K = 768 (197 rows; quantize + GEMM kernel 5.5, 6.5, 6.2, 7.4).  Threads per CTA,
+// Bound by its chain of latencies: an empty kernel takes 2.4-2.5 us from launch to launch, this one 2.4 us at K = 12, 3.0 at K = 192 and
+// 3.3 at K = 384 (197 rows, replayed from a graph; 2.5, 3.1 and 3.5 while one thread in a branch of its own issued the MMAs; as quantize + GEMM
+// kernel 5.5, 6.5, 6.2).  Threads per CTA,
 // 197 x 384 -> 192: 128 4.7 us, 256 3.9, 384 3.7, 512 4.0.  kMinCtas = 1 leaves 95 registers a thread, which keeps the
 // four rows of a thread interleaved; 2 (80 registers) costs 0.15 us and is taken where the grid needs two CTAs per SM.
 #pragma once
