@@ -635,10 +635,10 @@ ONE_KERNEL = "ptq_small_kernel or ptq_short_k_kernel"       # a forward pass tha
 # DRAM traffic per launch (dram__bytes_read.sum + dram__bytes_write.sum) from the ncu captures summarised
 # under profiles/; keyed by (kernel, workload, layer).  An entry is removed when its kernel changes.
 TRAFFIC = {
-    ("ptq_gemm_dequant_panel_kernel", "c3", "in_proj"): 41.221376e6 + 247.186176e6,
-    ("ptq_gemm_dequant_kernel", "c3", "out_proj"): 78.688512e6 + 22.753792e6,
-    ("ptq_quantize_kernel", "c3", "in_proj"): 77.500416e6 + 4.891648e6,
-    ("ptq_quantize_kernel", "c3", "out_proj"): 154.999808e6 + 19.248128e6,
+    ("ptq_gemm_dequant_panel_kernel", "c3", "in_proj"): 41.145856e6 + 246.88256e6,
+    ("ptq_gemm_dequant_kernel", "c3", "out_proj"): 78.681856e6 + 22.382848e6,
+    ("ptq_quantize_kernel", "c3", "in_proj"): 77.500928e6 + 5.625344e6,
+    ("ptq_quantize_kernel", "c3", "out_proj"): 155.00544e6 + 19.924736e6,
 }
 
 
