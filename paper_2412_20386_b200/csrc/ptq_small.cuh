@@ -119,7 +119,9 @@ ptq_small_kernel(const __grid_constant__ CUtensorMap tmW, const SmallParams p)
     volatile uint32_t *tmem_holder = reinterpret_cast<volatile uint32_t *>(tab + 3 * kTN) + 4;
     volatile uint32_t *abort_flag = tmem_holder + 1;
 
-    const int tid = static_cast<int>(threadIdx.x), warp = uniform_warp(), lane = tid & 31;
+    // A warp number known to be uniform (uniform_warp) speeds the signed instances and slows the unsigned one, replayed from a graph, us, without
+    // and with it: 197 x 384 -> 192 4.36 / 4.20 signed, 4.13 / 4.33 unsigned, 980 x 8 -> 128 unsigned 2.79 / 2.97, 3479 x 96 -> 200 3.87 / 4.04.
+    const int tid = static_cast<int>(threadIdx.x), warp = kMode == kCodeU8 ? tid >> 5 : uniform_warp(), lane = tid & 31;
     const int m_tile = static_cast<int>(fd_div(blockIdx.x, p.fd_n_tiles));
     const int n0 = (static_cast<int>(blockIdx.x) - m_tile * p.n_tiles) * kSmallRows;
     const int m0 = m_tile * kTN;
@@ -205,7 +207,8 @@ ptq_small_kernel(const __grid_constant__ CUtensorMap tmW, const SmallParams p)
     // Codes of rows beyond M and of channels beyond K are whatever lies there: those columns are not read, and the weights
     // are zero beyond K.
     if (warp == 0) {
-        const bool ok = mbar_wait_warp(wbar, 0u, abort_flag, p.status);
+        // (one vote, behind the wait: the weights have been there since long before; mbar_wait_warp's two cost 0.05 us)
+        const bool ok = __all_sync(0xffffffffu, mbar_wait(wbar, 0u, abort_flag, p.status));
         if (ok) {
             tc_fence_after_sync();
             const uint32_t idesc = make_idesc_i8(kSmallRows, kTN, false, kMode == kCodeU8);
