@@ -228,6 +228,13 @@ int ptq_linear_code_pitch(const ptq_linear_t *h);
 int ptq_linear_gemm_variant(const ptq_linear_t *h, int B);
 
 /*
+ * The same answer, and how that kernel cuts the output: *tile_cols is the number of columns of an output tile, *piece_cols
+ * that of the pieces which the streaming kernel makes of the tiles of its last round (0 where they stay whole).  Either pointer
+ * may be NULL; both are set to 0 where -1 is returned.
+ */
+int ptq_linear_gemm_tiling(const ptq_linear_t *h, int B, int *tile_cols, int *piece_cols);
+
+/*
  * Measurement aid; the paper has no counterpart.  Times one of five stand-alone kernels that move bytes the way
  * the GEMM + dequantization kernel does (Sec. 5.1; Appendix B.1, parts 3-4) but compute nothing, so that a
  * roofline discussion can quote what THIS GPU does with nothing else running:

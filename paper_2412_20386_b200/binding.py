@@ -66,6 +66,8 @@ def load_library() -> ctypes.CDLL:
     L.ptq_probe.argtypes = [ci, vp, sz, ci, ctypes.POINTER(ctypes.c_double), vp]
     L.ptq_linear_gemm_variant.restype = ci
     L.ptq_linear_gemm_variant.argtypes = [vp, ci]
+    L.ptq_linear_gemm_tiling.restype = ci
+    L.ptq_linear_gemm_tiling.argtypes = [vp, ci, ctypes.POINTER(ci), ctypes.POINTER(ci)]
     L.ptq_linear_forward_static.restype = ci
     L.ptq_linear_forward_static.argtypes = [vp, vp, ci, vp, vp]
     L.ptq_linear_workspace_bytes_dynamic.restype = sz
@@ -380,6 +382,12 @@ class PtqLinear:
     def gemm_variant(self, B: int) -> int:
         """``ptq_linear_gemm_variant``: 0 streaming kernel, 1 resident weights, 2 resident panel of codes."""
         return int(self._L.ptq_linear_gemm_variant(self._h, int(B)))
+
+    def gemm_tiling(self, B: int):
+        """``ptq_linear_gemm_tiling``: (variant, columns of a tile, columns of a piece of the last round or 0)."""
+        tile, piece = ctypes.c_int(), ctypes.c_int()
+        variant = self._L.ptq_linear_gemm_tiling(self._h, int(B), ctypes.byref(tile), ctypes.byref(piece))
+        return int(variant), tile.value, piece.value
 
     def gemm_dequant(self, q, B: int, y=None, stream=None):
         """``ptq_linear_gemm_dequant``: int8 codes [B*T, code_pitch()] -> y fp16 [B,T,N]."""

@@ -149,7 +149,7 @@ struct ptq_linear {
     long long l2_bytes = 0;
     unsigned char *d_all = nullptr;   // the one allocation that holds all of the following
     int8_t *d_w = nullptr;     // [n_tiles*BN, w_pitch], zero padded
-    float *d_dw = nullptr, *d_bias = nullptr;            // [n_tiles*BN rounded up to 64, +64], zero padded
+    float *d_dw = nullptr, *d_bias = nullptr;            // [n_tiles*BN rounded up to 64, +256], zero padded
     float *d_s = nullptr, *d_rs = nullptr;               // [round_up(K,16)]
     float *d_dx = nullptr;                               // [T]
     float2 *d_dx2 = nullptr;                             // [T] {dx, 1/dx}
@@ -510,6 +510,22 @@ void set_bn(const ptq_linear *h, ptq::GemmParams &p, int bn)
     p.fd_n_tiles = ptq::make_fastdiv(static_cast<unsigned>(p.n_tiles));
 }
 
+// Which of the streaming and the resident kernel takes a launch, with tiles of how many columns, and of how many each piece of its
+// last round (0: whole).  p.BN and the numbers of tiles are set to it.
+struct Tiling {
+    int bn = 0, cut = 0;
+    bool resident = false;
+};
+Tiling choose_tiling(const ptq_linear *h, ptq::GemmParams &p, bool tma_store)
+{
+    Tiling t;
+    t.bn = choose_bn(h, p);
+    if (t.bn != h->BN) set_bn(h, p, t.bn);
+    t.resident = tma_store && takes_resident(h, p.m_tiles, p.n_tiles);
+    t.cut = t.resident ? 0 : cut_cols(h, p, t.bn);
+    return t;
+}
+
 // Parameters of the GEMM kernels at the layer's own tile width.
 void set_gemm_params(const ptq_linear *h, ptq::GemmParams &p, long long M, void *y, void *acc_out, bool tma_store, const float *dx_rows)
 {
@@ -620,16 +636,14 @@ ptq_status_t launch_gemm(const ptq_linear *h, const void *codes, long long M, vo
         PTQ_CUDA(cudaGetLastError());
         return PTQ_OK;
     }
-    const int bn = choose_bn(h, p);
-    if (bn != h->BN) set_bn(h, p, bn);
+    const Tiling tiling = choose_tiling(h, p, tma_store);
+    const int bn = tiling.bn, cut = tiling.cut;
     const CUtensorMap &tmW = bn != h->BN ? h->tmWbn[bn / 64 - 1] : h->tmW;
     const long long tiles = static_cast<long long>(p.m_tiles) * p.n_tiles;
-    const bool resident = tma_store && takes_resident(h, p.m_tiles, p.n_tiles);
-    const int cut = resident ? 0 : cut_cols(h, p, bn);
     const int grid = static_cast<int>(tiles < h->num_sms ? tiles : h->num_sms);
     auto go = [&](auto debug, auto asym) -> ptq_status_t {
         constexpr bool kDbg = decltype(debug)::value, kAsym = decltype(asym)::value;
-        if (resident) {
+        if (tiling.resident) {
             constexpr auto kKern = ptq::ptq_gemm_dequant_resident_kernel<kDbg, kAsym>;
             p.fd_n_tiles = ptq::make_fastdiv(static_cast<unsigned>(p.m_tiles));
             const ptq_status_t es = ensure_smem<kKern>(h->device, ptq::kResSmemMax);
@@ -1203,23 +1217,25 @@ int ptq_linear_describe(const ptq_linear_t *h, char *buf, int buf_bytes)
 
 int ptq_linear_code_pitch(const ptq_linear_t *h) { return h ? h->Kpad : 0; }
 
-int ptq_linear_gemm_variant(const ptq_linear_t *h, int B)
+int ptq_linear_gemm_variant(const ptq_linear_t *h, int B) { return ptq_linear_gemm_tiling(h, B, nullptr, nullptr); }
+
+int ptq_linear_gemm_tiling(const ptq_linear_t *h, int B, int *tile_cols, int *piece_cols)
 {
+    if (tile_cols) *tile_cols = 0;
+    if (piece_cols) *piece_cols = 0;
     if (!h || B < 1) return -1;
     const long long M = static_cast<long long>(B) * h->T;
-    if (h->N % 8 != 0) return 0;
+    const bool tma_store = h->N % 8 == 0;
     ptq::GemmParams p = {};
-    p.BN = h->BN;
-    p.n_tiles = h->n_tiles;
-    p.m_tiles = static_cast<int>((M + ptq::kBM - 1) / ptq::kBM);
-    p.k_blocks = h->k_blocks;
-    p.has_bias = h->has_bias ? 1 : 0;
-    set_vectors(h, p);
-    const bool short_k = h->k_blocks <= kShortMainLoop;
-    p.boxes = short_k ? 2 : 1;
-    if (plan_panel(h, p, true)) return 2;
-    set_bn(h, p, choose_bn(h, p));
-    return takes_resident(h, p.m_tiles, p.n_tiles) ? 1 : 0;
+    set_gemm_params(h, p, M, nullptr, nullptr, tma_store, nullptr);
+    if (plan_panel(h, p, tma_store)) {
+        if (tile_cols) *tile_cols = h->BN;
+        return 2;
+    }
+    const Tiling t = choose_tiling(h, p, tma_store);
+    if (tile_cols) *tile_cols = t.bn;
+    if (piece_cols) *piece_cols = t.cut;
+    return t.resident ? 1 : 0;
 }
 
 ptq_status_t ptq_linear_gemm_dequant(const ptq_linear_t *h, const void *q_int8, int B, void *y_fp16, void *stream)

@@ -79,7 +79,7 @@ struct GemmParams {
     int k_blocks;      // ceil(K / 128)
     int last_mmas;     // MMAs (K = 32 each) in the last k-block: ceil((K - 128 (k_blocks-1)) / 32)
     const float *dx;   // [T]
-    const float *dw;   // [>= n_tiles*BN + 64], zero padded
+    const float *dw;   // [N + 256 and more], zero padded: a tile of any width may be read whole
     const float *bias; // same length, zeros when the layer has no bias
     int has_bias;      // 0: bias is all zeros and need not be read
     int vectors;       // scale vectors kept in shared memory: steps, bias where the layer has one, row sums if ws_copy
@@ -98,7 +98,7 @@ struct GemmParams {
     // accumulates sum_k c * Wq, and the epilogue subtracts z[t] * sum_k Wq[n,k] to obtain the offset-free
     // accumulator sum_k (c - z[t]) * Wq[n,k] exactly (all int32).  nullptr for symmetric layers.
     const int *zp;     // [T]
-    const int *wsum;   // [>= n_tiles*BN + 64] row sums of Wq, zero padded
+    const int *wsum;   // row sums of Wq, padded like dw
     // Panel kernel only: a work unit is one 128-row panel of codes times `group` adjacent N tiles; `groups`
     // units cover a panel; the weight ring has `b_stages` slots of `b_stage_bytes` (= BN * 128) each.
     int group, groups;

@@ -76,6 +76,10 @@ def test_null_handles_are_refused_not_dereferenced(lib):
     assert lib.ptq_linear_workspace_bytes(None, 4, 0) == 0
     assert lib.ptq_linear_fused_supported(None) == 0
     assert lib.ptq_linear_gemm_variant(None, 1) == -1
+    tile, piece = ctypes.c_int(9), ctypes.c_int(9)
+    assert lib.ptq_linear_gemm_tiling(None, 1, ctypes.byref(tile), ctypes.byref(piece)) == -1
+    assert (tile.value, piece.value) == (0, 0)
+    assert lib.ptq_linear_gemm_tiling(None, 1, None, None) == -1
     out = ctypes.c_double(-1.0)
     assert lib.ptq_probe(0, None, 0, 10, None, None) == 1                      # PTQ_ERR_NULL: no result pointer
     assert lib.ptq_probe(9, None, 0, 10, ctypes.byref(out), None) == 3         # PTQ_ERR_VALUE: unknown kind
