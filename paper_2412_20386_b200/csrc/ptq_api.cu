@@ -451,9 +451,12 @@ double epilogue_cycles(int cols) { return 360.0 + 670.0 * (((cols + 63) / 64 + 1
 
 // Columns per piece of the streaming kernel's last round with tiles of `bn` columns, 0 where it is not cut: at least one full
 // round before it, SMs enough for all pieces at once (narrow ones first), and a long main loop: the epilogue gains little by
-// a narrower tile.  Layer, both kernels, us, whole and cut: 6304 x 1536 -> 768 (dynamic) 21.4 -> 19.7, 6304 x 768 -> 3072 (dynamic) 24.5 -> 24.0,
-// 1568 x 768 -> 3072 10.8 -> 9.8, 3136 x 768 -> 3072 13.9 -> 13.2; with K <= 384 25088 x 384 -> 192 11.6 -> 11.7, 12608 x 192 -> 768 10.3 -> 10.3,
-// and a pair of layers with 6304 x 384 -> 1536 24.75 -> 24.9.
+// a narrower tile.  GEMM kernel alone, us, whole and cut, at the width that is chosen: 6304 x 1536 -> 768 (256 columns) 10.7 -> 8.9,
+// 6304 x 768 -> 3072 (256) 15.8 -> 14.8, 1568 x 768 -> 3072 (192) 7.0 -> 6.7, 3136 x 768 -> 3072 (256) 10.2 -> 9.5; with K <= 384 25088 x 384 -> 192
+// (192) 5.12 -> 5.14, 12608 x 192 -> 768 (192) 6.3 -> 6.3, 6304 x 384 -> 1536 (192) 6.8 -> 6.8.  (Of whole forward passes with K <= 384 one gained by a
+// cut: 25088 x 384 -> 192 16.5 -> 15.9; 12608 x 192 -> 768 10.7 -> 10.7, 6304 x 384 -> 768 9.6 -> 9.4.)
+// Every tile of the round counts with all its pieces: those of an N tile that ends early and lie wholly beyond N are issued too, load zero
+// weights, multiply and store nothing.
 int cut_cols(const ptq_linear *h, const ptq::GemmParams &p, int bn)
 {
     const long long tiles = static_cast<long long>(p.m_tiles) * ((h->N + bn - 1) / bn), last = tiles % h->num_sms;
@@ -484,8 +487,11 @@ double gemm_cycles(const ptq_linear *h, const ptq::GemmParams &p, int bn)
 // us, own width -> the one chosen: 2793 x 1536 -> 768 (256 -> 128) 7.4 -> 5.3, 1568 x 1536 -> 768 (256 -> 128) 7.3 -> 4.9, 3152 x 768 -> 384 (192 -> 128)
 // 4.7 -> 3.8, 12544 x 768 -> 384 (192, cut -> 128) 6.6 -> 6.1, 11229 x 520 -> 600 (256 -> 128) 8.9 -> 8.6, 12608 x 192 -> 768 (256 -> 192) 6.6 -> 6.3.
 // The margin keeps what the model cannot tell apart: 25216 x 768 -> 384 (192 -> 128, predicted -1.6 %) 10.7 -> 10.9.  What it gets wrong: 6304 x 768 ->
-// 384 keeps 192 columns, 5.0, where 128 with a cut round take 4.5, and 6304 x 384 -> 192 takes 128, 3.4, where 64 take 3.1.  Widths that lead to the
-// resident kernel are not compared: with several rounds and a short main loop the widths are within 3 % of one another either way.
+// 384 keeps 192 columns, 5.0, where 128 with a cut round take 4.5, and 6304 x 384 -> 192 takes 128, 3.4, where 64 take 3.1.  Whole forward passes of 1536
+// random layers, every width: the chosen one 0.4 % above the best on average; the furthest off 1078 x 46 -> 3072 with a bias (192 columns, 7.7,
+// where 256 take 6.9), 13867 x 298 -> 384 (128, 15.2, where 192 take 14.1) and 5047 x 576 -> 600 dynamic (128, cut, 14.0, where 256 take 13.0).  Wider
+// margins, less belief in the cut and a second round forbidden were tried on them: each slows as many layers as it mends.  Widths that lead to
+// the resident kernel are not compared: with several rounds and a short main loop the widths are within 3 % of one another either way.
 int choose_bn(const ptq_linear *h, const ptq::GemmParams &p)
 {
     auto resident = [&](int bn) { return takes_resident(h, p.m_tiles, (h->N + bn - 1) / bn); };

@@ -160,8 +160,8 @@ __device__ __forceinline__ bool quantize8_screen(uint32_t x0, uint32_t x1, uint3
 // when the chunk has to go to the slower routes: a value within the tie band, a magnitude above
 // 127.25 (saturation is not handled here), or a NaN / infinity: the running magnitude maximum
 // propagates NaN, and an infinity exceeds the limit, so both fail the one comparison on `big`.
-// kBounded: the caller knows that no |v'| exceeds 127 and passes a bound of them as `big`; NaN is then caught in the maximum of
-// the tie distances, and the maximum of the magnitudes is saved.
+// kBounded: the caller knows that no |v'| exceeds 127 (1 + 1e-6), so that none is above 127.25, and passes their largest, to a few 2^-24 of it,
+// as `big`; NaN is then caught in the maximum of the tie distances, and the maximum of the magnitudes is saved.
 template <int kMode = kCodeS8, bool kBounded = false>
 __device__ __forceinline__ bool quantize8_magic(uint32_t x0, uint32_t x1, uint32_t x2, uint32_t x3,
                                                 const float (&c8)[8], uint32_t &lo, uint32_t &hi, float big = 0.0f)

@@ -283,7 +283,9 @@ __global__ void __launch_bounds__(256, dyn_row_ctas_per_sm(kChunks)) ptq_quantiz
                 const float2 c0 = __fmul2_rn(make_float2(ra.x, ra.y), rd2), c1 = __fmul2_rn(make_float2(ra.z, ra.w), rd2);
                 const float2 c2 = __fmul2_rn(make_float2(rb.x, rb.y), rd2), c3 = __fmul2_rn(make_float2(rb.z, rb.w), rd2);
                 const float c8[8] = {c0.x, c0.y, c1.x, c1.y, c2.x, c2.y, c3.x, c3.y};
-                // |v'| <= 127: no saturation; cm is within 2^-24 of the chunk's largest |x/s|, far inside the slack of the band's slope
+                // No saturation: dx = RN(max / 127) and six roundings leave |v'| <= 127 (1 + 1e-6), code 127.  cm is within 2^-23 of the chunk's
+                // largest |x/s| (two roundings), cm * rdx within 4 * 2^-24 of its largest |v'|: a part in 4e6 of a band of 4e-7 |v'| that has
+                // 4e-8 |v'| to spare.
                 exact = quantize8_magic<kCodeS8, true>(v[j].x, v[j].y, v[j].z, v[j].w, c8, out.x, out.y, __fmul_rn(cm[j], rdx));
             }
             if (exact) quantize8_exact<false, kCodeS8>(v[j].x, v[j].y, v[j].z, v[j].w, s_s + 8 * c, nullptr, dx, rdx, out.x, out.y);

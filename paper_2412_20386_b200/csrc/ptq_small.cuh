@@ -119,8 +119,8 @@ ptq_small_kernel(const __grid_constant__ CUtensorMap tmW, const SmallParams p)
     volatile uint32_t *tmem_holder = reinterpret_cast<volatile uint32_t *>(tab + 3 * kTN) + 4;
     volatile uint32_t *abort_flag = tmem_holder + 1;
 
-    // A warp number known to be uniform (uniform_warp) speeds the signed instances and slows the unsigned one, replayed from a graph, us, without
-    // and with it: 197 x 384 -> 192 4.36 / 4.20 signed, 4.13 / 4.33 unsigned, 980 x 8 -> 128 unsigned 2.79 / 2.97, 3479 x 96 -> 200 3.87 / 4.04.
+    // A warp number known to be uniform (uniform_warp) speeds the signed instances and slows the unsigned one, replayed from a graph, one value
+    // in 7000 saturating, us, without and with it: 197 x 384 -> 192 4.36 / 4.20 signed, 4.13 / 4.33 unsigned, 980 x 8 -> 128 unsigned 2.79 / 2.97, 3479 x 96 -> 200 3.87 / 4.04.
     const int tid = static_cast<int>(threadIdx.x), warp = kMode == kCodeU8 ? tid >> 5 : uniform_warp(), lane = tid & 31;
     const int m_tile = static_cast<int>(fd_div(blockIdx.x, p.fd_n_tiles));
     const int n0 = (static_cast<int>(blockIdx.x) - m_tile * p.n_tiles) * kSmallRows;

@@ -294,9 +294,12 @@ __device__ __forceinline__ void tc_fence_after_sync()
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 }
 
-// The warps that issue MMAs, TMA loads and TMA stores run their loops with all 32 lanes and elect one inside the statement that
-// issues, so that control flow, addresses and descriptors are uniform over the warp for the compiler.  In a branch of one lane an MMA took 57 +
-// 0.54 N cycles of issue, whatever the tensor pipe needed; so 30 to 40 less, and the GEMM kernels 20 registers less.  Layers, both
+// All single-CTA kernels issue their MMAs with all 32 lanes of a warp and elect one inside the statement that issues, so that
+// control flow, addresses and descriptors are uniform over the warp for the compiler; the streaming, the panel and the resident
+// kernel their TMA loads and stores too.  (One lane in a branch of its own: the loads of the fused, the few-channels and the few-rows kernel, the
+// stores of the fused kernel, loads and MMAs of the CTA-pair kernel.)  In such a branch an MMA took 57 + 0.54 N cycles of issue, whatever the
+// tensor pipe needed; so 30 to 40 less, and the GEMM kernels of symmetric layers 133, 132 and 143 registers instead of 152, 154 and 164
+// (streaming, panel, resident; of asymmetric ones 158, 158 and 167 instead of 168).  Layers, both
 // kernels, us: 12608 x 192 -> 768 10.3 -> 9.7, 25216 x 384 -> 1536 26.0 -> 23.7, 2793 x 1536 -> 768 11.1 -> 9.9, 1568 x 1536 -> 768 9.5 -> 8.3,
 // 50432 x 768 -> 3072 131 -> 126; one kernel, 197 x 384 -> 192 3.46 -> 3.27.  (Loads and stores alone are 1.5 to 2.5 % of that.)
 //
