@@ -1409,13 +1409,14 @@ static ptq_status_t search_impl(int K, int T, const void *xcal_fp16, int Bc, con
     p.K = K;
     p.n_grid = n_grid;
     p.j_lo = j_lo;
+    p.vec = K % 8 == 0 && reinterpret_cast<uintptr_t>(xcal_fp16) % 16 == 0;
     p.fd_K = ptq::make_fastdiv(static_cast<unsigned>(K));
     const ptq::SearchPlan plan = ptq::search_plan(Bc * K, T, C, sms);
     const dim3 grid(static_cast<unsigned>(T), static_cast<unsigned>((C + plan.candidates - 1) / plan.candidates));
     if (plan.candidates == ptq::kSearchMany)
-        ptq::ptq_search_loss_kernel<ptq::kSearchMany><<<grid, plan.threads, 0, s>>>(p);
+        ptq::ptq_search_loss_kernel<ptq::kSearchGroups><<<grid, plan.block(), 0, s>>>(p);
     else
-        ptq::ptq_search_loss_kernel<ptq::kSearchFew><<<grid, plan.threads, 0, s>>>(p);
+        ptq::ptq_search_loss_kernel<1><<<grid, plan.block(), 0, s>>>(p);
     ptq::ptq_search_pick_kernel<<<(T + 3) / 4, 128, 0, s>>>(d_loss, d_base, T, n_grid, j_lo, d_best, d_dx);
     g_launches.fetch_add(2, std::memory_order_relaxed);
     PTQ_CUDA(cudaGetLastError());

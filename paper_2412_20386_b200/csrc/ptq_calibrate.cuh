@@ -289,11 +289,13 @@ __global__ void __launch_bounds__(128) ptq_calib_step_asym_kernel(const unsigned
 // non-finite u skipped.  One block per (position, group of candidates); threads
 // stride over the Bc*K elements of the position, keep one binary64 partial sum per candidate, and the
 // block reduces them in a fixed order (shuffles, then warp by warp), so a launch is reproducible.
-constexpr int kSearchSub = 9;                            // candidates whose integers are in registers at a time
-constexpr int kSearchFew = kSearchSub, kSearchMany = 3 * kSearchSub;   // candidates per block, the two kernels
+constexpr int kSearchSub = 9;                            // candidates of a thread
+constexpr int kSearchGroups = 3;                         // groups of threads with candidates of their own, in the kernel for many
+constexpr int kSearchFew = kSearchSub, kSearchMany = kSearchGroups * kSearchSub;   // candidates per block, the two kernels
 constexpr int kSearchTile = 2048;                        // elements whose x/s are in shared memory at a time
-constexpr int kSearchThreads = 256;                      // per block, at most
-constexpr int kSearchBlocksFew = 3, kSearchBlocksMany = 2;   // blocks of so many threads that an SM's registers hold
+constexpr int kSearchThreads = 256;                      // that walk the elements in a block with 9 candidates, at most
+constexpr int kSearchBlocksFew = 3, kSearchBlocksMany = 2;   // blocks of so many threads that an SM's registers hold (with 27: of half as many per group)
+constexpr int kSearchBlockMax = kSearchGroups * kSearchThreads / 2;
 
 struct SearchParams {
     const __half *x;     // [Bc,T,K]
@@ -302,6 +304,7 @@ struct SearchParams {
     double *loss;        // [T, n_grid - j_lo + 1]
     int Bc, T, K;
     int n_grid, j_lo;
+    int vec;             // K % 8 == 0, x 16-byte aligned: eight elements per load
     FastDiv fd_K;
 };
 
@@ -319,16 +322,17 @@ __device__ __forceinline__ float search_candidate_step(float base, int j, int n_
     return __fmul_rn(base, __fdiv_rn(static_cast<float>(j), static_cast<float>(n_grid)));
 }
 
-// Candidates per block and threads of a launch.  A block's threads each form the candidates' steps and, at the end, reduce
-// their sums: about as much work as 10 elements, so a block has as few threads as still fill the chip (256 threads where
-// blocks are few, 64 where they are many).  27 candidates share the loading and dividing of an element, 60 instructions, but
-// hold 128 registers: taken with three blocks per SM or more and at most an eighth of the candidates idle, else 9.
-// Kernel, us, with 9 candidates and 64 / 128 / 256 threads, with 27 and the same:
-//   8 x 197 x 384    8 candidates  24.6 / 15.2 / 11.0   42.6 / 27.4 / 21.8      81   40.0 / 41.4 / 48.0   47.8 / 35.1 / 40.6
-//   4 x 3136 x 96    8             14.2 / 17.3 / 28.2   35.0 / 47.0 / 75.1      81   95.7 / 128 / 222     93.4 / 127 / 213
-//   16 x 49 x 1536   8             168 / 88.7 / 53.9    290 / 155 / 96.7        81   190 / 109 / 79.7     296 / 158 / 96.9
+// Candidates per block and threads of a launch.  A thread has nine candidates: 27 of them took 128 registers and spilled, 16 warps
+// per SM at 57 % of the issue slots.  A block's threads each form the candidates' steps and, at the end, reduce their sums: about
+// as much work as 10 elements, so a block has as few threads as still fill the chip (256 threads where blocks are few, 64, or 32 in a
+// group, where they are many).  Three groups of threads in a block share the loading and dividing of the elements: taken with
+// three blocks per SM or more and at most an eighth of the candidates idle.  A whole call, us, one group of 64 / 128 / 256 threads, and three
+// of 32 / 64 / 128 (36 us of it are the copies, two launches and the wait for them):
+//   8 x 197 x 384   81 candidates   66 / 80 / 76      75 / 65 / 71        8 x 197 x 768   81   91 / 93 / 100     101 / 89 / 89
+//   4 x 3136 x 96   81              136 / 174 / 250   112 / 145 / 190     16 x 49 x 1536  81   156 / 113 / 100   217 / 156 / 105
 struct SearchPlan {
-    int candidates, threads;
+    int candidates, threads;   // three groups have half as many threads each: block()
+    __host__ __device__ int block() const { return candidates == kSearchMany ? kSearchGroups * threads / 2 : threads; }
 };
 __host__ __device__ inline SearchPlan search_plan(int elements, int T, int C, int sms)
 {
@@ -341,27 +345,38 @@ __host__ __device__ inline SearchPlan search_plan(int elements, int T, int C, in
     return {wide ? kSearchMany : kSearchFew, threads};
 }
 
+// max(a, |b|, |c|) in one instruction; NaN operands are dropped.
+__device__ __forceinline__ float search_max3_abs(float a, float b, float c)
+{
+    float r;
+    asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(fabsf(b)), "f"(fabsf(c)));
+    return r;
+}
+
 // Bound by issue: 49 M (element, candidate) pairs at 8 x 197 x 384 x 81, 9 instructions each.  The integer r = rne(u / Delta)
 // is taken from one FMA, t = RN(u * RN(1/Delta) + 1.5*2^23), whose low mantissa bits hold it; u * RN(1/Delta) is within
 // 1.2e-7 |v| of the defined quotient v, and beyond |v| = 128 every r clamps alike, so r can only be wrong where the distance
 // to r exceeds 0.49998: those elements (3 in 10^4) take the IEEE divisions.
-// 8 x 197 x 384 x 81: 71 us with IEEE divisions and 8 candidates per block, 40.6 with 27 and 256 threads, 35.1 so.
-template <int C>
-__global__ void __launch_bounds__(kSearchThreads, C == kSearchFew ? kSearchBlocksFew : kSearchBlocksMany) ptq_search_loss_kernel(SearchParams p)
+// 8 x 197 x 384 x 81, the kernel: 71 us with IEEE divisions and 8 candidates per block, 35 with 27 per thread; 8 x 197 x 768 x 81: 69.7 us so
+// (spills, 3.9 warps per scheduler), 59.0 with nine per thread in three groups and clamps only for the elements that need one, 51.5 with eight
+// elements per load (index arithmetic, load and division of one at a time were a fifth of the instructions).
+template <int kGroups>
+__global__ void __launch_bounds__(kSearchBlockMax, 2) ptq_search_loss_kernel(SearchParams p)
 {
     constexpr int S = kSearchSub;
     constexpr float kMagic = 12582912.0f;
-    __shared__ double partial[kSearchThreads / 32][C];
-    __shared__ float u_s[kSearchTile];
+    __shared__ double partial[kSearchBlockMax / 32][S];
+    __shared__ __align__(16) float u_s[kSearchTile];
+    const int per_group = static_cast<int>(blockDim.x) / kGroups;                // threads, whole warps
+    const int group = kGroups == 1 ? 0 : static_cast<int>(threadIdx.x) / per_group, at = static_cast<int>(threadIdx.x) - group * per_group;
     const int t = blockIdx.x;
-    const int j0 = p.j_lo + static_cast<int>(blockIdx.y) * C;
-    const int ncand = min(C, p.n_grid - j0 + 1);
+    const int j0 = p.j_lo + (static_cast<int>(blockIdx.y) * kGroups + group) * S;
     const float base = __ldg(p.base + t);
-    float delta[C], rdelta[C];
-    double acc[C];
+    float delta[S], rdelta[S];
+    double acc[S];
     bool fast = true;
 #pragma unroll
-    for (int c = 0; c < C; ++c) {
+    for (int c = 0; c < S; ++c) {
         delta[c] = search_candidate_step(base, min(j0 + c, p.n_grid), p.n_grid);
         rdelta[c] = __fdiv_rn(1.0f, delta[c]);
         fast = fast && delta[c] >= 9.313225746154785e-10f && delta[c] <= 1073741824.0f;      // 2^-30 .. 2^30
@@ -370,49 +385,67 @@ __global__ void __launch_bounds__(kSearchThreads, C == kSearchFew ? kSearchBlock
     for (SearchTiles tile(p.Bc * p.K); tile.valid(); tile.next()) {
         const int n = tile.count();
         __syncthreads();
+        if (p.vec) {
+            for (int i = 8 * static_cast<int>(threadIdx.x); i < n; i += 8 * static_cast<int>(blockDim.x)) {
+                const int b = static_cast<int>(fd_div(tile.at + i, p.fd_K));
+                const int k = static_cast<int>(tile.at + i) - b * p.K;
+                const CalibChunk<8> x = calib_load<8>(p.x + (static_cast<long long>(b) * p.T + t) * p.K + k);
+                const float4 s0 = __ldg(reinterpret_cast<const float4 *>(p.s + k)), s1 = __ldg(reinterpret_cast<const float4 *>(p.s + k) + 1);
+                float4 *u = reinterpret_cast<float4 *>(u_s + i);
+                u[0] = make_float4(__fdiv_rn(calib_channel(x, 0), s0.x), __fdiv_rn(calib_channel(x, 1), s0.y),
+                                   __fdiv_rn(calib_channel(x, 2), s0.z), __fdiv_rn(calib_channel(x, 3), s0.w));
+                u[1] = make_float4(__fdiv_rn(calib_channel(x, 4), s1.x), __fdiv_rn(calib_channel(x, 5), s1.y),
+                                   __fdiv_rn(calib_channel(x, 6), s1.z), __fdiv_rn(calib_channel(x, 7), s1.w));
+            }
+        } else {
 #pragma unroll 4
-        for (int i = threadIdx.x; i < n; i += blockDim.x) {
-            const int b = static_cast<int>(fd_div(tile.at + i, p.fd_K));
-            const int k = static_cast<int>(tile.at + i) - b * p.K;
-            u_s[i] = __fdiv_rn(__half2float(__ldg(p.x + (static_cast<long long>(b) * p.T + t) * p.K + k)), __ldg(p.s + k));
+            for (int i = threadIdx.x; i < n; i += blockDim.x) {
+                const int b = static_cast<int>(fd_div(tile.at + i, p.fd_K));
+                const int k = static_cast<int>(tile.at + i) - b * p.K;
+                u_s[i] = __fdiv_rn(__half2float(__ldg(p.x + (static_cast<long long>(b) * p.T + t) * p.K + k)), __ldg(p.s + k));
+            }
         }
         __syncthreads();
-        for (int i = threadIdx.x; i < n; i += blockDim.x) {
+        for (int i = at; i < n; i += per_group) {
             const float u = u_s[i];
             if (!(fabsf(u) <= 3.402823466e38f)) continue;      // inf and NaN do not enter the loss
+            float r[S], d[S];
 #pragma unroll
-            for (int c0 = 0; c0 < C; c0 += S) {
-                float r[S], worst = 0.0f;
+            for (int c = 0; c < S; ++c) {
+                r[c] = __fadd_rn(__fmaf_rn(u, rdelta[c], kMagic), -kMagic);
+                d[c] = __fmaf_rn(u, rdelta[c], -r[c]);
+            }
+            float worst = fabsf(d[0]);
 #pragma unroll
-                for (int c = 0; c < S; ++c) {
-                    r[c] = __fadd_rn(__fmaf_rn(u, rdelta[c0 + c], kMagic), -kMagic);
-                    worst = fmaxf(worst, fabsf(__fmaf_rn(u, rdelta[c0 + c], -r[c])));
-                }
-                if (!fast || worst > 0.49998f) {
+            for (int c = 1; c < S; c += 2) worst = search_max3_abs(worst, d[c], d[c + 1]);
+            if (!fast || worst > 0.49998f) {
 #pragma unroll
-                    for (int c = 0; c < S; ++c) r[c] = rintf(__fdiv_rn(u, delta[c0 + c]));
-                }
+                for (int c = 0; c < S; ++c) r[c] = rintf(__fdiv_rn(u, delta[c]));
+            }
+            if (!(fabsf(r[0]) <= 127.0f)) {                    // the group's smallest step: its largest quotient
 #pragma unroll
-                for (int c = 0; c < S; ++c) {
-                    const double e = static_cast<double>(__fmaf_rn(-delta[c0 + c], fminf(fmaxf(r[c], -128.0f), 127.0f), u));
-                    acc[c0 + c] = fma(e, e, acc[c0 + c]);
-                }
+                for (int c = 0; c < S; ++c) r[c] = fminf(fmaxf(r[c], -128.0f), 127.0f);
+            }
+#pragma unroll
+            for (int c = 0; c < S; ++c) {
+                const double e = static_cast<double>(__fmaf_rn(-delta[c], r[c], u));
+                acc[c] = fma(e, e, acc[c]);
             }
         }
     }
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
-    for (int c = 0; c < C; ++c) {
+    for (int c = 0; c < S; ++c) {
         double v = acc[c];
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
         if (lane == 0) partial[warp][c] = v;
     }
     __syncthreads();
-    if (threadIdx.x < ncand) {
+    if (at < S && j0 + at <= p.n_grid) {
         double v = 0.0;
-        for (int w = 0; w < static_cast<int>(blockDim.x) / 32; ++w) v += partial[w][threadIdx.x];
-        p.loss[static_cast<long long>(t) * (p.n_grid - p.j_lo + 1) + (j0 - p.j_lo) + threadIdx.x] = v;
+        for (int w = 0; w < per_group / 32; ++w) v += partial[group * (per_group / 32) + w][at];
+        p.loss[static_cast<long long>(t) * (p.n_grid - p.j_lo + 1) + (j0 - p.j_lo) + at] = v;
     }
 }
 

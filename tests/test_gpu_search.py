@@ -91,6 +91,26 @@ def test_search_block_shapes(env, K, T, Bc, C):
     check_search(ptq, torch, x, s, rng.uniform(0.02, 0.06, T).astype(F32), 100, 101 - C)
 
 
+@pytest.mark.parametrize("K,T,Bc,C", [(64, 12, 33, 9), (8, 450, 257, 27), (264, 450, 2, 80)])
+def test_search_loads_and_clamps(env, K, T, Bc, C):
+    """Eight elements per load (K a multiple of 8) with last tiles that are not full, against the same values at an address that is not
+    16-byte aligned: bit for bit the same sums.  Steps so small that the quotients reach 5 to 500, so that of one thread's nine
+    candidates some clamp, all clamp or none does; infinities and NaN among the elements."""
+    ptq, torch = env
+    rng = np.random.default_rng(K + C)
+    x = (rng.standard_t(3, (Bc, T, K)) * np.exp(rng.normal(0, 1, (1, T, 1)))).astype(np.float16)
+    x[0, 1, 3], x[-1, 2, 5], x[0, 3, 0] = np.inf, np.nan, -np.inf
+    s = np.exp(rng.uniform(-1, 1, K)).astype(F32)
+    base = rng.uniform(0.005, 0.2, T).astype(F32)
+    check_search(ptq, torch, x, s, base, 100, 101 - C)
+    buf = torch.empty(x.size + 1, dtype=torch.float16, device="cuda")
+    shifted = buf[1:].view(x.shape)
+    shifted.copy_(torch.from_numpy(x))
+    aligned = ptq.search_act_step(torch.from_numpy(x).cuda(), s, base, 100, 101 - C, want_loss=True)
+    for a, b in zip(aligned, ptq.search_act_step(shifted, s, base, 100, 101 - C, want_loss=True)):
+        assert a.tobytes() == b.tobytes()
+
+
 def test_search_argument_errors(env):
     ptq, torch = env
     x = torch.zeros((2, 3, 8), dtype=torch.float16, device="cuda")
