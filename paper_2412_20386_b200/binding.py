@@ -131,7 +131,8 @@ def _load_native():
             raise ImportError("%s: build it with `python -m paper_2412_20386_b200.build`. There is no fallback." % e) from e
         _ptq_torch.bind(*(ctypes.cast(f, ctypes.c_void_p).value for f in (
             L.ptq_linear_forward, L.ptq_linear_forward_static, L.ptq_linear_forward_dynamic,
-            L.ptq_linear_workspace_bytes, L.ptq_linear_workspace_bytes_dynamic)))
+            L.ptq_linear_workspace_bytes, L.ptq_linear_workspace_bytes_dynamic,
+            L.ptq_calibrate_in, L.ptq_search_act_step_in)))
         _native = _ptq_torch
     return _native
 
@@ -172,13 +173,19 @@ def _scratch(nbytes: int, device, stream):
     return torch.empty(max(int(nbytes), 16), dtype=torch.uint8, device=device)
 
 
-def _offline_workspace(nbytes: int, device, stream):
-    """`_scratch` for the offline steps, whose callers see a failed allocation as the library's PTQ_ERR_NOMEM."""
+def _offline(call, nbytes: int, stream, ints, xcal, *arrays):
+    """An offline step of the extension on `stream` (None: the current one) in a workspace of `_scratch`: a device allocation
+    per call costs more than the calibration.  Its callers see a failed allocation as the library's PTQ_ERR_NOMEM."""
     import torch
     try:
-        return _scratch(nbytes, device, stream)
+        ws = _scratch(nbytes, xcal.device, stream)
     except torch.OutOfMemoryError as e:
         raise PtqError(7, str(e)) from e
+    if stream is None:
+        _check(call(*ints, xcal, ws, *arrays))
+    else:
+        with torch.cuda.stream(stream):
+            _check(call(*ints, xcal, ws, *arrays))
 
 
 def kernel_launch_count() -> int:
@@ -432,9 +439,7 @@ CALIB_PTS, CALIB_PER_TENSOR, CALIB_ASYM, CALIB_W4A4 = 0, 1, 2, 3
 
 
 def _calibrate(scheme, xcal, w, w_step, stream, packed_K=None):
-    """``ptq_calibrate_in`` in a workspace from torch's caching allocator (a device allocation per call costs more than
-    the calibration)."""
-    L = load_library()
+    """``ptq_calibrate_in``"""
     Bc, T, K = _xcal(xcal, packed_K)
     w = _host(w, np.uint8 if scheme == CALIB_W4A4 else np.int8)
     N = int(w.shape[0])
@@ -447,9 +452,8 @@ def _calibrate(scheme, xcal, w, w_step, stream, packed_K=None):
     s = np.empty(K, np.float32)
     dx = np.empty(T, np.float32)
     z = np.empty(T, np.int32) if scheme == CALIB_ASYM else None
-    ws = _offline_workspace(L.ptq_calibrate_workspace_bytes(K, N, T), xcal.device, stream)
-    _check(L.ptq_calibrate_in(scheme, K, N, T, xcal.data_ptr(), Bc, _hp(w), _hp(w_step), _hp(s), _hp(dx), _hp(z),
-                              ws.data_ptr(), ws.numel(), _stream_ptr(stream)))
+    _offline(_load_native().calibrate, load_library().ptq_calibrate_workspace_bytes(K, N, T), stream, (scheme, K, N, T, Bc), xcal,
+             w, w_step, s, dx, z)
     return (s, dx) if z is None else (s, dx, z)
 
 
@@ -466,16 +470,14 @@ def calibrate_asym(xcal, w_q, w_step, stream=None):
 
 def search_act_step(xcal, smooth, base_step, n_grid: int = 100, j_lo: int = 20, want_loss: bool = False, stream=None):
     """``ptq_search_act_step``: device fp16 [Bc,T,K] -> (dx fp32 [T], best j int32 [T], loss fp64 [T,C] or None)."""
-    L = load_library()
     Bc, T, K = _xcal(xcal)
     smooth = _host(smooth, np.float32, (K,))
     base_step = _host(base_step, np.float32, (T,))
     dx = np.empty(T, np.float32)
     best = np.empty(T, np.int32)
     loss = np.empty((T, max(n_grid - j_lo + 1, 1)), np.float64) if want_loss else None
-    ws = _offline_workspace(L.ptq_search_workspace_bytes(K, T, n_grid, j_lo), xcal.device, stream)
-    _check(L.ptq_search_act_step_in(K, T, xcal.data_ptr(), Bc, _hp(smooth), _hp(base_step), n_grid, j_lo, _hp(dx),
-                                    _hp(best), _hp(loss), ws.data_ptr(), ws.numel(), _stream_ptr(stream)))
+    _offline(_load_native().search, load_library().ptq_search_workspace_bytes(K, T, n_grid, j_lo), stream, (K, T, Bc, n_grid, j_lo),
+             xcal, smooth, base_step, dx, best, loss)
     return dx, best, loss
 
 

@@ -1,6 +1,8 @@
 // The forward calls of binding.PtqLinear on torch tensors, without Python in between: checks, allocation of what the
 // caller did not pass, the current stream and the C ABI call.  Through Python attribute access and ctypes the same steps
 // took 6 to 11 us a call, more than the two kernel launches they lead to (5 us), and bound every layer below that time.
+// The offline steps (calibration, step search) go the same way, with host arrays through the buffer protocol: a calibration of
+// 8 x 197 x 384 with 192 outputs takes 60 us a call, 78 through ctypes, of which 36 are its copies, launches and the wait for them.
 // The C ABI's functions are handed over as addresses by the binding, so this module does not link the library.
 #define PY_SSIZE_T_CLEAN
 #include <Python.h>
@@ -19,6 +21,8 @@ decltype(&ptq_linear_forward_static) f_static = nullptr;
 decltype(&ptq_linear_forward_dynamic) f_dynamic = nullptr;
 decltype(&ptq_linear_workspace_bytes) f_ws = nullptr;
 decltype(&ptq_linear_workspace_bytes_dynamic) f_ws_dynamic = nullptr;
+decltype(&ptq_calibrate_in) f_calibrate = nullptr;
+decltype(&ptq_search_act_step_in) f_search = nullptr;
 
 // Arguments of every call: handle, T, K, N, x, y, workspace (the last two may be None).
 struct Call {
@@ -163,26 +167,110 @@ PyObject *py_forward_static(PyObject *, PyObject *const *args, Py_ssize_t n)
     });
 }
 
+// Memory of a contiguous host array (buffer protocol), or null for None.
+struct Host {
+    Py_buffer view;
+    bool held = false;
+    void *ptr = nullptr;
+    bool read(PyObject *o, bool writable)
+    {
+        if (o == Py_None) return true;
+        if (PyObject_GetBuffer(o, &view, writable ? PyBUF_WRITABLE | PyBUF_C_CONTIGUOUS : PyBUF_C_CONTIGUOUS) != 0) return false;
+        held = true;
+        ptr = view.buf;
+        return true;
+    }
+    Host() = default;
+    Host(const Host &) = delete;
+    Host &operator=(const Host &) = delete;
+    ~Host()
+    {
+        if (held) PyBuffer_Release(&view);
+    }
+};
+
+// The integers, the two tensors (activations, workspace) and the host arrays of an offline step: two that the library reads, three
+// that it writes.  Shapes and types are the binding's to check.
+struct Offline {
+    int v[5];
+    const void *x;
+    void *ws, *stream;
+    size_t ws_bytes;
+    Host h[5];
+};
+bool read_offline(PyObject *const *args, Py_ssize_t n, Offline &o)
+{
+    if (n != 12 || !THPVariable_Check(args[5]) || !THPVariable_Check(args[6])) {
+        PyErr_SetString(PyExc_TypeError, "five integers, two tensors and five arrays are wanted");
+        return false;
+    }
+    for (int i = 0; i < 5; ++i) o.v[i] = static_cast<int>(PyLong_AsLong(args[i]));
+    if (PyErr_Occurred()) return false;
+    for (int i = 0; i < 5; ++i)
+        if (!o.h[i].read(args[7 + i], i >= 2)) return false;
+    const at::Tensor &ws = THPVariable_Unpack(args[6]);
+    o.x = THPVariable_Unpack(args[5]).const_data_ptr();
+    o.ws = ws.data_ptr();
+    o.ws_bytes = ws.nbytes();
+    o.stream = c10::cuda::getCurrentCUDAStream().stream();
+    return true;
+}
+
+// calibrate(scheme, K, N, T, Bc, xcal, workspace, w, w_step, s, dx, z) -> status
+PyObject *py_calibrate(PyObject *, PyObject *const *args, Py_ssize_t n)
+{
+    return guarded([&]() -> PyObject * {
+        Offline o;
+        if (!read_offline(args, n, o)) return nullptr;
+        ptq_status_t st;
+        Py_BEGIN_ALLOW_THREADS
+        st = f_calibrate(o.v[0], o.v[1], o.v[2], o.v[3], o.x, o.v[4], o.h[0].ptr, static_cast<const float *>(o.h[1].ptr),
+                         static_cast<float *>(o.h[2].ptr), static_cast<float *>(o.h[3].ptr), static_cast<int32_t *>(o.h[4].ptr), o.ws,
+                         o.ws_bytes, o.stream);
+        Py_END_ALLOW_THREADS
+        return PyLong_FromLong(st);
+    });
+}
+
+// search(K, T, Bc, n_grid, j_lo, xcal, workspace, s, base, dx, best, loss) -> status
+PyObject *py_search(PyObject *, PyObject *const *args, Py_ssize_t n)
+{
+    return guarded([&]() -> PyObject * {
+        Offline o;
+        if (!read_offline(args, n, o)) return nullptr;
+        ptq_status_t st;
+        Py_BEGIN_ALLOW_THREADS
+        st = f_search(o.v[0], o.v[1], o.x, o.v[2], static_cast<const float *>(o.h[0].ptr), static_cast<const float *>(o.h[1].ptr), o.v[3],
+                      o.v[4], static_cast<float *>(o.h[2].ptr), static_cast<int32_t *>(o.h[3].ptr), static_cast<double *>(o.h[4].ptr), o.ws,
+                      o.ws_bytes, o.stream);
+        Py_END_ALLOW_THREADS
+        return PyLong_FromLong(st);
+    });
+}
+
 PyObject *py_bind(PyObject *, PyObject *const *args, Py_ssize_t n)
 {
-    if (n != 5) {
-        PyErr_SetString(PyExc_TypeError, "five addresses are wanted");
+    if (n != 7) {
+        PyErr_SetString(PyExc_TypeError, "seven addresses are wanted");
         return nullptr;
     }
-    void *p[5];
-    for (int i = 0; i < 5; ++i) p[i] = PyLong_AsVoidPtr(args[i]);
+    void *p[7];
+    for (int i = 0; i < 7; ++i) p[i] = PyLong_AsVoidPtr(args[i]);
     if (PyErr_Occurred()) return nullptr;
     f_forward = reinterpret_cast<decltype(f_forward)>(p[0]);
     f_static = reinterpret_cast<decltype(f_static)>(p[1]);
     f_dynamic = reinterpret_cast<decltype(f_dynamic)>(p[2]);
     f_ws = reinterpret_cast<decltype(f_ws)>(p[3]);
     f_ws_dynamic = reinterpret_cast<decltype(f_ws_dynamic)>(p[4]);
+    f_calibrate = reinterpret_cast<decltype(f_calibrate)>(p[5]);
+    f_search = reinterpret_cast<decltype(f_search)>(p[6]);
     Py_RETURN_NONE;
 }
 
 #define PTQ_METHOD(name, fn) {name, reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(fn)), METH_FASTCALL, nullptr}
 PyMethodDef methods[] = {PTQ_METHOD("bind", py_bind), PTQ_METHOD("forward", py_forward),
                          PTQ_METHOD("forward_static", py_forward_static), PTQ_METHOD("forward_dynamic", py_forward_dynamic),
+                         PTQ_METHOD("calibrate", py_calibrate), PTQ_METHOD("search", py_search),
                          {nullptr, nullptr, 0, nullptr}};
 PyModuleDef module = {PyModuleDef_HEAD_INIT, "_ptq_torch", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};
 

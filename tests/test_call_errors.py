@@ -26,6 +26,24 @@ def test_bad_arguments_are_refused_before_the_library_is_called(native, call):
             f(0, 1, 1, 1, x, None, None)
 
 
+@pytest.mark.parametrize("call", ["calibrate", "search"])
+def test_bad_arguments_of_the_offline_steps_are_refused_before_the_library_is_called(native, call):
+    import torch
+    f, t, a = getattr(native, call), torch.zeros(1), np.ones(1, np.float32)
+    fixed = a.copy()
+    fixed.flags.writeable = False
+    with pytest.raises(TypeError):
+        f(0, 1, 1, 1, 1, t, t, a, a)
+    with pytest.raises(TypeError):
+        f(0, 1, 1, 1, 1, a, t, a, a, a, a, a)                                        # no tensor
+    with pytest.raises(TypeError):
+        f(0, 1, 1, 1, 1, t, t, 1.0, a, a, a, a)                                      # no array
+    with pytest.raises((BufferError, ValueError)):
+        f(0, 1, 1, 1, 1, t, t, a, a, fixed, a, a)                                    # an output that cannot be written
+    with pytest.raises((BufferError, ValueError)):
+        f(0, 1, 1, 1, 1, t, t, np.ones((4, 4), np.int8)[:, ::2], a, a, a, a)         # not contiguous
+
+
 def test_offline_steps_report_a_failed_allocation_as_the_librarys_error(native, monkeypatch):
     import torch
     import paper_2412_20386_b200 as ptq
