@@ -444,6 +444,17 @@ bool takes_resident(const ptq_linear *h, int m_tiles, int n_tiles)
     return h->k_blocks <= kShortMainLoop && static_cast<long long>(m_tiles) * n_tiles >= kResidentMinRounds * h->num_sms;
 }
 
+// N tiles per unit of the kernel with resident weights: all of them where their weights fit in shared memory and the busiest CTA gets no more
+// tiles, else one.  A row panel's codes are then loaded once, and its output is written as whole rows at a time.  Both kernels, us, one / all:
+// 200704 x 96 -> 384 43.8 / 38.6, 50176 x 128 -> 512 17.6 / 16.5, the same asymmetric 20.8 / 20.4, 50176 x 96 -> 384 14.2 / 13.7; with a tile more for the
+// busiest CTA 100352 x 96 -> 384 (11 / 12 tiles) 22.1 / 22.6.  Some of them gain nothing: 50176 x 48 -> 1000 in pairs of four 36.9 / 36.7.
+int resident_group(const ptq_linear *h, const ptq::GemmParams &p)
+{
+    const long long sms = h->num_sms, tiles = static_cast<long long>(p.m_tiles) * p.n_tiles;
+    if (p.n_tiles == 1 || ptq::res_smem_bytes(p.k_blocks, p.n_tiles, p.BN, p.vectors) > ptq::kResSmemMax) return 1;
+    return (p.m_tiles + sms - 1) / sms * p.n_tiles <= (tiles + sms - 1) / sms ? p.n_tiles : 1;
+}
+
 // Cycles of one tile of `cols` columns in the streaming kernel, as fitted to timings of 24 shapes at all widths: an MMA of K = 32
 // takes 35 + 0.52 cols; the eight epilogue warps take 360 per tile and 670 per pair of 64-column steps.
 double mma_cycles(const ptq_linear *h, int cols) { return (h->K + 31) / 32 * (35.0 + 0.52 * cols); }
@@ -652,10 +663,15 @@ ptq_status_t launch_gemm(const ptq_linear *h, const void *codes, long long M, vo
         if (tiling.resident) {
             constexpr auto kKern = ptq::ptq_gemm_dequant_resident_kernel<kDbg, kAsym>;
             p.fd_n_tiles = ptq::make_fastdiv(static_cast<unsigned>(p.m_tiles));
+            p.group = resident_group(h, p);
+            p.groups = (p.n_tiles + p.group - 1) / p.group;
+            const long long units = static_cast<long long>(p.m_tiles) * p.groups;
+            const int rgrid = static_cast<int>(units < h->num_sms ? units : h->num_sms);
+            p.fd_groups = ptq::make_fastdiv(static_cast<unsigned>(rgrid));
             const ptq_status_t es = ensure_smem<kKern>(h->device, ptq::kResSmemMax);
             if (es != PTQ_OK) return es;
-            const int smem = ptq::res_smem_bytes(p.k_blocks, p.BN, p.vectors);
-            PTQ_CUDA(launch_pdl(kKern, grid, ptq::kGemmThreads, smem, stream, tmA, tmW, tmY, p));
+            const int smem = ptq::res_smem_bytes(p.k_blocks, p.group, p.BN, p.vectors);
+            PTQ_CUDA(launch_pdl(kKern, rgrid, ptq::kGemmThreads, smem, stream, tmA, tmW, tmY, p));
         } else if (cut) {
             constexpr auto kKern = ptq::ptq_gemm_dequant_kernel<kDbg, kAsym, ptq::GemmCutParams>;
             ptq::GemmCutParams cp;
@@ -907,6 +923,7 @@ ptq_status_t launch_short_k(const ptq_linear *h, const void *x, long long M, voi
     sp.ld_bytes = x_align % 16 == 0 ? 16 : x_align % 8 == 0 ? 8 : 2;
     const long long units = static_cast<long long>(p.m_tiles) * p.groups;
     const int grid = static_cast<int>(units < h->num_sms ? units : h->num_sms);
+    p.fd_groups = ptq::make_fastdiv(static_cast<unsigned>(grid));
     const int smem = ptq::short_k_smem_bytes(p.group * p.BN * ptq::kBK, p.vectors);
     auto go = [&](auto chunks, auto mode, auto debug) -> ptq_status_t {
         constexpr auto kKern = ptq::ptq_short_k_kernel<decltype(chunks)::value, decltype(mode)::value, decltype(debug)::value>;

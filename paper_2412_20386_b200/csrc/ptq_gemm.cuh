@@ -103,7 +103,7 @@ struct GemmParams {
     // units cover a panel; the weight ring has `b_stages` slots of `b_stage_bytes` (= BN * 128) each.
     int group, groups;
     int b_stages, b_stage_bytes;
-    FastDiv fd_T, fd_n_tiles, fd_groups;   // divisors T, n_tiles (resident kernel: m_tiles), groups
+    FastDiv fd_T, fd_n_tiles, fd_groups;   // divisors T, n_tiles, groups (kernels with resident weights: T, m_tiles, CTAs)
 };
 
 // --- epilogue helpers -------------------------------------------------------------------------
@@ -517,16 +517,46 @@ __device__ __forceinline__ bool team_all(bool pred, int team)
 }
 __device__ __forceinline__ void team_sync(int team) { asm volatile("bar.sync %0, 128;" ::"r"(1 + team) : "memory"); }
 
-// The CTA's tiles in the order the MMA thread produces them.  Tiles are numbered with the row tiles of an N tile adjacent;
-// with several N tiles a CTA takes a contiguous share, so that its weights change at most once or twice, with a single one it
-// strides over them, so that the CTAs read and write neighbouring rows at a time (200704 x 384 -> 96: 60.0 -> 58.5 us).
-struct TileCursor {
-    int tile, end, step, m_tiles;
-    FastDiv fd_m;
-    __device__ bool valid() const { return tile < end; }
-    __device__ void advance() { tile += step; }
-    __device__ int n_tile() const { return static_cast<int>(fd_div(static_cast<unsigned>(tile), fd_m)); }
-    __device__ int m_tile() const { return tile - n_tile() * m_tiles; }
+// The CTA's units (a row tile times a group of N tiles, numbered with the row tiles of a group adjacent) and, within a unit, its N
+// tiles.  With several groups a CTA takes a contiguous share, so that its weights change at most once or twice, with a single one it
+// strides over the units, so that the CTAs read and write neighbouring rows at a time (200704 x 384 -> 96: 60.0 -> 58.5 us).
+struct UnitCursor {
+    int unit, end, step, m, group_at, count, g;                // unit = group_at * m_tiles + m; N tile g of `count`
+    int m_tiles, n_tiles, group;
+    __device__ UnitCursor(const GemmParams &p) : g(0), m_tiles(p.m_tiles), n_tiles(p.n_tiles), group(p.group)
+    {
+        const int total = p.m_tiles * p.groups, grid = static_cast<int>(gridDim.x), cta = static_cast<int>(blockIdx.x);
+        const int share = static_cast<int>(fd_div(static_cast<unsigned>(total), p.fd_groups)), extra = total - share * grid;   // fd_groups: by the grid
+        const bool strided = p.groups == 1;
+        unit = strided ? cta : cta * share + min(cta, extra);
+        end = strided ? total : unit + share + (cta < extra ? 1 : 0);
+        step = strided ? grid : 1;
+        group_at = static_cast<int>(fd_div(static_cast<unsigned>(unit), p.fd_n_tiles));                                        // fd_n_tiles: by m_tiles
+        m = unit - group_at * m_tiles;
+        count = min(group, n_tiles - group_at * group);
+    }
+    __device__ bool valid() const { return unit < end; }
+    __device__ int grp() const { return group_at; }
+    __device__ int m_tile() const { return m; }
+    __device__ int n_tile() const { return group_at * group + g; }
+    __device__ int size() const { return count; }
+    __device__ void next_unit()
+    {
+        unit += step;
+        m += step;
+        if (m >= m_tiles) {                                    // several groups: step 1.  A single one: past the end
+            m -= m_tiles;
+            ++group_at;
+            count = min(group, n_tiles - group_at * group);
+        }
+    }
+    __device__ void advance()
+    {
+        if (++g == count) {
+            g = 0;
+            next_unit();
+        }
+    }
 };
 
 template <bool kDebugAcc, bool kAsym, class Cursor>
@@ -1141,6 +1171,14 @@ ptq_gemm_dequant_panel_kernel(const __grid_constant__ CUtensorMap tmA, const __g
 // 200704 x 96 -> 384: 43.2 -> 41.3 us; 200704 x 192 -> 384: 53.8 -> 52.2; 50176 x 192 -> 768: 24.2 -> 23.5; 25216 x 384 -> 1536:
 // 26.5 -> 26.1; 200704 x 64 -> 256: 33.5 -> 29-31.  The narrowest outputs gain nothing: 200704 x 192 -> 96: 32.8 -> 32.9.
 //
+// An SM writes 32 bytes per clock to L2 at most, whatever kind of store and however many SMs write (30.3 measured with all of them), and
+// its loads, 109 bytes per clock alone, take their time from the stores: fewer bytes in are more bytes out.
+//
+// Where the weights of ALL N tiles fit (K <= 128 mostly), the unit is a row panel with its N tiles in turn: the codes are loaded
+// once per panel and whole rows of y are written at a time (`group`; else 1).  200704 x 96 -> 384: 43.9 -> 36.2 us, 50176 x 128 -> 512 17.9 -> 16.8.
+// Part of that is the cursor, which steps without divisions: 25216 x 384 -> 1536 (group 1) 23.5 -> 23.2, 200704 x 192 -> 96 31.5 -> 31.0; what
+// loses is 200704 x 64 -> 256, 26.3 -> 26.6.
+//
 // Three stages of codes: two cost 2 to 10 % (200704 x 384 -> 96: 65 us, not 58.5), and with eight the loads run so far ahead
 // of the stores that 200704 x 192 -> 96 takes 34.0 us, not 33.0; the other shapes cannot tell three from eight.
 //
@@ -1149,13 +1187,13 @@ ptq_gemm_dequant_panel_kernel(const __grid_constant__ CUtensorMap tmA, const __g
 constexpr int kResMaxKBlocks = 3;
 constexpr int kResStages = 3;
 constexpr int kResNumBarriers = 2 * kResStages + 2 + 4;
-__host__ __device__ constexpr int res_smem_bytes(int k_blocks, int bn, int vectors)
+__host__ __device__ constexpr int res_smem_bytes(int k_blocks, int group, int bn, int vectors)
 {
-    return k_blocks * bn * kBK + kResStages * kATileBytes + 2 * kNumEpiWarps * kStreamStagingPerWarp + 2 * vectors * kScaleBufBytes +
+    return group * k_blocks * bn * kBK + kResStages * kATileBytes + 2 * kNumEpiWarps * kStreamStagingPerWarp + 2 * vectors * kScaleBufBytes +
            kResNumBarriers * 8 + 16;
 }
-constexpr int kResSmemMax = res_smem_bytes(kResMaxKBlocks, kMaxBN, 3);
-static_assert(kResSmemMax <= 232448, "resident kernel exceeds the shared memory of one CTA");
+constexpr int kResSmemMax = 232448;
+static_assert(res_smem_bytes(kResMaxKBlocks, 1, kMaxBN, 3) <= kResSmemMax, "resident kernel exceeds the shared memory of one CTA");
 
 template <bool kDebugAcc, bool kAsym>
 __global__ void __launch_bounds__(kGemmThreads, 1)
@@ -1170,7 +1208,8 @@ ptq_gemm_dequant_resident_kernel(const __grid_constant__ CUtensorMap tmA, const 
     }
     constexpr uint32_t nstages = kResStages;
     const uint32_t w_bytes = static_cast<uint32_t>(p.BN) * kBK;                   // one k-block of weights
-    const uint32_t a_off = static_cast<uint32_t>(p.k_blocks) * w_bytes;
+    const uint32_t w_tile_bytes = static_cast<uint32_t>(p.k_blocks) * w_bytes;
+    const uint32_t a_off = static_cast<uint32_t>(p.group) * w_tile_bytes;
     const uint32_t staging_off = a_off + nstages * kATileBytes;
     const uint32_t scale_off = staging_off + 2 * kNumEpiWarps * kStreamStagingPerWarp;
     const uint32_t bar_off = scale_off + 2 * p.vectors * kScaleBufBytes;
@@ -1213,39 +1252,34 @@ ptq_gemm_dequant_resident_kernel(const __grid_constant__ CUtensorMap tmA, const 
     const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_holder, 0);
     griddep_launch_dependents();         // the codes (and row steps) of the kernel before are read behind griddep_wait() only
 
-    const int total = p.m_tiles * p.n_tiles, grid = static_cast<int>(gridDim.x), cta = static_cast<int>(blockIdx.x);
-    const int share = total / grid, extra = total - share * grid;
-    TileCursor cur;
-    const bool strided = p.n_tiles == 1;
-    cur.tile = strided ? cta : cta * share + min(cta, extra);
-    cur.end = strided ? total : cur.tile + share + (cta < extra ? 1 : 0);
-    cur.step = strided ? grid : 1;
-    cur.m_tiles = p.m_tiles;
-    cur.fd_m = p.fd_n_tiles;
+    UnitCursor cur(p);
 
     if (warp == 0) {
         // ------------------------------------------------------------------ TMA producer
         if (cur.valid()) {
             uint32_t stage = 0, phase = 0, issued = 0, w_loads = 0;
-            int w_tile = -1;
-            auto load_weights = [&](int n_tile) {
-                mbar_arrive_expect_tx_warp(wfull_bar, static_cast<uint32_t>(p.k_blocks) * w_bytes);
-                for (int kb = 0; kb < p.k_blocks; ++kb)
-                    tma_load_2d_warp(base + static_cast<uint32_t>(kb) * w_bytes, &tmW, kb * kBK, n_tile * p.BN, wfull_bar);
-                w_tile = n_tile;
+            int held = -1;
+            auto load_weights = [&] {
+                const int n = cur.size();
+                held = cur.grp();
+                mbar_arrive_expect_tx_warp(wfull_bar, static_cast<uint32_t>(n) * w_tile_bytes);
+                for (int i = 0; i < n; ++i)
+                    for (int kb = 0; kb < p.k_blocks; ++kb)
+                        tma_load_2d_warp(base + static_cast<uint32_t>(i) * w_tile_bytes + static_cast<uint32_t>(kb) * w_bytes, &tmW, kb * kBK,
+                                         (held * p.group + i) * p.BN, wfull_bar);
                 ++w_loads;
             };
-            load_weights(cur.n_tile());                                          // parameters: before the dependency wait
+            load_weights();                                                      // parameters: before the dependency wait
             griddep_wait();
             bool ok = true;
-            for (; cur.valid() && ok; cur.advance()) {
-                const int n_tile = cur.n_tile(), m_tile = cur.m_tile();
-                if (n_tile != w_tile) {
+            for (; cur.valid() && ok; cur.next_unit()) {
+                const int m_tile = cur.m_tile();
+                if (cur.grp() != held) {
                     if (!mbar_wait_warp(wempty_bar, (w_loads - 1u) & 1u, abort_flag, p.status)) {
                         ok = false;
                         break;
                     }
-                    load_weights(n_tile);
+                    load_weights();
                 }
                 for (int kb = 0; kb < p.k_blocks; ++kb) {
                     if (!mbar_wait_warp(empty_bar(stage), phase ^ 1u, abort_flag, p.status)) {
@@ -1277,39 +1311,48 @@ ptq_gemm_dequant_resident_kernel(const __grid_constant__ CUtensorMap tmA, const 
         // ------------------------------------------------------------------ MMA issuer
         const uint32_t idesc = make_idesc_s8(kBM, p.BN, kAsym);
         uint32_t stage = 0, phase = 0, buf = 0, bphase = 0, w_uses = 0;
-        int w_tile = -1;
+        int held = -1;
         bool ok = true;
         while (cur.valid() && ok) {
-            const int n_tile = cur.n_tile();
-            if (n_tile != w_tile) {
+            const int n = cur.size();
+            if (cur.grp() != held) {
                 if (!mbar_wait_warp(wfull_bar, w_uses & 1u, abort_flag, p.status)) break;
-                w_tile = n_tile;
+                held = cur.grp();
                 ++w_uses;
             }
-            if (!mbar_wait_warp(tempty_bar(buf), bphase ^ 1u, abort_flag, p.status)) break;
-            tc_fence_after_sync();
-            const uint32_t d_tmem = tmem_base + buf * kMaxBN;
-            for (int kb = 0; kb < p.k_blocks; ++kb) {
-                if (!mbar_wait_warp(full_bar(stage), phase, abort_flag, p.status)) {
+            const uint32_t stage0 = stage, phase0 = phase;                       // of the unit's codes, read again for each of its N tiles
+            for (int i = 0; i < n && ok; ++i) {
+                if (!mbar_wait_warp(tempty_bar(buf), bphase ^ 1u, abort_flag, p.status)) {
                     ok = false;
                     break;
                 }
                 tc_fence_after_sync();
-                mma_i8_ss_kblock(d_tmem, make_smem_desc_sw128(base + a_off + stage * kATileBytes),
-                                 make_smem_desc_sw128(base + static_cast<uint32_t>(kb) * w_bytes), idesc, kb != 0 ? 1u : 0u,
-                                 kb == p.k_blocks - 1 ? p.last_mmas : kBK / 32);
-                mma_commit(empty_bar(stage));
-                if (++stage == nstages) {
-                    stage = 0;
-                    phase ^= 1u;
+                const uint32_t d_tmem = tmem_base + buf * kMaxBN, w_tile = base + static_cast<uint32_t>(i) * w_tile_bytes;
+                stage = stage0;
+                phase = phase0;
+                for (int kb = 0; kb < p.k_blocks; ++kb) {
+                    if (i == 0 && !mbar_wait_warp(full_bar(stage), phase, abort_flag, p.status)) {
+                        ok = false;
+                        break;
+                    }
+                    tc_fence_after_sync();
+                    mma_i8_ss_kblock(d_tmem, make_smem_desc_sw128(base + a_off + stage * kATileBytes),
+                                     make_smem_desc_sw128(w_tile + static_cast<uint32_t>(kb) * w_bytes), idesc, kb != 0 ? 1u : 0u,
+                                     kb == p.k_blocks - 1 ? p.last_mmas : kBK / 32);
+                    if (i == n - 1) mma_commit(empty_bar(stage));
+                    if (++stage == nstages) {
+                        stage = 0;
+                        phase ^= 1u;
+                    }
                 }
+                if (!ok) break;
+                mma_commit(tfull_bar(buf));      // accumulator complete
+                buf ^= 1u;
+                if (buf == 0u) bphase ^= 1u;
             }
             if (!ok) break;
-            mma_commit(tfull_bar(buf));          // accumulator complete
-            buf ^= 1u;
-            if (buf == 0u) bphase ^= 1u;
-            cur.advance();
-            if (cur.valid() && cur.n_tile() != w_tile) mma_commit(wempty_bar);   // the weights have been read for the last time
+            cur.next_unit();
+            if (cur.valid() && cur.grp() != held) mma_commit(wempty_bar);        // the weights have been read for the last time
         }
     } else {
         // ------------------------------------------------------------------ epilogue warps, two teams

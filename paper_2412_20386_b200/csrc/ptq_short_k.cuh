@@ -45,25 +45,6 @@ struct ShortKParams {
     int ld_bytes;         // bytes per load of x: 16, 8 or 2 (alignment of its rows)
 };
 
-// The CTA's units (numbered with the row tiles of a group adjacent) and, within a unit, its N tiles.
-struct UnitCursor {
-    int unit, end, step, m_tiles, n_tiles, group, g;
-    FastDiv fd_m;
-    __device__ bool valid() const { return unit < end; }
-    __device__ int grp() const { return static_cast<int>(fd_div(static_cast<unsigned>(unit), fd_m)); }
-    __device__ int m_tile() const { return unit - grp() * m_tiles; }
-    __device__ int n_tile() const { return grp() * group + g; }
-    __device__ int size() const { return min(group, n_tiles - grp() * group); }
-    __device__ void next_unit() { unit += step; }
-    __device__ void advance()
-    {
-        if (++g == size()) {
-            g = 0;
-            next_unit();
-        }
-    }
-};
-
 // kChunks: chunks of 8 channels per row, at most (K <= 8 kChunks).
 template <int kChunks, int kMode, bool kDebugAcc>
 __global__ void __launch_bounds__(kShortKThreads, 1)
@@ -127,18 +108,7 @@ ptq_short_k_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constan
     const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_holder, 0);
     griddep_launch_dependents();
 
-    const int total = p.m_tiles * p.groups, grid = static_cast<int>(gridDim.x), cta = static_cast<int>(blockIdx.x);
-    const int share = total / grid, extra = total - share * grid;
-    const bool strided = p.groups == 1;                        // see TileCursor
-    UnitCursor cur;
-    cur.unit = strided ? cta : cta * share + min(cta, extra);
-    cur.end = strided ? total : cur.unit + share + (cta < extra ? 1 : 0);
-    cur.step = strided ? grid : 1;
-    cur.m_tiles = p.m_tiles;
-    cur.n_tiles = p.n_tiles;
-    cur.group = p.group;
-    cur.g = 0;
-    cur.fd_m = p.fd_n_tiles;
+    UnitCursor cur(p);
 
     if (warp == 0) {
         // ------------------------------------------------------------------ TMA producer of the weights (parameters: no dependency wait)

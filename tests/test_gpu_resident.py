@@ -30,6 +30,12 @@ def env():
     (40, 60000, 67, 3, False, False),      # two row tiles: a share crosses several N tiles
     (384, 58000, 64, 4, False, True),
     (256, 16, 7, 8121, False, False),      # a single 16-column step per tile
+    # the weights of all N tiles at once, row panels as units: two and three N tiles (of a panel's odd number each team has the other half of
+    # the tiles in the next panel), last tiles and panels that are not full, two k-blocks
+    (96, 384, 784, 48, False, False),
+    (128, 488, 37, 1024, True, False),
+    (33, 648, 197, 192, False, True),
+    (200, 264, 50, 740, True, False),
 ])
 def test_resident_weights(env, K, N, T, B, bias, asym):
     ptq, torch = env
