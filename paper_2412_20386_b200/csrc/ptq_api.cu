@@ -455,6 +455,18 @@ int resident_group(const ptq_linear *h, const ptq::GemmParams &p)
     return (p.m_tiles + sms - 1) / sms * p.n_tiles <= (tiles + sms - 1) / sms ? p.n_tiles : 1;
 }
 
+// The order of a kernel with resident weights: a CTA keeps to one group of N tiles and strides over the row tiles, so that neighbouring CTAs
+// write the pieces of the same rows at about the same time, unless the busiest CTA would get more than with contiguous shares.  Both kernels, us,
+// contiguous shares (all rows of a group, then the next group) / spread: 50176 x 48 -> 1000 37.3 / 28.1 and 50176 x 384 -> 1000 asymmetric 45.7 / 41.0 (rows
+// of 2000 bytes: pieces that end inside a 32-byte sector reached DRAM separately), 100352 x 96 -> 384 22.4 / 21.3, 50176 x 256 -> 512 20.1 / 19.6,
+// 50176 x 192 -> 768 21.43 / 21.36.  Nine units for the busiest CTA instead of eight: 25216 x 384 -> 1536 23.2 / 24.0, so not.
+void set_spread(ptq::GemmParams &p, int grid)
+{
+    const int ctas = grid / p.groups;                    // of a group, at least
+    p.spread = ctas >= 1 && (p.m_tiles + ctas - 1) / ctas <= (static_cast<long long>(p.m_tiles) * p.groups + grid - 1) / grid;
+    p.fd_spread = ptq::make_fastdiv(static_cast<unsigned>(p.groups));
+}
+
 // Cycles of one tile of `cols` columns in the streaming kernel, as fitted to timings of 24 shapes at all widths: an MMA of K = 32
 // takes 35 + 0.52 cols; the eight epilogue warps take 360 per tile and 670 per pair of 64-column steps.
 double mma_cycles(const ptq_linear *h, int cols) { return (h->K + 31) / 32 * (35.0 + 0.52 * cols); }
@@ -668,6 +680,7 @@ ptq_status_t launch_gemm(const ptq_linear *h, const void *codes, long long M, vo
             const long long units = static_cast<long long>(p.m_tiles) * p.groups;
             const int rgrid = static_cast<int>(units < h->num_sms ? units : h->num_sms);
             p.fd_groups = ptq::make_fastdiv(static_cast<unsigned>(rgrid));
+            set_spread(p, rgrid);
             const ptq_status_t es = ensure_smem<kKern>(h->device, ptq::kResSmemMax);
             if (es != PTQ_OK) return es;
             const int smem = ptq::res_smem_bytes(p.k_blocks, p.group, p.BN, p.vectors);
@@ -924,6 +937,7 @@ ptq_status_t launch_short_k(const ptq_linear *h, const void *x, long long M, voi
     const long long units = static_cast<long long>(p.m_tiles) * p.groups;
     const int grid = static_cast<int>(units < h->num_sms ? units : h->num_sms);
     p.fd_groups = ptq::make_fastdiv(static_cast<unsigned>(grid));
+    set_spread(p, grid);
     const int smem = ptq::short_k_smem_bytes(p.group * p.BN * ptq::kBK, p.vectors);
     auto go = [&](auto chunks, auto mode, auto debug) -> ptq_status_t {
         constexpr auto kKern = ptq::ptq_short_k_kernel<decltype(chunks)::value, decltype(mode)::value, decltype(debug)::value>;

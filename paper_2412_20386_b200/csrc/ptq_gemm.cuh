@@ -103,6 +103,8 @@ struct GemmParams {
     // units cover a panel; the weight ring has `b_stages` slots of `b_stage_bytes` (= BN * 128) each.
     int group, groups;
     int b_stages, b_stage_bytes;
+    int spread;            // kernels with resident weights: every CTA keeps to one group of N tiles and strides over the row tiles
+    FastDiv fd_spread;
     FastDiv fd_T, fd_n_tiles, fd_groups;   // divisors T, n_tiles, groups (kernels with resident weights: T, m_tiles, CTAs)
 };
 
@@ -501,9 +503,10 @@ __device__ __forceinline__ RowStep load_row_step(const GemmParams &p, int m_tile
 // 18.3 us instead of 18.2, and in the few-channels kernel 12608 x 12 -> 384 5.66 instead of 5.52, 50432 x 24 -> 768 16.7 instead of 16.0.
 __device__ __forceinline__ void team_sync(int team) { asm volatile("bar.sync %0, 128;" ::"r"(1 + team) : "memory"); }
 
-// The CTA's units (a row tile times a group of N tiles, numbered with the row tiles of a group adjacent) and, within a unit, its N
-// tiles.  With several groups a CTA takes a contiguous share, so that its weights change at most once or twice, with a single one it
-// strides over the units, so that the CTAs read and write neighbouring rows at a time (200704 x 384 -> 96: 60.0 -> 58.5 us).
+// The CTA's units (a row tile times a group of N tiles) and, within a unit, its N tiles.  `spread`: the CTA keeps to the group of its number and
+// strides over the row tiles, so that the CTAs read and write neighbouring rows at a time (a single group is always so: 200704 x 384 -> 96 60.0 ->
+// 58.5 us).  Else the units are numbered with the row tiles of a group adjacent and the CTA takes a contiguous share: its weights change at most
+// once or twice.
 struct UnitCursor {
     int unit, end, step, m, group_at, count, g;                // unit = group_at * m_tiles + m; N tile g of `count`
     int m_tiles, n_tiles, group;
@@ -511,12 +514,19 @@ struct UnitCursor {
     {
         const int total = p.m_tiles * p.groups, grid = static_cast<int>(gridDim.x), cta = static_cast<int>(blockIdx.x);
         const int share = static_cast<int>(fd_div(static_cast<unsigned>(total), p.fd_groups)), extra = total - share * grid;   // fd_groups: by the grid
-        const bool strided = p.groups == 1;
-        unit = strided ? cta : cta * share + min(cta, extra);
-        end = strided ? total : unit + share + (cta < extra ? 1 : 0);
-        step = strided ? grid : 1;
-        group_at = static_cast<int>(fd_div(static_cast<unsigned>(unit), p.fd_n_tiles));                                        // fd_n_tiles: by m_tiles
-        m = unit - group_at * m_tiles;
+        if (p.spread) {
+            const int lane = static_cast<int>(fd_div(static_cast<unsigned>(cta), p.fd_spread));                                // fd_spread: by the groups
+            group_at = cta - lane * p.groups;
+            unit = m = lane;
+            end = m_tiles;
+            step = (grid - group_at + p.groups - 1) / p.groups;
+        } else {
+            unit = cta * share + min(cta, extra);
+            end = unit + share + (cta < extra ? 1 : 0);
+            step = 1;
+            group_at = static_cast<int>(fd_div(static_cast<unsigned>(unit), p.fd_n_tiles));                                    // fd_n_tiles: by m_tiles
+            m = unit - group_at * m_tiles;
+        }
         count = min(group, n_tiles - group_at * group);
     }
     __device__ bool valid() const { return unit < end; }
