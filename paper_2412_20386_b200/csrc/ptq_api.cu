@@ -455,16 +455,30 @@ int resident_group(const ptq_linear *h, const ptq::GemmParams &p)
     return (p.m_tiles + sms - 1) / sms * p.n_tiles <= (tiles + sms - 1) / sms ? p.n_tiles : 1;
 }
 
-// The order of a kernel with resident weights: a CTA keeps to one group of N tiles and strides over the row tiles, so that neighbouring CTAs
-// write the pieces of the same rows at about the same time, unless the busiest CTA would get more than with contiguous shares.  Both kernels, us,
-// contiguous shares (all rows of a group, then the next group) / spread: 50176 x 48 -> 1000 37.3 / 28.1 and 50176 x 384 -> 1000 asymmetric 45.7 / 41.0 (rows
-// of 2000 bytes: pieces that end inside a 32-byte sector reached DRAM separately), 100352 x 96 -> 384 22.4 / 21.3, 50176 x 256 -> 512 20.1 / 19.6,
-// 50176 x 192 -> 768 21.43 / 21.36.  Nine units for the busiest CTA instead of eight: 25216 x 384 -> 1536 23.2 / 24.0, so not.
-void set_spread(ptq::GemmParams &p, int grid)
+// The order of a kernel with resident weights on `grid` CTAs: as many CTAs as make whole sets of groups keep to one group each and stride over the
+// row tiles, so that neighbouring CTAs write the pieces of the same rows at about the same time; the few CTAs that are over take the row
+// tiles that are left.  Contiguous shares for all where the busiest CTA would get more so.  Both kernels, us, contiguous shares (all
+// rows of a group, then the next group) / spread: 50176 x 48 -> 1000 37.3 / 28.1 and 50176 x 384 -> 1000 asymmetric 45.7 / 41.0 (rows of 2000 bytes: pieces
+// that end inside a 32-byte sector reached DRAM separately), 100352 x 96 -> 384 22.4 / 21.3, 50176 x 256 -> 512 20.1 / 19.6; with row
+// tiles left over 18816 x 384 -> 1536 19.3 / 18.7, 50432 x 24 -> 768 16.0 / 15.2, 25216 x 384 -> 1536 23.0 / 23.0, 25807 x 376 -> 1504 25.3 / 25.4.
+void set_units(ptq::GemmParams &p, int grid)
 {
-    const int ctas = grid / p.groups;                    // of a group, at least
-    p.spread = ctas >= 1 && (p.m_tiles + ctas - 1) / ctas <= (static_cast<long long>(p.m_tiles) * p.groups + grid - 1) / grid;
+    const long long total = static_cast<long long>(p.m_tiles) * p.groups;
+    const int rounds = static_cast<int>((total + grid - 1) / grid), ctas = grid / p.groups, over = grid - ctas * p.groups;
+    long long rows = static_cast<long long>(ctas) * rounds;                            // that the spread CTAs take
+    if (rows > p.m_tiles) rows = p.m_tiles;
+    const long long left = (p.m_tiles - rows) * p.groups;
+    const bool spread = ctas >= 1 && left <= static_cast<long long>(over) * rounds;
+    p.spread = spread ? ctas * p.groups : 0;
+    p.spread_rows = spread ? static_cast<int>(rows) : 0;
+    p.spread_step = spread ? ctas : 1;
+    const long long rest = spread ? left : total;
+    const int rest_ctas = grid - p.spread;
+    p.rest_share = rest_ctas > 0 ? static_cast<int>(rest / rest_ctas) : 0;
+    p.rest_extra = rest_ctas > 0 ? static_cast<int>(rest % rest_ctas) : 0;
     p.fd_spread = ptq::make_fastdiv(static_cast<unsigned>(p.groups));
+    const int rest_rows = p.m_tiles - p.spread_rows;
+    p.fd_n_tiles = ptq::make_fastdiv(static_cast<unsigned>(rest_rows > 0 ? rest_rows : 1));
 }
 
 // Cycles of one tile of `cols` columns in the streaming kernel, as fitted to timings of 24 shapes at all widths: an MMA of K = 32
@@ -674,13 +688,11 @@ ptq_status_t launch_gemm(const ptq_linear *h, const void *codes, long long M, vo
         constexpr bool kDbg = decltype(debug)::value, kAsym = decltype(asym)::value;
         if (tiling.resident) {
             constexpr auto kKern = ptq::ptq_gemm_dequant_resident_kernel<kDbg, kAsym>;
-            p.fd_n_tiles = ptq::make_fastdiv(static_cast<unsigned>(p.m_tiles));
             p.group = resident_group(h, p);
             p.groups = (p.n_tiles + p.group - 1) / p.group;
             const long long units = static_cast<long long>(p.m_tiles) * p.groups;
             const int rgrid = static_cast<int>(units < h->num_sms ? units : h->num_sms);
-            p.fd_groups = ptq::make_fastdiv(static_cast<unsigned>(rgrid));
-            set_spread(p, rgrid);
+            set_units(p, rgrid);
             const ptq_status_t es = ensure_smem<kKern>(h->device, ptq::kResSmemMax);
             if (es != PTQ_OK) return es;
             const int smem = ptq::res_smem_bytes(p.k_blocks, p.group, p.BN, p.vectors);
@@ -927,7 +939,6 @@ ptq_status_t launch_short_k(const ptq_linear *h, const void *x, long long M, voi
             p.groups = groups;
         }
     }
-    p.fd_n_tiles = ptq::make_fastdiv(static_cast<unsigned>(p.m_tiles));
     sp.x = static_cast<const __half *>(x);
     sp.s = h->d_s;
     sp.rs = h->d_rs;
@@ -936,8 +947,7 @@ ptq_status_t launch_short_k(const ptq_linear *h, const void *x, long long M, voi
     sp.ld_bytes = x_align % 16 == 0 ? 16 : x_align % 8 == 0 ? 8 : 2;
     const long long units = static_cast<long long>(p.m_tiles) * p.groups;
     const int grid = static_cast<int>(units < h->num_sms ? units : h->num_sms);
-    p.fd_groups = ptq::make_fastdiv(static_cast<unsigned>(grid));
-    set_spread(p, grid);
+    set_units(p, grid);
     const int smem = ptq::short_k_smem_bytes(p.group * p.BN * ptq::kBK, p.vectors);
     auto go = [&](auto chunks, auto mode, auto debug) -> ptq_status_t {
         constexpr auto kKern = ptq::ptq_short_k_kernel<decltype(chunks)::value, decltype(mode)::value, decltype(debug)::value>;

@@ -103,9 +103,9 @@ struct GemmParams {
     // units cover a panel; the weight ring has `b_stages` slots of `b_stage_bytes` (= BN * 128) each.
     int group, groups;
     int b_stages, b_stage_bytes;
-    int spread;            // kernels with resident weights: every CTA keeps to one group of N tiles and strides over the row tiles
+    int spread, spread_rows, spread_step, rest_share, rest_extra;   // kernels with resident weights: see UnitCursor
     FastDiv fd_spread;
-    FastDiv fd_T, fd_n_tiles, fd_groups;   // divisors T, n_tiles, groups (kernels with resident weights: T, m_tiles, CTAs)
+    FastDiv fd_T, fd_n_tiles, fd_groups;   // divisors T, n_tiles (kernels with resident weights: see UnitCursor), groups
 };
 
 // --- epilogue helpers -------------------------------------------------------------------------
@@ -503,29 +503,29 @@ __device__ __forceinline__ RowStep load_row_step(const GemmParams &p, int m_tile
 // 18.3 us instead of 18.2, and in the few-channels kernel 12608 x 12 -> 384 5.66 instead of 5.52, 50432 x 24 -> 768 16.7 instead of 16.0.
 __device__ __forceinline__ void team_sync(int team) { asm volatile("bar.sync %0, 128;" ::"r"(1 + team) : "memory"); }
 
-// The CTA's units (a row tile times a group of N tiles) and, within a unit, its N tiles.  `spread`: the CTA keeps to the group of its number and
-// strides over the row tiles, so that the CTAs read and write neighbouring rows at a time (a single group is always so: 200704 x 384 -> 96 60.0 ->
-// 58.5 us).  Else the units are numbered with the row tiles of a group adjacent and the CTA takes a contiguous share: its weights change at most
-// once or twice.
+// The CTA's units (a row tile times a group of N tiles) and, within a unit, its N tiles.  The first `spread` CTAs keep to the group of their
+// number and stride over the first `spread_rows` row tiles, so that the CTAs read and write neighbouring rows at a time (a single group
+// is always so: 200704 x 384 -> 96 60.0 -> 58.5 us).  The other CTAs take contiguous shares of what is left (of everything, where
+// nothing is spread), numbered with the row tiles of a group adjacent: their weights change once or twice.
 struct UnitCursor {
-    int unit, end, step, m, group_at, count, g;                // unit = group_at * m_tiles + m; N tile g of `count`
-    int m_tiles, n_tiles, group;
-    __device__ UnitCursor(const GemmParams &p) : g(0), m_tiles(p.m_tiles), n_tiles(p.n_tiles), group(p.group)
+    int unit, end, step, m, group_at, count, g;                // N tile g of the `count` of unit (group_at, m)
+    int m_begin, m_tiles, n_tiles, group;
+    __device__ UnitCursor(const GemmParams &p) : g(0), m_begin(p.spread_rows), m_tiles(p.m_tiles), n_tiles(p.n_tiles), group(p.group)
     {
-        const int total = p.m_tiles * p.groups, grid = static_cast<int>(gridDim.x), cta = static_cast<int>(blockIdx.x);
-        const int share = static_cast<int>(fd_div(static_cast<unsigned>(total), p.fd_groups)), extra = total - share * grid;   // fd_groups: by the grid
-        if (p.spread) {
-            const int lane = static_cast<int>(fd_div(static_cast<unsigned>(cta), p.fd_spread));                                // fd_spread: by the groups
+        const int cta = static_cast<int>(blockIdx.x);
+        if (cta < p.spread) {
+            const int lane = static_cast<int>(fd_div(static_cast<unsigned>(cta), p.fd_spread));      // fd_spread: by the groups
             group_at = cta - lane * p.groups;
             unit = m = lane;
-            end = m_tiles;
-            step = (grid - group_at + p.groups - 1) / p.groups;
+            end = m_begin;
+            step = p.spread_step;
         } else {
-            unit = cta * share + min(cta, extra);
-            end = unit + share + (cta < extra ? 1 : 0);
+            const int rows = m_tiles - m_begin, at = cta - p.spread;
+            unit = at * p.rest_share + min(at, p.rest_extra);
+            end = unit + p.rest_share + (at < p.rest_extra ? 1 : 0);
             step = 1;
-            group_at = static_cast<int>(fd_div(static_cast<unsigned>(unit), p.fd_n_tiles));                                    // fd_n_tiles: by m_tiles
-            m = unit - group_at * m_tiles;
+            group_at = static_cast<int>(fd_div(static_cast<unsigned>(unit), p.fd_n_tiles));          // fd_n_tiles: by the rows that are left
+            m = m_begin + unit - group_at * rows;
         }
         count = min(group, n_tiles - group_at * group);
     }
@@ -538,8 +538,8 @@ struct UnitCursor {
     {
         unit += step;
         m += step;
-        if (m >= m_tiles) {                                    // several groups: step 1.  A single one: past the end
-            m -= m_tiles;
+        if (m >= m_tiles) {                                    // of a contiguous share: the next group (spread: past the end)
+            m = m_begin;
             ++group_at;
             count = min(group, n_tiles - group_at * group);
         }

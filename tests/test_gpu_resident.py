@@ -36,7 +36,7 @@ def env():
     (128, 488, 37, 1024, True, False),
     (33, 648, 197, 192, False, True),
     (200, 264, 50, 740, True, False),
-    (64, 1536, 197, 128, False, False),    # six N tiles that 148 CTAs do not share evenly: contiguous shares
+    (64, 1536, 197, 128, False, False),    # six N tiles: 24 CTAs on each, and four that share the row tiles that are left
     (104, 1000, 70, 301, True, False),     # four N tiles, every CTA on one: 37 CTAs each, rows of 2000 bytes
 ])
 def test_resident_weights(env, K, N, T, B, bias, asym):
