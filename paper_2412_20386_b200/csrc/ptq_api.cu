@@ -433,15 +433,19 @@ bool plan_panel(const ptq_linear *h, ptq::GemmParams &p, bool tma_store)
     return true;
 }
 
-// Whether the kernel with resident weights (and its epilogue in two teams) is taken: short main loop (K <= 384) and three tiles
-// per CTA (and TMA stores).  GEMM kernel alone, us, streaming / resident.  Below three the streaming kernel's shorter latency of a tile wins
-// mostly: 25088 x 384 -> 192 (1.3 tiles per CTA) 5.3 / 5.4, 12608 x 192 -> 768 (2.0) 6.6 / 6.8, 6304 x 384 -> 1536 (2.0) 7.1 / 7.6; at 2.7 it
-// depends, 6304 x 384 -> 1536 in 192 columns 6.8 / 7.2, 50176 x 384 -> 192 8.7 / 8.4.  With four and more this one does: 12544 x 384 -> 1536 10.8 /
-// 10.4, 25088 x 192 -> 768 9.55 / 9.2, 25216 x 384 -> 1536 18.9 / 17.3.
-constexpr long long kResidentMinRounds = 3;
+// Whether the kernel with resident weights (and its epilogue in two teams) is taken: short main loop (K <= 384) and TMA stores.  Symmetric layers
+// from more than one tile for the busiest CTA: against the streaming kernel below three, 116 random layers with 1 to 14 tiles per CTA
+// (33 <= K <= 384), each replayed alone, take 0.957 of the time, 18321 x 298 -> 592 17.4 / 15.4 us, 50176 x 384 -> 192 17.4 / 16.8, 12608 x 192 -> 768 9.78 /
+// 9.43; slower by more than 1 %: 10047 x 64 -> 1176 9.73 / 9.90 and 17927 x 48 -> 96 6.41 / 6.50.  Among other layers less of it is left, because
+// every further kernel in turn has to be fetched into the SMs again: in_proj and out_proj of Vim-Ti at batch 64 take 18.6 us with both
+// in one kernel and 19.1 with one in each.  So a layer of one tile per CTA, which alone does not gain, takes it where there are rows enough that the
+// other layers on them do; with few rows the long ones run in the streaming kernel (788 x 384 -> 1536 among 768 -> 56, 24 -> 768 and 768 -> 384,
+// twice: 41.8 us in the streaming kernel, 42.3).  Asymmetric layers from three tiles: 6304 x 384 -> 1536 alone 12.2 / 11.9, but with 6304 x 768 -> 384
+// behind it 24.4 / 24.55.
 bool takes_resident(const ptq_linear *h, int m_tiles, int n_tiles)
 {
-    return h->k_blocks <= kShortMainLoop && static_cast<long long>(m_tiles) * n_tiles >= kResidentMinRounds * h->num_sms;
+    const long long tiles = static_cast<long long>(m_tiles) * n_tiles;
+    return h->k_blocks <= kShortMainLoop && (h->asym ? tiles >= 3ll * h->num_sms : tiles > h->num_sms || 2ll * m_tiles >= h->num_sms);
 }
 
 // N tiles per unit of the kernel with resident weights: all of them where their weights fit in shared memory and the busiest CTA gets no more
@@ -461,7 +465,7 @@ int resident_group(const ptq_linear *h, const ptq::GemmParams &p)
 // rows of a group, then the next group) / spread: 50176 x 48 -> 1000 37.3 / 28.1 and 50176 x 384 -> 1000 asymmetric 45.7 / 41.0 (rows of 2000 bytes: pieces
 // that end inside a 32-byte sector reached DRAM separately), 100352 x 96 -> 384 22.4 / 21.3, 50176 x 256 -> 512 20.1 / 19.6; with row
 // tiles left over 18816 x 384 -> 1536 19.3 / 18.7, 50432 x 24 -> 768 16.0 / 15.2, 25216 x 384 -> 1536 23.0 / 23.0, 25807 x 376 -> 1504 25.3 / 25.4.
-void set_units(ptq::GemmParams &p, int grid)
+void set_units(ptq::UnitParams &p, int grid)
 {
     const long long total = static_cast<long long>(p.m_tiles) * p.groups;
     const int rounds = static_cast<int>((total + grid - 1) / grid), ctas = grid / p.groups, over = grid - ctas * p.groups;
@@ -527,16 +531,21 @@ double gemm_cycles(const ptq_linear *h, const ptq::GemmParams &p, int bn)
 // 384 keeps 192 columns, 5.0, where 128 with a cut round take 4.5, and 6304 x 384 -> 192 takes 128, 3.4, where 64 take 3.1.  Whole forward passes of 1536
 // random layers, every width: the chosen one 0.4 % above the best on average; the furthest off 1078 x 46 -> 3072 with a bias (192 columns, 7.7,
 // where 256 take 6.9), 13867 x 298 -> 384 (128, 15.2, where 192 take 14.1) and 5047 x 576 -> 600 dynamic (128, cut, 14.0, where 256 take 13.0).  Wider
-// margins, less belief in the cut and a second round forbidden were tried on them: each slows as many layers as it mends.  Widths that lead to
-// the resident kernel are not compared: with several rounds and a short main loop the widths are within 3 % of one another either way.
+// margins, less belief in the cut and a second round forbidden were tried on them: each slows as many layers as it mends.  With a
+// short main loop and three rounds or more the widths are not compared: they are within 3 % of one another either way.  With fewer the
+// kernel with resident weights takes the width chosen here (116 random layers: 1.3 % above the best of the four widths on average; furthest off
+// 14578 x 320 -> 640 asymmetric, 256 columns 14.9 where 128 take 12.6).
+constexpr long long kOwnWidthRounds = 3;
 int choose_bn(const ptq_linear *h, const ptq::GemmParams &p)
 {
-    auto resident = [&](int bn) { return takes_resident(h, p.m_tiles, (h->N + bn - 1) / bn); };
+    auto many = [&](int bn) {
+        return h->k_blocks <= kShortMainLoop && static_cast<long long>(p.m_tiles) * ((h->N + bn - 1) / bn) >= kOwnWidthRounds * h->num_sms;
+    };
     int best = h->BN;
-    if (resident(best)) return best;
+    if (many(best)) return best;
     double best_cost = 0.975 * gemm_cycles(h, p, best);
     for (int bn = 64; bn <= ptq::kMaxBN && bn < h->N + 64; bn += 64) {
-        if (resident(bn)) continue;
+        if (many(bn)) continue;
         const double cost = gemm_cycles(h, p, bn);
         if (cost < best_cost) {
             best = bn;
@@ -688,15 +697,17 @@ ptq_status_t launch_gemm(const ptq_linear *h, const void *codes, long long M, vo
         constexpr bool kDbg = decltype(debug)::value, kAsym = decltype(asym)::value;
         if (tiling.resident) {
             constexpr auto kKern = ptq::ptq_gemm_dequant_resident_kernel<kDbg, kAsym>;
-            p.group = resident_group(h, p);
-            p.groups = (p.n_tiles + p.group - 1) / p.group;
-            const long long units = static_cast<long long>(p.m_tiles) * p.groups;
+            ptq::UnitParams rp;
+            static_cast<ptq::GemmParams &>(rp) = p;
+            rp.group = resident_group(h, p);
+            rp.groups = (p.n_tiles + rp.group - 1) / rp.group;
+            const long long units = static_cast<long long>(p.m_tiles) * rp.groups;
             const int rgrid = static_cast<int>(units < h->num_sms ? units : h->num_sms);
-            set_units(p, rgrid);
+            set_units(rp, rgrid);
             const ptq_status_t es = ensure_smem<kKern>(h->device, ptq::kResSmemMax);
             if (es != PTQ_OK) return es;
-            const int smem = ptq::res_smem_bytes(p.k_blocks, p.group, p.BN, p.vectors);
-            PTQ_CUDA(launch_pdl(kKern, rgrid, ptq::kGemmThreads, smem, stream, tmA, tmW, tmY, p));
+            const int smem = ptq::res_smem_bytes(p.k_blocks, rp.group, p.BN, p.vectors);
+            PTQ_CUDA(launch_pdl(kKern, rgrid, ptq::kGemmThreads, smem, stream, tmA, tmW, tmY, rp));
         } else if (cut) {
             constexpr auto kKern = ptq::ptq_gemm_dequant_kernel<kDbg, kAsym, ptq::GemmCutParams>;
             ptq::GemmCutParams cp;
@@ -926,7 +937,7 @@ ptq_status_t launch_short_k(const ptq_linear *h, const void *x, long long M, voi
                                     static_cast<unsigned long long>(M), static_cast<unsigned long long>(h->N) * 2, ptq::kStreamBoxCols, 32);
     if (st != PTQ_OK) return st;
     ptq::ShortKParams sp;
-    ptq::GemmParams &p = sp.g;
+    ptq::UnitParams &p = sp.g;
     set_gemm_params(h, p, M, y, acc_out, true, nullptr);
     // N tiles per unit: the number that leaves the busiest CTA the fewest tiles; the larger one (rows quantized less often) if equal
     long long fewest = 0;

@@ -103,9 +103,7 @@ struct GemmParams {
     // units cover a panel; the weight ring has `b_stages` slots of `b_stage_bytes` (= BN * 128) each.
     int group, groups;
     int b_stages, b_stage_bytes;
-    int spread, spread_rows, spread_step, rest_share, rest_extra;   // kernels with resident weights: see UnitCursor
-    FastDiv fd_spread;
-    FastDiv fd_T, fd_n_tiles, fd_groups;   // divisors T, n_tiles (kernels with resident weights: see UnitCursor), groups
+    FastDiv fd_T, fd_n_tiles, fd_groups;   // divisors T, n_tiles, groups
 };
 
 // --- epilogue helpers -------------------------------------------------------------------------
@@ -507,14 +505,18 @@ __device__ __forceinline__ void team_sync(int team) { asm volatile("bar.sync %0,
 // number and stride over the first `spread_rows` row tiles, so that the CTAs read and write neighbouring rows at a time (a single group
 // is always so: 200704 x 384 -> 96 60.0 -> 58.5 us).  The other CTAs take contiguous shares of what is left (of everything, where
 // nothing is spread), numbered with the row tiles of a group adjacent: their weights change once or twice.
+struct UnitParams : GemmParams {       // only where they are used: parameters that a launch carries for nothing cost 0.4 to 1.3 % of a small layer
+    int spread, spread_rows, spread_step, rest_share, rest_extra;
+    FastDiv fd_spread;                 // divisor groups; fd_n_tiles divides by the row tiles that are left
+};
 struct UnitCursor {
     int unit, end, step, m, group_at, count, g;                // N tile g of the `count` of unit (group_at, m)
     int m_begin, m_tiles, n_tiles, group;
-    __device__ UnitCursor(const GemmParams &p) : g(0), m_begin(p.spread_rows), m_tiles(p.m_tiles), n_tiles(p.n_tiles), group(p.group)
+    __device__ UnitCursor(const UnitParams &p) : g(0), m_begin(p.spread_rows), m_tiles(p.m_tiles), n_tiles(p.n_tiles), group(p.group)
     {
         const int cta = static_cast<int>(blockIdx.x);
         if (cta < p.spread) {
-            const int lane = static_cast<int>(fd_div(static_cast<unsigned>(cta), p.fd_spread));      // fd_spread: by the groups
+            const int lane = static_cast<int>(fd_div(static_cast<unsigned>(cta), p.fd_spread));
             group_at = cta - lane * p.groups;
             unit = m = lane;
             end = m_begin;
@@ -524,7 +526,7 @@ struct UnitCursor {
             unit = at * p.rest_share + min(at, p.rest_extra);
             end = unit + p.rest_share + (at < p.rest_extra ? 1 : 0);
             step = 1;
-            group_at = static_cast<int>(fd_div(static_cast<unsigned>(unit), p.fd_n_tiles));          // fd_n_tiles: by the rows that are left
+            group_at = static_cast<int>(fd_div(static_cast<unsigned>(unit), p.fd_n_tiles));
             m = m_begin + unit - group_at * rows;
         }
         count = min(group, n_tiles - group_at * group);
@@ -1182,6 +1184,9 @@ ptq_gemm_dequant_panel_kernel(const __grid_constant__ CUtensorMap tmA, const __g
 // Three stages of codes: two cost 2 to 10 % (200704 x 384 -> 96: 65 us, not 58.5), and with eight the loads run so far ahead
 // of the stores that 200704 x 192 -> 96 takes 34.0 us, not 33.0; the other shapes cannot tell three from eight.
 //
+// 128 registers on symmetric layers (143 without the limit): the next kernel's quantizer CTAs find room beside it.  24 layers 12608 x 192 -> 768
+// in turn 237.8 -> 234.2 us; asymmetric ones would spill.
+//
 // Barriers: full/empty per stage of codes, wfull/wempty for the weights (the MMA thread frees them with a commit behind the
 // last tile that uses them), tfull/tempty per accumulator.  The epilogue runs in two teams.
 constexpr int kResMaxKBlocks = 3;
@@ -1196,9 +1201,9 @@ constexpr int kResSmemMax = 232448;
 static_assert(res_smem_bytes(kResMaxKBlocks, 1, kMaxBN, 3) <= kResSmemMax, "resident kernel exceeds the shared memory of one CTA");
 
 template <bool kDebugAcc, bool kAsym>
-__global__ void __launch_bounds__(kGemmThreads, 1)
+__global__ void __maxnreg__(kAsym ? 168 : 136)
 ptq_gemm_dequant_resident_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmW,
-                                 const __grid_constant__ CUtensorMap tmY, const GemmParams p)
+                                 const __grid_constant__ CUtensorMap tmY, const UnitParams p)
 {
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     const uint32_t base = smem_u32(smem_raw);

@@ -37,7 +37,7 @@ static_assert(kShortKSmemMax <= 232448, "short-K kernel exceeds the shared memor
 static_assert(kBM == kShortKQuantThreads, "a quantizer thread has one row");
 
 struct ShortKParams {
-    GemmParams g;
+    UnitParams g;
     const __half *x;      // [M,K]
     const float *s;       // [round_up(K,16)]
     const float *rs;      // RN(1/s)
@@ -50,7 +50,7 @@ template <int kChunks, int kMode, bool kDebugAcc>
 __global__ void __launch_bounds__(kShortKThreads, 1)
 ptq_short_k_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmY, const ShortKParams sp)
 {
-    const GemmParams &p = sp.g;
+    const UnitParams &p = sp.g;
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     const uint32_t base = smem_u32(smem_raw);
     if ((base & 1023u) != 0u) {

@@ -38,6 +38,9 @@ def env():
     (200, 264, 50, 740, True, False),
     (64, 1536, 197, 128, False, False),    # six N tiles: 24 CTAs on each, and four that share the row tiles that are left
     (104, 1000, 70, 301, True, False),     # four N tiles, every CTA on one: 37 CTAs each, rows of 2000 bytes
+    (300, 600, 64, 150, True, False),      # few tiles: one and two per CTA
+    (96, 48, 197, 60, False, False),       # fewer tiles than SMs
+    (384, 40, 128, 149, False, False),     # one tile more than CTAs
 ])
 def test_resident_weights(env, K, N, T, B, bias, asym):
     ptq, torch = env
