@@ -393,20 +393,29 @@ __device__ __noinline__ void copy_box_rows(__half *y, long long M, int N, int co
     }
 }
 
-template <bool kDebugAcc, bool kAsym>
+// kRelease: the warp arrives on `tempty` as soon as its part of the accumulator is in registers, not behind its last store; else the caller does.
+template <bool kDebugAcc, bool kAsym, bool kRelease = false>
 __device__ __forceinline__ uint32_t epilogue_tile_stream(const GemmParams &p, const CUtensorMap *tmY, uint32_t tmem_row,
                                                          long long m_row0, int n0, float dxr, uint32_t staging,
                                                          const float *dw_s, const float *bias_s, const int *ws_s, uint32_t nboxes,
-                                                         int lane, int c_begin, int c_stride, int cols, int zr, bool two_boxes)
+                                                         int lane, int c_begin, int c_stride, int cols, int zr, bool two_boxes,
+                                                         uint32_t tempty = 0u)
 {
     const long long m = m_row0 + lane;
     const bool row_ok = m < p.M;
+    auto release = [&] {
+        tc_fence_before_sync();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(tempty);
+    };
+    if (kRelease && c_begin >= cols) release();                // no step of this tile is the warp's
     for (int c0 = c_begin; c0 < cols; c0 += c_stride) {
         const int n_first = n0 + c0;
         uint32_t v0[32], v1[32];
         tmem_ld_32x32(tmem_row + c0, v0);
         tmem_ld_32x32(tmem_row + c0 + 32, v1);
         tmem_ld_wait();
+        if (kRelease && c0 + c_stride >= cols) release();
         if (kAsym) {
             // offset-free accumulator: acc - z[t] * sum_k Wq[n,k]
 #pragma unroll
@@ -1141,11 +1150,10 @@ ptq_gemm_dequant_panel_kernel(const __grid_constant__ CUtensorMap tmA, const __g
             const int *ws_s = !kAsym ? nullptr
                               : p.ws_copy ? reinterpret_cast<const int *>(scale_s) + (2u * p.vectors - 2u + (it & 1u)) * kMaxBN
                                           : p.wsum + n_tile * p.BN;
-            nboxes = epilogue_tile_stream<kDebugAcc, kAsym>(p, &tmY, tmem_row, m_row0, n_tile * p.BN, dxr, staging, dw_s, bias_s,
-                                                     ws_s, nboxes, lane, col_half * kEpiStepCols, 2 * kEpiStepCols, p.BN, zr, two_boxes);
-            tc_fence_before_sync();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(tempty_bar(buf));
+            // released early: 50432 x 768 -> 3072, both kernels, 127.8 -> 126.4 us (the other kernels gain nothing or lose 1 %)
+            nboxes = epilogue_tile_stream<kDebugAcc, kAsym, true>(p, &tmY, tmem_row, m_row0, n_tile * p.BN, dxr, staging, dw_s, bias_s,
+                                                                  ws_s, nboxes, lane, col_half * kEpiStepCols, 2 * kEpiStepCols, p.BN, zr, two_boxes,
+                                                                  tempty_bar(buf));
             buf ^= 1u;
             if (buf == 0u) bphase ^= 1u;
             publish_scales((it + 1u) & 1u);
