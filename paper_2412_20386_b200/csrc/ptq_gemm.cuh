@@ -99,7 +99,8 @@ struct GemmParams {
     // accumulator sum_k (c - z[t]) * Wq[n,k] exactly (all int32).  nullptr for symmetric layers.
     const int *zp;     // [T]
     const int *wsum;   // row sums of Wq, padded like dw
-    // Panel kernel only: a work unit is one 128-row panel of codes times `group` adjacent N tiles; `groups`
+    // Panel kernel (`group` and `groups` also the kernels with resident weights): a work unit is one 128-row panel of codes times `group` adjacent
+    // N tiles; `groups`
     // units cover a panel; the weight ring has `b_stages` slots of `b_stage_bytes` (= BN * 128) each.
     int group, groups;
     int b_stages, b_stage_bytes;
