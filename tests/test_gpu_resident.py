@@ -35,6 +35,8 @@ def env():
     (96, 384, 784, 48, False, False),
     (128, 488, 37, 1024, True, False),
     (33, 648, 197, 192, False, True),
+    (40, 512, 128, 103, False, False),     # code rows of 48 bytes, weights read in lines of 128
+    (80, 528, 128, 115, True, False),
     (200, 264, 50, 740, True, False),
     (64, 1536, 197, 128, False, False),    # six N tiles: 24 CTAs on each, and four that share the row tiles that are left
     (104, 1000, 70, 301, True, False),     # four N tiles, every CTA on one: 37 CTAs each, rows of 2000 bytes
