@@ -459,32 +459,6 @@ int resident_group(const ptq_linear *h, const ptq::GemmParams &p)
     return (p.m_tiles + sms - 1) / sms * p.n_tiles <= (tiles + sms - 1) / sms ? p.n_tiles : 1;
 }
 
-// The order of a kernel with resident weights on `grid` CTAs: as many CTAs as make whole sets of groups keep to one group each and stride over the
-// row tiles, so that neighbouring CTAs write the pieces of the same rows at about the same time; the few CTAs that are over take the row
-// tiles that are left.  Contiguous shares for all where the busiest CTA would get more so.  Both kernels, us, contiguous shares (all
-// rows of a group, then the next group) / spread: 50176 x 48 -> 1000 37.3 / 28.1 and 50176 x 384 -> 1000 asymmetric 45.7 / 41.0 (rows of 2000 bytes: pieces
-// that end inside a 32-byte sector reached DRAM separately), 100352 x 96 -> 384 22.4 / 21.3, 50176 x 256 -> 512 20.1 / 19.6; with row
-// tiles left over 18816 x 384 -> 1536 19.3 / 18.7, 50432 x 24 -> 768 16.0 / 15.2, 25216 x 384 -> 1536 23.0 / 23.0, 25807 x 376 -> 1504 25.3 / 25.4.
-void set_units(ptq::UnitParams &p, int grid)
-{
-    const long long total = static_cast<long long>(p.m_tiles) * p.groups;
-    const int rounds = static_cast<int>((total + grid - 1) / grid), ctas = grid / p.groups, over = grid - ctas * p.groups;
-    long long rows = static_cast<long long>(ctas) * rounds;                            // that the spread CTAs take
-    if (rows > p.m_tiles) rows = p.m_tiles;
-    const long long left = (p.m_tiles - rows) * p.groups;
-    const bool spread = ctas >= 1 && left <= static_cast<long long>(over) * rounds;
-    p.spread = spread ? ctas * p.groups : 0;
-    p.spread_rows = spread ? static_cast<int>(rows) : 0;
-    p.spread_step = spread ? ctas : 1;
-    const long long rest = spread ? left : total;
-    const int rest_ctas = grid - p.spread;
-    p.rest_share = rest_ctas > 0 ? static_cast<int>(rest / rest_ctas) : 0;
-    p.rest_extra = rest_ctas > 0 ? static_cast<int>(rest % rest_ctas) : 0;
-    p.fd_spread = ptq::make_fastdiv(static_cast<unsigned>(p.groups));
-    const int rest_rows = p.m_tiles - p.spread_rows;
-    p.fd_n_tiles = ptq::make_fastdiv(static_cast<unsigned>(rest_rows > 0 ? rest_rows : 1));
-}
-
 // Cycles of one tile of `cols` columns in the streaming kernel, as fitted to timings of 24 shapes at all widths: an MMA of K = 32
 // takes 35 + 0.52 cols; the eight epilogue warps take 360 per tile and 670 per pair of 64-column steps.
 double mma_cycles(const ptq_linear *h, int cols) { return (h->K + 31) / 32 * (35.0 + 0.52 * cols); }
@@ -703,7 +677,7 @@ ptq_status_t launch_gemm(const ptq_linear *h, const void *codes, long long M, vo
             rp.groups = (p.n_tiles + rp.group - 1) / rp.group;
             const long long units = static_cast<long long>(p.m_tiles) * rp.groups;
             const int rgrid = static_cast<int>(units < h->num_sms ? units : h->num_sms);
-            set_units(rp, rgrid);
+            ptq::set_units(rp, rgrid);
             const ptq_status_t es = ensure_smem<kKern>(h->device, ptq::kResSmemMax);
             if (es != PTQ_OK) return es;
             const int smem = ptq::res_smem_bytes(p.k_blocks, rp.group, p.BN, p.vectors);
@@ -958,7 +932,7 @@ ptq_status_t launch_short_k(const ptq_linear *h, const void *x, long long M, voi
     sp.ld_bytes = x_align % 16 == 0 ? 16 : x_align % 8 == 0 ? 8 : 2;
     const long long units = static_cast<long long>(p.m_tiles) * p.groups;
     const int grid = static_cast<int>(units < h->num_sms ? units : h->num_sms);
-    set_units(p, grid);
+    ptq::set_units(p, grid);
     const int smem = ptq::short_k_smem_bytes(p.group * p.BN * ptq::kBK, p.vectors);
     auto go = [&](auto chunks, auto mode, auto debug) -> ptq_status_t {
         constexpr auto kKern = ptq::ptq_short_k_kernel<decltype(chunks)::value, decltype(mode)::value, decltype(debug)::value>;

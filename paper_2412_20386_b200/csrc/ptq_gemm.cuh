@@ -514,17 +514,54 @@ __device__ __forceinline__ void team_sync(int team) { asm volatile("bar.sync %0,
 // The CTA's units (a row tile times a group of N tiles) and, within a unit, its N tiles.  The first `spread` CTAs keep to the group of their
 // number and stride over the first `spread_rows` row tiles, so that the CTAs read and write neighbouring rows at a time (a single group
 // is always so: 200704 x 384 -> 96 60.0 -> 58.5 us).  The other CTAs take contiguous shares of what is left (of everything, where
-// nothing is spread), numbered with the row tiles of a group adjacent: their weights change once or twice.
+// nothing is spread), numbered with the row tiles of a group adjacent: in shares of everything the weights change once (at every unit where
+// there are more groups than CTAs), in shares of a few left-over row tiles more often.
 struct UnitParams : GemmParams {       // only where they are used: parameters that a launch carries for nothing cost 0.4 to 1.3 % of a small layer
     int spread, spread_rows, spread_step, rest_share, rest_extra;
     FastDiv fd_spread;                 // divisor groups; fd_n_tiles divides by the row tiles that are left
 };
+
+// The order on `grid` CTAs.  As many CTAs as make whole sets of groups are spread: the pieces of a row of y are then written at about the same time.
+// With ceil(units / CTAs) rounds for each of them, the CTAs that are over always have room for the row tiles that are left.
+// Both kernels, us, contiguous shares (all rows of a group, then the next group) / spread: 50176 x 48 -> 1000 37.3 / 28.1 and 50176 x 384 -> 1000
+// asymmetric 45.7 / 41.0 (rows of 2000 bytes: pieces that end inside a 32-byte sector reached DRAM separately), 100352 x 96 -> 384 22.4 / 21.3,
+// 50176 x 256 -> 512 20.1 / 19.6; with row tiles left over 18816 x 384 -> 1536 19.3 / 18.7, 50432 x 24 -> 768 16.0 / 15.2,
+// 25216 x 384 -> 1536 23.0 / 23.0.
+// Not spread where changes of weights would make a left-over CTA the one that the launch waits for: a change costs it about a sixth of a tile, half
+// of that with one k-block, and the spread order is worth about a twenty-fifth; where rows of y end inside a sector it is worth more than that.
+// 18944 x 384 -> 1792 (one CTA with a row of seven tiles and seven loads) 24.5 / 26.5, 18944 x 96 -> 1792 17.0 / 17.3, 4736 x 384 -> 3072 (three
+// tiles, three loads) 12.5 / 13.2, 7552 x 384 -> 1280 (two and two) 11.9 / 12.2; nearest on the other side 11648 x 48 -> 3136 (eight tiles, four loads)
+// 19.2 / 17.9, 24320 x 300 -> 1664 (seven tiles in nine rounds, seven loads) 32.5 / 32.3, 4736 x 192 -> 3064 (three and three, rows that
+// end inside a sector) 11.9 / 11.4; against the rule 18944 x 48 -> 1664 17.1 / 16.8 and, nothing left over, 7296 x 96 -> 3232 13.3 / 14.1.
+inline void set_units(UnitParams &p, int grid)
+{
+    const long long total = static_cast<long long>(p.m_tiles) * p.groups;
+    const int rounds = static_cast<int>((total + grid - 1) / grid), ctas = grid / p.groups, over = grid - ctas * p.groups;
+    long long rows = static_cast<long long>(ctas) * rounds;                            // that the spread CTAs take
+    if (rows > p.m_tiles) rows = p.m_tiles;
+    const long long left_rows = p.m_tiles - rows, left = left_rows * p.groups;
+    bool spread = ctas >= 1;
+    if (spread && left > 0) {
+        const long long share = (left + over - 1) / over, loads = (share + left_rows - 2) / left_rows + 1;   // of the busiest, at most
+        spread = p.N % 16 != 0 || 24 * share + (p.k_blocks > 1 ? 4 : 2) * (loads - 1) <= 25ll * rounds;
+    }
+    p.spread = spread ? ctas * p.groups : 0;
+    p.spread_rows = spread ? static_cast<int>(rows) : 0;
+    p.spread_step = spread ? ctas : 1;
+    const long long rest = spread ? left : total;
+    const int rest_ctas = grid - p.spread;
+    p.rest_share = rest_ctas > 0 ? static_cast<int>(rest / rest_ctas) : 0;
+    p.rest_extra = rest_ctas > 0 ? static_cast<int>(rest % rest_ctas) : 0;
+    p.fd_spread = make_fastdiv(static_cast<unsigned>(p.groups));
+    const int rest_rows = p.m_tiles - p.spread_rows;
+    p.fd_n_tiles = make_fastdiv(static_cast<unsigned>(rest_rows > 0 ? rest_rows : 1));
+}
+
 struct UnitCursor {
     int unit, end, step, m, group_at, count, g;                // N tile g of the `count` of unit (group_at, m)
     int m_begin, m_tiles, n_tiles, group;
-    __device__ UnitCursor(const UnitParams &p) : g(0), m_begin(p.spread_rows), m_tiles(p.m_tiles), n_tiles(p.n_tiles), group(p.group)
+    __host__ __device__ UnitCursor(const UnitParams &p, int cta) : g(0), m_begin(p.spread_rows), m_tiles(p.m_tiles), n_tiles(p.n_tiles), group(p.group)
     {
-        const int cta = static_cast<int>(blockIdx.x);
         if (cta < p.spread) {
             const int lane = static_cast<int>(fd_div(static_cast<unsigned>(cta), p.fd_spread));
             group_at = cta - lane * p.groups;
@@ -541,12 +578,12 @@ struct UnitCursor {
         }
         count = min(group, n_tiles - group_at * group);
     }
-    __device__ bool valid() const { return unit < end; }
-    __device__ int grp() const { return group_at; }
-    __device__ int m_tile() const { return m; }
-    __device__ int n_tile() const { return group_at * group + g; }
-    __device__ int size() const { return count; }
-    __device__ void next_unit()
+    __host__ __device__ bool valid() const { return unit < end; }
+    __host__ __device__ int grp() const { return group_at; }
+    __host__ __device__ int m_tile() const { return m; }
+    __host__ __device__ int n_tile() const { return group_at * group + g; }
+    __host__ __device__ int size() const { return count; }
+    __host__ __device__ void next_unit()
     {
         unit += step;
         m += step;
@@ -556,7 +593,7 @@ struct UnitCursor {
             count = min(group, n_tiles - group_at * group);
         }
     }
-    __device__ void advance()
+    __host__ __device__ void advance()
     {
         if (++g == count) {
             g = 0;
@@ -1266,7 +1303,7 @@ ptq_gemm_dequant_resident_kernel(const __grid_constant__ CUtensorMap tmA, const 
     const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_holder, 0);
     griddep_launch_dependents();         // the codes (and row steps) of the kernel before are read behind griddep_wait() only
 
-    UnitCursor cur(p);
+    UnitCursor cur(p, static_cast<int>(blockIdx.x));
 
     if (warp == 0) {
         // ------------------------------------------------------------------ TMA producer

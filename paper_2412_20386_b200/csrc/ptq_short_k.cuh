@@ -108,7 +108,7 @@ ptq_short_k_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constan
     const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_holder, 0);
     griddep_launch_dependents();
 
-    UnitCursor cur(p);
+    UnitCursor cur(p, static_cast<int>(blockIdx.x));
 
     if (warp == 0) {
         // ------------------------------------------------------------------ TMA producer of the weights (parameters: no dependency wait)

@@ -43,9 +43,13 @@ __host__ __device__ inline FastDiv make_fastdiv(unsigned d)
     f.magic = d > 1u ? 0xFFFFFFFFFFFFFFFFull / d + 1ull : 0ull;
     return f;
 }
-__device__ __forceinline__ unsigned fd_div(unsigned n, const FastDiv &f)
+__host__ __device__ __forceinline__ unsigned fd_div(unsigned n, const FastDiv &f)
 {
+#ifdef __CUDA_ARCH__
     return f.d == 1u ? n : static_cast<unsigned>(__umul64hi(f.magic, static_cast<unsigned long long>(n)));
+#else
+    return n / f.d;
+#endif
 }
 
 // ---------------------------------------------------------------- mbarrier

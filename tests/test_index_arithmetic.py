@@ -14,7 +14,9 @@ PROGRAM = r"""
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <vector>
 #include "ptq_calibrate.cuh"
+#include "ptq_gemm.cuh"
 #include "ptq_quantize.cuh"
 
 // quant images chunks_per_image sms: images between two of a thread, ring depth, images of one launch
@@ -53,12 +55,46 @@ static int plan(char **a)
     return 0;
 }
 
+// units m_tiles n_tiles group sms k_blocks: tiles visited other than once, most units of a CTA, most of a CTA's 24 per unit and 4 per change of
+// its weights, 1 where CTAs keep to their groups
+static int units(char **a)
+{
+    ptq::UnitParams p = {};
+    p.m_tiles = atoi(a[0]);
+    p.n_tiles = atoi(a[1]);
+    p.group = atoi(a[2]);
+    p.groups = (p.n_tiles + p.group - 1) / p.group;
+    p.N = 256 * p.n_tiles;
+    p.k_blocks = atoi(a[4]);
+    const long long total = (long long)p.m_tiles * p.groups;
+    const int grid = (int)(total < atoi(a[3]) ? total : atoi(a[3]));
+    ptq::set_units(p, grid);
+    std::vector<int> visits((size_t)p.m_tiles * p.n_tiles, 0);
+    int most = 0, cost = 0;
+    for (int cta = 0; cta < grid; ++cta) {
+        int own = 0, loads = 0, held = -1;
+        for (ptq::UnitCursor c(p, cta); c.valid(); ++own) {
+            if (c.grp() != held) ++loads;
+            held = c.grp();
+            for (int n = c.size(); n > 0; --n, c.advance())
+                if (c.m_tile() < p.m_tiles && c.n_tile() < p.n_tiles) ++visits[(size_t)c.m_tile() * p.n_tiles + c.n_tile()];
+        }
+        if (own > most) most = own;
+        if (24 * own + 4 * (loads - 1) > cost) cost = 24 * own + 4 * (loads - 1);
+    }
+    long long wrong = 0;
+    for (int v : visits) wrong += v != 1;
+    printf("%lld %d %d %d\n", wrong, most, cost, p.spread > 0 ? 1 : 0);
+    return 0;
+}
+
 int main(int argc, char **argv)
 {
     if (argc > 1 && !strcmp(argv[1], "quant")) return quant(argv + 2);
     if (argc > 1 && !strcmp(argv[1], "tiles")) return tiles(argv + 2);
     if (argc > 1 && !strcmp(argv[1], "shares")) return shares(argv + 2);
     if (argc > 1 && !strcmp(argv[1], "plan")) return plan(argv + 2);
+    if (argc > 1 && !strcmp(argv[1], "units")) return units(argv + 2);
     return 2;
 }
 """
@@ -112,3 +148,26 @@ def test_calibration_shares_cover_every_image(program, Bc, T):
     (1, 1, 1, [9, 64]), (INT_MAX, 1, 4096, [9, 128]), (INT_MAX, 1048576, 4096, [27, 64])])
 def test_search_blocks_fill_the_chip_and_no_more(program, elements, T, C, want):
     assert program("plan", elements, T, C, 148) == want
+
+
+# row tiles, N tiles, N tiles per unit: groups that divide the CTAs and do not, left-over row tiles with few and with many changes of the
+# weights, fewer units than CTAs, more groups than CTAs, last groups that are smaller
+@pytest.mark.parametrize("m,n,group", [(1, 1, 1), (148, 7, 1), (190, 7, 1), (253, 7, 1), (37, 12, 1), (37, 11, 1), (59, 5, 1), (148, 5, 1), (394, 3, 1),
+                                       (147, 6, 1), (113, 13, 1), (105, 2, 2), (1568, 2, 2), (100, 5, 2), (85, 8, 3), (291, 10, 2), (2, 235, 1),
+                                       (3, 149, 1), (1, 400, 3), (200000, 7, 1)])
+@pytest.mark.parametrize("sms", [148, 132])
+def test_unit_order_visits_every_tile_once(program, m, n, group, sms):
+    """No CTA has more units than an even split gives the busiest, and where there are CTAs enough for one group each, changes of the
+    weights make no left-over CTA the one that the launch waits for by more than a twenty-fifth."""
+    units = m * -(-n // group)
+    rounds = -(-units // min(units, sms))
+    groups = -(-n // group)
+    for k_blocks in (1, 3):
+        wrong, most, cost, spread = program("units", m, n, group, sms, k_blocks)
+        assert wrong == 0 and most == rounds
+        if groups <= min(units, sms) and k_blocks > 1:
+            assert cost <= max(25 * rounds, 24 * rounds + 4)
+        if groups == 1:
+            assert spread == 1
+        if (m, n, group, sms) in ((148, 7, 1, 148), (37, 12, 1, 148)):
+            assert spread == 0
