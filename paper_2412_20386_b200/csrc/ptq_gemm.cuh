@@ -1227,7 +1227,7 @@ ptq_gemm_dequant_panel_kernel(const __grid_constant__ CUtensorMap tmA, const __g
 // Part of that is the cursor, which steps without divisions: 25216 x 384 -> 1536 (group 1) 23.5 -> 23.2, 200704 x 192 -> 96 31.5 -> 31.0; what
 // loses is 200704 x 64 -> 256, 26.3 -> 26.6.
 //
-// Three stages of codes: two cost 2 to 10 % (200704 x 384 -> 96: 65 us, not 58.5), and with eight the loads run so far ahead
+// Three stages of codes, which hold a whole panel (they must: see below): two cost 2 to 10 % (200704 x 384 -> 96: 65 us, not 58.5), and with eight the loads run so far ahead
 // of the stores that 200704 x 192 -> 96 takes 34.0 us, not 33.0; the other shapes cannot tell three from eight.
 //
 // 128 registers on symmetric layers (143 without the limit): the next kernel's quantizer CTAs find room beside it.  24 layers 12608 x 192 -> 768
@@ -1245,6 +1245,8 @@ __host__ __device__ constexpr int res_smem_bytes(int k_blocks, int group, int bn
 }
 constexpr int kResSmemMax = 232448;
 static_assert(res_smem_bytes(kResMaxKBlocks, 1, kMaxBN, 3) <= kResSmemMax, "resident kernel exceeds the shared memory of one CTA");
+// A panel's stages are freed behind its last N tile, and the first N tile reads all of them.
+static_assert(kResMaxKBlocks <= kResStages, "a unit's codes stay in the ring for all its N tiles");
 
 template <bool kDebugAcc, bool kAsym>
 __global__ void __maxnreg__(kAsym ? 168 : 136)
