@@ -304,7 +304,7 @@ struct SearchParams {
     double *loss;        // [T, n_grid - j_lo + 1]
     int Bc, T, K;
     int n_grid, j_lo;
-    int vec;             // K % 8 == 0, x 16-byte aligned: eight elements per load
+    int vec;             // eight elements per load: K % 8 == 0, x 16-byte aligned, elements enough
     FastDiv fd_K;
 };
 

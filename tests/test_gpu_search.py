@@ -91,11 +91,11 @@ def test_search_block_shapes(env, K, T, Bc, C):
     check_search(ptq, torch, x, s, rng.uniform(0.02, 0.06, T).astype(F32), 100, 101 - C)
 
 
-@pytest.mark.parametrize("K,T,Bc,C", [(64, 12, 33, 9), (8, 450, 257, 27), (264, 450, 2, 80)])
+@pytest.mark.parametrize("K,T,Bc,C", [(64, 12, 33, 9), (8, 450, 257, 27), (264, 450, 2, 80), (8, 197, 11, 3), (16, 40, 8, 5)])
 def test_search_loads_and_clamps(env, K, T, Bc, C):
-    """Eight elements per load (K a multiple of 8) with last tiles that are not full, against the same values at an address that is not
-    16-byte aligned: bit for bit the same sums.  Steps so small that the quotients reach 5 to 500, so that of one thread's nine
-    candidates some clamp, all clamp or none does; infinities and NaN among the elements."""
+    """Eight elements per load (K a multiple of 8) with last tiles that are not full, on both sides of two elements per thread, against the
+    same values at an address that is not 16-byte aligned: bit for bit the same sums.  Steps so small that the quotients reach 5 to 500,
+    so that of one thread's nine candidates some clamp, all clamp or none does; infinities and NaN among the elements."""
     ptq, torch = env
     rng = np.random.default_rng(K + C)
     x = (rng.standard_t(3, (Bc, T, K)) * np.exp(rng.normal(0, 1, (1, T, 1)))).astype(np.float16)
