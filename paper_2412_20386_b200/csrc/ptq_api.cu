@@ -913,17 +913,8 @@ ptq_status_t launch_short_k(const ptq_linear *h, const void *x, long long M, voi
     ptq::ShortKParams sp;
     ptq::UnitParams &p = sp.g;
     set_gemm_params(h, p, M, y, acc_out, true, nullptr);
-    // N tiles per unit: the number that leaves the busiest CTA the fewest tiles; the larger one (rows quantized less often) if equal
-    long long fewest = 0;
-    for (int group = 1; group <= p.n_tiles && group <= ptq::kShortKMaxGroup; ++group) {
-        const int groups = (p.n_tiles + group - 1) / group;
-        const long long tiles = (static_cast<long long>(p.m_tiles) * groups + h->num_sms - 1) / h->num_sms * group;
-        if (group == 1 || tiles <= fewest) {
-            fewest = tiles;
-            p.group = group;
-            p.groups = groups;
-        }
-    }
+    p.group = ptq::short_k_group(p.m_tiles, p.n_tiles, h->num_sms);
+    p.groups = (p.n_tiles + p.group - 1) / p.group;
     sp.x = static_cast<const __half *>(x);
     sp.s = h->d_s;
     sp.rs = h->d_rs;

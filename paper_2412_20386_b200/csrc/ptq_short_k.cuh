@@ -45,6 +45,22 @@ struct ShortKParams {
     int ld_bytes;         // bytes per load of x: 16, 8 or 2 (alignment of its rows)
 };
 
+// N tiles per unit: the number that leaves the busiest CTA the fewest tiles; the larger one (rows quantized less often) if equal.
+__host__ inline int short_k_group(int m_tiles, int n_tiles, int sms)
+{
+    int best = 1;
+    long long fewest = 0;
+    for (int group = 1; group <= n_tiles && group <= kShortKMaxGroup; ++group) {
+        const long long groups = (n_tiles + group - 1) / group;
+        const long long tiles = (m_tiles * groups + sms - 1) / sms * group;
+        if (group == 1 || tiles <= fewest) {
+            fewest = tiles;
+            best = group;
+        }
+    }
+    return best;
+}
+
 // kChunks: chunks of 8 channels per row, at most (K <= 8 kChunks).
 template <int kChunks, int kMode, bool kDebugAcc>
 __global__ void __launch_bounds__(kShortKThreads, 1)

@@ -1,8 +1,8 @@
-"""The GEMM kernel that keeps its weights in shared memory (K <= 384, three tiles and more per CTA), where its tile order and
-its weight reloads can go wrong: a single N tile (CTAs stride over the rows), shares that run over one and over several N
-tiles, one to three k-blocks with ragged K, ragged N, asymmetric layers and layers with a bias.  Oracle: the integer
-accumulators computed on the host from the codes and weights, every element, and the scaled output within the repository's bound
-max(2^-10 |y|, 1e-3)."""
+"""The GEMM kernel that keeps its weights in shared memory (K <= 384), where its order of tiles and its weight reloads can go wrong: a
+single N tile (CTAs stride over the rows), CTAs on one group each with and without left-over row tiles, contiguous shares that cross one and
+several N tiles, one to three k-blocks with ragged K, ragged N, asymmetric layers, layers with a bias, one tile per CTA and fewer.  Oracle:
+the integer accumulators computed on the host from the codes and weights, every element, and the scaled output within the repository's
+bound max(2^-10 |y|, 1e-3)."""
 import numpy as np
 import pytest
 
@@ -26,7 +26,8 @@ def env():
 @pytest.mark.parametrize("K,N,T,B,bias,asym", [
     (96, 96, 784, 80, False, False),       # one N tile, strided
     (384, 200, 197, 300, True, True),      # one N tile, three k-blocks
-    (200, 600, 197, 110, True, False),     # a share crosses one N tile; K and N ragged
+    (200, 600, 197, 110, True, False),     # K and N ragged, CTAs on one N tile each
+    (384, 1792, 128, 148, True, False),    # seven N tiles on 148 row tiles: contiguous shares, which cross one N tile
     (40, 60000, 67, 3, False, False),      # two row tiles: a share crosses several N tiles
     (384, 58000, 64, 4, False, True),
     (256, 16, 7, 8121, False, False),      # a single 16-column step per tile

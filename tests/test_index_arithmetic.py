@@ -6,6 +6,7 @@ import subprocess
 import pytest
 
 from paper_2412_20386_b200 import build as lib_build
+from test_gpu_short_k import RELOADS
 
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2412_20386_b200", "csrc")
 INT_MAX = 2 ** 31 - 1
@@ -18,6 +19,7 @@ PROGRAM = r"""
 #include "ptq_calibrate.cuh"
 #include "ptq_gemm.cuh"
 #include "ptq_quantize.cuh"
+#include "ptq_short_k.cuh"
 
 // quant images chunks_per_image sms: images between two of a thread, ring depth, images of one launch
 static int quant(char **a)
@@ -55,14 +57,14 @@ static int plan(char **a)
     return 0;
 }
 
-// units m_tiles n_tiles group sms k_blocks: tiles visited other than once, most units of a CTA, most of a CTA's 24 per unit and 4 per change of
-// its weights, 1 where CTAs keep to their groups
+// units m_tiles n_tiles group sms k_blocks (group 0: as the few-channels kernel takes it): tiles visited other than once, most units of a CTA, most of a CTA's 24 per unit and 4 per change of
+// its weights, 1 where CTAs keep to their groups, most loads of weights of a CTA
 static int units(char **a)
 {
     ptq::UnitParams p = {};
     p.m_tiles = atoi(a[0]);
     p.n_tiles = atoi(a[1]);
-    p.group = atoi(a[2]);
+    p.group = atoi(a[2]) ? atoi(a[2]) : ptq::short_k_group(p.m_tiles, p.n_tiles, atoi(a[3]));
     p.groups = (p.n_tiles + p.group - 1) / p.group;
     p.N = 256 * p.n_tiles;
     p.k_blocks = atoi(a[4]);
@@ -70,7 +72,7 @@ static int units(char **a)
     const int grid = (int)(total < atoi(a[3]) ? total : atoi(a[3]));
     ptq::set_units(p, grid);
     std::vector<int> visits((size_t)p.m_tiles * p.n_tiles, 0);
-    int most = 0, cost = 0;
+    int most = 0, cost = 0, reloads = 0;
     for (int cta = 0; cta < grid; ++cta) {
         int own = 0, loads = 0, held = -1;
         for (ptq::UnitCursor c(p, cta); c.valid(); ++own) {
@@ -80,11 +82,12 @@ static int units(char **a)
                 if (c.m_tile() < p.m_tiles && c.n_tile() < p.n_tiles) ++visits[(size_t)c.m_tile() * p.n_tiles + c.n_tile()];
         }
         if (own > most) most = own;
+        if (loads > reloads) reloads = loads;
         if (24 * own + 4 * (loads - 1) > cost) cost = 24 * own + 4 * (loads - 1);
     }
     long long wrong = 0;
     for (int v : visits) wrong += v != 1;
-    printf("%lld %d %d %d\n", wrong, most, cost, p.spread > 0 ? 1 : 0);
+    printf("%lld %d %d %d %d\n", wrong, most, cost, p.spread > 0 ? 1 : 0, reloads);
     return 0;
 }
 
@@ -163,7 +166,7 @@ def test_unit_order_visits_every_tile_once(program, m, n, group, sms):
     rounds = -(-units // min(units, sms))
     groups = -(-n // group)
     for k_blocks in (1, 3):
-        wrong, most, cost, spread = program("units", m, n, group, sms, k_blocks)
+        wrong, most, cost, spread, _ = program("units", m, n, group, sms, k_blocks)
         assert wrong == 0 and most == rounds
         if groups <= min(units, sms) and k_blocks > 1:
             assert cost <= max(25 * rounds, 24 * rounds + 4)
@@ -171,3 +174,10 @@ def test_unit_order_visits_every_tile_once(program, m, n, group, sms):
             assert spread == 1
         if (m, n, group, sms) in ((148, 7, 1, 148), (37, 12, 1, 148)):
             assert spread == 0
+
+
+def test_few_channel_layers_reload_their_weights(program):
+    """The layers that the few-channels kernel is tested with for a change of weights within a CTA have one."""
+    for K, N, T, M, bias, off in RELOADS:
+        wrong, _, _, spread, loads = program("units", -(-M // 128), -(-N // 256), 0, 148, 1)
+        assert wrong == 0 and loads > 1
