@@ -9,7 +9,7 @@
 // form for K <= 128 with chunks spread over the threads took 58 us for 200704 x 96 -> 384 (two kernels 41), with eight quantizer
 // warps, for which the epilogue's registers spill, 48.
 //
-// Warps: 0 TMA producer of the weights, 1 TMEM owner and MMA issuer, 2..9 epilogue in two teams, 10..13 quantizers.
+// Warps: 0 TMA producer of the weights, which also has the rows of x brought into L2, 1 TMEM owner and MMA issuer, 2..9 epilogue in two teams, 10..13 quantizers.
 // Barriers: afull/aempty per stage of codes (filled by the quantizer warps, freed by the commit after the unit's last N tile),
 // wfull/wempty for the weights, tfull/tempty per accumulator.
 #pragma once
@@ -59,6 +59,23 @@ __host__ inline int short_k_group(int m_tiles, int n_tiles, int sms)
         }
     }
     return best;
+}
+
+// Asks for the rows of x of the CTA's next units, before the dependency wait.  CTAs with the groups of one row tile read them at the same time, and
+// each unit waited for DRAM, beside the stores: whole forward, us, without and with, 15360 x 24 -> 1696 17.3 / 15.8, 10880 x 24 -> 2000 15.6 / 14.4,
+// 47104 x 5 -> 496 12.8 / 11.5, 38528 x 22 -> 384 15.2 / 13.8; where the stores are all of it nothing, 50432 x 24 -> 768 20.1 / 20.2.
+// By the weights' producer, which has nothing else to do, and for so many units at most: asked for by a quantizer thread, for all 42 units of
+// the CTA, 802816 x 6 -> 192 took 53.0 us, 51.2 so, and 791791 x 2 -> 32 36.7 / 35.5 (51.4 and 35.5 without).
+constexpr int kShortKAhead = 16;
+__device__ __forceinline__ void prefetch_rows(const ShortKParams &sp, UnitCursor at)
+{
+    const uintptr_t x0 = reinterpret_cast<uintptr_t>(sp.x);
+    for (int i = 0; i < kShortKAhead && at.valid(); ++i, at.next_unit()) {
+        const long long first = static_cast<long long>(at.m_tile()) * kBM, last = min(first + kBM, sp.g.M);
+        const uintptr_t begin = (x0 + 2 * static_cast<uintptr_t>(first * sp.g.K) + 15u) & ~static_cast<uintptr_t>(15);
+        const uintptr_t end = (x0 + 2 * static_cast<uintptr_t>(last * sp.g.K)) & ~static_cast<uintptr_t>(15);
+        if (end > begin) l2_prefetch(reinterpret_cast<const void *>(begin), static_cast<uint32_t>(end - begin));
+    }
 }
 
 // kChunks: chunks of 8 channels per row, at most (K <= 8 kChunks).
@@ -143,7 +160,7 @@ ptq_short_k_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constan
                 mbar_arrive_expect_tx(wfull_bar, static_cast<uint32_t>(n) * w_bytes);
                 for (int i = 0; i < n; ++i) tma_load_2d(base + static_cast<uint32_t>(i) * w_bytes, &tmW, 0, (grp * p.group + i) * p.BN, wfull_bar);
                 held = grp;
-                ++loads;
+                if (loads++ == 0u) prefetch_rows(sp, cur);
             }
             if (!ok) {   // error path only: the loads land before the CTA gives up its shared memory (bounded)
                 for (int i = 0; i < 200000 && !mbar_try_wait(wfull_bar, (loads - 1u) & 1u); ++i) {
@@ -205,19 +222,6 @@ ptq_short_k_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constan
                 if (j < cpr) next[j] = load_chunk_regs(src + 8 * j, p.K - 8 * j, sp.ld_bytes);
             d_next = __ldg(sp.dx2 + (m - fd_div(m, p.fd_T) * p.fd_T.d));
         };
-        // The rows of all the CTA's units are asked for at once.  CTAs with the groups of one row tile read them at the same time, and each unit
-        // waited for DRAM, beside the stores: whole forward, us, without and with, 15360 x 24 -> 1696 17.3 / 15.8, 10880 x 24 -> 2000 15.6 / 14.4,
-        // 47104 x 5 -> 496 12.8 / 11.5, 38528 x 22 -> 384 15.2 / 13.8; where the stores are all of it nothing, 50432 x 24 -> 768 20.1 / 20.2.
-        if (row == 0) {
-            const uintptr_t x0 = reinterpret_cast<uintptr_t>(sp.x);
-            for (UnitCursor ahead = cur; ahead.valid(); ahead.next_unit()) {
-                const long long first = static_cast<long long>(ahead.m_tile()) * kBM, last = min(first + kBM, p.M);
-                const uintptr_t begin = (x0 + 2 * static_cast<uintptr_t>(first * p.K) + 15u) & ~static_cast<uintptr_t>(15);
-                const uintptr_t end = (x0 + 2 * static_cast<uintptr_t>(last * p.K)) & ~static_cast<uintptr_t>(15);
-                if (end > begin) l2_prefetch(reinterpret_cast<const void *>(begin), static_cast<uint32_t>(end - begin));
-            }
-        }
-        __syncwarp();
         griddep_wait();
         if (cur.valid()) fetch(cur.m_tile());
         uint32_t stage = 0, phase = 0;

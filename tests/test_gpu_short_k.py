@@ -1,5 +1,5 @@
 """The one-kernel path for layers of a few channels at the sizes where it can go wrong: K around a chunk of 8 and at the largest,
-row tiles and shares that end raggedly, one to seven N tiles (units of one, two and three tiles, the last group smaller), CTAs
+row tiles and shares that end raggedly, more units per CTA than are prefetched, one to seven N tiles (units of one, two and three tiles, the last group smaller), CTAs
 that change their weights (RELOADS), rows of x at every alignment, saturating, infinite and NaN inputs, 4-bit codes, and the sizes on either
 side of its rule.  Codes and accumulators bit for bit."""
 import numpy as np
@@ -31,7 +31,7 @@ RELOADS = [(16, 1280, 64, 7552, False, 0), (24, 768, 197, 25216, True, 0), (8, 1
 @pytest.mark.parametrize("K,N,T,M,bias,off", RELOADS + [
     (1, 8, 7, 9800, False, 0), (8, 64, 19, 19000, True, 0), (9, 72, 197, 10047, False, 1), (12, 384, 197, 4925, True, 0),
     (12, 384, 197, 25216, False, 4), (16, 1280, 64, 6400, False, 0), (24, 768, 49, 10045, True, 2), (31, 1000, 3, 3999, False, 0),
-    (32, 256, 1, 20001, True, 0), (5, 1600, 128, 12800, False, 0)])
+    (32, 256, 1, 20001, True, 0), (5, 1600, 128, 12800, False, 0), (3, 24, 7, 329287, True, 1)])
 def test_few_channels_match_oracle(env, K, N, T, M, bias, off):
     ptq, torch = env
     spec = wl.LinearSpec(16, K % 83, N % 7, "short_k", M // T, T, K, N, bias=bias)
