@@ -74,3 +74,16 @@ def test_resident_weights(env, K, N, T, B, bias, asym):
             ref = ref + torch.from_numpy(b).cuda().double()
         assert_y_close(y[m0:m0 + 8192].cpu().numpy(), ref.cpu().numpy(), "rows from %d" % m0)
     layer.close()
+
+
+@pytest.mark.parametrize("K,N,rows,variant", [
+    (384, 192, 74, 1), (384, 192, 73, 0), (384, 200, 99, 0), (206, 208, 140, 0), (128, 64, 148, 1),    # one tile per CTA: layers that narrow by half
+    (128, 512, 74, 0), (128, 512, 75, 1),                                                              # 148 and 150 tiles
+])
+def test_which_short_layers_keep_their_weights(env, K, N, rows, variant):
+    ptq, torch = env
+    if torch.cuda.get_device_properties(0).multi_processor_count != 148:
+        pytest.skip("row counts for 148 SMs")
+    layer = ptq.PtqLinear(np.ones((N, K), np.int8), np.ones(N, np.float32), np.ones(K, np.float32), np.ones(1, np.float32))
+    assert layer.gemm_variant(128 * rows) == variant
+    layer.close()
