@@ -676,6 +676,7 @@ ptq_status_t launch_gemm(const ptq_linear *h, const void *codes, long long M, vo
             ptq::UnitParams rp;
             static_cast<ptq::GemmParams &>(rp) = p;
             rp.group = resident_group(h, p);
+            rp.stages = ptq::res_stages(h->K, h->N);
             rp.groups = (p.n_tiles + rp.group - 1) / rp.group;
             const long long units = static_cast<long long>(p.m_tiles) * rp.groups;
             const int rgrid = static_cast<int>(units < h->num_sms ? units : h->num_sms);

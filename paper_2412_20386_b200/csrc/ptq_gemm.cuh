@@ -1248,6 +1248,12 @@ static_assert(res_smem_bytes(kResMaxKBlocks, 1, kMaxBN, 3) <= kResSmemMax, "resi
 // A panel's stages are freed behind its last N tile, and the first N tile reads all of them.
 static_assert(kResMaxKBlocks <= kResStages, "a unit's codes stay in the ring for all its N tiles");
 
+// Two stages where a row of codes is 16 bytes and a row of y at most 128: little is stored per tile, and with three the loads run ahead of the
+// stores as above.  Both kernels, us, three / two: 802816 x 16 -> 16 38.5 / 36.4, 802816 x 8 -> 32 35.3 / 33.0, 678027 x 6 -> 8 31.8 / 30.2,
+// 517930 x 13 -> 32 30.8 / 29.3, 249235 x 13 -> 48 18.1 / 17.5, below 100000 rows the same; others mostly lose: 713300 x 24 -> 40 35.0 / 35.7,
+// 604093 x 55 -> 32 61.2 / 63.8, 265825 x 14 -> 104 22.0 / 22.2 (802816 x 48 -> 32 58.0 / 56.9).
+__host__ inline int res_stages(int K, int N) { return K <= 16 && N <= 64 ? 2 : kResStages; }
+
 template <bool kDebugAcc, bool kAsym>
 __global__ void __maxnreg__(kAsym ? 168 : 136)
 ptq_gemm_dequant_resident_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmW,
@@ -1259,11 +1265,11 @@ ptq_gemm_dequant_resident_kernel(const __grid_constant__ CUtensorMap tmA, const 
         if (threadIdx.x == 0) atomicOr(p.status, PTQ_DEV_SMEM_ALIGN);
         return;
     }
-    constexpr uint32_t nstages = kResStages;
+    const uint32_t nstages = static_cast<uint32_t>(p.stages);                     // at most kResStages: res_stages
     const uint32_t w_bytes = static_cast<uint32_t>(p.BN) * kBK;                   // one k-block of weights
     const uint32_t w_tile_bytes = static_cast<uint32_t>(p.k_blocks) * w_bytes;
     const uint32_t a_off = static_cast<uint32_t>(p.group) * w_tile_bytes;
-    const uint32_t staging_off = a_off + nstages * kATileBytes;
+    const uint32_t staging_off = a_off + kResStages * kATileBytes;
     const uint32_t scale_off = staging_off + 2 * kNumEpiWarps * kStreamStagingPerWarp;
     const uint32_t bar_off = scale_off + 2 * p.vectors * kScaleBufBytes;
     const uint32_t bar_base = base + bar_off;

@@ -31,6 +31,8 @@ def env():
     (40, 60000, 67, 3, False, False),      # two row tiles: a share crosses several N tiles
     (384, 58000, 64, 4, False, True),
     (256, 16, 7, 8121, False, False),      # a single 16-column step per tile
+    (16, 64, 37, 1800, True, False),       # two stages of codes: four tiles per CTA
+    (13, 8, 64, 900, False, True),
     # the weights of all N tiles at once, row panels as units: two and three N tiles (of a panel's odd number each team has the other half of
     # the tiles in the next panel), last tiles and panels that are not full, two k-blocks
     (96, 384, 784, 48, False, False),
