@@ -345,14 +345,6 @@ __host__ __device__ inline SearchPlan search_plan(int elements, int T, int C, in
     return {wide ? kSearchMany : kSearchFew, threads};
 }
 
-// max(a, |b|, |c|) in one instruction; NaN operands are dropped.
-__device__ __forceinline__ float search_max3_abs(float a, float b, float c)
-{
-    float r;
-    asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(fabsf(b)), "f"(fabsf(c)));
-    return r;
-}
-
 // Bound by issue: 49 M (element, candidate) pairs at 8 x 197 x 384 x 81, 9 instructions each.  The integer r = rne(u / Delta)
 // is taken from one FMA, t = RN(u * RN(1/Delta) + 1.5*2^23), whose low mantissa bits hold it; u * RN(1/Delta) is within
 // 1.2e-7 |v| of the defined quotient v, and beyond |v| = 128 every r clamps alike, so r can only be wrong where the distance
@@ -417,7 +409,7 @@ __global__ void __launch_bounds__(kSearchBlockMax, 2) ptq_search_loss_kernel(Sea
             }
             float worst = fabsf(d[0]);
 #pragma unroll
-            for (int c = 1; c < S; c += 2) worst = search_max3_abs(worst, d[c], d[c + 1]);
+            for (int c = 1; c < S; c += 2) worst = max3_abs(worst, d[c], d[c + 1]);
             if (!fast || worst > 0.49998f) {
 #pragma unroll
                 for (int c = 0; c < S; ++c) r[c] = rintf(__fdiv_rn(u, delta[c]));

@@ -104,15 +104,7 @@ __device__ __forceinline__ float dist_to_integer(float v)
     return fabsf(__fadd_rn(v, -r));
 }
 
-// max(a, |b|, |c|) in one instruction (three-input max of sm_100); NaN operands are dropped like fmaxf does.
-__device__ __forceinline__ float max3_abs(float a, float b, float c)
-{
-    float r;
-    asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(fabsf(b)), "f"(fabsf(c)));
-    return r;
-}
-
-// The same, but a NaN operand makes the result NaN (and keeps it NaN through a chain of these).
+// max3_abs, but a NaN operand makes the result NaN (and keeps it NaN through a chain of these).
 __device__ __forceinline__ float max3_abs_nan(float a, float b, float c)
 {
     float r;
