@@ -436,7 +436,7 @@ bool plan_panel(const ptq_linear *h, ptq::GemmParams &p, bool tma_store)
 // Whether the kernel with resident weights (and its epilogue in two teams) is taken: short main loop (K <= 384) and TMA stores.  Symmetric layers
 // from more than one tile for the busiest CTA: against the streaming kernel below three, 116 random layers with 1 to 14 tiles per CTA
 // (33 <= K <= 384), each replayed alone, take 0.957 of the time, 18321 x 298 -> 592 17.4 / 15.4 us, 50176 x 384 -> 192 17.4 / 16.8, 12608 x 192 -> 768 9.78 /
-// 9.43; slower by more than 1 %: 10047 x 64 -> 1176 9.73 / 9.90 and 17927 x 48 -> 96 6.41 / 6.50.  Among other layers less of it is left, because
+// 9.43; none is slower by more than 1 % (10047 x 64 -> 1176 10.0 / 9.9, 17927 x 48 -> 96 6.5 / 6.2).  Among other layers less of it is left, because
 // every further kernel in turn has to be fetched into the SMs again: in_proj and out_proj of Vim-Ti at batch 64 take 18.6 us with both
 // in one kernel and 19.1 with one in each.  So a layer of one tile per CTA that narrows by half, as the last of a block does, takes it where there
 // are rows enough that the block's wide first layer does (streaming / resident after 128 -> 512 on 99 row tiles 16.4 / 15.8, after 192 -> 768 on 74 17.6 / 17.2,
@@ -452,7 +452,7 @@ bool takes_resident(const ptq_linear *h, int m_tiles, int n_tiles)
 
 // N tiles per unit of the kernel with resident weights: all of them where their weights fit in shared memory and the busiest CTA gets no more
 // tiles, else one.  A row panel's codes are then loaded once, and its output is written as whole rows at a time.  Both kernels, us, one / all:
-// 200704 x 96 -> 384 43.8 / 38.6, 50176 x 128 -> 512 17.6 / 16.5, the same asymmetric 20.8 / 20.4, 50176 x 96 -> 384 14.2 / 13.7; with a tile more for the
+// 200704 x 96 -> 384 41.3 / 39.7, 50176 x 128 -> 512 17.7 / 17.3, the same asymmetric 20.9 / 20.9, 50176 x 96 -> 384 14.6 / 14.1; with a tile more for the
 // busiest CTA 100352 x 96 -> 384 (11 / 12 tiles) 22.1 / 22.6.  Some of them gain nothing: 50176 x 48 -> 1000 in pairs of four 36.9 / 36.7.
 int resident_group(const ptq_linear *h, const ptq::GemmParams &p)
 {
@@ -499,8 +499,8 @@ double gemm_cycles(const ptq_linear *h, const ptq::GemmParams &p, int bn)
     return cut ? 0.9 * busiest(cut) + 0.1 * busiest(bn) : busiest(bn);
 }
 
-// Tile width of the streaming kernel for this many rows: the layer's own (as few N tiles as possible), unless another
-// leaves the busiest CTA clearly less to do: idle SMs in a single round, or a last round that is nearly empty.  GEMM kernel alone,
+// Tile width for this many rows, in the streaming kernel and below three rounds in the one with resident weights: the layer's own (as few N
+// tiles as possible), unless another leaves the busiest CTA clearly less to do: idle SMs in a single round, or a last round that is nearly empty.  GEMM kernel alone,
 // us, own width -> the one chosen: 2793 x 1536 -> 768 (256 -> 128) 7.4 -> 5.3, 1568 x 1536 -> 768 (256 -> 128) 7.3 -> 4.9, 3152 x 768 -> 384 (192 -> 128)
 // 4.7 -> 3.8, 12544 x 768 -> 384 (192, cut -> 128) 6.6 -> 6.1, 11229 x 520 -> 600 (256 -> 128) 8.9 -> 8.6, 12608 x 192 -> 768 (256 -> 192) 6.6 -> 6.3.
 // The margin keeps what the model cannot tell apart: 25216 x 768 -> 384 (192 -> 128, predicted -1.6 %) 10.7 -> 10.9.  What it gets wrong: 6304 x 768 ->

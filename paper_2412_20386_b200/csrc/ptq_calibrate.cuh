@@ -323,7 +323,7 @@ __device__ __forceinline__ float search_candidate_step(float base, int j, int n_
 }
 
 // Candidates per block and threads of a launch.  A thread has nine candidates: 27 of them took 128 registers and spilled, 16 warps
-// per SM at 57 % of the issue slots.  A block's threads each form the candidates' steps and, at the end, reduce their sums: about
+// per SM at 53.5 % of the issue slots.  A block's threads each form the candidates' steps and, at the end, reduce their sums: about
 // as much work as 10 elements, so a block has as few threads as still fill the chip (256 threads where blocks are few, 64, or 32 in a
 // group, where they are many).  Three groups of threads in a block share the loading and dividing of the elements: taken with
 // three blocks per SM or more and at most an eighth of the candidates idle.  A whole call, us, one group of 64 / 128 / 256 threads, and three

@@ -99,9 +99,8 @@ struct GemmParams {
     // accumulator sum_k (c - z[t]) * Wq[n,k] exactly (all int32).  nullptr for symmetric layers.
     const int *zp;     // [T]
     const int *wsum;   // row sums of Wq, padded like dw
-    // Panel kernel (`group` and `groups` also the kernels with resident weights): a work unit is one 128-row panel of codes times `group` adjacent
-    // N tiles; `groups`
-    // units cover a panel; the weight ring has `b_stages` slots of `b_stage_bytes` (= BN * 128) each.
+    // Panel kernel and kernels with resident weights: a work unit is one 128-row panel of codes times `group` adjacent N tiles; `groups` units
+    // cover a panel.  The panel kernel's weight ring has `b_stages` slots of `b_stage_bytes` (= BN * 128) each.
     int group, groups;
     int b_stages, b_stage_bytes;
     FastDiv fd_T, fd_n_tiles, fd_groups;   // divisors T, n_tiles, groups
@@ -1212,10 +1211,10 @@ ptq_gemm_dequant_panel_kernel(const __grid_constant__ CUtensorMap tmA, const __g
 
 // --- weights resident ---------------------------------------------------------------------------
 //
-// Same computation for layers with a short main loop (K <= 384) and several tiles per CTA.  Such a layer is bound by its
+// Same computation for layers with a short main loop (K <= 384), mostly with several tiles per CTA.  Such a layer is bound by its
 // output: the SM moves 2 x BN bytes of y per row against K bytes of codes, and the loads share its TMA unit and the way to L2
 // with the stores.  The weights of one N tile (at most 96 KB) therefore stay in shared memory and only the codes stream:
-// 128 x K bytes per output tile instead of (128 + BN) x K, a third at BN = 256.  Whole forward, streamed weights -> resident:
+// 128 x K bytes per output tile instead of (128 + BN) x K, a third at BN = 256.  Whole forward, streamed weights -> resident, one N tile at a time:
 // 200704 x 96 -> 384: 43.2 -> 41.3 us; 200704 x 192 -> 384: 53.8 -> 52.2; 50176 x 192 -> 768: 24.2 -> 23.5; 25216 x 384 -> 1536:
 // 26.5 -> 26.1; 200704 x 64 -> 256: 33.5 -> 29-31.  The narrowest outputs gain nothing: 200704 x 192 -> 96: 32.8 -> 32.9.
 //
@@ -1223,12 +1222,15 @@ ptq_gemm_dequant_panel_kernel(const __grid_constant__ CUtensorMap tmA, const __g
 // its loads, 109 bytes per clock alone, take their time from the stores: fewer bytes in are more bytes out.
 //
 // Where the weights of ALL N tiles fit (K <= 128 mostly), the unit is a row panel with its N tiles in turn: the codes are loaded
-// once per panel and whole rows of y are written at a time (`group`; else 1).  200704 x 96 -> 384: 43.9 -> 36.2 us, 50176 x 128 -> 512 17.9 -> 16.8.
-// Part of that is the cursor, which steps without divisions: 25216 x 384 -> 1536 (group 1) 23.5 -> 23.2, 200704 x 192 -> 96 31.5 -> 31.0; what
-// loses is 200704 x 64 -> 256, 26.3 -> 26.6.
+// once per panel and whole rows of y are written at a time (`group`; else 1).  Whole forward on another box, one N tile at a time / all:
+// 200704 x 96 -> 384 41.3 / 39.7 us, 200704 x 192 -> 384 57.4 / 55.0, 50176 x 96 -> 384 14.6 / 14.1, 50176 x 128 -> 512 17.7 / 17.3.  What the cursor (no
+// divisions), the order of units, scales copied once per N tile and 128 registers give beside that, before them / with them, one N tile at a time:
+// 200704 x 96 -> 384 46.5 / 41.3, 200704 x 192 -> 384 60.9 / 57.4, 25216 x 384 -> 1536 25.9 / 26.2, 200704 x 192 -> 96 38.8 / 38.2; 200704 x 64 -> 256, as it
+// is now, loses 1 %, 28.3 / 28.5.
 //
-// Three stages of codes, which hold a whole panel (they must: see below): two cost 2 to 10 % (200704 x 384 -> 96: 65 us, not 58.5), and with eight the loads run so far ahead
-// of the stores that 200704 x 192 -> 96 takes 34.0 us, not 33.0; the other shapes cannot tell three from eight.
+// Three stages of codes, which hold a whole panel (they must: see below): two cost 2 to 10 % (200704 x 384 -> 96: 65 us, not 58.5) but where
+// a tile stores little (res_stages), and with eight the loads run so far ahead of the stores that 200704 x 192 -> 96 takes 34.0 us, not
+// 33.0; the other shapes cannot tell three from eight.
 //
 // 128 registers on symmetric layers (143 without the limit): the next kernel's quantizer CTAs find room beside it.  24 layers 12608 x 192 -> 768
 // in turn 237.8 -> 234.2 us; asymmetric ones would spill.
