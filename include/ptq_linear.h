@@ -220,8 +220,7 @@ int ptq_linear_code_pitch(const ptq_linear_t *h);
  *   0  ptq_gemm_dequant_kernel          operand stages streamed per tile, eight epilogue warps per tile
  *   1  ptq_gemm_dequant_resident_kernel the weights of an N tile resident in shared memory, the epilogue
  *                                       warps in two teams, one per accumulator (K <= 384 and more tiles
- *                                       than SMs, or half as many row tiles and 2 N <= K; asymmetric three tiles
- *                                       per SM)
+ *                                       than SMs; some with fewer and 2 N <= K; asymmetric three tiles per SM)
  *   2  ptq_gemm_dequant_panel_kernel    the codes of a row panel resident in shared memory for a group
  *                                       of N tiles (512 <= K <= 768, several N tiles, many tiles per SM)
  * Returns -1 for a NULL handle or B < 1.  All variants produce the same bits.

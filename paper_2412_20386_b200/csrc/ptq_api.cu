@@ -438,16 +438,23 @@ bool plan_panel(const ptq_linear *h, ptq::GemmParams &p, bool tma_store)
 // (33 <= K <= 384), each replayed alone, take 0.957 of the time, 18321 x 298 -> 592 17.4 / 15.4 us, 50176 x 384 -> 192 17.4 / 16.8, 12608 x 192 -> 768 9.78 /
 // 9.43; none is slower by more than 1 % (10047 x 64 -> 1176 10.0 / 9.9, 17927 x 48 -> 96 6.5 / 6.2).  Among other layers less of it is left, because
 // every further kernel in turn has to be fetched into the SMs again: in_proj and out_proj of Vim-Ti at batch 64 take 18.6 us with both
-// in one kernel and 19.1 with one in each.  So a layer of one tile per CTA that narrows by half, as the last of a block does, takes it where there
-// are rows enough that the block's wide first layer does (streaming / resident after 128 -> 512 on 99 row tiles 16.4 / 15.8, after 192 -> 768 on 74 17.6 / 17.2,
-// on 120 21.8 / 21.4; on 60 and fewer the same).  Others do not: they lose, 206 -> 208 and 75 -> 33 on 140 row tiles 19.8 / 21.1,
-// 128 -> 512 and 256 -> 128 on 74 13.1 / 13.4, 91 -> 179 among 463 -> 199 and two narrow ones on 96 37.2 / 37.9; beside K > 384 narrowing ones
-// lose too, up to 3 % (298 -> 112 before 596 -> 190 on 80 23.0 / 23.7), which a layer cannot know.  Asymmetric layers from three tiles: 6304 x 384 -> 1536 alone 12.2 / 11.9, but with 6304 x 768 -> 384
+// in one kernel and 19.1 with one in each.  So a layer of one tile per CTA that narrows by half, as the last of a block does, takes it where
+// the block's first one, on the same rows and four times as wide as this one, makes more tiles than SMs, with half as many row tiles as SMs or more
+// (below that no difference).  Both streaming / both resident / so, us: 128 -> 512 and 256 -> 128 on 92 row tiles, twice, 32.5 / 31.3 / 31.5, 112 -> 448 and
+// 224 -> 112 on 148 37.8 / 36.8 / 34.8; where the first one is a tile per CTA too, 64 -> 256 and 128 -> 64 on 130, 26.4 / 26.4 / 26.4, 27.2 with one in
+// each.  Up to 48 columns it is taken below two thirds of the SMs, where that costs nothing (48 -> 192 and 96 -> 48 on 76 24.6 / 24.0, with one
+// in each 24.8; on 148 26.4 / 27.0 / 27.3).  Others do not take it, they lose, 206 -> 208 and 75 -> 33 on 140 row tiles 19.8 / 21.1, 91 -> 179 among
+// 463 -> 199 and two narrow ones on 96 37.2 / 37.9; beside K > 384 narrowing ones lose too, up to 3 % (298 -> 112 before 596 -> 190 on 80
+// 23.0 / 23.7), which a layer cannot know.  Asymmetric layers from three tiles: 6304 x 384 -> 1536 alone 12.2 / 11.9, but with 6304 x 768 -> 384
 // behind it 24.4 / 24.55.
 bool takes_resident(const ptq_linear *h, int m_tiles, int n_tiles)
 {
-    const long long tiles = static_cast<long long>(m_tiles) * n_tiles;
-    return h->k_blocks <= kShortMainLoop && (h->asym ? tiles >= 3ll * h->num_sms : tiles > h->num_sms || (2ll * m_tiles >= h->num_sms && 2 * h->N <= h->K));
+    if (h->k_blocks > kShortMainLoop) return false;
+    const long long sms = h->num_sms, rows = m_tiles, tiles = rows * n_tiles;
+    if (h->asym) return tiles >= 3 * sms;
+    if (tiles > sms) return true;
+    const long long first_tiles = rows * ((4ll * h->N + ptq::kMaxBN - 1) / ptq::kMaxBN);
+    return 2ll * h->N <= h->K && 2 * rows >= sms && (first_tiles > sms || (h->N <= 48 && 3 * rows < 2 * sms));
 }
 
 // N tiles per unit of the kernel with resident weights: all of them where their weights fit in shared memory and the busiest CTA gets no more

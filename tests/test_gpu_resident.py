@@ -79,7 +79,9 @@ def test_resident_weights(env, K, N, T, B, bias, asym):
 
 
 @pytest.mark.parametrize("K,N,rows,variant", [
-    (384, 192, 74, 1), (384, 192, 73, 0), (384, 200, 99, 0), (206, 208, 140, 0), (128, 64, 148, 1),    # one tile per CTA: layers that narrow by half
+    (384, 192, 74, 1), (384, 192, 73, 0), (384, 200, 99, 0), (206, 208, 140, 0),      # one tile per CTA: layers that narrow by half, behind
+    (256, 128, 75, 1), (256, 128, 74, 0), (128, 64, 148, 0),                          # a four times wider one with more tiles than SMs,
+    (96, 48, 98, 1), (96, 48, 99, 0),                                                 # or up to 48 columns on less than two thirds of the SMs
     (128, 512, 74, 0), (128, 512, 75, 1),                                                              # 148 and 150 tiles
 ])
 def test_which_short_layers_keep_their_weights(env, K, N, rows, variant):
